@@ -335,8 +335,10 @@ struct ecris_ctx {
     unsigned long long* d_cstat = nullptr;   // scan tile status words and ticket counter
     unsigned long long* d_ckeys = nullptr;
     int collide_grid = 0;
-    // two sets of particle arrays; the sort moves the particles from the
-    // current set (index cur) to the other
+    // two sets of particle arrays, each the eight arrays of one allocation
+    // (d_set: 8 cap words, so that a set not in use also serves as cap 32-byte
+    // records); the sort moves the particles from the current set to the other
+    uint32_t* d_set[2] = {nullptr, nullptr};
     float* d_soa[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     uint32_t* d_meta = nullptr;
     uint32_t* d_id = nullptr;
@@ -446,12 +448,7 @@ void free_graphs(ecris_ctx* ctx)
 void free_ions(ecris_ctx* ctx)
 {
     free_graphs(ctx);
-    for (auto& p : ctx->d_soa) free_async(ctx, p);
-    free_async(ctx, ctx->d_meta);
-    free_async(ctx, ctx->d_id);
-    for (auto& p : ctx->d_soa2) free_async(ctx, p);
-    free_async(ctx, ctx->d_meta2);
-    free_async(ctx, ctx->d_id2);
+    for (auto& p : ctx->d_set) free_async(ctx, p);
     free_async(ctx, ctx->d_hist);
     free_async(ctx, ctx->d_hoff);
     free_async(ctx, ctx->d_hblk);
@@ -931,15 +928,19 @@ ecris_status sort_particles(ecris_ctx* ctx)
     dst.meta = ctx->d_meta2;
     dst.id = ctx->d_id2;
     // the first sort after a load sees the load order: it moves 32-byte
-    // records through a scratch buffer taken from the stream's pool for it
+    // records into the other set's memory and unpacks them back into the
+    // current set, which stays current
     const size_t cap4 = 4 * ctx->n4;
-    uint4* aos = nullptr;
-    if (ctx->fresh) CK(cudaMallocAsync((void**)&aos, 2 * cap4 * sizeof(uint4), ctx->stream));
+    uint4* aos = ctx->fresh ? reinterpret_cast<uint4*>(dst.x) : nullptr;
     CK(timed(ctx, kKindOther, [&] {
         return launch_sort(*ctx->h_run, (uint32_t)cap4, dst, ctx->d_hist, ctx->d_hoff, ctx->d_hblk, aos,
                            ctx->stream);
     }, aos ? 7 : 6));
-    if (aos) CK(cudaFreeAsync(aos, ctx->stream));
+    ctx->since_sort = 0;
+    if (ctx->fresh) {
+        ctx->fresh = false;
+        return ECRIS_OK;
+    }
     for (int k = 0; k < 6; ++k) std::swap(ctx->d_soa[k], ctx->d_soa2[k]);
     std::swap(ctx->d_meta, ctx->d_meta2);
     std::swap(ctx->d_id, ctx->d_id2);
@@ -952,8 +953,6 @@ ecris_status sort_particles(ecris_ctx* ctx)
     R.vz = ctx->d_soa[5];
     R.meta = ctx->d_meta;
     R.id = ctx->d_id;
-    ctx->since_sort = 0;
-    ctx->fresh = false;
     ctx->parity ^= 1;
     return ECRIS_OK;
 }
@@ -1218,19 +1217,18 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
     }
     CK(cudaSetDevice(ctx->device));
     const size_t n4 = (n + 3) / 4;
-    const size_t cap = n4 > 0 ? 4 * n4 : 4;
+    const size_t cap = n4 > 0 ? (4 * n4 + 31) / 32 * 32 : 32;   // arrays of a set start at 128-byte boundaries
     const size_t nc = (size_t)h.nx * h.ny * h.nz;
     // device buffers are kept across loads while they are large enough
     if (!ctx->have_ions || cap > ctx->cap || nc != ctx->cap_cells) {
         free_ions(ctx);
-        for (int k = 0; k < 6; ++k)
-            CK(cudaMallocAsync((void**)&ctx->d_soa[k], cap * sizeof(float), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_meta, cap * sizeof(uint32_t), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_id, cap * sizeof(uint32_t), ctx->stream));
-        for (int k = 0; k < 6; ++k)
-            CK(cudaMallocAsync((void**)&ctx->d_soa2[k], cap * sizeof(float), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_meta2, cap * sizeof(uint32_t), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_id2, cap * sizeof(uint32_t), ctx->stream));
+        for (int set = 0; set < 2; ++set) {
+            CK(cudaMallocAsync((void**)&ctx->d_set[set], 8 * cap * sizeof(uint32_t), ctx->stream));
+            for (int k = 0; k < 6; ++k)
+                (set ? ctx->d_soa2 : ctx->d_soa)[k] = reinterpret_cast<float*>(ctx->d_set[set] + k * cap);
+            (set ? ctx->d_meta2 : ctx->d_meta) = ctx->d_set[set] + 6 * cap;
+            (set ? ctx->d_id2 : ctx->d_id) = ctx->d_set[set] + 7 * cap;
+        }
         CK(cudaMallocAsync((void**)&ctx->d_hist, (2 * nc + 1) * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_hoff, (2 * nc + 2) * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_hblk, (size_t)sort_scan_blocks((uint32_t)(2 * nc + 1)) * sizeof(uint32_t),
@@ -1557,12 +1555,12 @@ ecris_status ecris_get_state(ecris_ctx* ctx, float* const xyzv[6], uint32_t* met
         // by their ids (into the caller's device arrays, or via the spare set)
         if (dst_is_device) {
             CK(launch_export_ordered(*ctx->h_run, (uint32_t)n, (uint32_t)(4 * ctx->n4), xyzv, meta, sxy, sz,
-                                     ctx->stream));
+                                     reinterpret_cast<uint4*>(ctx->d_soa2[0]), ctx->stream));
         } else {
             float* spare[6];
             for (int k = 0; k < 6; ++k) spare[k] = (xyzv && xyzv[k]) ? ctx->d_soa2[k] : nullptr;
             CK(launch_export_ordered(*ctx->h_run, (uint32_t)n, (uint32_t)(4 * ctx->n4), spare,
-                                     meta ? ctx->d_meta2 : nullptr, sxy, sz, ctx->stream));
+                                     meta ? ctx->d_meta2 : nullptr, sxy, sz, nullptr, ctx->stream));
             for (int k = 0; k < 6; ++k)
                 if (spare[k])
                     CK(cudaMemcpyAsync(xyzv[k], spare[k], n * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));

@@ -436,16 +436,18 @@ struct ParticleSet {
 // Counting sort of the run's particles (in R) by (ion/atom, cell) into `dst`:
 // live ions first, then live atoms, each by cell; frozen and padding slots
 // last.  hist (2 Nc + 1 words) must be zero and is left zero; off (2 Nc + 2)
-// and blk (scan block totals) are scratch.  aos (2 cap uint4 of scratch, or
-// NULL): move through 32-byte records, for input in arbitrary order (the
-// first sort after a load); NULL writes the destination arrays directly.
+// and blk (scan block totals) are scratch.  aos (the memory of `dst` as cap
+// 32-byte records, or NULL): for input in arbitrary order (the first sort
+// after a load), move records there and unpack them back into the arrays of
+// R, which then hold the sorted particles; NULL writes `dst` directly.
 cudaError_t launch_sort(const RunDev& R, uint32_t cap, const ParticleSet& dst, uint32_t* hist, uint32_t* off,
                         uint32_t* blk, uint4* aos, cudaStream_t s);
 int sort_scan_blocks(uint32_t nbins);
 // state in load order: out[id[slot]] = state[slot] for id < n (positions to
-// metres), into device arrays
+// metres), into device arrays; rec: scratch of n 32-byte records (not `out`),
+// or NULL
 cudaError_t launch_export_ordered(const RunDev& R, uint32_t n, uint32_t cap, float* const out[6], uint32_t* meta_out,
-                                  double sxy, double sz, cudaStream_t s);
+                                  double sxy, double sz, uint4* rec, cudaStream_t s);
 cudaError_t launch_census(const RunDev& R, uint32_t n4, unsigned long long* census, cudaStream_t s);
 // add the current particles to the probes' sums (probe.cu)
 cudaError_t launch_probe(const RunDev& R, const ProbeDev& P, uint32_t n4, int sm_count, cudaStream_t s);
