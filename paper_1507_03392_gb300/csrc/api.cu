@@ -867,8 +867,8 @@ ecris_status get_cells(ecris_ctx* ctx, float* ne, float* delta_x, float* delta_y
     return ECRIS_OK;
 }
 
-// the kernel sequence of one step, captured once per particle set and
-// parameter block and replayed as a CUDA graph
+// the kernel sequence of one step with collisions between ions, captured once
+// per particle set and parameter block and replayed as a CUDA graph
 ecris_status step_graph(ecris_ctx* ctx, int kind, cudaGraphExec_t* out)
 {
     const int p = ctx->parity;
@@ -886,7 +886,6 @@ ecris_status step_graph(ecris_ctx* ctx, int kind, cudaGraphExec_t* out)
         cudaGraphExecDestroy(ctx->gexec[p][kind]);
         ctx->gexec[p][kind] = nullptr;
     }
-    const bool coulomb = (ctx->h.mcc.flags & kFCoulomb) != 0;
     const uint32_t nc = (uint32_t)((size_t)ctx->h.nx * ctx->h.ny * ctx->h.nz);
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
@@ -894,11 +893,8 @@ ecris_status step_graph(ecris_ctx* ctx, int kind, cudaGraphExec_t* out)
     // kind 0, the whole step; kind 1, the collision kernels alone (timed
     // steps launch the step kernel on its own before them).  With collisions
     // the scan kernel also runs the leaver pass.
-    if (kind == 0) {
-        e = launch_step(*ctx->h_run, ctx->ntiles, ctx->step_grid, ctx->stream);
-        if (e == cudaSuccess && !coulomb) e = launch_leave(*ctx->h_run, ctx->d_ticket, 1, ctx->stream);
-    }
-    if (e == cudaSuccess && coulomb)
+    if (kind == 0) e = launch_step(*ctx->h_run, ctx->ntiles, ctx->step_grid, ctx->stream);
+    if (e == cudaSuccess)
         e = launch_coulomb(*ctx->h_run, nc, ctx->ntiles, ctx->d_ticket, ctx->collide_grid, (uint32_t)kLeaveBlocks,
                            1, ctx->stream);
     const cudaError_t e2 = cudaStreamEndCapture(ctx->stream, &g);
@@ -912,6 +908,18 @@ ecris_status step_graph(ecris_ctx* ctx, int kind, cudaGraphExec_t* out)
     ctx->gkey[p][kind] = key;
     *out = x;
     return ECRIS_OK;
+}
+
+// Steps of the next window of a run without collisions between ions: at most
+// `left`, and no further than the next sort and the next deposit fold.  Timed
+// steps go one by one.
+uint32_t window_steps(const ecris_ctx* ctx, uint32_t left, bool one_by_one)
+{
+    if (one_by_one) return 1;
+    uint32_t K = std::min(left, kMaxWindow);
+    K = std::min(K, ctx->fold_every - std::min(ctx->since_fold, ctx->fold_every - 1));
+    if (ctx->n4 > 0) K = std::min(K, ctx->sort_every - std::min(ctx->since_sort, ctx->sort_every - 1));
+    return K;
 }
 
 // Regroup the particles by (ion/atom, cell) into the other set of arrays and
@@ -1246,7 +1254,7 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
         CK(cudaMallocAsync((void**)&ctx->d_leave, cap * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_birth, cap * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_fptd, kFptdWords * sizeof(unsigned long long), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_nleave, sizeof(uint32_t), ctx->stream));
+        CK(cudaMallocAsync((void**)&ctx->d_nleave, 2 * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_ticket, sizeof(unsigned int), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_bad, 2 * sizeof(unsigned int), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_err, sizeof(uint32_t), ctx->stream));
@@ -1300,7 +1308,7 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
         if (pst != ECRIS_OK) return pst;
     }
     CK(cudaMemsetAsync(ctx->d_step, 0, sizeof(uint32_t), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_nleave, 0, sizeof(uint32_t), ctx->stream));
+    CK(cudaMemsetAsync(ctx->d_nleave, 0, 2 * sizeof(uint32_t), ctx->stream));
     CK(cudaMemsetAsync(ctx->d_ticket, 0, sizeof(unsigned int), ctx->stream));
     CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(uint32_t), ctx->stream));
     CK(cudaMemsetAsync(ctx->d_bad, 0, sizeof(unsigned int), ctx->stream));
@@ -1372,14 +1380,20 @@ ecris_status ecris_step(ecris_ctx* ctx, uint32_t nsteps, double dt)
     if (st != ECRIS_OK) return st;
     const bool coulomb = (ctx->h.mcc.flags & kFCoulomb) != 0;
     const uint32_t nc = (uint32_t)((size_t)ctx->h.nx * ctx->h.ny * ctx->h.nz);
-    for (uint32_t s = 0; s < nsteps; ++s) {
+    for (uint32_t s = 0; s < nsteps;) {
         const bool due = ctx->since_sort >= ctx->sort_every ||
                          (ctx->fresh && s == 0 && (nsteps >= kSortAfterLoad || ctx->calls_since_load > 0));
         if (due && ctx->n4 > 0) {
             st = sort_particles(ctx);
             if (st != ECRIS_OK) return st;
         }
-        if (!ctx->timer.on) {
+        uint32_t K = 1;   // steps taken together
+        if (!coulomb) {
+            K = window_steps(ctx, nsteps - s, ctx->timer.on);
+            CK(timed(ctx, kKindStep, [&] {
+                return launch_window(*ctx->h_run, K, ctx->d_ticket, ctx->sm_count, ctx->stream);
+            }));
+        } else if (!ctx->timer.on) {
             // the whole step as one graph launch
             cudaGraphExec_t x = nullptr;
             st = step_graph(ctx, 0, &x);
@@ -1390,22 +1404,20 @@ ecris_status ecris_step(ecris_ctx* ctx, uint32_t nsteps, double dt)
             CK(timed(ctx, kKindStep, [&] {
                 return launch_step(*ctx->h_run, ctx->ntiles, ctx->step_grid, ctx->stream);
             }));
-            if (!coulomb)
-                CK(timed(ctx, kKindOther, [&] { return launch_leave(*ctx->h_run, ctx->d_ticket, 1, ctx->stream); }));
-            if (coulomb) {
-                cudaGraphExec_t x = nullptr;
-                st = step_graph(ctx, 1, &x);
-                if (st != ECRIS_OK) return st;
-                CK(timed(ctx, kKindCoulomb, [&] { return cudaGraphLaunch(x, ctx->stream); }, kCoulombKernels));
-            }
+            cudaGraphExec_t x = nullptr;
+            st = step_graph(ctx, 1, &x);
+            if (st != ECRIS_OK) return st;
+            CK(timed(ctx, kKindCoulomb, [&] { return cudaGraphLaunch(x, ctx->stream); }, kCoulombKernels));
         }
-        if (++ctx->since_fold >= ctx->fold_every) {
+        ctx->since_fold += K;
+        if (ctx->since_fold >= ctx->fold_every) {
             CK(timed(ctx, kKindOther, [&] {
                 return launch_fold(*ctx->h_run, nc, ctx->d_count, ctx->d_charge, ctx->stream);
             }));
             ctx->since_fold = 0;
         }
-        ++ctx->since_sort;
+        ctx->since_sort += K;
+        s += K;
     }
     ctx->steps_done += nsteps;
     ++ctx->calls_since_load;
@@ -1616,6 +1628,7 @@ struct ecris_batch {
     int blocks_per_sm = 0;          // 0: as many as fit
     int shape = kDefaultShape;      // launch shape of the batched step kernel
     int max_bps[kStepShapes] = {};  // resident blocks per SM of each shape
+    int window_bps[kStepShapes] = {};   // and of the window kernels
     uint32_t sort_every = 32;
     size_t budget = 0, used = 0;
     std::string err;
@@ -1626,6 +1639,8 @@ struct ecris_batch {
     RunDev* h_runs = nullptr;       // pinned staging of the same
     cudaEvent_t staged = nullptr;   // the last upload from h_runs has finished
     size_t runs_cap = 0;
+    uint32_t* d_pref = nullptr;     // scratch of a window's active pass (runs_cap + 1)
+    bool any_coulomb = false;       // some run has collisions between ions: the batch steps one by one
     uint2* d_items = nullptr;       // work list (handle, tile)
     size_t items_cap = 0;
     uint32_t nitems = 0;
@@ -1722,6 +1737,8 @@ ecris_status batch_upload(ecris_batch* b)
         if (b->h_runs) b->old_host.push_back(b->h_runs);
         b->runs_cap = nr + 16;
         BCK(cudaMallocAsync((void**)&b->d_runs, b->runs_cap * sizeof(RunDev), b->stream));
+        if (b->d_pref) cudaFreeAsync(b->d_pref, b->stream);
+        BCK(cudaMallocAsync((void**)&b->d_pref, (b->runs_cap + 1) * sizeof(uint32_t), b->stream));
         BCK(cudaMallocHost((void**)&b->h_runs, b->runs_cap * sizeof(RunDev)));
         b->graph_dirty = true;
     } else {
@@ -1773,19 +1790,23 @@ ecris_status batch_items(ecris_batch* b)
         BCK(cudaEventRecord(b->items_staged, b->stream));
     }
     b->nitems = (uint32_t)items.size();
-    b->variants = false;
-    for (auto* c : b->runs)
+    b->variants = b->any_coulomb = false;
+    for (auto* c : b->runs) {
         if (c && ((c->h.mcc.flags & kFVariants) || !c->h.ax_y.empty())) b->variants = true;
+        if (c && (c->h.mcc.flags & kFCoulomb)) b->any_coulomb = true;
+    }
     b->layout_dirty = false;
     b->graph_dirty = true;
     return ECRIS_OK;
 }
 
-// one step of every run: the batched step kernel, the collision kernels of
-// the runs that have them, and the step counters of the others
+// resident blocks per SM of the batch's step kernels: the most that fit, and
+// as many as the tuning asks for
+int batch_most_bps(const ecris_batch* b) { return (b->any_coulomb ? b->max_bps : b->window_bps)[b->shape]; }
+
 int batch_bps(const ecris_batch* b)
 {
-    const int m = b->max_bps[b->shape];
+    const int m = batch_most_bps(b);
     return b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, m) : m;
 }
 
@@ -1915,7 +1936,10 @@ ecris_status ecris_batch_create(ecris_batch** out, int device, void* cuda_stream
         delete b;
         return ECRIS_ECUDA;
     }
-    for (int k = 0; k < kStepShapes; ++k) b->max_bps[k] = step_batch_blocks_per_sm(k);
+    for (int k = 0; k < kStepShapes; ++k) {
+        b->max_bps[k] = step_batch_blocks_per_sm(k);
+        b->window_bps[k] = window_blocks_per_sm(kShapeThreads[k]);
+    }
     *out = b;
     return ECRIS_OK;
 }
@@ -1929,6 +1953,7 @@ void ecris_batch_destroy(ecris_batch* b)
         if (c) ecris_destroy(c);
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     if (b->d_runs) cudaFreeAsync(b->d_runs, b->stream);
+    if (b->d_pref) cudaFreeAsync(b->d_pref, b->stream);
     if (b->d_items) cudaFreeAsync(b->d_items, b->stream);
     if (b->d_ticket) cudaFreeAsync(b->d_ticket, b->stream);
     cudaStreamSynchronize(b->stream);
@@ -2039,7 +2064,7 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
         ecris_status st = batch_items(b);
         if (st != ECRIS_OK) return st;
     }
-    for (uint32_t s = 0; s < nsteps; ++s) {
+    for (uint32_t s = 0; s < nsteps;) {
         // regroup the particles of the runs that are due; their parameter
         // blocks change (the arrays swap), and so does the captured graph
         // when a run's collision kernels take the block by value
@@ -2078,7 +2103,18 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
             ecris_status st = batch_upload(b);
             if (st != ECRIS_OK) return st;
         }
-        if (!b->timer.on) {
+        uint32_t K = 1;   // steps taken together
+        if (!b->any_coulomb) {
+            K = nsteps - s;
+            for (auto* c : b->runs)
+                if (c) K = std::min(K, window_steps(c, K, b->timer.on));
+            const int threads = kShapeThreads[b->shape];
+            BCK(b->timer.run(kKindStep, b->stream, [&] {
+                return launch_window_batch(b->d_runs, (uint32_t)b->runs.size(), b->d_items, b->nitems,
+                                           shape_tile(b->shape), threads, b->sm_count * batch_bps(b), b->variants, K,
+                                           b->d_pref, b->d_ticket, b->stream);
+            }));
+        } else if (!b->timer.on) {
             ecris_status st = batch_graph(b);
             if (st != ECRIS_OK) return st;
             BCK(cudaGraphLaunch(b->gexec, b->stream));
@@ -2102,10 +2138,11 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
         for (size_t r = 0; r < b->runs.size(); ++r) {
             ecris_ctx* c = b->runs[r];
             if (!c) continue;
-            c->steps_done += 1;
-            c->time_s += b->dt[r];
-            ++c->since_sort;
-            if (++c->since_fold >= c->fold_every) {
+            c->steps_done += K;
+            for (uint32_t k = 0; k < K; ++k) c->time_s += b->dt[r];
+            c->since_sort += K;
+            c->since_fold += K;
+            if (c->since_fold >= c->fold_every) {
                 const uint32_t nc = (uint32_t)((size_t)c->h.nx * c->h.ny * c->h.nz);
                 BCK(b->timer.run(kKindOther, b->stream, [&] {
                     return launch_fold(*c->h_run, nc, c->d_count, c->d_charge, b->stream);
@@ -2113,6 +2150,7 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
                 c->since_fold = 0;
             }
         }
+        s += K;
     }
     return ECRIS_OK;
 }
@@ -2439,7 +2477,8 @@ ecris_status batch_autotune(ecris_batch* b, uint32_t trial_steps, bool cadence, 
     }
     // 2. resident blocks per SM of that shape
     best = 1e30f;
-    for (int bps = 1; bps <= b->max_bps[best_shape] && st == ECRIS_OK; ++bps) {
+    if (st == ECRIS_OK) apply(best_shape, 0, orig_sort);
+    for (int bps = 1; bps <= batch_most_bps(b) && st == ECRIS_OK; ++bps) {
         apply(best_shape, bps, orig_sort);
         st = time_steps(b, trial_steps, true, &ms);
         if (st == ECRIS_OK && ms < best) {

@@ -168,7 +168,8 @@ struct alignas(16) RunDev {
     float nanbu_lnlo, nanbu_inv_dln;
     uint32_t *step;              // device step counter of the run
     uint32_t *leave;             // slots of the particles that left the chamber this step
-    uint32_t *nleave;            // their number (zero between steps)
+    uint32_t *nleave;            // their number (zero between steps); in a window of steps two counts:
+                                 // ions listed from the front of `leave`, atoms listed from its back
     uint32_t *err;               // device error word: 0, or ECRIS_ETIMEOUT after a bounded wait ran out
     uint32_t *birth;             // by particle id: step of the last ionisation from Q = 0 (~0: unknown)
     unsigned long long *fptd;    // [Q][kFptdBins] extraction counts by age bin, [Q] summed ages (steps),
@@ -390,13 +391,25 @@ struct ProbeDev {
 // one pass of the fused step kernel over the run's ntiles tiles of kTile
 // particles; the particles that left the chamber are listed in R.leave
 cudaError_t launch_step(const RunDev& R, uint32_t ntiles, int grid, cudaStream_t s);
-// the leaver pass after it: crossing, tallies, re-emission and deposit of the
-// listed particles; the list is cleared; bump_step: advance the step counter
-// (ticket: a zeroed device word, left zero)
+// the leaver pass of a batch after it: crossing, tallies, re-emission and
+// deposit of the listed particles of every run; the lists are cleared (ticket:
+// a zeroed device word, left zero).  A run alone has it in the collisions'
+// scan kernel (launch_coulomb).
 constexpr int kLeaveBlocks = 64;
-cudaError_t launch_leave(const RunDev& R, unsigned int* ticket, int bump_step, cudaStream_t s);
-// the same for every run of a batch (step counters untouched)
 cudaError_t launch_leave_batch(const RunDev* runs, uint32_t nruns, unsigned int* ticket, cudaStream_t s);
+// Up to kMaxWindow steps of a run without collisions between ions in two
+// launches (k_quiet, k_active): the atoms that neither leave nor ionise in the
+// window, then every other particle; the step counter advances by K.  R.leave
+// and R.nleave hold the list in between (ticket: a zeroed device word).
+constexpr uint32_t kMaxWindow = 32;
+constexpr uint32_t kActiveTile = 128;   // listed particles a block takes at a time
+cudaError_t launch_window(const RunDev& R, uint32_t K, unsigned int* ticket, int sm_count, cudaStream_t s);
+// the same for every run of a batch: items are the (run, tile) work list of
+// `tile` particles a tile, pref nruns + 1 words of scratch, grid the blocks
+int window_blocks_per_sm(int threads);
+cudaError_t launch_window_batch(const RunDev* runs, uint32_t nruns, const uint2* items, uint32_t nitems, uint32_t tile,
+                                int threads, int grid, bool variants, uint32_t K, uint32_t* pref,
+                                unsigned int* ticket, cudaStream_t s);
 cudaError_t launch_fold(const RunDev& R, uint32_t ncells, unsigned long long* count,
                         unsigned long long* charge, cudaStream_t s);
 // words of the rate table after its 8 kQSlots rates and shares: the atom gate and the

@@ -15,6 +15,9 @@
 // is only listed by the step kernel; a second, small pass does its crossing
 // geometry (FP64), tallies and re-emission, so the step kernel carries no
 // FP64 code and no per-tile tally traffic.
+//
+// Runs without collisions between ions take their steps in windows instead
+// (k_quiet, k_active below).
 #include "ecris_internal.cuh"
 
 namespace ecris {
@@ -856,21 +859,6 @@ __device__ __forceinline__ bool last_block(unsigned int* ticket)
     return last != 0;
 }
 
-// one run; the last block clears the list and, with bump_step, advances the
-// run's step counter (runs with Coulomb collisions advance it in the
-// collision kernels)
-__global__ void __launch_bounds__(256) k_leave(const __grid_constant__ RunDev R, unsigned int* ticket, int bump_step)
-{
-    pdl_wait();
-    pdl_trigger();
-    const uint32_t n = *R.nleave;
-    leave_run(R, n, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
-    if (last_block(ticket) && threadIdx.x == 0) {
-        *R.nleave = 0u;
-        if (bump_step) *R.step += 1u;
-    }
-}
-
 // every run of a batch: block b takes runs b, b + grid, ...; the last block
 // clears the lists and advances the step counter of every run without
 // Coulomb collisions (nothing reads those counters again in this step; the
@@ -889,6 +877,428 @@ __global__ void __launch_bounds__(256) k_leave_batch(const RunDev* __restrict__ 
             if (runs[r].step) {
                 *runs[r].nleave = 0u;
                 if (!(runs[r].flags & kFCoulomb)) *runs[r].step += 1u;
+            }
+}
+
+// ---------------------------------------------------------------------------
+// Windows of steps.  Without collisions between ions no particle's step
+// depends on another's, so a call's steps run in windows of up to kMaxWindow:
+// each particle's state is read once, stepped through the window in registers
+// and written once.
+//
+// k_quiet takes the atoms.  An atom moves on a straight line by the same whole
+// number of grid units every step, so its place after the window is one
+// multiply away; it stays in the chamber throughout if it does at the window's
+// end (the chamber is convex, and the box and r <= R0 tests are exact in the
+// integers).  What is left of its steps is the ionisation word: one Philox
+// block a step, of which the first two rounds hardly depend on both the
+// particle and the step (see quiet_rng), compared with the atom gate.  An atom
+// that neither leaves nor ionises in the window is done: moved, its deposits
+// added, its events cleared.  All other particles (ions, and atoms with an
+// event to come) are listed by slot.
+//
+// k_active takes the listed particles through step_particle and, for those
+// that leave the chamber, leave_particle, step by step.  Ions are listed from
+// the front of the list and atoms from its back, so that a warp has one kind.
+//
+// Against a step kernel and a leaver pass a step, which read and wrote every
+// particle each time and were bound by instruction issue: 32 steps of the 32
+// oxygen runs of a gas-flow scan (2.6e7 particles, dt 1 ns) took 11.8 ms and
+// take 5.2 (k_quiet 1.7, k_active 3.4); 1000 steps of 1e4 particles, bound by
+// the latency of two launches a step, 9.1 ms and 2.2.
+// ---------------------------------------------------------------------------
+
+// The part of an atom's Philox blocks in a window that does not depend on the
+// step, and a step's part that does not depend on the particle.  With the
+// counter (pid, 0, c, 0), c = 4 step, the first round leaves (hi(M1 c) ^ k0,
+// lo(M1 c), hi(M0 pid) ^ k1, lo(M0 pid)): two words of the step and two of
+// the particle.  The second multiplies word 0 (the step's) and word 2 (the
+// particle's), so its products need no particle-and-step multiply either.
+struct QuietAtom { uint32_t p0, p1, p2; };
+
+__device__ __forceinline__ QuietAtom quiet_atom(const RunDev& R, uint32_t pid)
+{
+    const uint32_t a = __umulhi(0xD2511F53u, pid) ^ R.seed_hi, b = 0xD2511F53u * pid;
+    return QuietAtom{__umulhi(0xCD9E8D57u, a), 0xCD9E8D57u * a, b};
+}
+
+// a step's words after two rounds: to be xored into words 0 and 2, and word 3
+__device__ __forceinline__ uint4 quiet_step(const RunDev& R, uint32_t step)
+{
+    const uint32_t c = 4u * step;
+    const uint32_t u0 = __umulhi(0xCD9E8D57u, c) ^ R.seed_lo, lo1 = 0xCD9E8D57u * c;
+    return make_uint4(lo1 ^ (R.seed_lo + 0x9E3779B9u), __umulhi(0xD2511F53u, u0) ^ (R.seed_hi + 0xBB67AE85u),
+                      0xD2511F53u * u0, 0u);
+}
+
+// word 0 of the block: rounds 3 to 10
+__device__ __forceinline__ uint32_t quiet_word0(const RunDev& R, const QuietAtom& a, const uint4& st)
+{
+    uint32_t c0 = a.p0 ^ st.x, c1 = a.p1, c2 = a.p2 ^ st.y, c3 = st.z;
+    uint32_t k0 = R.seed_lo + 2u * 0x9E3779B9u, k1 = R.seed_hi + 2u * 0xBB67AE85u;
+#pragma unroll
+    for (int r = 2; r < 10; ++r) {
+        const unsigned long long p0 = (unsigned long long)0xD2511F53u * c0;
+        const unsigned long long p1 = (unsigned long long)0xCD9E8D57u * c2;
+        const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ k0;
+        const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ k1;
+        c0 = n0; c1 = (uint32_t)p1; c2 = n2; c3 = (uint32_t)p0;
+        k0 += 0x9E3779B9u;
+        k1 += 0xBB67AE85u;
+    }
+    return c0;
+}
+
+constexpr int kQuietMaxTile = 2048;   // particles a block takes at a time (threads x particles per thread)
+
+struct QuietShared {
+    uint4 rng[kMaxWindow];            // quiet_step of the window's steps
+    uint32_t list[kQuietMaxTile];     // the tile's listed slots: ions from the front, atoms from the back
+    uint32_t cnt[2], base[2];
+};
+
+// Does the atom (at X, Y, Z, moving DX, DY, DZ a step) ionise in one of the
+// window's K steps?  Taken only when a word lies below the atom gate: the
+// decision of step_particle in the cell the atom is in at that step.
+__device__ __forceinline__ bool atom_ionizes(const RunDev& R, const QuietShared& S, const QuietAtom& a, uint32_t K,
+                                             int32_t X, int32_t Y, int32_t Z, int32_t DX, int32_t DY, int32_t DZ)
+{
+    for (uint32_t s = 0; s < K; ++s) {
+        X += DX;
+        Y += DY;
+        Z += DZ;
+        const uint32_t w0 = quiet_word0(R, a, S.rng[s]);
+        if (!atom_may_ionize(R, w0)) continue;
+        const float4 cr = __ldg(R.cell + ngp_cell(R, X, Y, Z));
+        const int zone = cr.y > 0.5f ? 1 : 0;
+        if (fires(w0, event_prob(cr.x * __ldg(R.kdt + zone * kQSlots)))) return true;
+    }
+    return false;
+}
+
+// Deposit of the whole warp's particles: each lane `count` visits and `charge`
+// in all to `cell` (kNoCell: none), one reduction per run of neighbouring lanes
+// in the same cell
+__device__ __forceinline__ void deposit_sums(const RunDev& R, uint32_t cell, uint32_t count, uint32_t charge)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, cell, 1);
+    const uint32_t heads = __ballot_sync(0xFFFFFFFFu, lane == 0 || prev != cell);
+    const uint32_t h = 31u - (uint32_t)__clz(heads & (0xFFFFFFFFu >> (31u - lane)));   // first lane of the run
+    uint32_t n = count, q = charge;
+    const uint32_t any_q = __any_sync(0xFFFFFFFFu, charge != 0u);
+#pragma unroll
+    for (uint32_t d = 1; d < 32u; d <<= 1) {
+        const uint32_t on = __shfl_up_sync(0xFFFFFFFFu, n, d);
+        const bool in = lane >= h + d;   // lane - d lies in the same run
+        if (in) n += on;
+        if (any_q) {
+            const uint32_t oq = __shfl_up_sync(0xFFFFFFFFu, q, d);
+            if (in) q += oq;
+        }
+    }
+    const bool last = lane == 31u || ((heads >> (lane + 1u)) & 1u);
+    if (last && cell != kNoCell) atomicAdd(R.dep + cell, ((unsigned long long)n << 32) | (unsigned long long)q);
+}
+
+// One tile of k_quiet: particles [t * tile, (t + 1) * tile) of the run
+__device__ __forceinline__ void quiet_tile(const RunDev& R, QuietShared& S, uint32_t t, uint32_t tile, uint32_t K)
+{
+    const uint32_t tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
+    const uint32_t nslot = 4u * R.n4;
+    for (uint32_t j = tid; j < tile; j += T) {
+        const uint32_t i = t * tile + j;
+        const uint32_t meta = i < nslot ? R.meta[i] : kStPad;
+        const uint32_t status = meta & 0xFFFF0000u, Q = meta & kQMask;
+        const bool live = !(status & (kStFrozen | kStPad));
+        bool listed = live && Q > 0u;
+        uint32_t dep_cell = kNoCell;
+        if (live && Q == 0u) {
+            int32_t X = R.x[i], Y = R.y[i], Z = R.z[i];
+            const uint32_t id = R.id[i];
+            float dx = 0.0f, dy = 0.0f, dz = 0.0f;
+            if (R.flags & kFPush) {
+                dx = R.vx[i] * R.dt_sxy;
+                dy = R.vy[i] * R.dt_sxy;
+                dz = R.vz[i] * R.dt_sz;
+            }
+            listed = !(fmaxf(fabsf(dx), fmaxf(fabsf(dy), fabsf(dz))) < 1.0e9f);
+            if (!listed) {
+                const int32_t DX = __float2int_rn(dx), DY = __float2int_rn(dy), DZ = __float2int_rn(dz);
+                const long long xe = X + (long long)K * DX, ye = Y + (long long)K * DY, ze = Z + (long long)K * DZ;
+                bool out_r, out_0, out_L;
+                outside(xe, ye, ze, out_r, out_0, out_L);
+                listed = out_r | out_0 | out_L;
+                if (!listed && (R.flags & kFIonize)) {
+                    const QuietAtom a = quiet_atom(R, id);
+                    uint32_t w = 0xFFFFFFFFu;
+#pragma unroll 2
+                    for (uint32_t s = 0; s < K; ++s) w = min(w, quiet_word0(R, a, S.rng[s]));
+                    if (atom_may_ionize(R, w)) listed = atom_ionizes(R, S, a, K, X, Y, Z, DX, DY, DZ);
+                }
+                if (!listed) {
+                    // the cells it visits: the same one throughout if the
+                    // first and the last step share it (each coordinate is
+                    // monotone)
+                    const int32_t xl = (int32_t)xe, yl = (int32_t)ye, zl = (int32_t)ze;
+                    dep_cell = ngp_cell(R, xl, yl, zl);
+                    if (K > 1u && ngp_cell(R, X + DX, Y + DY, Z + DZ) != dep_cell) {
+                        uint32_t at = kNoCell, n = 0u;
+                        for (uint32_t s = 0; s < K; ++s) {
+                            X += DX;
+                            Y += DY;
+                            Z += DZ;
+                            const uint32_t c = ngp_cell(R, X, Y, Z);
+                            if (c != at) {
+                                if (n) atomicAdd(R.dep + at, (unsigned long long)n << 32);
+                                at = c;
+                                n = 0u;
+                            }
+                            ++n;
+                        }
+                        atomicAdd(R.dep + at, (unsigned long long)n << 32);
+                        dep_cell = kNoCell;
+                    }
+                    R.x[i] = xl;
+                    R.y[i] = yl;
+                    R.z[i] = zl;
+                }
+            }
+        }
+        if (!listed && i < nslot && meta != (status | Q)) R.meta[i] = status | Q;   // its events are over
+        // the deposits of the atoms that kept their cell, K visits each
+        {
+            const uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, dep_cell, 1);
+            const uint32_t heads = __ballot_sync(0xFFFFFFFFu, lane == 0 || prev != dep_cell);
+            const bool last = lane == 31u || ((heads >> (lane + 1u)) & 1u);
+            const uint32_t h = 31u - (uint32_t)__clz(heads & (0xFFFFFFFFu >> (31u - lane)));
+            if (last && dep_cell != kNoCell)
+                atomicAdd(R.dep + dep_cell, (unsigned long long)((lane - h + 1u) * K) << 32);
+        }
+        // the listed slots, ions and atoms apart
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, listed);
+        if (m) {
+            const uint32_t mi = __ballot_sync(0xFFFFFFFFu, listed && Q > 0u);
+            const uint32_t ma = m & ~mi, below = (1u << lane) - 1u;
+            uint32_t bi = 0u, ba = 0u;
+            if (lane == 0) {
+                if (mi) bi = atomicAdd(&S.cnt[0], (uint32_t)__popc(mi));
+                if (ma) ba = atomicAdd(&S.cnt[1], (uint32_t)__popc(ma));
+            }
+            bi = __shfl_sync(0xFFFFFFFFu, bi, 0);
+            ba = __shfl_sync(0xFFFFFFFFu, ba, 0);
+            if (listed) {
+                if (Q > 0u) S.list[bi + (uint32_t)__popc(mi & below)] = i;
+                else S.list[tile - 1u - (ba + (uint32_t)__popc(ma & below))] = i;
+            }
+        }
+    }
+    // the tile's slots to the run's lists: one atomic a list and tile (many
+    // warps adding to one word would queue for it)
+    __syncthreads();
+    if (tid < 2u) S.base[tid] = S.cnt[tid] ? atomicAdd(R.nleave + tid, S.cnt[tid]) : 0u;
+    __syncthreads();
+    const uint32_t ni = S.cnt[0], na = S.cnt[1];
+    for (uint32_t k = tid; k < ni; k += T) R.leave[S.base[0] + k] = S.list[k];
+    for (uint32_t k = tid; k < na; k += T) R.leave[nslot - 1u - (S.base[1] + k)] = S.list[tile - 1u - k];
+    __syncthreads();
+    if (tid < 2u) S.cnt[tid] = 0u;
+    __syncthreads();
+}
+
+__device__ __forceinline__ void quiet_start(const RunDev& R, QuietShared& S, uint32_t K)
+{
+    if (threadIdx.x < K) S.rng[threadIdx.x] = quiet_step(R, *R.step + threadIdx.x);
+    if (threadIdx.x < 2) S.cnt[threadIdx.x] = 0u;
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(512, 3) k_quiet(const __grid_constant__ RunDev R, uint32_t ntiles, uint32_t tile,
+                                                  uint32_t K)
+{
+    __shared__ QuietShared S;
+    pdl_wait();
+    pdl_trigger();
+    quiet_start(R, S, K);
+    for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) quiet_tile(R, S, t, tile, K);
+}
+
+// the block's copy of a run's parameter block (all threads call it)
+__device__ __forceinline__ void stage_run(RunDev& rs, const RunDev* src)
+{
+    const uint32_t* from = reinterpret_cast<const uint32_t*>(src);
+    uint32_t* to = reinterpret_cast<uint32_t*>(&rs);
+    for (uint32_t k = threadIdx.x; k < sizeof(RunDev) / 4; k += blockDim.x) to[k] = from[k];
+}
+
+// entries of a run's list: its ions, padded to whole warps, then its atoms
+__device__ __forceinline__ uint32_t list_entries(uint32_t ni, uint32_t na) { return ((ni + 31u) & ~31u) + na; }
+
+// every run of a batch; the last block works out where each run's tiles of
+// listed particles start in the active pass (pref[r], nruns + 1 entries)
+__global__ void __launch_bounds__(512, 3) k_quiet_batch(const RunDev* __restrict__ runs, const uint2* __restrict__ items,
+                                                        uint32_t nitems, uint32_t tile, uint32_t K, uint32_t nruns,
+                                                        uint32_t* __restrict__ pref, unsigned int* ticket)
+{
+    __shared__ QuietShared S;
+    __shared__ RunDev rs;
+    __shared__ uint32_t s_sum[512];
+    pdl_wait();
+    pdl_trigger();
+    uint32_t cur = 0xFFFFFFFFu;
+    for (uint32_t i = blockIdx.x; i < nitems; i += gridDim.x) {
+        const uint2 it = items[i];
+        if (it.x != cur) {
+            cur = it.x;
+            stage_run(rs, runs + cur);
+            __syncthreads();
+            quiet_start(rs, S, K);
+        }
+        quiet_tile(rs, S, it.y, tile, K);
+    }
+    if (!last_block(ticket)) return;
+    const uint32_t tid = threadIdx.x, T = blockDim.x;
+    uint32_t carry = 0u;
+    for (uint32_t r0 = 0; r0 < nruns; r0 += T) {
+        const uint32_t r = r0 + tid;
+        uint32_t v = 0u;
+        if (r < nruns && runs[r].step) {
+            const volatile uint32_t* nl = runs[r].nleave;
+            v = (list_entries(nl[0], nl[1]) + kActiveTile - 1u) / kActiveTile;
+        }
+        s_sum[tid] = v;
+        __syncthreads();
+        for (uint32_t d = 1; d < T; d <<= 1) {
+            const uint32_t o = tid >= d ? s_sum[tid - d] : 0u;
+            __syncthreads();
+            s_sum[tid] += o;
+            __syncthreads();
+        }
+        if (r < nruns) pref[r] = carry + s_sum[tid] - v;
+        carry += s_sum[T - 1u];
+        __syncthreads();
+    }
+    if (tid == 0) pref[nruns] = carry;
+}
+
+// a particle that left the chamber, out of line: its FP64 geometry's registers
+// are not the step's
+struct Left {
+    int32_t X, Y, Z;
+    float vx, vy, vz;
+    uint32_t meta, cell;
+};
+
+__device__ __noinline__ Left leave_call(const RunDev& R, uint32_t pid, uint32_t step, int32_t X, int32_t Y, int32_t Z,
+                                        float vx, float vy, float vz, uint32_t meta)
+{
+    Left l{X, Y, Z, vx, vy, vz, meta, kNoCell};
+    l.cell = leave_particle(R, pid, step, l.X, l.Y, l.Z, l.vx, l.vy, l.vz, l.meta);
+    return l;
+}
+
+// One tile of k_active: entries [t * kActiveTile, ...) of the run's list, K steps each
+template <bool kVar>
+__device__ __forceinline__ void active_tile(const RunDev& R, uint32_t t, uint32_t K, uint32_t ni, uint32_t na)
+{
+    const uint32_t step0 = *R.step, ni32 = (ni + 31u) & ~31u, nslot = 4u * R.n4;
+    for (uint32_t j = threadIdx.x; j < kActiveTile; j += blockDim.x) {
+        const uint32_t e = t * kActiveTile + j;
+        bool in = e < ni || (e >= ni32 && e - ni32 < na);
+        if (!__any_sync(0xFFFFFFFFu, in)) continue;
+        uint32_t i = 0u, id = 0u, meta = kStPad;
+        int32_t x = 0, y = 0, z = 0;
+        float vx = 0.0f, vy = 0.0f, vz = 0.0f;
+        if (in) {
+            i = R.leave[e < ni ? e : nslot - 1u - (e - ni32)];
+            meta = R.meta[i];
+            id = R.id[i];
+            x = R.x[i]; y = R.y[i]; z = R.z[i];
+            vx = R.vx[i]; vy = R.vy[i]; vz = R.vz[i];
+        }
+        // deposits: summed while the particle stays in a cell
+        uint32_t at = kNoCell, n = 0u, q = 0u;
+#pragma unroll 1
+        for (uint32_t s = 0; s < K; ++s) {
+            uint32_t ck, dc;
+            if (step_particle<kVar>(R, id, step0 + s, x, y, z, vx, vy, vz, meta, ck, dc)) {
+                const Left l = leave_call(R, id, step0 + s, x, y, z, vx, vy, vz, meta);
+                x = l.X; y = l.Y; z = l.Z;
+                vx = l.vx; vy = l.vy; vz = l.vz;
+                meta = l.meta;
+                dc = l.cell;   // (as an atom: no charge)
+            }
+            if (dc != at) {
+                if (n) atomicAdd(R.dep + at, ((unsigned long long)n << 32) | (unsigned long long)q);
+                at = dc;
+                n = q = 0u;
+            }
+            if (dc != kNoCell) {
+                ++n;
+                q += meta & kQMask;
+            }
+        }
+        deposit_sums(R, at, n, q);
+        if (in) {
+            R.x[i] = x; R.y[i] = y; R.z[i] = z;
+            R.vx[i] = vx; R.vy[i] = vy; R.vz[i] = vz;
+            R.meta[i] = meta;
+        }
+    }
+}
+
+// the last block clears the lists and advances the step counter
+template <bool kVar>
+__global__ void __launch_bounds__(512, 2) k_active(const __grid_constant__ RunDev R, uint32_t K, unsigned int* ticket)
+{
+    pdl_wait();
+    pdl_trigger();
+    const uint32_t ni = R.nleave[0], na = R.nleave[1];
+    const uint32_t nt = (list_entries(ni, na) + kActiveTile - 1u) / kActiveTile;
+    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) active_tile<kVar>(R, t, K, ni, na);
+    if (last_block(ticket) && threadIdx.x == 0) {
+        R.nleave[0] = 0u;
+        R.nleave[1] = 0u;
+        *R.step += K;
+    }
+}
+
+template <bool kVar>
+__global__ void __launch_bounds__(512, 2) k_active_batch(const RunDev* __restrict__ runs, uint32_t nruns,
+                                                         const uint32_t* __restrict__ pref, uint32_t K,
+                                                         unsigned int* ticket)
+{
+    __shared__ RunDev rs;
+    __shared__ uint32_t s_run, s_base;
+    pdl_wait();
+    pdl_trigger();
+    const uint32_t nt = pref[nruns];
+    uint32_t cur = 0xFFFFFFFFu;
+    for (uint32_t v = blockIdx.x; v < nt; v += gridDim.x) {
+        // the run whose tiles hold tile v
+        for (uint32_t r = threadIdx.x; r < nruns; r += blockDim.x) {
+            const uint32_t lo = pref[r];
+            if (lo <= v && v < pref[r + 1]) {
+                s_run = r;
+                s_base = lo;
+            }
+        }
+        __syncthreads();
+        const uint32_t r = s_run, t = v - s_base;
+        if (r != cur) {
+            cur = r;
+            stage_run(rs, runs + cur);
+        }
+        __syncthreads();
+        active_tile<kVar>(rs, t, K, rs.nleave[0], rs.nleave[1]);
+        __syncthreads();
+    }
+    if (last_block(ticket))
+        for (uint32_t r = threadIdx.x; r < nruns; r += blockDim.x)
+            if (runs[r].step) {
+                runs[r].nleave[0] = 0u;
+                runs[r].nleave[1] = 0u;
+                *runs[r].step += K;
             }
 }
 
@@ -1274,16 +1684,67 @@ cudaError_t launch_step(const RunDev& R, uint32_t ntiles, int grid, cudaStream_t
     return cudaGetLastError();
 }
 
+template <class K>
+static int blocks_per_sm(K kernel, int threads)
+{
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, 0) != cudaSuccess || b < 1) b = 1;
+    return b;
+}
+
+int window_blocks_per_sm(int threads)
+{
+    const int a = blocks_per_sm(k_active_batch<false>, threads), b = blocks_per_sm(k_active_batch<true>, threads);
+    return a < b ? a : b;
+}
+
+// Tile of the quiet pass of one run: 128 threads, each with as many particles
+// (up to 8) as leaves every resident block a tile
+static uint32_t quiet_tile_of(uint32_t slots, int sm_count)
+{
+    const uint32_t blocks = 8u * (uint32_t)sm_count;
+    uint32_t v = 8u;
+    while (v > 1u && slots < blocks * 128u * v) v >>= 1;
+    return 128u * v;
+}
+
+cudaError_t launch_window(const RunDev& R, uint32_t K, unsigned int* ticket, int sm_count, cudaStream_t s)
+{
+    const uint32_t slots = 4u * R.n4;
+    if (slots) {
+        const uint32_t tile = quiet_tile_of(slots, sm_count), nt = (slots + tile - 1u) / tile;
+        const uint32_t most = 12u * (uint32_t)sm_count;
+        const cudaError_t e = launch_pdl(k_quiet, dim3(nt < most ? nt : most), dim3(128), 0, s, R, nt, tile, K);
+        if (e != cudaSuccess) return e;
+    }
+    // as many blocks as the list could need, at most one wave
+    const uint32_t need = slots / kActiveTile + 2u, most = 8u * (uint32_t)sm_count;
+    const dim3 grid(need < most ? need : most);
+    if ((R.flags & kFVariants) || R.btab) return launch_pdl(k_active<true>, grid, dim3(kActiveTile), 0, s, R, K, ticket);
+    return launch_pdl(k_active<false>, grid, dim3(kActiveTile), 0, s, R, K, ticket);
+}
+
+cudaError_t launch_window_batch(const RunDev* runs, uint32_t nruns, const uint2* items, uint32_t nitems, uint32_t tile,
+                                int threads, int grid, bool variants, uint32_t K, uint32_t* pref,
+                                unsigned int* ticket, cudaStream_t s)
+{
+    if (nruns == 0) return cudaSuccess;
+    const uint32_t g = nitems < 1u ? 1u : (nitems < (uint32_t)grid ? nitems : (uint32_t)grid);
+    cudaError_t e = launch_pdl(k_quiet_batch, dim3(g), dim3(threads), 0, s, runs, items, nitems, tile, K, nruns, pref,
+                               ticket);
+    if (e != cudaSuccess) return e;
+    if (variants)
+        return launch_pdl(k_active_batch<true>, dim3(grid), dim3(threads), 0, s, runs, nruns, (const uint32_t*)pref, K,
+                          ticket);
+    return launch_pdl(k_active_batch<false>, dim3(grid), dim3(threads), 0, s, runs, nruns, (const uint32_t*)pref, K,
+                      ticket);
+}
+
 cudaError_t launch_scan(const RunDev& R, uint32_t ncells, uint32_t nscan, uint32_t leave_blocks, int do_leave,
                         cudaStream_t s)
 {
     return launch_pdl(k_scan, dim3(nscan + leave_blocks), dim3(kScanThreads), 0, s, R, ncells, nscan + leave_blocks,
                       nscan, do_leave);
-}
-
-cudaError_t launch_leave(const RunDev& R, unsigned int* ticket, int bump_step, cudaStream_t s)
-{
-    return launch_pdl(k_leave, dim3(kLeaveBlocks), dim3(256), 0, s, R, ticket, bump_step);
 }
 
 cudaError_t launch_leave_batch(const RunDev* runs, uint32_t nruns, unsigned int* ticket, cudaStream_t s)
