@@ -54,7 +54,7 @@ typedef enum {
     ECRIS_EINVAL = 1,   /* invalid argument; nothing was changed */
     ECRIS_ENOMEM = 2,   /* device or host allocation failed */
     ECRIS_ECUDA = 3,    /* a CUDA call failed; the message names it */
-    ECRIS_ETIMEOUT = 4, /* a bounded device wait ran out */
+    ECRIS_ETIMEOUT = 4, /* a bounded device wait ran out (no kernel waits at present) */
     ECRIS_ESTATE = 5    /* call out of order (e.g. step before load), or the
                            context is unusable after an earlier device error */
 } ecris_status;
@@ -323,13 +323,12 @@ ecris_status ecris_get_state(ecris_ctx* ctx, float* const xyzv[6], uint32_t* met
  * CUDA events; ecris_get_profile synchronises and reports, per kernel kind,
  * the number of launches and their summed device time since the last reset. */
 typedef struct {
-    int64_t step_launches;     /* fused push/MCC/boundary/deposit kernel */
+    int64_t step_launches;     /* push/MCC/boundary/deposit passes, counted once a step (the atoms' pass
+                                  and the pass over all other particles; timed steps are windows of one) */
     double step_ms;
-    int64_t coulomb_launches;  /* ion-ion collision kernels (binning, pairing; one run's leaver
-                                  pass runs inside them when the run has collisions) */
+    int64_t coulomb_launches;  /* ion-ion collision kernels */
     double coulomb_ms;
-    int64_t other_launches;    /* leaver pass of runs without collisions, sorts, deposit fold and
-                                  bookkeeping kernels */
+    int64_t other_launches;    /* sorts, deposit fold and bookkeeping kernels */
     double other_ms;
 } ecris_profile;
 
@@ -343,11 +342,12 @@ ecris_status ecris_get_profile(ecris_ctx* ctx, ecris_profile* out);
  * 32; >= 1).  ecris_get_state always returns particles in load order. */
 typedef struct {
     int32_t sort_every;
-    int32_t blocks_per_sm;  /* batches: resident step-kernel blocks per SM (0: as many as fit) */
-    int32_t threads;        /* batches: step-kernel threads per block, 128, 256 or 512 (0: 256) */
-    int32_t particles_per_thread;   /* batches: particles per thread and tile, 1, 2 or 4 (0: 2) */
-    int32_t stages;         /* batches: tiles held in shared memory per block, 2 or 3 (0: 3 where the
-                               shape has a three-stage form, else 2) */
+    int32_t blocks_per_sm;  /* batches: resident blocks per SM of the step's passes (0: as many as fit) */
+    int32_t threads;        /* batches: their threads per block, 128, 256 or 512 (0: 256) */
+    int32_t particles_per_thread;   /* batches: particles per thread and tile of the atoms' pass, 1, 2 or 4
+                               (0: 2) */
+    int32_t stages;         /* batches: 2, or 3 for 128 x 2, 256 x 1 and 256 x 2 (0: 3 for these, else 2);
+                               no pass has stages, so 2 and 3 are the same */
     int32_t reserved[3];    /* set to 0 */
 } ecris_tuning;
 ecris_status ecris_set_tuning(ecris_ctx* ctx, const ecris_tuning* t);
@@ -355,9 +355,8 @@ ecris_status ecris_set_tuning(ecris_ctx* ctx, const ecris_tuning* t);
 /* ------------------------------------------------------------------------ */
 /* Batched form: many runs advanced together (the paper's parameter scans of */
 /* Sec. III -- gas flow, microwave power via n_e and T_e -- run as one       */
-/* batch).  Every step of all active runs is one persistent launch of the     */
-/* step kernel over a work list of (run, tile) items, captured with the       */
-/* runs' collision kernels in one CUDA graph.  Each run keeps its particles   */
+/* batch).  Each pass of a step is one launch over all active runs, and each   */
+/* step's passes with collisions one CUDA graph.  Each run keeps its particles */
 /* resident on the device and gives exactly the results it gives alone.      */
 /* ------------------------------------------------------------------------ */
 typedef struct ecris_batch ecris_batch;
@@ -404,15 +403,14 @@ ecris_status ecris_batch_get_cells(ecris_batch* b, int32_t run, float* ne, float
 /* Bytes held by the batch's runs and its budget (0: none). */
 ecris_status ecris_batch_memory(const ecris_batch* b, size_t* used, size_t* budget);
 /* Kernel timing for a batch, as ecris_set_profiling / ecris_get_profile:
- * with profiling on, every step launches its kernels one by one (no graph)
- * between events; step_* is the batched step kernel, coulomb_* the collision
- * kernels of all runs, other_* sorts, deposit folds and step counters. */
+ * with profiling on, every step launches its kernels one by one (no graph, no
+ * windows of several steps) between events; step_* is the step's passes,
+ * coulomb_* the collision kernel of all runs, other_* sorts and deposit folds. */
 ecris_status ecris_batch_set_profiling(ecris_batch* b, int enable);
 ecris_status ecris_batch_get_profile(ecris_batch* b, ecris_profile* out);
 /* Launch-shape autotuner.  Times `trial_steps` steps of the batch (no sort
- * among them) in each launch shape of the step kernel -- threads per block
- * 128, 256 or 512 times particles per thread 1, 2 or 4 with two stages, and
- * 128 x 2, 256 x 1 and 256 x 2 with three -- with as many resident blocks as
+ * among them) in each launch shape of its passes -- threads per block 128, 256
+ * or 512 times particles per thread 1, 2 or 4 -- with as many resident blocks as
  * fit; then, in the fastest shape, each count of resident
  * blocks per SM; then each sort cadence (8, 32, 128, 256, 512 steps), in whole sort
  * periods that each start with a sort.  Keeps the fastest of each and returns
@@ -562,7 +560,7 @@ ecris_status ecris_server_calib_poll(ecris_server* s, int64_t job, ecris_calib_r
  * the device.  It runs the same Takizawa-Abe pairing and Nanbu scattering as
  * ecris_step (ECRIS_F_COULOMB) on caller-owned device arrays and keeps all its
  * working memory in one fixed-size array that the library holds on every GPU
- * that loads it (about 4.5 MB, until the process exits); it allocates nothing.
+ * that loads it (about 5 MB, until the process exits); it allocates nothing.
  *
  *   n            particles, at most 65536; arrays are indexed by particle id
  *                (the Philox counter word, as in ecris_step)
@@ -581,10 +579,8 @@ ecris_status ecris_server_calib_poll(ecris_server* s, int64_t job, ecris_calib_r
  *
  * Larger n or ncells return ECRIS_EINVAL with a message in
  * ecris_last_error(NULL).  Every call shares the one working array: calls whose
- * GPU work overlaps race and must be serialised by the caller.  If they do
- * overlap, a bounded wait inside the call can run out; a call given
- * collisions_out then returns ECRIS_ETIMEOUT (its velocities are not valid),
- * while a call without it returns at once and cannot report this.  The first
+ * GPU work overlaps race (their velocities are not valid) and must be
+ * serialised by the caller.  The first
  * call on a device sets that device up (a synchronous copy), so make it before
  * any stream capture begins.  That set-up lasts for the life of the process: a
  * device reset (cudaDeviceReset) is not supported. */

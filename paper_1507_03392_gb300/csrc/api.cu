@@ -294,8 +294,6 @@ constexpr uint32_t kSortAfterLoad = 8;   // steps of one ecris_step call that so
 // the launch shapes
 struct GraphKey {
     RunDev R;
-    uint32_t ntiles;
-    int step_grid, collide_grid;
 };
 
 struct ecris_ctx {
@@ -303,7 +301,6 @@ struct ecris_ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int sm_count = 0;
-    int step_grid = 0;
     std::string err;
     bool failed = false;
 
@@ -324,17 +321,22 @@ struct ecris_ctx {
     uint8_t* d_q8 = nullptr;
     unsigned int* d_bad = nullptr;
     uint32_t* d_err = nullptr;
-    uint4* d_plist = nullptr;
-    float4* d_pvel = nullptr;
-    uint32_t* d_tcount = nullptr;
-    float4* d_crec = nullptr;
+    // Coulomb collisions: see RunDev
+    uint4* d_crec = nullptr;
+    uint32_t* d_cnext = nullptr;
+    uint32_t* d_chead = nullptr;
     uint32_t* d_ccount = nullptr;
-    uint32_t* d_cstart = nullptr;
-    uint32_t* d_crange = nullptr;   // collision ranges: size this step, largest cell count seen
-    uint32_t* d_coff = nullptr;
-    unsigned long long* d_cstat = nullptr;   // scan tile status words and ticket counter
-    unsigned long long* d_ckeys = nullptr;
-    int collide_grid = 0;
+    uint4* d_cbkt = nullptr;
+    uint4* d_pcell = nullptr;
+    uint32_t* d_pcount = nullptr;
+    uint32_t* d_rstart = nullptr;
+    uint32_t* d_xcell = nullptr;
+    uint32_t* d_cidx = nullptr;
+    uint32_t* d_cord = nullptr;
+    uint32_t* d_cword = nullptr;
+    unsigned long long* d_plan = nullptr;   // block sums of the plan
+    bool planned = false;       // the buckets were planned since the load
+    int collide_grid = 0;       // most blocks of the collision kernel
     // two sets of particle arrays, each the eight arrays of one allocation
     // (d_set: 8 cap words, so that a set not in use also serves as cap 32-byte
     // records); the sort moves the particles from the current set to the other
@@ -360,8 +362,6 @@ struct ecris_ctx {
     // re-instantiate its graph)
     cudaGraphExec_t gexec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     GraphKey gkey[2][2];
-    uint32_t* d_cslot = nullptr;
-    uint32_t* d_sslot = nullptr;
     unsigned long long* d_dep = nullptr;
     unsigned long long* d_count = nullptr;
     unsigned long long* d_charge = nullptr;
@@ -384,9 +384,6 @@ struct ecris_ctx {
     unsigned long long* d_fptd = nullptr;   // first-passage histogram and age sums
     uint32_t* d_nleave = nullptr;
     unsigned int* d_ticket = nullptr;
-    uint32_t ntiles = 0;
-    uint32_t tile = kTile;      // particles per tile of the step kernel (a batch sets its launch shape's)
-    uint32_t btiles = 0;        // tiles of the run in its batch's launch shape
     RunDev* h_run = nullptr;    // parameter block passed by value to every kernel
     float* h_kdt = nullptr;     // pinned staging copy of the rate table
     double weight = 0.0;
@@ -452,8 +449,6 @@ void free_ions(ecris_ctx* ctx)
     free_async(ctx, ctx->d_hist);
     free_async(ctx, ctx->d_hoff);
     free_async(ctx, ctx->d_hblk);
-    free_async(ctx, ctx->d_cslot);
-    free_async(ctx, ctx->d_sslot);
     free_async(ctx, ctx->d_dep);
     free_async(ctx, ctx->d_count);
     free_async(ctx, ctx->d_charge);
@@ -470,16 +465,19 @@ void free_ions(ecris_ctx* ctx)
     free_async(ctx, ctx->d_q8);
     free_async(ctx, ctx->d_bad);
     free_async(ctx, ctx->d_err);
-    free_async(ctx, ctx->d_plist);
-    free_async(ctx, ctx->d_pvel);
-    free_async(ctx, ctx->d_tcount);
     free_async(ctx, ctx->d_crec);
+    free_async(ctx, ctx->d_cnext);
+    free_async(ctx, ctx->d_chead);
     free_async(ctx, ctx->d_ccount);
-    free_async(ctx, ctx->d_cstart);
-    free_async(ctx, ctx->d_crange);
-    free_async(ctx, ctx->d_coff);
-    free_async(ctx, ctx->d_cstat);
-    free_async(ctx, ctx->d_ckeys);
+    free_async(ctx, ctx->d_cbkt);
+    free_async(ctx, ctx->d_pcell);
+    free_async(ctx, ctx->d_pcount);
+    free_async(ctx, ctx->d_rstart);
+    free_async(ctx, ctx->d_xcell);
+    free_async(ctx, ctx->d_cidx);
+    free_async(ctx, ctx->d_cord);
+    free_async(ctx, ctx->d_cword);
+    free_async(ctx, ctx->d_plan);
     ctx->have_ions = false;
     ctx->loaded = false;
     ctx->cap = ctx->cap_cells = 0;
@@ -599,19 +597,19 @@ void fill_rundev(ecris_ctx* ctx, double dt, RunDev& R)
     R.inv_h = ctx->h.ax_y.empty() ? 0.0f : (float)((double)R.nseg / ctx->h.geo.L);
     R.dep = ctx->d_dep;
     R.tally = ctx->d_tally;
-    R.plist = ctx->d_plist;
-    R.pvel = ctx->d_pvel;
-    R.tcount = ctx->d_tcount;
     R.crec = ctx->d_crec;
+    R.cpool = R.cover = (uint32_t)ctx->cap;
+    R.cnext = ctx->d_cnext;
+    R.chead = ctx->d_chead;
     R.ccount = ctx->d_ccount;
-    R.cstart = ctx->d_cstart;
-    R.crange = ctx->d_crange;
-    R.coff = ctx->d_coff;
-    R.cstat = ctx->d_cstat;
-    R.cctr = ctx->d_cstat ? ctx->d_cstat + coulomb_scan_blocks((uint32_t)ctx->cap_cells) : nullptr;
-    R.ckeys = ctx->d_ckeys;
-    R.cslot = ctx->d_cslot;
-    R.sslot = ctx->d_sslot;
+    R.cbkt = ctx->d_cbkt;
+    R.pcell = ctx->d_pcell;
+    R.pcount = ctx->d_pcount;
+    R.rstart = ctx->d_rstart;
+    R.xcell = ctx->d_xcell;
+    R.cidx = ctx->d_cidx;
+    R.cord = ctx->d_cord;
+    R.cword = ctx->d_cword;
     R.nanbu = ctx->d_nanbu;
     R.nanbu_lnlo = (float)std::log(kNanbuSLo);
     R.nanbu_inv_dln = (float)((kNanbuN - 1) / std::log(kNanbuSHi / kNanbuSLo));
@@ -624,7 +622,6 @@ void fill_rundev(ecris_ctx* ctx, double dt, RunDev& R)
     R.n = (uint32_t)ctx->n;
     R.n4 = (uint32_t)ctx->n4;
     R.ncells = (uint32_t)((size_t)h.nx * h.ny * h.nz);
-    R.tile = ctx->tile;
 }
 
 // The per-cell records the kernels read, {n_e, zone, delta_x, delta_y}, from
@@ -867,17 +864,15 @@ ecris_status get_cells(ecris_ctx* ctx, float* ne, float* delta_x, float* delta_y
     return ECRIS_OK;
 }
 
-// the kernel sequence of one step with collisions between ions, captured once
-// per particle set and parameter block and replayed as a CUDA graph
+// the kernel sequence of one step with collisions between ions (after the
+// window's quiet pass), captured once per particle set and parameter block and
+// replayed as a CUDA graph
 ecris_status step_graph(ecris_ctx* ctx, int kind, cudaGraphExec_t* out)
 {
     const int p = ctx->parity;
     GraphKey key;
     std::memset(&key, 0, sizeof key);
     std::memcpy(&key.R, ctx->h_run, sizeof(RunDev));   // the block was zeroed before it was filled
-    key.ntiles = ctx->ntiles;
-    key.step_grid = ctx->step_grid;
-    key.collide_grid = ctx->collide_grid;
     if (ctx->gexec[p][kind] && std::memcmp(&ctx->gkey[p][kind], &key, sizeof key) == 0) {
         *out = ctx->gexec[p][kind];
         return ECRIS_OK;
@@ -886,17 +881,14 @@ ecris_status step_graph(ecris_ctx* ctx, int kind, cudaGraphExec_t* out)
         cudaGraphExecDestroy(ctx->gexec[p][kind]);
         ctx->gexec[p][kind] = nullptr;
     }
-    const uint32_t nc = (uint32_t)((size_t)ctx->h.nx * ctx->h.ny * ctx->h.nz);
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
     // kind 0, the whole step; kind 1, the collision kernels alone (timed
-    // steps launch the step kernel on its own before them).  With collisions
-    // the scan kernel also runs the leaver pass.
-    if (kind == 0) e = launch_step(*ctx->h_run, ctx->ntiles, ctx->step_grid, ctx->stream);
+    // steps launch the ions' pass on its own before them)
+    if (kind == 0) e = launch_ions(*ctx->h_run, ctx->sm_count, ctx->stream);
     if (e == cudaSuccess)
-        e = launch_coulomb(*ctx->h_run, nc, ctx->ntiles, ctx->d_ticket, ctx->collide_grid, (uint32_t)kLeaveBlocks,
-                           1, ctx->stream);
+        e = launch_coulomb(*ctx->h_run, (uint32_t)ctx->n, ctx->collide_grid, ctx->stream);
     const cudaError_t e2 = cudaStreamEndCapture(ctx->stream, &g);
     CK(e);
     CK(e2);
@@ -910,9 +902,8 @@ ecris_status step_graph(ecris_ctx* ctx, int kind, cudaGraphExec_t* out)
     return ECRIS_OK;
 }
 
-// Steps of the next window of a run without collisions between ions: at most
-// `left`, and no further than the next sort and the next deposit fold.  Timed
-// steps go one by one.
+// Steps of the next window: at most `left`, and no further than the next sort
+// and the next deposit fold.  Timed steps go one by one.
 uint32_t window_steps(const ecris_ctx* ctx, uint32_t left, bool one_by_one)
 {
     if (one_by_one) return 1;
@@ -941,10 +932,13 @@ ecris_status sort_particles(ecris_ctx* ctx)
     const size_t cap4 = 4 * ctx->n4;
     uint4* aos = ctx->fresh ? reinterpret_cast<uint4*>(dst.x) : nullptr;
     CK(timed(ctx, kKindOther, [&] {
-        return launch_sort(*ctx->h_run, (uint32_t)cap4, dst, ctx->d_hist, ctx->d_hoff, ctx->d_hblk, aos,
+        return launch_sort(*ctx->h_run, (uint32_t)cap4, dst, ctx->d_hist, ctx->d_hoff, ctx->d_hblk, ctx->d_plan, aos,
                            ctx->stream);
-    }, aos ? 7 : 6));
+    }, (aos ? 7 : 6) + (ctx->d_plan ? 3 : 0)));
     ctx->since_sort = 0;
+    if (ctx->d_ccount && !ctx->planned)   // the load's counts were for a plan that is not needed now
+        CK(cudaMemsetAsync(ctx->d_ccount, 0, ctx->cap_cells * sizeof(uint32_t), ctx->stream));
+    ctx->planned = true;
     if (ctx->fresh) {
         ctx->fresh = false;
         return ECRIS_OK;
@@ -1008,8 +1002,7 @@ ecris_status ecris_create(ecris_ctx** out, int device, void* cuda_stream)
         delete ctx;
         return ECRIS_ECUDA;
     }
-    ctx->step_grid = ctx->sm_count * step_blocks_per_sm();   // one wave of resident blocks
-    ctx->collide_grid = ctx->sm_count * collide_blocks_per_sm();
+    ctx->collide_grid = collide_blocks(ctx->sm_count);
     *out = ctx;
     return ECRIS_OK;
 }
@@ -1157,8 +1150,9 @@ ecris_status ecris_init_fields(ecris_ctx* ctx, const ecris_geometry* geo, const 
     h.bmag = bm;
     std::vector<float4> cell;
     cell_records(h, ne, zone, cell);
-    std::vector<float4> E(nc, make_float4(0.f, 0.f, 0.f, 0.f));
+    std::vector<float4> E;   // (an all-zero grid is not kept: the push then gathers nothing)
     if (grid->E) {
+        E.resize(nc);
         for (size_t c = 0; c < nc; ++c) {
             const float ex = grid->E[3 * c], ey = grid->E[3 * c + 1], ez = grid->E[3 * c + 2];
             if (!std::isfinite(ex) || !std::isfinite(ey) || !std::isfinite(ez))
@@ -1168,7 +1162,7 @@ ecris_status ecris_init_fields(ecris_ctx* ctx, const ecris_geometry* geo, const 
         }
     }
     CK(cudaMallocAsync((void**)&ctx->d_cell, nc * sizeof(float4), ctx->stream));
-    CK(cudaMallocAsync((void**)&ctx->d_E, nc * sizeof(float4), ctx->stream));
+    if (h.has_e) CK(cudaMallocAsync((void**)&ctx->d_E, nc * sizeof(float4), ctx->stream));
     CK(cudaMallocAsync((void**)&ctx->d_kdt, kKdtWords * sizeof(float), ctx->stream));
     CK(cudaMallocAsync((void**)&ctx->d_rlc, nc * sizeof(double), ctx->stream));
     // R_L n_e per cell for the device's rebuild of delta, in the order the
@@ -1199,7 +1193,7 @@ ecris_status ecris_init_fields(ecris_ctx* ctx, const ecris_geometry* geo, const 
     CK(cudaMemcpyAsync(ctx->d_cell, cell.data(), nc * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(ctx->d_rlc, rlc.data(), nc * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(ctx->d_kdt + kGateWord, gate_words, sizeof gate_words, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(ctx->d_E, E.data(), nc * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream));
+    if (h.has_e) CK(cudaMemcpyAsync(ctx->d_E, E.data(), nc * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream));
     // the host vectors die at return: wait for the copies
     CK(cudaStreamSynchronize(ctx->stream));
     ctx->have_fields = true;
@@ -1254,25 +1248,27 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
         CK(cudaMallocAsync((void**)&ctx->d_leave, cap * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_birth, cap * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_fptd, kFptdWords * sizeof(unsigned long long), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_nleave, 2 * sizeof(uint32_t), ctx->stream));
+        CK(cudaMallocAsync((void**)&ctx->d_nleave, 3 * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_ticket, sizeof(unsigned int), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_bad, 2 * sizeof(unsigned int), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_err, sizeof(uint32_t), ctx->stream));
         if (h.mcc.flags & kFCoulomb) {
-            // participant lists for tiles of up to kMaxTile particles
-            const size_t slots = cap + kMaxTile;
-            CK(cudaMallocAsync((void**)&ctx->d_plist, slots * sizeof(uint4), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_cslot, cap * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_sslot, cap * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_pvel, slots * sizeof(float4), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_tcount, (cap / kMinTile + 1) * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_ckeys, cap * sizeof(unsigned long long), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_crec, cap * sizeof(float4), ctx->stream));
+            const size_t cells = std::min(nc, cap);   // most cells with ions
+            CK(cudaMallocAsync((void**)&ctx->d_crec, 2 * cap * 2 * sizeof(uint4), ctx->stream));
+            CK(cudaMallocAsync((void**)&ctx->d_cnext, cap * sizeof(uint32_t), ctx->stream));
+            CK(cudaMallocAsync((void**)&ctx->d_chead, nc * sizeof(uint32_t), ctx->stream));
             CK(cudaMallocAsync((void**)&ctx->d_ccount, nc * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_cstart, (cap / kCellIonsMin + 2) * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_crange, 2 * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_coff, (nc + 1) * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_cstat, (size_t)(coulomb_scan_blocks((uint32_t)nc) + 1) * sizeof(unsigned long long),
+            CK(cudaMallocAsync((void**)&ctx->d_cbkt, nc * sizeof(uint4), ctx->stream));
+            CK(cudaMallocAsync((void**)&ctx->d_pcell, cells * sizeof(uint4), ctx->stream));
+            CK(cudaMallocAsync((void**)&ctx->d_pcount, cells * sizeof(uint32_t), ctx->stream));
+            // the cells' room is at most 9/8 of the ions and 4 a cell
+            CK(cudaMallocAsync((void**)&ctx->d_rstart, ((9 * cap / 8 + 4 * cells) / kRange + 3) * sizeof(uint32_t),
+                               ctx->stream));
+            CK(cudaMallocAsync((void**)&ctx->d_xcell, cells * sizeof(uint32_t), ctx->stream));
+            CK(cudaMallocAsync((void**)&ctx->d_cidx, cap * sizeof(uint32_t), ctx->stream));
+            CK(cudaMallocAsync((void**)&ctx->d_cord, cap * sizeof(uint32_t), ctx->stream));
+            CK(cudaMallocAsync((void**)&ctx->d_cword, kCwWords * sizeof(uint32_t), ctx->stream));
+            CK(cudaMallocAsync((void**)&ctx->d_plan, plan_blocks((uint32_t)nc) * sizeof(unsigned long long),
                                ctx->stream));
         }
         ctx->cap = cap;
@@ -1281,21 +1277,19 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
     }
     ctx->n = n;
     ctx->n4 = n4;
-    ctx->ntiles = (uint32_t)((n4 + kTileGroups - 1) / kTileGroups);
     const cudaMemcpyKind kind = src_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     if (n) {
         for (int k = 0; k < 6; ++k)
             CK(cudaMemcpyAsync(ctx->d_soa[k], xyzv[k], n * sizeof(float), kind, ctx->stream));
         CK(cudaMemcpyAsync(ctx->d_q8, q, n, kind, ctx->stream));
     }
-    if (ctx->d_ccount) CK(cudaMemsetAsync(ctx->d_ccount, 0, nc * sizeof(uint32_t), ctx->stream));
-    if (ctx->d_crange) {
-        static const uint32_t crange0[2] = {(uint32_t)kCellIons, 0u};
-        CK(cudaMemcpyAsync(ctx->d_crange, crange0, sizeof crange0, cudaMemcpyHostToDevice, ctx->stream));
+    if (ctx->d_ccount) {
+        CK(cudaMemsetAsync(ctx->d_ccount, 0, nc * sizeof(uint32_t), ctx->stream));
+        CK(cudaMemsetAsync(ctx->d_chead, 0, nc * sizeof(uint32_t), ctx->stream));
+        CK(cudaMemsetAsync(ctx->d_pcount, 0, std::min(nc, ctx->cap) * sizeof(uint32_t), ctx->stream));
+        CK(cudaMemsetAsync(ctx->d_cword, 0, kCwWords * sizeof(uint32_t), ctx->stream));
     }
-    if (ctx->d_cstat)
-        CK(cudaMemsetAsync(ctx->d_cstat, 0, (size_t)(coulomb_scan_blocks((uint32_t)nc) + 1) * sizeof(unsigned long long),
-                           ctx->stream));
+    ctx->planned = false;
     CK(cudaMemsetAsync(ctx->d_dep, 0, nc * sizeof(unsigned long long), ctx->stream));
     CK(cudaMemsetAsync(ctx->d_count, 0, nc * sizeof(unsigned long long), ctx->stream));
     CK(cudaMemsetAsync(ctx->d_charge, 0, nc * sizeof(unsigned long long), ctx->stream));
@@ -1308,7 +1302,7 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
         if (pst != ECRIS_OK) return pst;
     }
     CK(cudaMemsetAsync(ctx->d_step, 0, sizeof(uint32_t), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_nleave, 0, 2 * sizeof(uint32_t), ctx->stream));
+    CK(cudaMemsetAsync(ctx->d_nleave, 0, 3 * sizeof(uint32_t), ctx->stream));
     CK(cudaMemsetAsync(ctx->d_ticket, 0, sizeof(unsigned int), ctx->stream));
     CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(uint32_t), ctx->stream));
     CK(cudaMemsetAsync(ctx->d_bad, 0, sizeof(unsigned int), ctx->stream));
@@ -1328,6 +1322,10 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
         lc.inv_sz_hi = (float)b;
         lc.inv_sz_lo = (float)(b - (double)lc.inv_sz_hi);
     }
+    lc.nx = h.nx;
+    lc.ny = h.ny;
+    lc.nz = h.nz;
+    lc.count = ctx->d_ccount;
     CK(launch_load_init(lc, ctx->d_soa, ctx->d_q8, ctx->d_meta, ctx->d_id, (uint32_t)n, (uint32_t)cap, ctx->d_bad,
                         ctx->stream));
     unsigned int bad[2] = {0u, 0u};
@@ -1336,7 +1334,6 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
     if (bad[0]) {
         ctx->n = 0;
         ctx->n4 = 0;
-        ctx->ntiles = 0;
         ctx->loaded = false;
         return fail(ctx, ECRIS_EINVAL,
                     "load_ions: %u particle(s) outside the chamber, not finite or with Q > qmax "
@@ -1387,25 +1384,24 @@ ecris_status ecris_step(ecris_ctx* ctx, uint32_t nsteps, double dt)
             st = sort_particles(ctx);
             if (st != ECRIS_OK) return st;
         }
-        uint32_t K = 1;   // steps taken together
-        if (!coulomb) {
-            K = window_steps(ctx, nsteps - s, ctx->timer.on);
-            CK(timed(ctx, kKindStep, [&] {
-                return launch_window(*ctx->h_run, K, ctx->d_ticket, ctx->sm_count, ctx->stream);
-            }));
-        } else if (!ctx->timer.on) {
-            // the whole step as one graph launch
+        // a window of steps; timed steps launch the collision kernels of their
+        // one step as a graph of their own
+        const uint32_t K = window_steps(ctx, nsteps - s, ctx->timer.on);
+        if (coulomb && !ctx->planned && ctx->n4 > 0) {
+            // on the load order: from the load's counts
+            CK(launch_plan(*ctx->h_run, ctx->d_ccount, true, ctx->d_plan, ctx->stream));
+            ctx->planned = true;
+        }
+        const RunDev& R = *ctx->h_run;
+        CK(timed(ctx, kKindStep, [&] {
+            cudaError_t e = launch_quiet(R, K, ctx->sm_count, ctx->stream);
+            if (e == cudaSuccess && !coulomb) e = launch_active(R, K, ctx->d_ticket, ctx->sm_count, ctx->stream);
+            if (e == cudaSuccess && coulomb && ctx->timer.on) e = launch_ions(R, ctx->sm_count, ctx->stream);
+            return e;
+        }));
+        for (uint32_t k = 0; coulomb && k < K; ++k) {
             cudaGraphExec_t x = nullptr;
-            st = step_graph(ctx, 0, &x);
-            if (st != ECRIS_OK) return st;
-            CK(cudaGraphLaunch(x, ctx->stream));
-        } else {
-            // timed: the step kernel on its own, the collision kernels as a graph
-            CK(timed(ctx, kKindStep, [&] {
-                return launch_step(*ctx->h_run, ctx->ntiles, ctx->step_grid, ctx->stream);
-            }));
-            cudaGraphExec_t x = nullptr;
-            st = step_graph(ctx, 1, &x);
+            st = step_graph(ctx, ctx->timer.on ? 1 : 0, &x);
             if (st != ECRIS_OK) return st;
             CK(timed(ctx, kKindCoulomb, [&] { return cudaGraphLaunch(x, ctx->stream); }, kCoulombKernels));
         }
@@ -1487,7 +1483,7 @@ ecris_status ecris_diag(ecris_ctx* ctx, ecris_diag_out* out)
     CK(cudaStreamSynchronize(ctx->stream));
     if (err) {
         ctx->failed = true;
-        return fail(ctx, ECRIS_ETIMEOUT, "diag: a kernel's bounded wait for its tile copies ran out; reload");
+        return fail(ctx, ECRIS_ETIMEOUT, "diag: a kernel's bounded wait ran out; reload");
     }
     fill_diag(h, ctx->weight, tally, census, ctx->steps_done, ctx->time_s, out);
     return ECRIS_OK;
@@ -1626,9 +1622,8 @@ struct ecris_batch {
     bool own_stream = false;
     int sm_count = 0;
     int blocks_per_sm = 0;          // 0: as many as fit
-    int shape = kDefaultShape;      // launch shape of the batched step kernel
+    int shape = kDefaultShape;      // launch shape of the batch's passes
     int max_bps[kStepShapes] = {};  // resident blocks per SM of each shape
-    int window_bps[kStepShapes] = {};   // and of the window kernels
     uint32_t sort_every = 32;
     size_t budget = 0, used = 0;
     std::string err;
@@ -1639,8 +1634,8 @@ struct ecris_batch {
     RunDev* h_runs = nullptr;       // pinned staging of the same
     cudaEvent_t staged = nullptr;   // the last upload from h_runs has finished
     size_t runs_cap = 0;
-    uint32_t* d_pref = nullptr;     // scratch of a window's active pass (runs_cap + 1)
-    bool any_coulomb = false;       // some run has collisions between ions: the batch steps one by one
+    uint32_t* d_pref = nullptr;     // where each run's tiles of listed particles start, 2 (runs_cap + 1)
+    bool any_coulomb = false, any_plain = false;   // some run has collisions between ions, some run has none
     uint2* d_items = nullptr;       // work list (handle, tile)
     size_t items_cap = 0;
     uint32_t nitems = 0;
@@ -1651,13 +1646,10 @@ struct ecris_batch {
     bool graph_dirty = true;
     unsigned int* d_ticket = nullptr;   // last-block ticket of the leaver pass
     KernelTimer timer;              // ecris_batch_set_profiling
-    // side streams on which the captured graph runs the collision kernels of
-    // different runs side by side (small runs do not fill the GPU alone)
+    int collide_grid = 0;       // most blocks of the collision kernel
+    // side streams on which the layout sorts of the runs due for one run side
+    // by side (small runs do not fill the GPU alone)
     cudaStream_t side[kBatchSideStreams] = {};
-    cudaEvent_t side_join[kBatchSideStreams] = {};
-    cudaEvent_t side_fork = nullptr;
-    // the layout sorts of the runs due for one, spread over the same side
-    // streams outside the graph, with their own fork and join events
     cudaEvent_t sort_join[kBatchSideStreams] = {};
     cudaEvent_t sort_fork = nullptr;
     // added runs are set up on their own stream, so the batch's queued steps
@@ -1738,7 +1730,7 @@ ecris_status batch_upload(ecris_batch* b)
         b->runs_cap = nr + 16;
         BCK(cudaMallocAsync((void**)&b->d_runs, b->runs_cap * sizeof(RunDev), b->stream));
         if (b->d_pref) cudaFreeAsync(b->d_pref, b->stream);
-        BCK(cudaMallocAsync((void**)&b->d_pref, (b->runs_cap + 1) * sizeof(uint32_t), b->stream));
+        BCK(cudaMallocAsync((void**)&b->d_pref, 2 * (b->runs_cap + 1) * sizeof(uint32_t), b->stream));
         BCK(cudaMallocHost((void**)&b->h_runs, b->runs_cap * sizeof(RunDev)));
         b->graph_dirty = true;
     } else {
@@ -1762,13 +1754,8 @@ ecris_status batch_items(ecris_batch* b)
         ecris_ctx* c = b->runs[r];
         if (!c) continue;
         // the run's tiles in the batch's launch shape
-        c->tile = tile;
-        if (c->h_run->tile != tile) {
-            c->h_run->tile = tile;
-            b->params_dirty = true;
-        }
-        c->btiles = (uint32_t)((c->n4 + groups - 1) / groups);
-        for (uint32_t t = 0; t < c->btiles; ++t) items.push_back(make_uint2((uint32_t)r, t));
+        const uint32_t nt = (uint32_t)((c->n4 + groups - 1) / groups);
+        for (uint32_t t = 0; t < nt; ++t) items.push_back(make_uint2((uint32_t)r, t));
     }
     // the last upload must have read the staging copy before it is rewritten;
     // queued launches may still read the old device list, freed in stream order
@@ -1790,67 +1777,69 @@ ecris_status batch_items(ecris_batch* b)
         BCK(cudaEventRecord(b->items_staged, b->stream));
     }
     b->nitems = (uint32_t)items.size();
-    b->variants = b->any_coulomb = false;
+    b->variants = b->any_coulomb = b->any_plain = false;
     for (auto* c : b->runs) {
         if (c && ((c->h.mcc.flags & kFVariants) || !c->h.ax_y.empty())) b->variants = true;
-        if (c && (c->h.mcc.flags & kFCoulomb)) b->any_coulomb = true;
+        if (c) ((c->h.mcc.flags & kFCoulomb) ? b->any_coulomb : b->any_plain) = true;
     }
     b->layout_dirty = false;
     b->graph_dirty = true;
     return ECRIS_OK;
 }
 
-// resident blocks per SM of the batch's step kernels: the most that fit, and
-// as many as the tuning asks for
-int batch_most_bps(const ecris_batch* b) { return (b->any_coulomb ? b->max_bps : b->window_bps)[b->shape]; }
-
+// resident blocks per SM of the batch's passes: as many as the tuning asks for
 int batch_bps(const ecris_batch* b)
 {
-    const int m = batch_most_bps(b);
+    const int m = b->max_bps[b->shape];
     return b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, m) : m;
 }
 
 cudaError_t batch_side_streams(ecris_batch* b)
 {
-    if (b->side_fork) return cudaSuccess;
-    cudaError_t e = cudaEventCreateWithFlags(&b->side_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->sort_fork, cudaEventDisableTiming);
+    if (b->sort_fork) return cudaSuccess;
+    cudaError_t e = cudaEventCreateWithFlags(&b->sort_fork, cudaEventDisableTiming);
     for (int k = 0; e == cudaSuccess && k < kBatchSideStreams; ++k) {
         e = cudaStreamCreateWithFlags(&b->side[k], cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->side_join[k], cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->sort_join[k], cudaEventDisableTiming);
     }
     return e;
 }
 
-// The step of every run (captured into the batch graph): the batched step
-// kernel and leaver pass on the batch stream (the leaver pass advances the
-// step counters of the runs without collisions between ions); the collision
-// kernels of the runs that have them forked onto the side streams, so
-// different runs' collision kernels overlap, and joined back.
+// the first launch of a window: the quiet pass of every run, and the whole
+// window of the runs without collisions between ions
+cudaError_t batch_window(ecris_batch* b, uint32_t K)
+{
+    const uint32_t nr = (uint32_t)b->runs.size();
+    const int threads = kShapeThreads[b->shape], grid = b->sm_count * batch_bps(b);
+    if (nr == 0) return cudaSuccess;
+    cudaError_t e = launch_quiet_batch(b->d_runs, nr, b->d_items, b->nitems, shape_tile(b->shape), threads, grid, K,
+                                       b->d_pref, b->d_ticket, b->stream);
+    if (e == cudaSuccess && b->any_plain)
+        e = launch_active_batch(b->d_runs, nr, threads, grid, b->variants, K, b->d_pref, b->d_ticket, b->stream);
+    return e;
+}
+
+cudaError_t batch_ions(ecris_batch* b)
+{
+    return launch_ions_batch(b->d_runs, (uint32_t)b->runs.size(), kShapeThreads[b->shape],
+                             b->sm_count * batch_bps(b), b->variants, b->d_pref, b->stream);
+}
+
+// A step of every run with collisions between ions (captured into the batch
+// graph): the ions' pass of all of them, then their collisions
+cudaError_t batch_coulomb(ecris_batch* b)
+{
+    size_t n = 0;
+    for (auto* c : b->runs)
+        if (c && (c->h.mcc.flags & kFCoulomb)) n += c->n;
+    return launch_coulomb_batch(b->d_runs, (uint32_t)b->runs.size(), (uint32_t)std::min(n, (size_t)0xFFFFFFFFu),
+                                b->collide_grid, b->stream);
+}
+
 cudaError_t batch_launch(ecris_batch* b)
 {
-    cudaError_t e = launch_step_batch(b->d_runs, b->d_items, b->nitems, b->sm_count * batch_bps(b), b->variants,
-                                      b->shape, b->stream);
-    if (e == cudaSuccess) e = launch_leave_batch(b->d_runs, (uint32_t)b->runs.size(), b->d_ticket, b->stream);
-    if (e == cudaSuccess) e = batch_side_streams(b);
-    if (e == cudaSuccess) e = cudaEventRecord(b->side_fork, b->stream);
-    int used = 0;
-    for (size_t r = 0; e == cudaSuccess && r < b->runs.size(); ++r) {
-        ecris_ctx* c = b->runs[r];
-        if (!c || !(c->h.mcc.flags & kFCoulomb)) continue;
-        const int k = used % kBatchSideStreams;
-        if (used < kBatchSideStreams) e = cudaStreamWaitEvent(b->side[k], b->side_fork, 0);
-        ++used;
-        const uint32_t nc = (uint32_t)((size_t)c->h.nx * c->h.ny * c->h.nz);
-        if (e == cudaSuccess)
-            e = launch_coulomb(*c->h_run, nc, c->btiles, c->d_ticket, c->collide_grid, 0u, 0, b->side[k]);
-    }
-    for (int k = 0; e == cudaSuccess && k < used && k < kBatchSideStreams; ++k) {
-        e = cudaEventRecord(b->side_join[k], b->side[k]);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->side_join[k], 0);
-    }
-    return e;
+    const cudaError_t e = batch_ions(b);
+    return e == cudaSuccess ? batch_coulomb(b) : e;
 }
 
 ecris_status batch_graph(ecris_batch* b)
@@ -1936,9 +1925,9 @@ ecris_status ecris_batch_create(ecris_batch** out, int device, void* cuda_stream
         delete b;
         return ECRIS_ECUDA;
     }
+    b->collide_grid = collide_blocks(b->sm_count);
     for (int k = 0; k < kStepShapes; ++k) {
-        b->max_bps[k] = step_batch_blocks_per_sm(k);
-        b->window_bps[k] = window_blocks_per_sm(kShapeThreads[k]);
+        b->max_bps[k] = window_blocks_per_sm(kShapeThreads[k]);
     }
     *out = b;
     return ECRIS_OK;
@@ -1959,10 +1948,8 @@ void ecris_batch_destroy(ecris_batch* b)
     cudaStreamSynchronize(b->stream);
     for (int k = 0; k < kBatchSideStreams; ++k) {
         if (b->side[k]) cudaStreamDestroy(b->side[k]);
-        if (b->side_join[k]) cudaEventDestroy(b->side_join[k]);
         if (b->sort_join[k]) cudaEventDestroy(b->sort_join[k]);
     }
-    if (b->side_fork) cudaEventDestroy(b->side_fork);
     if (b->sort_fork) cudaEventDestroy(b->sort_fork);
     for (auto& g : b->old_graphs) {
         cudaGraphExecDestroy(g.second);
@@ -2066,8 +2053,7 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
     }
     for (uint32_t s = 0; s < nsteps;) {
         // regroup the particles of the runs that are due; their parameter
-        // blocks change (the arrays swap), and so does the captured graph
-        // when a run's collision kernels take the block by value
+        // blocks change (the arrays swap)
         // (several at once: the runs' sorts go to the side streams, whose
         // work the batch stream then waits for; timed steps sort one by one)
         int nsort = 0;
@@ -2093,7 +2079,6 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
             }
             if (st != ECRIS_OK) return bfail(b, st, "batch_step: " + c->err);
             b->params_dirty = true;
-            if (c->h.mcc.flags & kFCoulomb) b->graph_dirty = true;
         }
         for (int k = 0; k < nsort && k < kBatchSideStreams; ++k) {
             BCK(cudaEventRecord(b->sort_join[k], b->side[k]));
@@ -2103,37 +2088,23 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
             ecris_status st = batch_upload(b);
             if (st != ECRIS_OK) return st;
         }
-        uint32_t K = 1;   // steps taken together
-        if (!b->any_coulomb) {
-            K = nsteps - s;
-            for (auto* c : b->runs)
-                if (c) K = std::min(K, window_steps(c, K, b->timer.on));
-            const int threads = kShapeThreads[b->shape];
-            BCK(b->timer.run(kKindStep, b->stream, [&] {
-                return launch_window_batch(b->d_runs, (uint32_t)b->runs.size(), b->d_items, b->nitems,
-                                           shape_tile(b->shape), threads, b->sm_count * batch_bps(b), b->variants, K,
-                                           b->d_pref, b->d_ticket, b->stream);
-            }));
-        } else if (!b->timer.on) {
-            ecris_status st = batch_graph(b);
-            if (st != ECRIS_OK) return st;
-            BCK(cudaGraphLaunch(b->gexec, b->stream));
-        } else {
-            // timed: the same launches as the graph, one by one
-            BCK(b->timer.run(kKindStep, b->stream, [&] {
-                return launch_step_batch(b->d_runs, b->d_items, b->nitems, b->sm_count * batch_bps(b),
-                                         b->variants, b->shape, b->stream);
-            }));
-            BCK(b->timer.run(kKindOther, b->stream, [&] {
-                return launch_leave_batch(b->d_runs, (uint32_t)b->runs.size(), b->d_ticket, b->stream);
-            }));
-            for (auto* c : b->runs) {
-                if (!c || !(c->h.mcc.flags & kFCoulomb)) continue;
-                const uint32_t nc = (uint32_t)((size_t)c->h.nx * c->h.ny * c->h.nz);
-                BCK(b->timer.run(kKindCoulomb, b->stream, [&] {
-                    return launch_coulomb(*c->h_run, nc, c->btiles, c->d_ticket, c->collide_grid, 0u, 0, b->stream);
-                }, kCoulombKernels));
+        uint32_t K = nsteps - s;   // the window's steps
+        for (auto* c : b->runs)
+            if (c) K = std::min(K, window_steps(c, K, b->timer.on));
+        BCK(b->timer.run(kKindStep, b->stream, [&] {
+            cudaError_t e = batch_window(b, K);
+            if (e == cudaSuccess && b->timer.on && b->any_coulomb) e = batch_ions(b);
+            return e;
+        }));
+        for (uint32_t k = 0; b->any_coulomb && k < K; ++k) {
+            if (!b->timer.on) {
+                ecris_status st = batch_graph(b);
+                if (st != ECRIS_OK) return st;
+                BCK(cudaGraphLaunch(b->gexec, b->stream));
+                continue;
             }
+            // timed: the graph's collision kernels on their own
+            BCK(b->timer.run(kKindCoulomb, b->stream, [&] { return batch_coulomb(b); }, kCoulombKernels));
         }
         for (size_t r = 0; r < b->runs.size(); ++r) {
             ecris_ctx* c = b->runs[r];
@@ -2178,10 +2149,7 @@ ecris_status ecris_batch_update_ne(ecris_batch* b, int32_t run)
     ecris_status st = update_ne(c);
     if (st == ECRIS_OK) st = upload_dt(c, b->dt[run]);
     if (st != ECRIS_OK) return bfail(b, st, "batch_update_ne: " + c->err);
-    if (std::memcmp(&before, c->h_run, sizeof before) != 0) {
-        b->params_dirty = true;
-        if (c->h.mcc.flags & kFCoulomb) b->graph_dirty = true;
-    }
+    if (std::memcmp(&before, c->h_run, sizeof before) != 0) b->params_dirty = true;
     return ECRIS_OK;
 }
 
@@ -2381,6 +2349,10 @@ ecris_status snapshot_restore(ecris_batch* b, ecris_ctx* c, RunSnapshot& sn)
         off += (n + 255) & ~(size_t)255;
     });
     BCK(e);
+    // the step number goes back: neither set of the collisions' counters may
+    // hold what a trial step left
+    if (c->d_cword)
+        BCK(cudaMemsetAsync(c->d_cword + kCwUnplanned, 0, (kCwWords - kCwUnplanned) * sizeof(uint32_t), b->stream));
     BCK(cudaFreeAsync(sn.buf, b->stream));
     sn.buf = nullptr;
     c->steps_done = sn.steps_done;
@@ -2465,9 +2437,10 @@ ecris_status batch_autotune(ecris_batch* b, uint32_t trial_steps, bool cadence, 
         b->sort_every = every;
         b->graph_dirty = true;
     };
-    // 1. the launch shape (threads per block x particles per thread), as many
-    // resident blocks as fit, no sorts among the timed steps
-    for (int k = 0; k < kStepShapes && st == ECRIS_OK; ++k) {
+    // 1. the launch shape (threads per block x particles per thread: the first
+    // nine, the others differ from one of these in name only), as many resident
+    // blocks as fit, no sorts among the timed steps
+    for (int k = 0; k < 9 && st == ECRIS_OK; ++k) {
         apply(k, 0, orig_sort);
         st = time_steps(b, trial_steps, true, &ms);
         if (st == ECRIS_OK && ms < best) {
@@ -2477,8 +2450,7 @@ ecris_status batch_autotune(ecris_batch* b, uint32_t trial_steps, bool cadence, 
     }
     // 2. resident blocks per SM of that shape
     best = 1e30f;
-    if (st == ECRIS_OK) apply(best_shape, 0, orig_sort);
-    for (int bps = 1; bps <= batch_most_bps(b) && st == ECRIS_OK; ++bps) {
+    for (int bps = 1; bps <= b->max_bps[best_shape] && st == ECRIS_OK; ++bps) {
         apply(best_shape, bps, orig_sort);
         st = time_steps(b, trial_steps, true, &ms);
         if (st == ECRIS_OK && ms < best) {

@@ -2,89 +2,171 @@
 // collision block): Takizawa-Abe pairing of the ions of each cell and Nanbu's
 // scattering angle, Coulomb logarithm lnL_ii.
 //
-// Per step, after the fused step kernel has counted the ions that stayed inside
-// per cell (ccount) and published each one's (pid, cell) and (v, Q) record in
-// its tile's participant list:
-//   1. scan      exclusive scan of ccount -> coff (one pass, decoupled look-back;
-//                the kernel lives in step_kernel.cu beside the leaver pass it
-//                can run in extra blocks);
-//   2. scatter   each participant takes slot coff[cell] + (ccount[cell] counted
-//                down by one), which leaves ccount at zero for the next step;
-//                the slot receives key = (pairing hash << 32 | pid), the hash
-//                being word 0 of the particle's stream-1 Philox block, and the
-//                record (v, cell << 6 | Q), so each cell's records are contiguous;
-//   3. cells     each block takes the cells whose segments start in its
-//                range of participants (kCellIons at the first step after a
-//                load; later as many as keep the largest cell of the step
-//                before inside shared memory) and copies their keys,
-//                records and array slots to shared memory; one thread per
-//                participant counts the hashes of its cell that are smaller
-//                than its own, which is its place in the cell's order (by hash,
-//                then pid: a tie of hash words, about one pair in 2^32, sends
-//                the range to a count by the whole key), independent of the
-//                atomic arrival order.  Consecutive
-//                ranks pair up; a cell with an odd count puts ranks 0, 1, 2 in a
-//                triplet that collides (0,1), (1,2), (2,0) over dt/2 each.  The
-//                first ion of every pair and triplet is listed in shared memory
-//                and one thread per listed entry collides it and writes the
-//                velocities back.  A range too large for shared memory (a cell
-//                with thousands of ions) is done the same way in global memory.
+// The ions' pass of a step leaves a 32-byte record of every ion that stayed
+// inside, (v, Q) and (array slot, its three words of the stream-1 Philox
+// block), in its cell's bucket (place_warp in step_kernel.cu):
+//   - buckets are planned at every layout sort (and before the first step on
+//     the load order) from the cells' ion counts at that time: a cell of h ions
+//     gets room for h + h/8 + 4 (k_plan*), cells without ions none;
+//   - an ion that finds its cell's bucket full, or a cell without one, goes to
+//     the overflow part of the pool and is chained to its cell.
+// So a cell's records lie together without a count, a scan and a scatter in
+// every step.  Then k_collide orders each cell's ions by (first word, particle
+// id), which is independent of the order of arrival, pairs consecutive ones and
+// collides them; a cell with an odd count puts ranks 0, 1, 2 in a triplet that
+// collides (0,1), (1,2), (2,0) over dt/2 each:
+//   - a warp takes a range of planned cells (kRange records' room) or 32
+//     unplanned ones.  It sorts up to kWarpIons ions of several cells at once in
+//     registers, by cell, the first word's high 20 bits and the ion's place (a
+//     bitonic network over 32 lanes x 4); words that tie in those bits are put in
+//     order afterwards;
+//   - it ranks a cell of up to kWarpCell ions by counting into word buckets: ion j
+//     of a cell of m goes to bucket floor(word m / 2^32) of m, the counts are
+//     scanned, and the few ions that share a bucket compare their words, and
+//     their ids if the words tie;
+//   - triplets, three collisions in a row, and larger cells are put by for the
+//     block, whose threads take a triplet each and a large cell together (ranked
+//     the same way, or above kBlockIons by counting in global memory).
+//
 // A collision of ions a, b (same mass M, charges Qa, Qb) over time dt_c uses
 //   s = lnL/(4 pi) (Qa Qb e^2 / (eps0 mu))^2 n g^-3 dt_c,  mu = M/2,
 // n = w m / V_cell for the cell's m ions; A(s) from coth A - 1/A = e^-s
 // (tabulated in FP64 on the host, s >= 1e-3; 1/(1 - e^-s) below, where coth A
 // is 1 to working precision; isotropic for s > 6);
 //   cos chi = 1 + ln(U + (1-U) e^-2A) / A,  eps = 2 pi U'
-// (the logarithm's argument formed without cancellation in FP32, see collide_w);
+// (the logarithm's argument formed without cancellation in FP32, see collide);
 // the relative velocity g is turned by (chi, eps) and the change is shared
 // equally, which conserves momentum and energy of the pair.
+#include <algorithm>
+
 #include "ecris_internal.cuh"
 
 namespace ecris {
 
 namespace {
 
+// ---------------------------------------------------------------------------
+// The plan of the buckets
+// ---------------------------------------------------------------------------
+constexpr int kPlanThreads = 256;
+constexpr int kPlanPer = 8;
+constexpr uint32_t kPlanBlock = kPlanThreads * kPlanPer;
 
-// scatter the participants of each tile into their cells' segments; counting
-// ccount back down gives each its slot and leaves ccount zero for the next step.
-// Neighbouring list entries mostly share a cell (the step kernel sees the
-// particles sorted by cell), so each run of equal cells within a warp takes
-// its slots with one atomic.
-__global__ void k_scatter(const __grid_constant__ RunDev R, uint32_t ntiles)
+// room of a cell of h ions
+__device__ __forceinline__ uint32_t bucket_room(uint32_t h) { return h ? h + (h >> 3) + 4u : 0u; }
+
+__device__ __forceinline__ unsigned long long warp_incl64(unsigned long long v)
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(0xFFFFFFFFu, v, o);
+        if ((int)(threadIdx.x & 31) >= o) v += t;
+    }
+    return v;
+}
+
+// exclusive scan over the block of v; *total: the block's sum (kT threads)
+template <int kT>
+__device__ __forceinline__ unsigned long long block_excl64(unsigned long long v, unsigned long long* total)
+{
+    __shared__ unsigned long long ws[kT / 32 + 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned long long incl = warp_incl64(v);
+    if (lane == 31) ws[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned long long w = lane < kT / 32 ? ws[lane] : 0ull;
+        const unsigned long long wi = warp_incl64(w);
+        if (lane < kT / 32) ws[lane] = wi - w;
+        if (lane == kT / 32 - 1) ws[kT / 32] = wi;
+    }
+    __syncthreads();
+    *total = ws[kT / 32];
+    return ws[warp] + incl - v;
+}
+
+// (planned cells, room) of the blocks of kPlanBlock cells, packed (<< 32 |);
+// count: ions per cell
+__global__ void __launch_bounds__(kPlanThreads) k_plan_sum(const uint32_t* __restrict__ count, uint32_t ncells,
+                                                           unsigned long long* __restrict__ blk)
 {
     pdl_wait();
-    const uint32_t step = *R.step;
-    const uint32_t lane = threadIdx.x & 31;
-    for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const uint32_t np = R.tcount[t];
-        const uint32_t end = (np + 31u) & ~31u;   // whole warps iterate together
-        for (uint32_t i = threadIdx.x; i < end; i += blockDim.x) {
-            const bool in = i < np;
-            uint4 pc = make_uint4(0u, kNoCell, 0u, 0u);   // (array slot, cell, id, -)
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (in) {
-                pc = R.plist[t * R.tile + i];
-                v = R.pvel[t * R.tile + i];
-            }
-            const uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, pc.y, 1);
-            const uint32_t heads = __ballot_sync(0xFFFFFFFFu, lane == 0 || prev != pc.y);
-            const uint32_t upto = 0xFFFFFFFFu >> (31u - lane);             // lanes 0..lane
-            const uint32_t after = heads & ~upto;                           // run heads above this lane
-            const uint32_t tl = after ? (uint32_t)(__ffs(after) - 2) : 31u; // last lane of this lane's run
-            const uint32_t h = 31u - (uint32_t)__clz(heads & upto);          // first lane of this lane's run
-            uint32_t top = 0;
-            if (in && lane == tl) top = atomicSub(R.ccount + pc.y, tl - h + 1u);
-            top = __shfl_sync(0xFFFFFFFFu, top, tl);
-            if (!in) continue;
-            const uint32_t slot = R.coff[pc.y] + top - 1u - (tl - lane);
-            const Words w = rng_words(R, pc.z, step, 1u);
-            R.ckeys[slot] = ((unsigned long long)w.w0 << 32) | pc.z;
-            R.crec[slot] = make_float4(v.x, v.y, v.z, __uint_as_float((pc.y << 6) | __float_as_uint(v.w)));
-            R.cslot[slot] = pc.x;
+    pdl_trigger();
+    const uint32_t base = blockIdx.x * kPlanBlock + threadIdx.x;
+    unsigned long long v = 0ull, total;
+#pragma unroll
+    for (int j = 0; j < kPlanPer; ++j) {
+        const uint32_t c = base + j * kPlanThreads;
+        const uint32_t h = c < ncells ? count[c] : 0u;
+        v += ((unsigned long long)(h ? 1u : 0u) << 32) + bucket_room(h);
+    }
+    block_excl64<kPlanThreads>(v, &total);
+    if (threadIdx.x == 0) blk[blockIdx.x] = total;
+}
+
+// one block: exclusive scan of the block sums in place, and the plan's words
+__global__ void __launch_bounds__(1024) k_plan_scan(const __grid_constant__ RunDev R, unsigned long long* blk,
+                                                    uint32_t nb)
+{
+    pdl_wait();
+    pdl_trigger();
+    const uint32_t per = (nb + 1023u) / 1024u, base = threadIdx.x * per;
+    unsigned long long sum = 0ull, total;
+    for (uint32_t j = 0; j < per; ++j)
+        if (base + j < nb) sum += blk[base + j];
+    unsigned long long o = block_excl64<1024>(sum, &total);
+    for (uint32_t j = 0; j < per; ++j)
+        if (base + j < nb) {
+            const unsigned long long t = blk[base + j];
+            blk[base + j] = o;
+            o += t;
         }
+    if (threadIdx.x == 0) {
+        const uint32_t np = (uint32_t)(total >> 32), room = (uint32_t)total;
+        R.cword[kCwPlanned] = np;
+        R.cword[kCwRanges] = (room + kRange - 1u) / kRange;
+        R.rstart[0] = 0u;
+        R.rstart[(room + kRange - 1u) / kRange] = np;
     }
 }
 
+// every cell's bucket, the compact list of planned cells, and the ranges: range
+// b holds the planned cells whose room starts in [b kRange, (b + 1) kRange)
+__global__ void __launch_bounds__(kPlanThreads) k_plan_cells(const __grid_constant__ RunDev R,
+                                                             uint32_t* __restrict__ count,
+                                                             const unsigned long long* __restrict__ blk, int zero)
+{
+    pdl_wait();
+    const uint32_t base = blockIdx.x * kPlanBlock + threadIdx.x * kPlanPer;
+    uint32_t h[kPlanPer];
+    unsigned long long v = 0ull, total;
+#pragma unroll
+    for (int j = 0; j < kPlanPer; ++j) {
+        h[j] = base + j < R.ncells ? count[base + j] : 0u;
+        if (zero && h[j]) count[base + j] = 0u;
+        v += ((unsigned long long)(h[j] ? 1u : 0u) << 32) + bucket_room(h[j]);
+    }
+    unsigned long long o = blk[blockIdx.x] + block_excl64<kPlanThreads>(v, &total);
+#pragma unroll
+    for (int j = 0; j < kPlanPer; ++j) {
+        const uint32_t c = base + j;
+        if (c >= R.ncells) break;
+        const uint32_t room = bucket_room(h[j]), k = (uint32_t)(o >> 32), at = (uint32_t)o;
+        // (a bucket past the pool's bucket part is cut short; its ions overflow)
+        const uint32_t fits = at < R.cpool ? min(room, R.cpool - at) : 0u;
+        R.cbkt[c] = room ? make_uint4(at, fits, k, 0u) : make_uint4(kNoCell, 0u, 0u, 0u);
+        if (!room) continue;
+        R.pcell[k] = make_uint4(at, fits, c, 0u);
+        for (uint32_t b = at / kRange + 1u; b * kRange < at + room; ++b) R.rstart[b] = k + 1u;
+        // a range that starts just where the next cell's room does
+        if ((at + room) % kRange == 0u) R.rstart[(at + room) / kRange] = k + 1u;
+        o += (1ull << 32) + room;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// One collision
+// ---------------------------------------------------------------------------
 // A(s) for 1e-3 <= s <= 6 from the table of ln A, linear in ln s.  The
 // logarithm that indexes the table and the exponential of the interpolated
 // ln A use the fast intrinsics: their errors (below 1e-6 in ln s and a few
@@ -106,12 +188,12 @@ __device__ __forceinline__ float nanbu_A(const RunDev& R, float s)
 // One collision over time dtc of the records ra, rb (vx, vy, vz, Q bits),
 // with w1, w2 the stream-1 words 1 and 2 of the pair's first particle (the
 // angles); updates the records in place.
-__device__ __forceinline__ void collide_w(const RunDev& R, float4& ra, float4& rb, float dtc, float m_cell,
-                                          uint32_t w1, uint32_t w2)
+__device__ __forceinline__ void collide(const RunDev& R, float4& ra, float4& rb, float dtc, float m_cell, uint32_t w1,
+                                        uint32_t w2)
 {
     // (FMAs written out: this file is compiled without contraction, so that
-    // every inlined copy of this code rounds the same way, whichever path of
-    // the collision kernel takes a cell)
+    // every inlined copy of this code rounds the same way, whichever kernel
+    // takes a cell)
     const float gx = ra.x - rb.x, gy = ra.y - rb.y, gz = ra.z - rb.z;
     const float g2 = fmaf(gx, gx, fmaf(gy, gy, gz * gz));
     if (!(g2 > 0.0f)) return;
@@ -164,115 +246,14 @@ __device__ __forceinline__ void collide_w(const RunDev& R, float4& ra, float4& r
     rb.x -= dgx; rb.y -= dgy; rb.z -= dgz;
 }
 
-// the same with the words of particle `first` at this step
-__device__ __forceinline__ void collide(const RunDev& R, float4& ra, float4& rb, float dtc, float m_cell,
-                                        uint32_t first, uint32_t step)
-{
-    const Words w = rng_words(R, first, step, 1u);
-    collide_w(R, ra, rb, dtc, m_cell, w.w1, w.w2);
-}
-
 __device__ __forceinline__ void write_back(const RunDev& R, uint32_t slot, const float4& r)
 {
     R.vx[slot] = r.x;
     R.vy[slot] = r.y;
     R.vz[slot] = r.z;
-    atomicOr(R.meta + slot, kEvCoulomb);   // result unused: a fire-and-forget reduction
-}
-
-// Shared-memory image of one range of cells (see the header).  The pairing
-// key (hash << 32 | pid) is kept as its two words.
-struct CellSmem {
-    uint32_t hash[kCellCap];
-    uint32_t pid[kCellCap];
-    float4 rec[kCellCap];
-    uint32_t slot[kCellCap];
-    uint32_t sidx[kCellCap];          // sorted position -> index in the range
-    uint2 start[kCellCap / 2 + 1];    // (sorted position, cell count): pairs from the front,
-                                      // triplets from the back, so a warp runs one kind
-    uint32_t claim[kCellCap / 32];    // sorted positions taken by the 32-bit ranking
-    uint32_t npair, ntrip;
-    uint32_t s0, s1;
-    int tie;                          // two keys of a cell share their hash word
-    unsigned long long ncoll;
-};
-
-// collide the pair (kind 0) or triplet (kind 1) starting at sorted position p
-// of a range (key / rec / slot indexed through sidx), m ions in the cell
-template <class K, class V, class S, class I>
-__device__ __forceinline__ uint32_t collide_entry(const RunDev& R, const K& key, const V& rec, const S& slot,
-                                                  const I& sidx, uint32_t p, uint32_t m, bool triplet,
-                                                  uint32_t step)
-{
-    const float dt = R.dt;
-    const uint32_t ia = sidx[p], ib = sidx[p + 1];
-    float4 ra = rec[ia], rb = rec[ib];
-    if (!triplet) {
-        collide(R, ra, rb, dt, (float)m, (uint32_t)key[ia], step);   // ids give the random words
-        write_back(R, slot[ia], ra);
-        write_back(R, slot[ib], rb);
-        return 1u;
-    }
-    // ranks 0, 1, 2: (0,1), (1,2), (2,0) over dt/2 each; the three pairs'
-    // random words do not depend on the velocities, so they are drawn first
-    const uint32_t ic = sidx[p + 2];
-    float4 rc = rec[ic];
-    const float mc = (float)m;
-    const Words wa = rng_words(R, (uint32_t)key[ia], step, 1u);
-    const Words wb = rng_words(R, (uint32_t)key[ib], step, 1u);
-    const Words wc = rng_words(R, (uint32_t)key[ic], step, 1u);
-    collide_w(R, ra, rb, 0.5f * dt, mc, wa.w1, wa.w2);
-    collide_w(R, rb, rc, 0.5f * dt, mc, wb.w1, wb.w2);
-    collide_w(R, rc, ra, 0.5f * dt, mc, wc.w1, wc.w2);
-    write_back(R, slot[ia], ra);
-    write_back(R, slot[ib], rb);
-    write_back(R, slot[ic], rc);
-    return 3u;
-}
-
-// rank of participant j (index in the range) within its cell: the number of
-// smaller keys among the cell's m; seg = the cell's first index in the range
-template <class K>
-__device__ __forceinline__ uint32_t rank_in_cell(const K& key, uint32_t seg, uint32_t m, unsigned long long mine)
-{
-    uint32_t r0 = 0, r1 = 0;
-    uint32_t i = 0;
-    for (; i + 2 <= m; i += 2) {
-        r0 += key[seg + i] < mine ? 1u : 0u;
-        r1 += key[seg + i + 1] < mine ? 1u : 0u;
-    }
-    if (i < m) r0 += key[seg + i] < mine ? 1u : 0u;
-    return r0 + r1;
-}
-
-// the same from the hash words alone: exact when the cell's hashes are
-// distinct (then the order by hash is the order by key); a tie gives two
-// participants the same rank, which the caller detects
-__device__ __forceinline__ uint32_t rank_in_cell32(const uint32_t* hash, uint32_t seg, uint32_t m, uint32_t mine)
-{
-    const uint32_t* h = hash + seg;
-    uint32_t r0 = 0, r1 = 0, r2 = 0, r3 = 0;
-    uint32_t i = 0;
-    for (; i + 4 <= m; i += 4) {
-        r0 += h[i] < mine ? 1u : 0u;
-        r1 += h[i + 1] < mine ? 1u : 0u;
-        r2 += h[i + 2] < mine ? 1u : 0u;
-        r3 += h[i + 3] < mine ? 1u : 0u;
-    }
-    for (; i < m; ++i) r0 += h[i] < mine ? 1u : 0u;
-    return (r0 + r1) + (r2 + r3);
-}
-
-// the rank by the whole key (hash, then pid) from the two word arrays
-__device__ __forceinline__ uint32_t rank_in_cell64(const uint32_t* hash, const uint32_t* pid, uint32_t seg,
-                                                   uint32_t m, uint32_t mh, uint32_t mp)
-{
-    uint32_t r = 0;
-    for (uint32_t i = 0; i < m; ++i) {
-        const uint32_t h = hash[seg + i];
-        r += (h < mh || (h == mh && pid[seg + i] < mp)) ? 1u : 0u;
-    }
-    return r;
+    // (a caller's event words are not the records' meta words)
+    if (R.pcell) R.meta[slot] = __float_as_uint(r.w) | kEvCoulomb;
+    else R.meta[slot] |= kEvCoulomb;
 }
 
 // kind of sorted place r in a cell of m: 1 starts a pair, 2 starts a triplet
@@ -286,176 +267,742 @@ __device__ __forceinline__ uint32_t start_kind(uint32_t r, uint32_t m)
     return (r & 1u) ? 0u : 1u;
 }
 
-__global__ void __launch_bounds__(256, 6) k_cells(const __grid_constant__ RunDev R, uint32_t ncells, unsigned int* ticket)
+struct Record {
+    float4 v;      // vx, vy, vz, Q as bits
+    uint4 w;       // array slot, words 0, 1, 2
+};
+
+__device__ __forceinline__ Record load_record(const RunDev& R, uint32_t p)
 {
-    extern __shared__ __align__(16) unsigned char cell_smem_raw[];
-    CellSmem& S = *reinterpret_cast<CellSmem*>(cell_smem_raw);
-    pdl_wait();
-    const uint32_t total = R.coff[ncells];
-    const uint32_t step = *R.step;
-    const uint32_t tid = threadIdx.x, lane = tid & 31;
-    if (tid == 0) S.ncoll = 0ull;
-    uint32_t ncoll = 0;
-    const uint32_t stride = R.crange[0];   // participants a range, as the scan marked them
-    for (uint32_t b = blockIdx.x; b * stride < total; b += gridDim.x) {
-        if (tid == 0) {
-            const uint32_t hi = (b + 1u) * stride;
-            S.s0 = R.cstart[b];
-            S.s1 = hi >= total ? total : R.cstart[b + 1];
-            S.npair = 0u;
-            S.ntrip = 0u;
-        }
-        __syncthreads();
-        const uint32_t s0 = S.s0, n = S.s1 - S.s0;
-        if (n <= (uint32_t)kCellCap) {
-            for (uint32_t j = tid; j < n; j += blockDim.x) {
-                const unsigned long long k = R.ckeys[s0 + j];
-                S.hash[j] = (uint32_t)(k >> 32);
-                S.pid[j] = (uint32_t)k;
-                S.rec[j] = R.crec[s0 + j];
-                S.slot[j] = R.cslot[s0 + j];
-            }
-            for (uint32_t w = tid; w < kCellCap / 32; w += blockDim.x) S.claim[w] = 0u;
-            if (tid == 0) S.tie = 0;
-            __syncthreads();
-            // ranks, and the list of pair / triplet starters.  First by the
-            // hash words alone, each participant claiming its sorted place;
-            // if two claim one place (hash words tie, about once in 2^32
-            // pairs), again by the whole key.
-            const uint32_t end = (n + 31u) & ~31u;
-            for (int exact = 0; exact < 2; ++exact) {
-                for (uint32_t j = tid; j < end; j += blockDim.x) {
-                    uint32_t kind = 0u, pos = 0u, m = 0u;
-                    if (j < n) {
-                        const uint32_t cell = __float_as_uint(S.rec[j].w) >> 6;
-                        const uint32_t seg = R.coff[cell] - s0;
-                        m = R.coff[cell + 1] - R.coff[cell];
-                        uint32_t r;
-                        if (!exact) {
-                            r = rank_in_cell32(S.hash, seg, m, S.hash[j]);
-                            const uint32_t bit = 1u << ((seg + r) & 31u);
-                            if (atomicOr(&S.claim[(seg + r) >> 5], bit) & bit) S.tie = 1;
-                        } else {
-                            r = rank_in_cell64(S.hash, S.pid, seg, m, S.hash[j], S.pid[j]);
-                        }
-                        pos = seg + r;
-                        S.sidx[pos] = j;
-                        kind = start_kind(r, m);
-                    }
-                    const uint32_t b1 = __ballot_sync(0xFFFFFFFFu, kind == 1u);
-                    const uint32_t b2 = __ballot_sync(0xFFFFFFFFu, kind == 2u);
-                    if (b1 | b2) {
-                        uint32_t base1 = 0, base2 = 0;
-                        if (lane == 0) {
-                            if (b1) base1 = atomicAdd(&S.npair, (uint32_t)__popc(b1));
-                            if (b2) base2 = atomicAdd(&S.ntrip, (uint32_t)__popc(b2));
-                        }
-                        base1 = __shfl_sync(0xFFFFFFFFu, base1, 0);
-                        base2 = __shfl_sync(0xFFFFFFFFu, base2, 0);
-                        const uint32_t below = (1u << lane) - 1u;
-                        if (kind == 1u) S.start[base1 + (uint32_t)__popc(b1 & below)] = make_uint2(pos, m);
-                        if (kind == 2u)
-                            S.start[kCellCap / 2 - (base2 + (uint32_t)__popc(b2 & below))] = make_uint2(pos, m);
-                    }
-                }
-                __syncthreads();
-                if (exact || !S.tie) break;
-                // a tie: rebuild the lists by the whole key
-                if (tid == 0) {
-                    S.npair = 0u;
-                    S.ntrip = 0u;
-                }
-                __syncthreads();
-            }
-            // triplets (three collisions in a row) first, so that they run
-            // beside the pairs instead of after them
-            const uint32_t np = S.npair, nt = S.ntrip;
-            for (uint32_t e = tid; e < nt + np; e += blockDim.x) {
-                const bool trip = e < nt;
-                const uint2 st = S.start[trip ? kCellCap / 2 - e : e - nt];
-                ncoll += collide_entry(R, S.pid, S.rec, S.slot, S.sidx, st.x, st.y, trip, step);
-            }
-        } else {
-            // the same in global memory: sorted positions in sslot
-            const unsigned long long* key = R.ckeys + s0;
-            const float4* rec = R.crec + s0;
-            const uint32_t* slot = R.cslot + s0;
-            uint32_t* sidx = R.sslot + s0;
-            for (uint32_t j = tid; j < n; j += blockDim.x) {
-                const uint32_t cell = __float_as_uint(rec[j].w) >> 6;
-                const uint32_t seg = R.coff[cell] - s0;
-                const uint32_t m = R.coff[cell + 1] - R.coff[cell];
-                sidx[seg + rank_in_cell(key, seg, m, key[j])] = j;
-            }
-            __syncthreads();
-            for (uint32_t p = tid; p < n; p += blockDim.x) {
-                const uint32_t cell = __float_as_uint(rec[sidx[p]].w) >> 6;
-                const uint32_t seg = R.coff[cell] - s0;
-                const uint32_t m = R.coff[cell + 1] - R.coff[cell];
-                const uint32_t kind = start_kind(p - seg, m);
-                if (kind) ncoll += collide_entry(R, key, rec, slot, sidx, p, m, kind == 2u, step);
-            }
-        }
-        __syncthreads();   // the range's shared memory is reused by the next one
+    uint32_t a[8];
+    asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7])
+                 : "l"(R.crec + 2 * (size_t)p));
+    return Record{make_float4(__uint_as_float(a[0]), __uint_as_float(a[1]), __uint_as_float(a[2]),
+                              __uint_as_float(a[3])),
+                  make_uint4(a[4], a[5], a[6], a[7])};
+}
+
+// collide the records ia, ib of the pool as a pair, m ions in the cell
+__device__ __forceinline__ void collide_pair(const RunDev& R, uint32_t ia, uint32_t ib, float m)
+{
+    Record a = load_record(R, ia), b = load_record(R, ib);
+    collide(R, a.v, b.v, R.dt, m, a.w.z, a.w.w);
+    write_back(R, a.w.x, a.v);
+    write_back(R, b.w.x, b.v);
+}
+
+// ranks 0, 1, 2: (0,1), (1,2), (2,0) over dt/2 each
+__device__ __forceinline__ void collide_triplet(const RunDev& R, uint32_t ia, uint32_t ib, uint32_t ic, float m)
+{
+    Record a = load_record(R, ia), b = load_record(R, ib), c = load_record(R, ic);
+    const float dtc = 0.5f * R.dt;
+#pragma unroll 1
+    for (int k = 0; k < 3; ++k) {
+        collide(R, a.v, b.v, dtc, m, a.w.z, a.w.w);
+        const Record t = a;   // the next pair to the front
+        a = b;
+        b = c;
+        c = t;
     }
+    write_back(R, a.w.x, a.v);
+    write_back(R, b.w.x, b.v);
+    write_back(R, c.w.x, c.v);
+}
+
+// ---------------------------------------------------------------------------
+// The cells
+// ---------------------------------------------------------------------------
+// Shared memory of a block that takes one cell of up to kBlockIons ions
+struct CellSmem {
+    uint32_t pidx[kBlockIons];            // record of each ion
+    uint32_t word[kBlockIons];            // its first word
+    uint32_t cnt[kBlockIons + 1];         // ions per word bucket, then their exclusive scan
+    uint32_t start[kBlockIons / 2 + 1];   // sorted places that start a pair
+    uint16_t pos[kBlockIons];             // arrival in the word bucket
+    uint16_t arr[kBlockIons];             // ions by word bucket
+    uint16_t ord[kBlockIons];             // ions in order
+};
+
+// particle id at an array slot (the slot where there are no ids)
+__device__ __forceinline__ uint32_t slot_id(const RunDev& R, uint32_t slot) { return R.id ? R.id[slot] : slot; }
+
+__device__ __forceinline__ uint32_t record_id(const RunDev& R, uint32_t p)
+{
+    return slot_id(R, R.crec[2 * (size_t)p + 1].x);
+}
+
+// a cell that takes a block: (first record, room, ions, chain)
+using BigCell = uint4;
+
+// Order and collide the ions of one cell by the block
+__device__ __forceinline__ void collide_cell(const RunDev& R, CellSmem& S, const BigCell& b)
+{
+    constexpr uint32_t T = 32 * kCollideWarps;
+    const uint32_t g = threadIdx.x, M = b.z, room = min(b.y, b.z);
+    for (uint32_t j = g; j <= M; j += T) S.cnt[j] = 0u;
+    for (uint32_t j = g; j < room; j += T) S.pidx[j] = b.x + j;
+    if (g == 0) {
+        uint32_t at = b.w;
+        for (uint32_t i = room; i < M; ++i) {
+            S.pidx[i] = at ? at - 1u : R.cpool;   // (a chain holds as many as the count says)
+            if (at) at = R.cnext[at - 1u - R.cpool];
+        }
+    }
+    __syncthreads();
+    for (uint32_t j = g; j < M; j += T) {
+        const uint32_t w = R.crec[2 * (size_t)S.pidx[j] + 1].y;
+        S.word[j] = w;
+        S.pos[j] = (uint16_t)atomicAdd(&S.cnt[__umulhi(w, M)], 1u);
+    }
+    __syncthreads();
+    // exclusive scan of the bucket counts
+    constexpr int kPer = kBlockIons / T;
+    uint32_t v[kPer], sum = 0u;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ncoll += __shfl_down_sync(0xFFFFFFFFu, ncoll, o);
-    if (lane == 0 && ncoll) atomicAdd(&S.ncoll, (unsigned long long)ncoll);
-    __shared__ int s_last;
+    for (int k = 0; k < kPer; ++k) {
+        v[k] = g * kPer + k < M ? S.cnt[g * kPer + k] : 0u;
+        sum += v[k];
+    }
+    unsigned long long total;
+    uint32_t o = (uint32_t)block_excl64<T>(sum, &total);
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        if (g * kPer + k < M) S.cnt[g * kPer + k] = o;
+        o += v[k];
+    }
+    if (g == 0) S.cnt[M] = M;
     __syncthreads();
-    if (tid == 0) {
-        if (S.ncoll) atomicAdd(R.tally + kTallyCoulomb, S.ncoll);
-        // the last block to finish advances the run's step counter
-        __threadfence();
-        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1 ? 1 : 0;
+    for (uint32_t j = g; j < M; j += T) S.arr[S.cnt[__umulhi(S.word[j], M)] + S.pos[j]] = (uint16_t)j;
+    __syncthreads();
+    for (uint32_t j = g; j < M; j += T) {
+        const uint32_t w = S.word[j], k = __umulhi(w, M);
+        const uint32_t lo = S.cnt[k], hi = S.cnt[k + 1];
+        uint32_t r = lo;
+        for (uint32_t t = lo; t < hi; ++t) {
+            const uint32_t i = S.arr[t], wi = S.word[i];
+            if (wi < w || (wi == w && i != j && record_id(R, S.pidx[i]) < record_id(R, S.pidx[j]))) ++r;
+        }
+        S.ord[r] = (uint16_t)j;
     }
     __syncthreads();
-    if (s_last && tid == 0) {
-        *R.step += 1u;
-        *ticket = 0u;
-        if (R.nleave) *R.nleave = 0u;   // the leaver pass of the step (if the scan did it) is over
-        // the next step's range size: as large as keeps this step's largest
-        // cell, with a range's cells whole, inside shared memory
-        const uint32_t mx = R.crange[1];
-        const uint32_t room = mx < (uint32_t)kCellCap ? (uint32_t)kCellCap - mx : 0u;
-        R.crange[0] = min(max(room, (uint32_t)kCellIonsMin), (uint32_t)kCellIonsMax);
-        R.crange[1] = 0u;
+    // the triplet to the last thread, the pairs from the first
+    const uint32_t first = (M & 1u) ? 3u : 0u, np = (M - first) / 2u;
+    if (first && g == T - 1u)
+        collide_triplet(R, S.pidx[S.ord[0]], S.pidx[S.ord[1]], S.pidx[S.ord[2]], (float)M);
+    for (uint32_t e = g; e < np; e += T)
+        collide_pair(R, S.pidx[S.ord[first + 2 * e]], S.pidx[S.ord[first + 2 * e + 1]], (float)M);
+    __syncthreads();   // the shared memory is used again
+}
+
+// collisions of a cell of m >= 2 ions
+__device__ __forceinline__ uint32_t collisions_of(uint32_t m) { return (m & 1u) ? 3u + (m - 3u) / 2u : m / 2u; }
+
+template <int kT>
+__device__ __forceinline__ void group_sync()
+{
+    if (kT == 32) __syncwarp();
+    else __syncthreads();
+}
+
+// A cell of more than kBlockIons ions, in global memory, by a warp or a block
+// of kT threads of which this is thread g (told: a word they share): its records'
+// indices to cidx, their places to cord, and the rank by counting smaller
+// (word, id)
+template <int kT>
+__device__ __forceinline__ void collide_huge(const RunDev& R, const BigCell b, uint32_t g, uint32_t* told)
+{
+    const uint32_t room = min(b.y, b.z), m = b.z;
+    if (g == 0) *told = atomicAdd(R.cword + kCwHuge, m);
+    group_sync<kT>();
+    const uint32_t off = *told;
+    group_sync<kT>();
+    if (off + m > R.cover) return;   // (the scratch holds every participant)
+    uint32_t* idx = R.cidx + off;
+    uint32_t* ord = R.cord + off;
+    for (uint32_t i = g; i < room; i += kT) idx[i] = b.x + i;
+    if (g == 0) {
+        uint32_t at = b.w;
+        for (uint32_t i = room; i < m; ++i) {
+            idx[i] = at ? at - 1u : R.cpool;
+            if (at) at = R.cnext[at - 1u - R.cpool];
+        }
     }
+    group_sync<kT>();
+    for (uint32_t j = g; j < m; j += kT) {
+        const uint32_t p = idx[j], w = R.crec[2 * (size_t)p + 1].y;
+        uint32_t r = 0u;
+        for (uint32_t i = 0; i < m; ++i) {
+            const uint32_t wo = R.crec[2 * (size_t)idx[i] + 1].y;
+            if (wo < w || (wo == w && i != j && record_id(R, idx[i]) < record_id(R, p))) ++r;
+        }
+        ord[r] = p;
+    }
+    group_sync<kT>();
+    const uint32_t first = (m & 1u) ? 3u : 0u;
+    if (first && g == 0) collide_triplet(R, ord[0], ord[1], ord[2], (float)m);
+    for (uint32_t p = first + 2u * g; p < m; p += 2u * kT) collide_pair(R, ord[p], ord[p + 1], (float)m);
+    group_sync<kT>();
+}
+
+// Shared memory of a warp: up to kWarpIons ions of up to 32 cells
+struct PackSmem {
+    float4 v[kWarpIons];             // the ions' records, cell after cell
+    uint4 w[kWarpIons];
+    uint4 cell[32];                  // (first record - first place, places in the bucket end, first place, ions)
+    uint32_t pidx[kWarpIons];        // where the records are in the pool
+    uint32_t list[kWarpIons];        // pairs; or the keys while ties are put in order
+};
+
+// or one cell of up to kWarpCell
+struct RankSmem {
+    uint32_t word[kWarpCell];        // first words
+    uint32_t cnt2[kWarpCell / 2 + 1];   // ions per word bucket, then their exclusive scan, two 16-bit counts a word
+    uint16_t pos[kWarpCell];         // arrival in the word bucket, then the ions in order
+    uint16_t arr[kWarpCell];         // ions by word bucket
+};
+
+union WarpSmem {
+    PackSmem pack;
+    RankSmem rank;
+};
+
+// what a block's warps put by for the block
+constexpr uint32_t kTrips = 128, kBigs = 32;
+struct Trip {
+    uint32_t a, b, c, m;
+    const RunDev* run;
+};
+struct WarpsSmem {
+    WarpSmem warp[kCollideWarps];
+    Trip trip[kTrips];
+};
+union AnySmem {
+    WarpsSmem w;
+    CellSmem cell;
+};
+struct BlockSmem {
+    AnySmem a;
+    BigCell big[kBigs];
+    const RunDev* big_run[kBigs];
+    uint32_t ntrip, nbig, off[kCollideWarps];
+};
+
+// element exchange of the bitonic network: keep the smaller or the larger
+__device__ __forceinline__ uint32_t keep(uint32_t a, uint32_t b, bool small) { return small ? min(a, b) : max(a, b); }
+
+// sort 128 keys, key r of lane l at place 4 l + r, ascending
+__device__ __forceinline__ void sort128(uint32_t (&k)[4])
+{
+    const uint32_t lane = threadIdx.x & 31;
+#pragma unroll
+    for (uint32_t size = 2; size <= 128u; size <<= 1) {
+#pragma unroll
+        for (uint32_t d = size >> 1; d > 0u; d >>= 1) {
+            if (d >= 4u) {
+                // partner 4 (lane ^ d/4) + r: the lower place keeps the smaller if its group ascends
+                const bool up = ((4u * lane) & size) == 0u, low = ((4u * lane) & d) == 0u;
+                const bool small = up == low;
+#pragma unroll
+                for (int r = 0; r < 4; ++r) k[r] = keep(k[r], __shfl_xor_sync(0xFFFFFFFFu, k[r], d / 4u), small);
+            } else {
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    if (r & (int)d) continue;
+                    const bool up = size >= 4u ? ((4u * lane) & size) == 0u || size > 64u : (r & 2) == 0;
+                    const uint32_t lo = min(k[r], k[r | (int)d]), hi = max(k[r], k[r | (int)d]);
+                    k[r] = up ? lo : hi;
+                    k[r | (int)d] = up ? hi : lo;
+                }
+            }
+        }
+    }
+}
+
+// Order and collide the nq cells described in S.cell (M <= kWarpIons ions in
+// all; starts: a bit at each cell's first place) by a warp.  Triplets go to
+// the block's list while there is room.  Returns the collisions.
+__device__ __forceinline__ uint32_t collide_warp(const RunDev& R, PackSmem& S, BlockSmem& B, uint32_t M,
+                                                 const uint32_t (&starts)[4])
+{
+    const uint32_t lane = threadIdx.x & 31, le = 0xFFFFFFFFu >> (31u - lane);
+    // the records, two a lane in flight (a lane past the last ion takes that one)
+    uint32_t key[4], before[4];
+    before[0] = 0u;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) before[r + 1] = before[r] + (uint32_t)__popc(starts[r]);
+#pragma unroll
+    for (int h = 0; h < 4; h += 2) {
+        uint32_t p[2], q[2];
+        Record rec[2];
+        if (h && M <= 64u) {
+            key[2] = key[3] = 0xFFFFFFFFu;
+            break;
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint32_t at = 32u * (h + k) + lane, j = min(at, M - 1u);
+            const uint32_t word = at < M ? (uint32_t)(h + k) : j >> 5;
+            const uint32_t st = word == 0u ? starts[0] : word == 1u ? starts[1] : word == 2u ? starts[2] : starts[3];
+            const uint32_t bf = word == 0u ? before[0] : word == 1u ? before[1] : word == 2u ? before[2] : before[3];
+            q[k] = bf + (uint32_t)__popc(st & (0xFFFFFFFFu >> (31u - (j & 31u)))) - 1u;
+            const uint4 c = S.cell[q[k]];
+            p[k] = j < c.y ? c.x + j : S.pidx[j];
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) rec[k] = load_record(R, p[k]);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint32_t j = 32u * (h + k) + lane;
+            key[h + k] = 0xFFFFFFFFu;
+            if (j < M) {
+                S.pidx[j] = p[k];
+                S.v[j] = rec[k].v;
+                S.w[j] = rec[k].w;
+                key[h + k] = (q[k] << 27) | ((rec[k].w.y >> 12) << 7) | j;
+            }
+        }
+    }
+    sort128(key);
+    // words of a cell that tie in their high bits: one lane puts them in order
+    uint32_t next = __shfl_down_sync(0xFFFFFFFFu, key[0], 1);
+    const uint32_t p0 = 4u * lane;
+    const bool tie = (p0 + 1u < M && (key[0] >> 7) == (key[1] >> 7)) ||
+                     (p0 + 2u < M && (key[1] >> 7) == (key[2] >> 7)) ||
+                     (p0 + 3u < M && (key[2] >> 7) == (key[3] >> 7)) || (p0 + 4u < M && (key[3] >> 7) == (next >> 7));
+    __syncwarp();
+    if (__any_sync(0xFFFFFFFFu, tie)) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) S.list[4u * lane + r] = key[r];
+        __syncwarp();
+        if (lane == 0) {
+            for (uint32_t i = 1; i < M; ++i)
+                for (uint32_t t = i; t > 0u && (S.list[t - 1] >> 7) == (S.list[t] >> 7); --t) {
+                    const uint32_t ka = S.list[t - 1], kb = S.list[t];
+                    const uint4 wa = S.w[ka & 127u], wb = S.w[kb & 127u];
+                    if (wa.y < wb.y || (wa.y == wb.y && slot_id(R, wa.x) < slot_id(R, wb.x))) break;
+                    S.list[t - 1] = kb;
+                    S.list[t] = ka;
+                }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < 4; ++r) key[r] = S.list[4u * lane + r];
+        next = __shfl_down_sync(0xFFFFFFFFu, key[0], 1);
+        __syncwarp();
+    }
+    const uint32_t next2 = __shfl_down_sync(0xFFFFFFFFu, key[1], 1);
+    uint32_t np = 0u, nt = 0u;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const uint32_t p = 4u * lane + r, q = key[r] >> 27;
+        const uint32_t kb = r < 3 ? key[r < 3 ? r + 1 : 0] : next;
+        const uint32_t kc = r < 2 ? key[r < 2 ? r + 2 : 0] : (r == 2 ? next : next2);
+        uint32_t kind = 0u, m = 0u;
+        if (p < M) {
+            const uint4 c = S.cell[q];
+            m = c.w;
+            kind = start_kind(p - c.z, m);
+        }
+        if (kind == 2u) {
+            const uint32_t ia = S.pidx[key[r] & 127u], ib = S.pidx[kb & 127u], ic = S.pidx[kc & 127u];
+            const uint32_t at = atomicAdd(&B.ntrip, 1u);
+            if (at < kTrips) B.a.w.trip[at] = Trip{ia, ib, ic, m, &R};
+            else collide_triplet(R, ia, ib, ic, (float)m);
+            S.w[key[r] & 127u].x = S.w[kb & 127u].x = S.w[kc & 127u].x = kNoCell;   // written back there
+        }
+        const uint32_t pairs = __ballot_sync(0xFFFFFFFFu, kind == 1u);
+        nt += (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, kind == 2u));
+        if (kind == 1u) S.list[np + (uint32_t)__popc(pairs & (le >> 1))] = (key[r] & 127u) | ((kb & 127u) << 7) | (q << 14);
+        np += (uint32_t)__popc(pairs);
+    }
+    __syncwarp();
+    for (uint32_t e = lane; e < np; e += 32u) {
+        const uint32_t l = S.list[e], ja = l & 127u, jb = (l >> 7) & 127u;
+        float4 a = S.v[ja], b = S.v[jb];
+        const uint4 wa = S.w[ja];
+        collide(R, a, b, R.dt, (float)S.cell[l >> 14].w, wa.z, wa.w);
+        S.v[ja] = a;
+        S.v[jb] = b;
+    }
+    __syncwarp();
+    // back to the arrays in the records' order, in which neighbours mostly are
+    // neighbours there too
+    for (uint32_t j = lane; j < M; j += 32u) {
+        const uint32_t slot = S.w[j].x;
+        if (slot != kNoCell) write_back(R, slot, S.v[j]);
+    }
+    __syncwarp();   // the shared memory is used again
+    return np + 3u * nt;
+}
+
+// ranges and groups of 32 unplanned cells of a run
+__device__ __forceinline__ uint32_t collide_items(const RunDev& R)
+{
+    const uint32_t nr = R.pcell ? R.cword[kCwRanges] : (R.ncells + R.ucells - 1u) / R.ucells;
+    return nr + (R.cword[R.cword[kCwSet] + kCwUnplanned] + 31u) / 32u;
+}
+
+// Order and collide one cell of kWarpIons to kWarpCell ions that all lie in its
+// bucket, by a warp
+__device__ __forceinline__ uint32_t collide_warp_cell(const RunDev& R, RankSmem& S, BlockSmem& B, uint32_t base,
+                                                      uint32_t M)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t* const cnt2 = S.cnt2;
+    const uint16_t* const cnt = reinterpret_cast<const uint16_t*>(S.cnt2);
+    for (uint32_t j = lane; j < (M + 2u) / 2u; j += 32u) cnt2[j] = 0u;
+    __syncwarp();
+#pragma unroll 4
+    for (uint32_t j = lane; j < M; j += 32u) {
+        const uint32_t w = R.crec[2 * (size_t)(base + j) + 1].y, k = __umulhi(w, M);
+        S.word[j] = w;
+        S.pos[j] = (uint16_t)(atomicAdd(cnt2 + (k >> 1), 1u << (16u * (k & 1u))) >> (16u * (k & 1u)));
+    }
+    __syncwarp();
+    // exclusive scan, 16 counts a lane
+    {
+        constexpr int kPer = kWarpCell / 32 / 2;
+        uint32_t v[kPer], sum = 0u;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const uint32_t i = lane * kPer + k;
+            v[k] = 2u * i < M ? cnt2[i] : 0u;
+            sum += (v[k] & 0xFFFFu) + (v[k] >> 16);
+        }
+        uint32_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= (uint32_t)o) incl += t;
+        }
+        uint32_t o = incl - sum;
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const uint32_t i = lane * kPer + k, lo = v[k] & 0xFFFFu;
+            if (2u * i < M) cnt2[i] = o | ((o + lo) << 16);
+            o += lo + (v[k] >> 16);
+        }
+        __syncwarp();
+        if (lane == 0) {   // the end: the high half of a word, or a word of its own
+            if (M & 1u) cnt2[M >> 1] = (cnt2[M >> 1] & 0xFFFFu) | (M << 16);
+            else cnt2[M >> 1] = M;
+        }
+    }
+    __syncwarp();
+    for (uint32_t j = lane; j < M; j += 32u) S.arr[cnt[__umulhi(S.word[j], M)] + S.pos[j]] = (uint16_t)j;
+    __syncwarp();
+    for (uint32_t j = lane; j < M; j += 32u) {
+        const uint32_t w = S.word[j], k = __umulhi(w, M);
+        const uint32_t lo = cnt[k], hi = cnt[k + 1];
+        uint32_t r = lo;
+        for (uint32_t t = lo; t < hi; ++t) {
+            const uint32_t i = S.arr[t], wi = S.word[i];
+            if (wi < w || (wi == w && i != j && record_id(R, base + i) < record_id(R, base + j))) ++r;
+        }
+        S.pos[r] = (uint16_t)j;   // (the arrivals are done with)
+    }
+    __syncwarp();
+    const uint32_t first = (M & 1u) ? 3u : 0u, np = (M - first) / 2u;
+    if (first && lane == 0) {
+        const uint32_t ia = base + S.pos[0], ib = base + S.pos[1], ic = base + S.pos[2];
+        const uint32_t at = atomicAdd(&B.ntrip, 1u);
+        if (at < kTrips) B.a.w.trip[at] = Trip{ia, ib, ic, M, &R};
+        else collide_triplet(R, ia, ib, ic, (float)M);
+    }
+    for (uint32_t e = lane; e < np; e += 32u)
+        collide_pair(R, base + S.pos[first + 2u * e], base + S.pos[first + 2u * e + 1u], (float)M);
+    __syncwarp();   // the shared memory is used again
+    return np + (first ? 3u : 0u);
+}
+
+// a lane's cell of an item: its bucket, its participants and chain
+struct ItemCell { uint32_t base, room, m, head; };
+
+// The cells of an item of a run, a lane each; their counts (and chains) are
+// taken and left zero for the next step
+__device__ __forceinline__ ItemCell item_cell(const RunDev& R, uint32_t item)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t nr = R.pcell ? R.cword[kCwRanges] : (R.ncells + R.ucells - 1u) / R.ucells;
+    uint32_t c = kNoCell;
+    uint32_t* count = nullptr;
+    ItemCell ic{0u, 0u, 0u, 0u};
+    if (item < nr) {
+        if (R.pcell) {
+            const uint32_t k = R.rstart[item] + lane;
+            if (k < R.rstart[item + 1]) {
+                const uint4 p = R.pcell[k];
+                ic.base = p.x;
+                ic.room = p.y;
+                c = p.z;
+                count = R.pcount + k;
+            }
+        } else if (lane < R.ucells && item * R.ucells + lane < R.ncells) {
+            c = item * R.ucells + lane;
+            ic.base = c * R.uroom;
+            ic.room = R.uroom;
+            count = R.pcount + c;
+        }
+    } else {
+        const uint32_t k = (item - nr) * 32u + lane;
+        if (k < R.cword[R.cword[kCwSet] + kCwUnplanned]) {
+            c = R.xcell[k];
+            count = R.ccount + c;
+        }
+    }
+    if (count) {
+        ic.m = *count;
+        if (ic.m) *count = 0u;
+        if (ic.m > ic.room) {
+            ic.head = R.chead[c];
+            R.chead[c] = 0u;
+        }
+        if (ic.m < 2u) ic.m = 0u;   // nothing to collide with
+    }
+    return ic;
+}
+
+// One item of a run by a warp
+__device__ __forceinline__ void collide_item(const RunDev& R, WarpSmem& S, BlockSmem& B, const ItemCell& ic)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t m = ic.m;
+    uint32_t ncoll = 0u;
+    uint32_t left = __ballot_sync(0xFFFFFFFFu, m > 0u);
+    while (left) {
+        // the next cells that fit together
+        const bool mine = (left >> lane) & 1u;
+        uint32_t incl = mine ? m : 0u;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= (uint32_t)o) incl += t;
+        }
+        const uint32_t take = __ballot_sync(0xFFFFFFFFu, mine && incl <= (uint32_t)kWarpIons);
+        if (!take) {   // the first of them goes alone
+            const int src = __ffs(left) - 1;
+            left &= left - 1u;
+            const uint32_t cm = __shfl_sync(0xFFFFFFFFu, m, src), room = __shfl_sync(0xFFFFFFFFu, ic.room, src);
+            const uint32_t base = __shfl_sync(0xFFFFFFFFu, ic.base, src);
+            if (cm <= (uint32_t)kWarpCell && cm <= room) {
+                ncoll += collide_warp_cell(R, S.rank, B, base, cm);
+                continue;
+            }
+            const BigCell big = make_uint4(base, room, cm, __shfl_sync(0xFFFFFFFFu, ic.head, src));
+            uint32_t at = 0u;
+            if (lane == 0) at = atomicAdd(&B.nbig, 1u);
+            at = __shfl_sync(0xFFFFFFFFu, at, 0);
+            if (at < kBigs) {
+                if (lane == 0) {
+                    B.big[at] = big;
+                    B.big_run[at] = &R;
+                }
+            } else {   // no room for it (more than kBigs such cells in a few items): the warp does it
+                collide_huge<32>(R, big, lane, B.off + threadIdx.x / 32u);
+                ncoll += collisions_of(cm);
+            }
+            continue;
+        }
+        left &= ~take;
+        const bool taken = (take >> lane) & 1u;
+        const uint32_t seg = incl - m;
+        if (taken)
+            S.pack.cell[__popc(take & ((1u << lane) - 1u))] = make_uint4(ic.base - seg, seg + min(ic.room, m), seg, m);
+        const uint32_t M = __shfl_sync(0xFFFFFFFFu, incl, 31 - __clz((int)take));
+        uint32_t starts[4];
+#pragma unroll
+        for (uint32_t r = 0; r < 4u; ++r)
+            starts[r] = __reduce_or_sync(0xFFFFFFFFu, taken && (seg >> 5) == r ? 1u << (seg & 31u) : 0u);
+        if (taken && m > ic.room) {   // ions past the bucket: walk the chain
+            uint32_t at = ic.head;
+            for (uint32_t i = ic.room; i < m; ++i) {
+                S.pack.pidx[seg + i] = at ? at - 1u : R.cpool;   // (a chain holds as many as the count says)
+                if (at) at = R.cnext[at - 1u - R.cpool];
+            }
+        }
+        __syncwarp();
+        ncoll += collide_warp(R, S.pack, B, M, starts);
+    }
+    if (lane == 0 && ncoll) atomicAdd(R.tally + kTallyCoulomb, (unsigned long long)ncoll);
+}
+
+// a large cell, by the block
+__device__ __forceinline__ void collide_big(const RunDev& R, BlockSmem& B, const BigCell& b)
+{
+    if (b.z <= (uint32_t)kBlockIons) collide_cell(R, B.a.cell, b);
+    else collide_huge<32 * kCollideWarps>(R, b, threadIdx.x, B.off);
+    if (threadIdx.x == 0) atomicAdd(R.tally + kTallyCoulomb, (unsigned long long)collisions_of(b.z));
+}
+
+// what the block's warps have put by (all threads call it, at the same point)
+__device__ __forceinline__ void collide_rest(BlockSmem& B)
+{
+    __syncthreads();
+    const uint32_t nt = min(B.ntrip, kTrips), nb = min(B.nbig, kBigs);
+    static_assert(kTrips == 32 * kCollideWarps, "a triplet a thread");
+    if (threadIdx.x < nt) {
+        const Trip t = B.a.w.trip[threadIdx.x];
+        collide_triplet(*t.run, t.a, t.b, t.c, (float)t.m);
+    }
+    __syncthreads();   // the list's memory is the large cells' too
+    for (uint32_t e = 0; e < nb; ++e) collide_big(*B.big_run[e], B, B.big[e]);
+    __syncthreads();
+    if (threadIdx.x == 0) B.ntrip = B.nbig = 0u;
+    __syncthreads();
+}
+
+// End of a run's step, by one thread at the start of the collision kernel: it
+// touches only what this kernel does not read (the step number, the window's
+// list and the counters of the next step)
+__device__ __forceinline__ void step_done(const RunDev& R)
+{
+    *R.step += 1u;
+    uint32_t* const other = R.cword + (2u - R.cword[kCwSet]);
+    other[kCwUnplanned] = 0u;
+    other[kCwOverflow] = 0u;
+    if (R.nleave && --R.nleave[2] == 0u) R.nleave[0] = R.nleave[1] = 0u;   // the window's list is done with
+}
+
+// items of each of up to kRunChunk runs at a time, and which run item v belongs to
+constexpr uint32_t kRunChunk = 256;
+
+// the runs' item counts (f(run)) as an exclusive prefix in s_pref[0..nr]; all
+// threads of the block call it
+template <class F>
+__device__ __forceinline__ void run_prefix(const RunDev* runs, uint32_t nr, uint32_t* s_pref, F f)
+{
+    __syncthreads();
+    for (uint32_t r = threadIdx.x; r < nr; r += blockDim.x)
+        s_pref[r + 1] = runs[r].step && (runs[r].flags & kFCoulomb) ? f(runs[r]) : 0u;
+    if (threadIdx.x == 0) s_pref[0] = 0u;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        uint32_t carry = 0u;
+        for (uint32_t r0 = 0; r0 < nr; r0 += 32u) {
+            uint32_t v = r0 + threadIdx.x < nr ? s_pref[r0 + threadIdx.x + 1] : 0u;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, v, o);
+                if ((threadIdx.x & 31u) >= (uint32_t)o) v += t;
+            }
+            if (r0 + threadIdx.x < nr) s_pref[r0 + threadIdx.x + 1] = carry + v;
+            carry += __shfl_sync(0xFFFFFFFFu, v, 31);
+        }
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ uint32_t run_of(const uint32_t* s_pref, uint32_t nr, uint32_t v)
+{
+    uint32_t lo = 0, hi = nr;   // s_pref[lo] <= v < s_pref[hi]
+    while (hi - lo > 1u) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (s_pref[mid] <= v) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// items a warp takes between two visits of the block to what was put by
+constexpr uint32_t kVisit = 4;
+
+__global__ void __launch_bounds__(32 * kCollideWarps, 8) k_collide(const __grid_constant__ RunDev R)
+{
+    __shared__ BlockSmem B;
+    pdl_wait();
+    pdl_trigger();
+    if (threadIdx.x == 0) B.ntrip = B.nbig = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 32) step_done(R);
+    __syncthreads();
+    const uint32_t total = collide_items(R), warp = threadIdx.x >> 5;
+    uint32_t n = 0u;
+    // the next item's cells are read while this one's collide
+    const uint32_t stride = gridDim.x * kCollideWarps;
+    uint32_t v0 = blockIdx.x * kCollideWarps;
+    ItemCell next{0u, 0u, 0u, 0u};
+    if (v0 + warp < total) next = item_cell(R, v0 + warp);
+    for (; v0 < total; v0 += stride) {
+        const ItemCell ic = next;
+        next = ItemCell{0u, 0u, 0u, 0u};
+        if (v0 + stride + warp < total) next = item_cell(R, v0 + stride + warp);
+        collide_item(R, B.a.w.warp[warp], B, ic);
+        if (++n % kVisit == 0u) collide_rest(B);
+    }
+    collide_rest(B);
+}
+
+// every run of a batch
+__global__ void __launch_bounds__(32 * kCollideWarps, 8) k_collide_batch(const RunDev* __restrict__ runs,
+                                                                        uint32_t nruns)
+{
+    __shared__ BlockSmem B;
+    __shared__ uint32_t s_pref[kRunChunk + 1];
+    pdl_wait();
+    pdl_trigger();
+    if (threadIdx.x == 0) B.ntrip = B.nbig = 0u;
+    if (blockIdx.x == 0)
+        for (uint32_t r = threadIdx.x; r < nruns; r += blockDim.x)
+            if (runs[r].step && (runs[r].flags & kFCoulomb)) step_done(runs[r]);
+    const uint32_t warp = threadIdx.x >> 5;
+    for (uint32_t r0 = 0; r0 < nruns; r0 += kRunChunk) {
+        const uint32_t nr = min(kRunChunk, nruns - r0);
+        run_prefix(runs + r0, nr, s_pref, [](const RunDev& R) { return collide_items(R); });
+        const uint32_t total = s_pref[nr];
+        uint32_t n = 0u;
+        for (uint32_t v0 = blockIdx.x * kCollideWarps; v0 < total; v0 += gridDim.x * kCollideWarps) {
+            const uint32_t v = v0 + warp;
+            if (v < total) {
+                const uint32_t r = run_of(s_pref, nr, v);
+                collide_item(runs[r0 + r], B.a.w.warp[warp], B, item_cell(runs[r0 + r], v - s_pref[r]));
+            }
+            if (++n % kVisit == 0u) collide_rest(B);
+        }
+        collide_rest(B);
+    }
+}
+
+template <class K>
+int resident(K kernel, int threads)
+{
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, 0) != cudaSuccess || b < 1) b = 1;
+    return b;
 }
 
 }  // namespace
 
-int coulomb_scan_blocks(uint32_t ncells) { return (int)((ncells + kScanBlock - 1) / kScanBlock); }
+uint32_t plan_blocks(uint32_t ncells) { return (ncells + kPlanBlock - 1u) / kPlanBlock; }
 
-int collide_blocks_per_sm()
+cudaError_t launch_plan(const RunDev& R, uint32_t* count, bool zero, unsigned long long* blk, cudaStream_t s)
 {
-    const int smem = (int)sizeof(CellSmem);
-    if (cudaFuncSetAttribute(k_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 1;
-    int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_cells, 256, smem) != cudaSuccess || b < 1) b = 1;
-    return b;
-}
-
-// the scatter's grid: at most 32 blocks an SM, each taking tiles b, b + grid, ...
-// (fewer, longer-lived blocks than one a tile took 1.4 us less a step at 4e6
-// particles)
-static uint32_t scatter_grid(uint32_t ntiles)
-{
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        return ntiles;
-    return min(ntiles, 32u * (uint32_t)sms);
-}
-
-cudaError_t launch_coulomb(const RunDev& R, uint32_t ncells, uint32_t ntiles, unsigned int* ticket, int grid,
-                           uint32_t leave_blocks, int do_leave, cudaStream_t s)
-{
-    const int nb = coulomb_scan_blocks(ncells);
-    cudaError_t e = launch_scan(R, ncells, (uint32_t)nb, leave_blocks, do_leave, s);
-    if (e == cudaSuccess && ntiles > 0) e = launch_pdl(k_scatter, dim3(scatter_grid(ntiles)), dim3(256), 0, s, R, ntiles);
-    if (e == cudaSuccess) e = launch_pdl(k_cells, dim3(grid), dim3(256), sizeof(CellSmem), s, R, ncells, ticket);
+    const uint32_t nb = plan_blocks(R.ncells);
+    cudaError_t e = launch_pdl(k_plan_sum, dim3(nb), dim3(kPlanThreads), 0, s, (const uint32_t*)count, R.ncells, blk);
+    if (e == cudaSuccess) e = launch_pdl(k_plan_scan, dim3(1), dim3(1024), 0, s, R, blk, nb);
+    if (e == cudaSuccess)
+        e = launch_pdl(k_plan_cells, dim3(nb), dim3(kPlanThreads), 0, s, R, count, (const unsigned long long*)blk,
+                       zero ? 1 : 0);
     return e;
+}
+
+int collide_blocks(int sm_count)
+{
+    return sm_count * std::min(resident(k_collide, 32 * kCollideWarps), resident(k_collide_batch, 32 * kCollideWarps));
+}
+
+// no more blocks than n particles can give work (an item holds two colliding
+// ions or more, few items hold fewer than 32)
+static int grid_for(int most, uint32_t n) { return (int)std::min((uint32_t)most, n / (kCollideWarps * 32u) + 2u); }
+
+cudaError_t launch_coulomb(const RunDev& R, uint32_t n, int most, cudaStream_t s)
+{
+    return launch_pdl(k_collide, dim3(grid_for(most, n)), dim3(32 * kCollideWarps), 0, s, R);
+}
+
+cudaError_t launch_coulomb_batch(const RunDev* runs, uint32_t nruns, uint32_t n, int most, cudaStream_t s)
+{
+    return launch_pdl(k_collide_batch, dim3(grid_for(most, n)), dim3(32 * kCollideWarps), 0, s, runs, nruns);
 }
 
 }  // namespace ecris

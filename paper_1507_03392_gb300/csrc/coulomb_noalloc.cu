@@ -8,13 +8,13 @@
 // device memory up front and forbid allocation afterwards, and plug-ins
 // running inside a larger simulation whose memory manager owns the device.
 // cudaMalloc can also synchronise the device, which such callers must avoid.
-// This entry point therefore keeps all its working memory (per-cell counts and
-// offsets, participant records and keys, the Nanbu table, counters) in one
+// This entry point therefore keeps all its working memory (per-cell counts,
+// participant records, the Nanbu table, counters) in one
 // file-scope device array of fixed size, and allocates nothing.
 //
 // Limits: at most kNaMaxIons particles and kNaMaxCells cells per call; larger
 // sizes are rejected with ECRIS_EINVAL.  The array (kNaScratchBytes, about
-// 4.5 MB) is held by every GPU that loads the library until the process exits.
+// 5 MB) is held by every GPU that loads the library until the process exits.
 // Every call shares it and finds the last call's contents there; what must
 // start at zero is cleared at the start of each call.  Calls whose GPU work
 // overlaps (different streams, or several host threads) race on the array
@@ -23,11 +23,8 @@
 // that first call before any stream capture begins.  That set-up is kept for
 // the life of the process: a device reset (cudaDeviceReset) is not supported,
 // and the entry point must not be called on a device after one.
-// A bounded wait inside the cell-count scan that runs out (possible only when
-// calls overlap) sets an error word in the array instead of faulting; a call
-// given collisions_out synchronises, reads that word and returns
-// ECRIS_ETIMEOUT.  A call without collisions_out returns at once and does not
-// report it.
+// There is no plan of the cells' buckets: the bucket records are shared out
+// evenly among the call's cells, and what does not fit overflows.
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -43,25 +40,19 @@ namespace {
 
 constexpr uint32_t kNaMaxIons = 65536;
 constexpr uint32_t kNaMaxCells = 65536;
-constexpr uint32_t kNaTiles = kNaMaxIons / kTile;
+constexpr uint32_t kNaPool = 49152;    // bucket records, shared out evenly among the call's cells
 constexpr size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // byte offsets of the sub-buffers inside the scratch array
-constexpr size_t kOffPlist = 0;
-constexpr size_t kOffPvel = kOffPlist + align256(sizeof(uint4) * kNaMaxIons);
-constexpr size_t kOffTcount = kOffPvel + align256(sizeof(float4) * kNaMaxIons);
-constexpr size_t kOffCcount = kOffTcount + align256(sizeof(uint32_t) * kNaTiles);
-constexpr size_t kOffCoff = kOffCcount + align256(sizeof(uint32_t) * kNaMaxCells);
-constexpr uint32_t kNaScanTiles = kNaMaxCells / kScanBlock + 1;
-constexpr size_t kOffCstat = kOffCoff + align256(sizeof(uint32_t) * (kNaMaxCells + 1));
-constexpr size_t kOffCkeys = kOffCstat + align256(sizeof(unsigned long long) * (kNaScanTiles + 1));
-constexpr size_t kOffCrec = kOffCkeys + align256(sizeof(unsigned long long) * kNaMaxIons);
-constexpr size_t kOffCslot = kOffCrec + align256(sizeof(float4) * kNaMaxIons);
-constexpr size_t kOffSslot = kOffCslot + align256(sizeof(uint32_t) * kNaMaxIons);
-constexpr size_t kOffCstart = kOffSslot + align256(sizeof(uint32_t) * kNaMaxIons);
-constexpr size_t kOffNanbu = kOffCstart + align256(sizeof(uint32_t) * (kNaMaxIons / kCellIonsMin + 2));
+constexpr size_t kOffRec = 0;
+constexpr size_t kOffNext = kOffRec + align256(2 * sizeof(uint4) * (kNaPool + kNaMaxIons));
+constexpr size_t kOffHead = kOffNext + align256(sizeof(uint32_t) * kNaMaxIons);
+constexpr size_t kOffCcount = kOffHead + align256(sizeof(uint32_t) * kNaMaxCells);
+constexpr size_t kOffIdx = kOffCcount + align256(sizeof(uint32_t) * kNaMaxCells);
+constexpr size_t kOffOrd = kOffIdx + align256(sizeof(uint32_t) * kNaMaxIons);
+constexpr size_t kOffNanbu = kOffOrd + align256(sizeof(uint32_t) * kNaMaxIons);
 constexpr size_t kOffWords = kOffNanbu + align256(sizeof(float) * kNanbuN);
-// words: step, ticket, error word, -, collision range size and largest cell count; then the tally block
+// words: step; from word 16 the collisions' counters; then the tally block
 constexpr size_t kOffTally = kOffWords + 256;
 constexpr size_t kNaScratchBytes = kOffTally + align256(sizeof(unsigned long long) * kTallyWords);
 
@@ -77,48 +68,40 @@ std::mutex g_setup_mutex;
 DeviceSetup g_setup[64];
 
 // clear the per-call counters and store the step index
-__global__ void k_na_init(unsigned char* base, uint32_t ncells, uint32_t tiles, uint32_t step)
+__global__ void k_na_init(unsigned char* base, uint32_t ncells, uint32_t step)
 {
     uint32_t* ccount = reinterpret_cast<uint32_t*>(base + kOffCcount);
-    uint32_t* tcount = reinterpret_cast<uint32_t*>(base + kOffTcount);
+    uint32_t* chead = reinterpret_cast<uint32_t*>(base + kOffHead);
     uint32_t* words = reinterpret_cast<uint32_t*>(base + kOffWords);
     unsigned long long* tally = reinterpret_cast<unsigned long long*>(base + kOffTally);
-    unsigned long long* cstat = reinterpret_cast<unsigned long long*>(base + kOffCstat);
     const uint32_t stride = gridDim.x * blockDim.x;
-    // scan status words and their ticket counter (the scan's tile count
-    // changes with ncells from call to call)
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i <= kNaScanTiles; i += stride) cstat[i] = 0ull;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < ncells; i += stride) ccount[i] = 0u;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < tiles; i += stride) tcount[i] = 0u;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        words[0] = step;
-        words[1] = 0u;   // the collision kernel's ticket
-        words[2] = 0u;   // error word: the scan sets ECRIS_ETIMEOUT if a bounded wait runs out
-        words[4] = (uint32_t)kCellIons;   // collision range size of this call
-        words[5] = 0u;
-    }
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < ncells; i += stride) ccount[i] = chead[i] = 0u;
+    // (the collisions' counters: the set of this step)
+    if (blockIdx.x == 0 && threadIdx.x < 16 + kCwWords)
+        words[threadIdx.x] = threadIdx.x == 0 ? step : (threadIdx.x == 16 + kCwSet ? 2u * (step & 1u) : 0u);
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < (uint32_t)kTallyWords; i += stride) tally[i] = 0ull;
 }
 
-// publish the participants (cell < ncells, Q >= 1) in their tile's list and
-// count them per cell, as the fused step kernel does for ecris_step
-__global__ void k_na_pack(unsigned char* base, uint32_t n, const uint32_t* __restrict__ cell,
-                          const uint8_t* __restrict__ q, const float* __restrict__ vx,
-                          const float* __restrict__ vy, const float* __restrict__ vz, uint32_t ncells)
+// record the participants (cell < ncells, Q >= 1) in their cells' buckets, as
+// the ions' pass does for ecris_step (whole warps: n rounded up)
+__global__ void k_na_pack(const __grid_constant__ RunDev R, uint32_t n, const uint32_t* __restrict__ cell,
+                          const uint8_t* __restrict__ q)
 {
-    uint4* plist = reinterpret_cast<uint4*>(base + kOffPlist);
-    float4* pvel = reinterpret_cast<float4*>(base + kOffPvel);
-    uint32_t* tcount = reinterpret_cast<uint32_t*>(base + kOffTcount);
-    uint32_t* ccount = reinterpret_cast<uint32_t*>(base + kOffCcount);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const uint32_t c = cell[i];
-        const uint32_t Q = q[i];
-        if (c >= ncells || Q == 0u || Q > 63u) continue;
-        const uint32_t t = i / kTile;
-        const uint32_t slot = t * kTile + atomicAdd(tcount + t, 1u);
-        plist[slot] = make_uint4(i, c, i, 0u);   // slot and id are both the array index
-        pvel[slot] = make_float4(vx[i], vy[i], vz[i], __uint_as_float(Q));
-        atomicAdd(ccount + c, 1u);
+    pdl_wait();
+    pdl_trigger();
+    const uint32_t end = (n + 31u) & ~31u;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < end; i += gridDim.x * blockDim.x) {
+        uint32_t c = kNoCell, Q = 0u;
+        float vx = 0.0f, vy = 0.0f, vz = 0.0f;
+        if (i < n) {
+            c = cell[i];
+            Q = q[i];
+            if (c >= R.ncells || Q == 0u || Q > 63u) c = kNoCell;
+            vx = R.vx[i];
+            vy = R.vy[i];
+            vz = R.vz[i];
+        }
+        place_warp(R, i, c, i, *R.step, vx, vy, vz, Q);   // slot and id are both the array index
     }
 }
 
@@ -173,14 +156,13 @@ extern "C" ecris_status ecris_coulomb_collide_noalloc(size_t n, const uint32_t* 
             e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             if (e != cudaSuccess) return na_cuda(e, "cudaDeviceGetAttribute");
             d.base = static_cast<unsigned char*>(p);
-            d.grid = sms * collide_blocks_per_sm();
+            d.grid = collide_blocks(sms);
             d.ready = true;
         }
         setup = d;
     }
     cudaStream_t s = (cudaStream_t)cuda_stream;
     unsigned char* base = setup.base;
-    const uint32_t tiles = (uint32_t)((n + kTile - 1) / kTile);
 
     // the parameter block the collision kernels read, pointing into the scratch
     RunDev R;
@@ -193,50 +175,37 @@ extern "C" ecris_status ecris_coulomb_collide_noalloc(size_t n, const uint32_t* 
     R.vy = vy;
     R.vz = vz;
     R.meta = events;
-    R.plist = reinterpret_cast<uint4*>(base + kOffPlist);
-    R.pvel = reinterpret_cast<float4*>(base + kOffPvel);
-    R.tcount = reinterpret_cast<uint32_t*>(base + kOffTcount);
-    R.ccount = reinterpret_cast<uint32_t*>(base + kOffCcount);
-    R.coff = reinterpret_cast<uint32_t*>(base + kOffCoff);
-    R.cstat = reinterpret_cast<unsigned long long*>(base + kOffCstat);
-    R.cctr = R.cstat + kNaScanTiles;
-    R.cstart = reinterpret_cast<uint32_t*>(base + kOffCstart);
-    R.crange = reinterpret_cast<uint32_t*>(base + kOffWords) + 4;
-    R.ckeys = reinterpret_cast<unsigned long long*>(base + kOffCkeys);
-    R.crec = reinterpret_cast<float4*>(base + kOffCrec);
-    R.cslot = reinterpret_cast<uint32_t*>(base + kOffCslot);
-    R.sslot = reinterpret_cast<uint32_t*>(base + kOffSslot);
-    R.tile = (uint32_t)kTile;   // the participant lists of k_na_pack, kTile slots a tile
+    R.ncells = ncells;
+    R.crec = reinterpret_cast<uint4*>(base + kOffRec);
+    R.cpool = kNaPool;
+    R.cover = kNaMaxIons;
+    R.cnext = reinterpret_cast<uint32_t*>(base + kOffNext);
+    R.chead = reinterpret_cast<uint32_t*>(base + kOffHead);
+    R.pcount = reinterpret_cast<uint32_t*>(base + kOffCcount);
+    R.uroom = kNaPool / ncells;
+    R.ucells = R.uroom > kRange ? 1u : (R.uroom < kRange / 32u ? 32u : kRange / R.uroom);
+    R.cidx = reinterpret_cast<uint32_t*>(base + kOffIdx);
+    R.cord = reinterpret_cast<uint32_t*>(base + kOffOrd);
+    R.cword = reinterpret_cast<uint32_t*>(base + kOffWords) + 16;
     R.nanbu = reinterpret_cast<const float*>(base + kOffNanbu);
     R.nanbu_lnlo = (float)std::log(kNanbuSLo);
     R.nanbu_inv_dln = (float)((kNanbuN - 1) / std::log(kNanbuSHi / kNanbuSLo));
     R.step = reinterpret_cast<uint32_t*>(base + kOffWords);
-    R.err = reinterpret_cast<uint32_t*>(base + kOffWords) + 2;
     R.tally = reinterpret_cast<unsigned long long*>(base + kOffTally);
-    unsigned int* ticket = reinterpret_cast<unsigned int*>(base + kOffWords) + 1;
 
-    const uint32_t span = ncells > tiles ? ncells : tiles;
-    k_na_init<<<(span + 255) / 256 > 0 ? (span + 255) / 256 : 1, 256, 0, s>>>(base, ncells, tiles, step);
-    if (n > 0)
-        k_na_pack<<<(uint32_t)((n + 255) / 256), 256, 0, s>>>(base, (uint32_t)n, cell, q, vx, vy, vz, ncells);
+    k_na_init<<<(ncells + 255) / 256, 256, 0, s>>>(base, ncells, step);
     e = cudaGetLastError();
+    if (e == cudaSuccess && n > 0)
+        e = launch_pdl(k_na_pack, dim3((uint32_t)((n + 255) / 256)), dim3(256), 0, s, R, (uint32_t)n, cell, q);
     if (e != cudaSuccess) return na_cuda(e, "launch");
-    e = launch_coulomb(R, ncells, tiles, ticket, setup.grid, 0u, 0, s);
+    e = launch_coulomb(R, (uint32_t)n, setup.grid, s);
     if (e != cudaSuccess) return na_cuda(e, "launch_coulomb");
     if (collisions_out) {
-        // the call synchronises: read the collision count and the error word
+        // the call synchronises: read the collision count
         unsigned long long c = 0;
-        uint32_t err = 0;
         e = cudaMemcpyAsync(&c, R.tally + kTallyCoulomb, sizeof c, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&err, R.err, sizeof err, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return na_cuda(e, "collision count");
-        if (err != 0u) {
-            ecris_internal_set_thread_error(
-                "coulomb_collide_noalloc: a bounded wait of the cell-count scan ran out (a call overlapping "
-                "this one on the GPU?); the velocities of this call are not valid");
-            return ECRIS_ETIMEOUT;
-        }
         *collisions_out = (int64_t)c;
     }
     return ECRIS_OK;

@@ -14,18 +14,6 @@
 namespace ecris {
 
 constexpr int kQSlots = 64;            // charge-state slots per tally array
-#ifndef ECRIS_TILE_VEC
-#define ECRIS_TILE_VEC 2
-#endif
-#ifndef ECRIS_STEP_MIN_BLOCKS
-#define ECRIS_STEP_MIN_BLOCKS 5
-#endif
-constexpr int kThreads = 256;                 // threads per block of the step kernel
-constexpr int kVec = ECRIS_TILE_VEC;          // particles per thread per tile
-constexpr int kTile = kThreads * kVec;        // particles per tile
-constexpr int kTileGroups = kTile / 4;        // float4 groups per tile
-constexpr int kStepMinBlocks = ECRIS_STEP_MIN_BLOCKS;   // resident step-kernel blocks per SM asked of ptxas
-
 // Tally words per run (u64): extracted[64], lost[64], kinetic energy of ions
 // that left (micro-eV), Coulomb pair collisions.
 constexpr int kTallyExtracted = 0;
@@ -71,20 +59,21 @@ constexpr uint32_t kFHasE = 1u << 16;   // internal: the run has a nonzero E gri
 
 constexpr uint32_t kNoCell = 0xFFFFFFFFu;
 
-// bounded waits: iterations of mbarrier.try_wait before a kernel gives up,
-// records ECRIS_ETIMEOUT (4) in the run's error word and stops its work
-constexpr uint32_t kWaitLimit = 1u << 20;
-constexpr uint32_t kErrTimeout = 4u;
-
 // Nanbu A(s) table: ln A tabulated on a uniform grid in ln s over [1e-3, 6]
 constexpr int kNanbuN = 2048;
 constexpr double kNanbuSLo = 1e-3;
 constexpr double kNanbuSHi = 6.0;
 
-// scan of the per-cell participant counts: cells per scan tile (one block)
-constexpr int kScanThreads = 256;
-constexpr int kScanPerThread = 8;     // a multiple of 4 (vector loads)
-constexpr int kScanBlock = kScanThreads * kScanPerThread;
+// words of RunDev::cword: the plan's planned cells and ranges; which of the two
+// sets of a step's counters is in use (the ions' pass of a step sets it, the
+// collision kernel clears the other set for the next step); the scratch
+// entries; then the sets, each the step's unplanned cells and overflow records
+constexpr int kCwPlanned = 0, kCwRanges = 1, kCwSet = 2, kCwHuge = 3, kCwUnplanned = 4, kCwOverflow = 5, kCwWords = 8;
+// Coulomb collisions: room (records) a range of cells spans; ions of several
+// cells that a warp sorts in registers, of one cell that a warp ranks, and of one
+// cell that a block holds in shared memory; warps a block
+constexpr uint32_t kRange = 128;
+constexpr int kWarpIons = 128, kWarpCell = 512, kBlockIons = 1024, kCollideWarps = 4;
 
 // Device parameter block of one run: FP32 constants of the kernels (built in
 // FP64 on the host) and the run's device arrays.
@@ -149,35 +138,37 @@ struct alignas(16) RunDev {
                                  // such bound), and the largest n_e of the cold and warm cells
     unsigned long long *dep;     // packed deposit accumulator: count << 32 | charge
     unsigned long long *tally;   // kTallyWords
-    uint4 *plist;                // Coulomb participants of each tile: (slot, cell, id, 0), `tile` slots a tile
-    float4 *pvel;                // their (vx, vy, vz, Q as bits), same slots
-    uint32_t *tcount;            // participants per tile
-    uint32_t *ccount;            // Coulomb participants per cell (counted up by the step kernel,
-                                 // counted back to zero by the scatter)
-    uint32_t *coff;              // exclusive scan of ccount, Nc + 1 entries
-    unsigned long long *cstat;   // scan tile status words (decoupled look-back), one per scan tile
-    unsigned long long *cctr;    // scan tile tickets handed out so far
-    uint32_t *cstart;            // first participant of each collision range (a range holds whole cells)
-    uint32_t *crange;            // [0] participants per range this step, [1] largest cell count seen by
-                                 // this step's scan (sets the next step's range size)
-    unsigned long long *ckeys;   // (pairing hash << 32 | pid) per participant, grouped by cell
-    float4 *crec;                // (vx, vy, vz, cell << 6 | Q as bits) per participant, grouped by cell
-    uint32_t *cslot;             // array slot of each participant, grouped by cell
-    uint32_t *sslot;             // scratch: pairing order of a range of cells too large for shared memory
+    uint4 *crec;                 // pool of 32-byte records of the step's Coulomb participants: (vx, vy, vz,
+                                 // meta word as bits), (array slot, words 0, 1, 2 of the stream-1 Philox block); the
+                                 // first cpool are the cells' buckets, the next cover the overflow
+    uint32_t cpool, cover;
+    uint32_t *cnext;             // per overflow record: the next of its cell's chain (record + 1, 0: none)
+    uint32_t *chead;             // per cell: its chain of overflow records (zero between steps)
+    uint32_t *ccount;            // per cell without a plan: its participants (zero between steps)
+    uint4 *cbkt;                 // per cell: its bucket (first record, room, planned place, 0); (kNoCell, 0, 0, 0):
+                                 // not planned
+    uint4 *pcell;                // planned cells by place: (first record, room, cell, 0) (nullptr: every cell c has
+                                 // place c and uroom records from c uroom)
+    uint32_t *pcount;            // their participants (zero between steps)
+    uint32_t *rstart;            // first planned place of each range
+    uint32_t ucells, uroom;      // without a plan: cells a range and records a cell
+    uint32_t *xcell;             // unplanned cells with participants this step
+    uint32_t *cidx, *cord;       // scratch of cells too large for shared memory, one word a participant each
+    uint32_t *cword;             // counters (kCw*)
     const float *nanbu;          // ln A at ln s = nanbu_lnlo + i / nanbu_inv_dln, i < kNanbuN
     float nanbu_lnlo, nanbu_inv_dln;
     uint32_t *step;              // device step counter of the run
-    uint32_t *leave;             // slots of the particles that left the chamber this step
-    uint32_t *nleave;            // their number (zero between steps); in a window of steps two counts:
-                                 // ions listed from the front of `leave`, atoms listed from its back
-    uint32_t *err;               // device error word: 0, or ECRIS_ETIMEOUT after a bounded wait ran out
+    uint32_t *leave;             // the window's listed particles by slot: ions from the front, atoms from the
+                                 // back (of 4 n4 entries)
+    uint32_t *nleave;            // [0], [1] their numbers (zero between windows), [2] with collisions between
+                                 // ions, the steps left in the window
+    uint32_t *err;               // device error word (0; a kernel that gave up would leave its status)
     uint32_t *birth;             // by particle id: step of the last ionisation from Q = 0 (~0: unknown)
     unsigned long long *fptd;    // [Q][kFptdBins] extraction counts by age bin, [Q] summed ages (steps),
                                  // [Q] summed extraction radii (nm)
     uint32_t n;                  // particles
     uint32_t n4;                 // float4 groups = ceil(n/4)
     uint32_t ncells;
-    uint32_t tile;               // particles per tile of the step kernel's launch shape
 };
 
 // ----------------------------------------------------------------------------
@@ -364,7 +355,8 @@ __device__ __forceinline__ int32_t to_fx_z(const RunDev& R, float z)
 
 // nearest-grid-point cell of a fixed-point position: with U = X + 2^31 the
 // cell is floor(U n / 2^32), the high word of a 32x32-bit product (exact)
-__device__ __forceinline__ uint32_t ngp_cell(const RunDev& R, int32_t X, int32_t Y, int32_t Z)
+template <class Mesh>
+__device__ __forceinline__ uint32_t ngp_cell(const Mesh& R, int32_t X, int32_t Y, int32_t Z)
 {
     const uint32_t ix = __umulhi((uint32_t)X ^ 0x80000000u, (uint32_t)R.nx);
     const uint32_t iy = __umulhi((uint32_t)Y ^ 0x80000000u, (uint32_t)R.ny);
@@ -388,28 +380,30 @@ struct ProbeDev {
 // ----------------------------------------------------------------------------
 // Launch wrappers (defined in step_kernel.cu / coulomb.cu)
 // ----------------------------------------------------------------------------
-// one pass of the fused step kernel over the run's ntiles tiles of kTile
-// particles; the particles that left the chamber are listed in R.leave
-cudaError_t launch_step(const RunDev& R, uint32_t ntiles, int grid, cudaStream_t s);
-// the leaver pass of a batch after it: crossing, tallies, re-emission and
-// deposit of the listed particles of every run; the lists are cleared (ticket:
-// a zeroed device word, left zero).  A run alone has it in the collisions'
-// scan kernel (launch_coulomb).
-constexpr int kLeaveBlocks = 64;
-cudaError_t launch_leave_batch(const RunDev* runs, uint32_t nruns, unsigned int* ticket, cudaStream_t s);
-// Up to kMaxWindow steps of a run without collisions between ions in two
-// launches (k_quiet, k_active): the atoms that neither leave nor ionise in the
-// window, then every other particle; the step counter advances by K.  R.leave
-// and R.nleave hold the list in between (ticket: a zeroed device word).
+// A window of up to kMaxWindow steps: launch_quiet takes the atoms that neither
+// leave nor ionise in it and lists every other particle (R.leave, R.nleave);
+// then launch_active takes the listed ones through all K steps and advances
+// the step counter by K (ticket: a zeroed device word, left zero), or, with
+// collisions between ions, each step is launch_ions and launch_coulomb, whose
+// last kernel advances the counter and, at the window's end, clears the list.
 constexpr uint32_t kMaxWindow = 32;
-constexpr uint32_t kActiveTile = 128;   // listed particles a block takes at a time
-cudaError_t launch_window(const RunDev& R, uint32_t K, unsigned int* ticket, int sm_count, cudaStream_t s);
+constexpr uint32_t kActiveTile = 128;   // threads a block of the passes over one run's list
+cudaError_t launch_quiet(const RunDev& R, uint32_t K, int sm_count, cudaStream_t s);
+cudaError_t launch_active(const RunDev& R, uint32_t K, unsigned int* ticket, int sm_count, cudaStream_t s);
+cudaError_t launch_ions(const RunDev& R, int sm_count, cudaStream_t s);
 // the same for every run of a batch: items are the (run, tile) work list of
-// `tile` particles a tile, pref nruns + 1 words of scratch, grid the blocks
+// `tile` particles a tile, pref 2 (nruns + 1) words of scratch, grid the
+// blocks; entries of runs with step == NULL are skipped.  variants: some run
+// has one of kFVariants or an on-axis table
+cudaError_t launch_quiet_batch(const RunDev* runs, uint32_t nruns, const uint2* items, uint32_t nitems, uint32_t tile,
+                               int threads, int grid, uint32_t K, uint32_t* pref, unsigned int* ticket,
+                               cudaStream_t s);
+cudaError_t launch_active_batch(const RunDev* runs, uint32_t nruns, int threads, int grid, bool variants, uint32_t K,
+                                const uint32_t* pref, unsigned int* ticket, cudaStream_t s);
+cudaError_t launch_ions_batch(const RunDev* runs, uint32_t nruns, int threads, int grid, bool variants,
+                              const uint32_t* pref, cudaStream_t s);
+// resident blocks per SM of the batch's passes
 int window_blocks_per_sm(int threads);
-cudaError_t launch_window_batch(const RunDev* runs, uint32_t nruns, const uint2* items, uint32_t nitems, uint32_t tile,
-                                int threads, int grid, bool variants, uint32_t K, uint32_t* pref,
-                                unsigned int* ticket, cudaStream_t s);
 cudaError_t launch_fold(const RunDev& R, uint32_t ncells, unsigned long long* count,
                         unsigned long long* charge, cudaStream_t s);
 // words of the rate table after its 8 kQSlots rates and shares: the atom gate and the
@@ -433,6 +427,8 @@ struct LoadCheck {
     float inlet_x, inlet_y, inlet_z;
     float inv_sxy_hi, inv_sxy_lo;   // metres -> fixed point, as an unevaluated FP32 sum
     float inv_sz_hi, inv_sz_lo;
+    int32_t nx, ny, nz;
+    uint32_t* count;                // ions per cell, added up for the first plan (nullptr: no collisions)
 };
 // check particles [0, n), convert their positions (metres, float) in place to
 // fixed point, build their meta words from q8 and ids, fill pads [n, cap);
@@ -449,12 +445,13 @@ struct ParticleSet {
 // Counting sort of the run's particles (in R) by (ion/atom, cell) into `dst`:
 // live ions first, then live atoms, each by cell; frozen and padding slots
 // last.  hist (2 Nc + 1 words) must be zero and is left zero; off (2 Nc + 2)
-// and blk (scan block totals) are scratch.  aos (the memory of `dst` as cap
+// and blk (scan block totals) are scratch.  plan (plan_blocks words, or
+// NULL): also plan the collisions' buckets from the counts.  aos (the memory of `dst` as cap
 // 32-byte records, or NULL): for input in arbitrary order (the first sort
 // after a load), move records there and unpack them back into the arrays of
 // R, which then hold the sorted particles; NULL writes `dst` directly.
 cudaError_t launch_sort(const RunDev& R, uint32_t cap, const ParticleSet& dst, uint32_t* hist, uint32_t* off,
-                        uint32_t* blk, uint4* aos, cudaStream_t s);
+                        uint32_t* blk, unsigned long long* plan, uint4* aos, cudaStream_t s);
 int sort_scan_blocks(uint32_t nbins);
 // state in load order: out[id[slot]] = state[slot] for id < n (positions to
 // metres), into device arrays; rec: scratch of n 32-byte records (not `out`),
@@ -465,29 +462,15 @@ cudaError_t launch_census(const RunDev& R, uint32_t n4, unsigned long long* cens
 // add the current particles to the probes' sums (probe.cu)
 cudaError_t launch_probe(const RunDev& R, const ProbeDev& P, uint32_t n4, int sm_count, cudaStream_t s);
 
-// resident blocks per SM of the step kernel
-int step_blocks_per_sm();
-// Launch shapes of the batched step kernel: threads per block x particles per
-// thread and tile, shape k = (kShapeThreads[k], kShapeVec[k]); tile sizes
-// from 128 to 2048 particles
+// Launch shapes of a batch's passes: threads per block x particles per thread
+// and tile of the atoms' pass.  (The stages of a shape belong to its name in
+// ecris_tuning; no kernel has stages.)
 constexpr int kStepShapes = 12;
-constexpr int kDefaultShape = 11;   // 256 x 2 with three stages
+constexpr int kDefaultShape = 11;
 constexpr int kShapeThreads[kStepShapes] = {128, 128, 128, 256, 256, 256, 512, 512, 512, 128, 256, 256};
 constexpr int kShapeVec[kStepShapes] = {1, 2, 4, 1, 2, 4, 1, 2, 4, 2, 1, 2};
 constexpr int kShapeStages[kStepShapes] = {2, 2, 2, 2, 2, 2, 2, 2, 2, 3, 3, 3};
-constexpr int kMinTile = 128, kMaxTile = 2048;
 inline uint32_t shape_tile(int k) { return (uint32_t)(kShapeThreads[k] * kShapeVec[k]); }
-int step_batch_blocks_per_sm(int shape);
-// batch form: one persistent step-kernel launch over the work items (run,
-// tile) of many runs whose parameter blocks are in device memory (it leaves
-// the step counters alone); the batch leaver pass then advances the counters
-// of the runs without Coulomb collisions (the collision kernels of the
-// others, launched after it, advance theirs); entries with step == NULL are
-// skipped
-// variants: launch the kernel with the opt-in processes' code (some run has
-// one of kFVariants)
-cudaError_t launch_step_batch(const RunDev* runs, const uint2* items, uint32_t nitems, int grid, bool variants,
-                              int shape, cudaStream_t s);
 // message returned by ecris_last_error(NULL) on the calling thread
 void ecris_internal_set_thread_error(const char* msg);
 // host: ln A(s) of Nanbu's scattering law on kNanbuN points uniform in ln s
@@ -516,30 +499,67 @@ ecris_status batch_autotune(ecris_batch* b, uint32_t trial_steps, bool cadence, 
 void batch_snapshot_diag(const ecris_batch* b, int32_t run, const TallySnapshot& snap, uint64_t steps,
                          ecris_diag_out* out);
 
-// Coulomb collisions of one run for the current step, after the step
-// kernel: scan of the cell counts, scatter of the pairing keys, and the
-// per-cell sort / pair / collide kernel, whose last block advances the step
-// counter and clears the leaver list.  leave_blocks extra blocks of the scan
-// kernel (the same count at every launch of a run: kLeaveBlocks for one run,
-// 0 in a batch) run the step's leaver pass if do_leave, in place of
-// launch_leave; else the leavers were finished before, by launch_leave or
-// the batch's pass.
-constexpr int kCoulombKernels = 3;   // kernels per launch_coulomb
-// participants per range of cells of the collision kernel: the first step
-// after a load takes kCellIons; each later step takes kCellCap minus the
-// largest cell count of the step before, within [kCellIonsMin, kCellIonsMax],
-// so that a range (its cells whole) still fits in shared memory while ranges
-// stay as large as it allows (fewer ranges, fewer per-range waits)
-constexpr int kCellIons = 512;
-constexpr int kCellIonsMin = 256, kCellIonsMax = 896;
-constexpr int kCellCap = 1024;       // participants of a range held in shared memory
-cudaError_t launch_coulomb(const RunDev& R, uint32_t ncells, uint32_t ntiles, unsigned int* ticket, int grid,
-                           uint32_t leave_blocks, int do_leave, cudaStream_t s);
-// the cell-count scan of the collisions, with leave_blocks extra blocks for
-// the leaver pass (step_kernel.cu)
-cudaError_t launch_scan(const RunDev& R, uint32_t ncells, uint32_t nscan, uint32_t leave_blocks, int do_leave,
-                        cudaStream_t s);
-int coulomb_scan_blocks(uint32_t ncells);
-int collide_blocks_per_sm();
+// Coulomb collisions (coulomb.cu).  launch_plan: the buckets of every cell
+// from `count` ions per cell (blk: plan_blocks words of scratch; zero: count is
+// left zero).  Any plan is valid, one of
+// the present counts is fast.  launch_coulomb: the collisions of one step
+// after its ions' pass, in a kernel that also advances the step counter and,
+// at the window's end, clears the list; n: the run's particles (all runs' in a
+// batch).
+uint32_t plan_blocks(uint32_t ncells);
+cudaError_t launch_plan(const RunDev& R, uint32_t* count, bool zero, unsigned long long* blk, cudaStream_t s);
+constexpr int kCoulombKernels = 1;   // kernels per launch_coulomb
+int collide_blocks(int sm_count);    // most blocks of the collision kernel
+cudaError_t launch_coulomb(const RunDev& R, uint32_t n, int most, cudaStream_t s);
+cudaError_t launch_coulomb_batch(const RunDev* runs, uint32_t nruns, uint32_t n, int most, cudaStream_t s);
+
+// a 32-byte record in one store: one full sector, one request to L2
+__device__ __forceinline__ void store_record(uint4* rec, size_t d, const uint4& a, const uint4& b)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(rec + 2 * d), "r"(a.x), "r"(a.y),
+                 "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+
+// Record this lane's Coulomb participant (ck != kNoCell) in its cell's bucket,
+// or in the overflow chained to the cell when the bucket is full; the whole warp
+// calls this.  One returning atomic per run of neighbouring lanes in the same
+// cell.
+__device__ __forceinline__ void place_warp(const RunDev& R, uint32_t slot, uint32_t ck, uint32_t id, uint32_t step,
+                                           float vx, float vy, float vz, uint32_t meta)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    const bool in = ck != kNoCell;
+    if (!__any_sync(0xFFFFFFFFu, in)) return;
+    const uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, ck, 1);
+    const uint32_t heads = __ballot_sync(0xFFFFFFFFu, lane == 0 || prev != ck);
+    const uint32_t upto = 0xFFFFFFFFu >> (31u - lane);              // lanes 0..lane
+    const uint32_t after = heads & ~upto;                            // run heads above this lane
+    const uint32_t tl = after ? (uint32_t)(__ffs(after) - 2) : 31u;  // last lane of this lane's run
+    const uint32_t h = 31u - (uint32_t)__clz(heads & upto);           // first lane of this lane's run
+    uint4 bk = make_uint4(0u, 0u, 0u, 0u);
+    if (in) bk = R.cbkt ? __ldg(R.cbkt + ck) : make_uint4(ck * R.uroom, R.uroom, ck, 0u);
+    uint32_t k = 0u;
+    if (in && lane == h) k = atomicAdd(bk.x == kNoCell ? R.ccount + ck : R.pcount + bk.z, tl - h + 1u);
+    const Words w = rng_words(R, id, step, 1u);
+    k = __shfl_sync(0xFFFFFFFFu, k, h) + (lane - h);
+    uint32_t p = k < bk.y ? bk.x + k : kNoCell;
+    const uint32_t over = __ballot_sync(0xFFFFFFFFu, in && k >= bk.y);
+    if (over) {
+        uint32_t o = 0u;
+        const uint32_t first = (uint32_t)(__ffs(over) - 1);
+        uint32_t* const words = R.cword + 2u * (step & 1u);   // the step's set of counters
+        if (lane == first) o = atomicAdd(words + kCwOverflow, (uint32_t)__popc(over));
+        o = __shfl_sync(0xFFFFFFFFu, o, first) + (uint32_t)__popc(over & (upto >> 1));
+        if (in && k >= bk.y && o < R.cover) {
+            p = R.cpool + o;
+            R.cnext[o] = atomicExch(R.chead + ck, p + 1u);
+            if (bk.x == kNoCell && k == 0u) R.xcell[atomicAdd(words + kCwUnplanned, 1u)] = ck;
+        }
+    }
+    if (in && p != kNoCell)
+        store_record(R.crec, p, make_uint4(__float_as_uint(vx), __float_as_uint(vy), __float_as_uint(vz), meta),
+                     make_uint4(slot, w.w0, w.w1, w.w2));
+}
 
 }  // namespace ecris

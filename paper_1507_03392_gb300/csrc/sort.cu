@@ -140,14 +140,6 @@ __global__ void __launch_bounds__(kSortThreads) k_scan3(uint32_t* __restrict__ o
         if (base + j < n) out[base + j] += add;
 }
 
-// a 32-byte record in one store: one full sector, one request to L2
-__device__ __forceinline__ void store_record(uint4* rec, uint32_t d, const uint4& a, const uint4& b)
-{
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(rec + 2 * (size_t)d), "r"(a.x),
-                 "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
-                 : "memory");
-}
-
 // kRecords: write 32-byte records to aos (unpacked by k_sort_unpack), else
 // the destination arrays
 template <bool kRecords>
@@ -285,7 +277,7 @@ int grid_for(uint32_t n, int threads, int cap_blocks)
 int sort_scan_blocks(uint32_t nbins) { return (int)((nbins + kSortScanBlock - 1) / kSortScanBlock); }
 
 cudaError_t launch_sort(const RunDev& R, uint32_t cap, const ParticleSet& dst, uint32_t* hist, uint32_t* off,
-                        uint32_t* blk, uint4* aos, cudaStream_t s)
+                        uint32_t* blk, unsigned long long* plan, uint4* aos, cudaStream_t s)
 {
     const uint32_t nbins = 2u * R.ncells + 1u;
     const int nb = sort_scan_blocks(nbins);
@@ -293,6 +285,10 @@ cudaError_t launch_sort(const RunDev& R, uint32_t cap, const ParticleSet& dst, u
     k_scan1<<<nb, kSortThreads, 0, s>>>(hist, off, blk, nbins);
     k_scan2<<<1, 1024, 0, s>>>(blk, (uint32_t)nb, off, nbins);
     k_scan3<<<nb, kSortThreads, 0, s>>>(off, blk, nbins);
+    if (plan) {
+        const cudaError_t e = launch_plan(R, hist, false, plan, s);
+        if (e != cudaSuccess) return e;
+    }
     if (aos) {
         k_sort_move<true><<<grid_for(cap, 256, 8192), 256, 0, s>>>(R, cap, dst, aos, hist, off);
         const ParticleSet src{R.x, R.y, R.z, R.vx, R.vy, R.vz, R.meta, R.id};
