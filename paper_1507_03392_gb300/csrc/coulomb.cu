@@ -26,7 +26,7 @@
 //     their ids if the words tie;
 //   - triplets, three collisions in a row, and larger cells are put by for the
 //     block, whose threads take a triplet each and a large cell together (ranked
-//     the same way, or above kBlockIons by counting in global memory).
+//     the same way, above kBlockIons ions in windows of their words).
 //
 // A collision of ions a, b (same mass M, charges Qa, Qb) over time dt_c uses
 //   s = lnL/(4 pi) (Qa Qb e^2 / (eps0 mu))^2 n g^-3 dt_c,  mu = M/2,
@@ -313,15 +313,14 @@ __device__ __forceinline__ void collide_triplet(const RunDev& R, uint32_t ia, ui
 // ---------------------------------------------------------------------------
 // The cells
 // ---------------------------------------------------------------------------
-// Shared memory of a block that takes one cell of up to kBlockIons ions
+// Shared memory of a block that ranks up to kBlockIons ions of one cell
 struct CellSmem {
-    uint32_t pidx[kBlockIons];            // record of each ion
-    uint32_t word[kBlockIons];            // its first word
-    uint32_t cnt[kBlockIons + 1];         // ions per word bucket, then their exclusive scan
-    uint32_t start[kBlockIons / 2 + 1];   // sorted places that start a pair
+    uint32_t word[kBlockIons];            // first words
+    uint32_t rec[kBlockIons];             // the ions' places in the cell
+    uint32_t cnt2[kBlockIons / 2 + 1];    // ions per word bucket, then their exclusive scan, two 16-bit counts a word
     uint16_t pos[kBlockIons];             // arrival in the word bucket
     uint16_t arr[kBlockIons];             // ions by word bucket
-    uint16_t ord[kBlockIons];             // ions in order
+    uint32_t n;
 };
 
 // particle id at an array slot (the slot where there are no ids)
@@ -335,114 +334,161 @@ __device__ __forceinline__ uint32_t record_id(const RunDev& R, uint32_t p)
 // a cell that takes a block: (first record, room, ions, chain)
 using BigCell = uint4;
 
-// Order and collide the ions of one cell by the block
-__device__ __forceinline__ void collide_cell(const RunDev& R, CellSmem& S, const BigCell& b)
+// the record of ion j of a cell (idx: those past its bucket)
+__device__ __forceinline__ uint32_t cell_record(const BigCell& b, const uint32_t* idx, uint32_t j)
+{
+    return j < b.y ? b.x + j : idx[j];
+}
+
+// Order and collide the ions of one cell by the block.  The words are uniform,
+// so a cell of more ions than the shared memory holds is ranked in windows of
+// equal word ranges, each of them holding 7/8 of kBlockIons on average (a window
+// that is too full all the same is halved); the order goes to global scratch.
+__device__ __forceinline__ void collide_cell(const RunDev& R, CellSmem& S, const BigCell& b, uint32_t* s_off)
 {
     constexpr uint32_t T = 32 * kCollideWarps;
-    const uint32_t g = threadIdx.x, M = b.z, room = min(b.y, b.z);
-    for (uint32_t j = g; j <= M; j += T) S.cnt[j] = 0u;
-    for (uint32_t j = g; j < room; j += T) S.pidx[j] = b.x + j;
+    const uint32_t g = threadIdx.x, M = b.z;
+    if (g == 0) *s_off = atomicAdd(R.cword + kCwHuge, M);
+    __syncthreads();
+    const uint32_t off = *s_off;
+    if (off + M > R.cover) return;   // (the scratch holds every participant)
+    uint32_t* const idx = R.cidx + off;
+    uint32_t* const ord = R.cord + off;
     if (g == 0) {
         uint32_t at = b.w;
-        for (uint32_t i = room; i < M; ++i) {
-            S.pidx[i] = at ? at - 1u : R.cpool;   // (a chain holds as many as the count says)
+        for (uint32_t i = b.y; i < M; ++i) {
+            idx[i] = at ? at - 1u : R.cpool;   // (a chain holds as many as the count says)
             if (at) at = R.cnext[at - 1u - R.cpool];
         }
     }
-    __syncthreads();
-    for (uint32_t j = g; j < M; j += T) {
-        const uint32_t w = R.crec[2 * (size_t)S.pidx[j] + 1].y;
-        S.word[j] = w;
-        S.pos[j] = (uint16_t)atomicAdd(&S.cnt[__umulhi(w, M)], 1u);
-    }
-    __syncthreads();
-    // exclusive scan of the bucket counts
-    constexpr int kPer = kBlockIons / T;
-    uint32_t v[kPer], sum = 0u;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        v[k] = g * kPer + k < M ? S.cnt[g * kPer + k] : 0u;
-        sum += v[k];
-    }
-    unsigned long long total;
-    uint32_t o = (uint32_t)block_excl64<T>(sum, &total);
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        if (g * kPer + k < M) S.cnt[g * kPer + k] = o;
-        o += v[k];
-    }
-    if (g == 0) S.cnt[M] = M;
-    __syncthreads();
-    for (uint32_t j = g; j < M; j += T) S.arr[S.cnt[__umulhi(S.word[j], M)] + S.pos[j]] = (uint16_t)j;
-    __syncthreads();
-    for (uint32_t j = g; j < M; j += T) {
-        const uint32_t w = S.word[j], k = __umulhi(w, M);
-        const uint32_t lo = S.cnt[k], hi = S.cnt[k + 1];
-        uint32_t r = lo;
-        for (uint32_t t = lo; t < hi; ++t) {
-            const uint32_t i = S.arr[t], wi = S.word[i];
-            if (wi < w || (wi == w && i != j && record_id(R, S.pidx[i]) < record_id(R, S.pidx[j]))) ++r;
+    unsigned long long width = (1ull << 32) / ((M + kBlockIons * 7u / 8u - 1u) / (kBlockIons * 7u / 8u)) + 1ull;
+    if (M <= (uint32_t)kBlockIons) width = 1ull << 32;
+    uint32_t done = 0u;
+    for (unsigned long long lo = 0ull; lo < (1ull << 32);) {
+        // the window's ions
+        __syncthreads();
+        if (g == 0) S.n = 0u;
+        for (uint32_t k = g; k < (uint32_t)kBlockIons / 2u + 1u; k += T) S.cnt2[k] = 0u;
+        __syncthreads();
+        for (uint32_t j = g; j < M; j += T) {
+            const uint32_t w = R.crec[2 * (size_t)cell_record(b, idx, j) + 1].y;
+            if (w < lo || w - lo >= width) continue;
+            const uint32_t at = atomicAdd(&S.n, 1u);
+            if (at < (uint32_t)kBlockIons) {
+                S.word[at] = w;
+                S.rec[at] = j;
+            }
         }
-        S.ord[r] = (uint16_t)j;
+        __syncthreads();
+        const uint32_t n = S.n;
+        if (n > (uint32_t)kBlockIons && width > 1ull) {
+            width = (width + 1ull) / 2ull;
+            continue;
+        }
+        if (n > (uint32_t)kBlockIons) {   // one word for so many ions: in the order of their ids
+            for (uint32_t j = g; j < M; j += T) {
+                const uint32_t p = cell_record(b, idx, j), id = record_id(R, p);
+                if (R.crec[2 * (size_t)p + 1].y != (uint32_t)lo) continue;
+                uint32_t r = 0u;
+                for (uint32_t i = 0; i < M; ++i) {
+                    const uint32_t pi = cell_record(b, idx, i);
+                    if (R.crec[2 * (size_t)pi + 1].y == (uint32_t)lo && record_id(R, pi) < id) ++r;
+                }
+                ord[done + r] = p;
+            }
+            done += n;
+            lo += 1ull;
+            continue;
+        }
+        // ranked by counting into n buckets of its range
+        const float scale = (float)n / (float)width;   // (any monotone rule will do)
+        const uint16_t* const cnt = reinterpret_cast<const uint16_t*>(S.cnt2);
+        auto bucket = [&](uint32_t w) { return min((uint32_t)((float)(w - (uint32_t)lo) * scale), n - 1u); };
+        for (uint32_t j = g; j < n; j += T) {
+            const uint32_t k = bucket(S.word[j]), sh = 16u * (k & 1u);
+            S.pos[j] = (uint16_t)(atomicAdd(&S.cnt2[k >> 1], 1u << sh) >> sh);
+        }
+        __syncthreads();
+        {
+            constexpr int kPer = kBlockIons / 2 / (int)T;
+            uint32_t v[kPer], sum = 0u;
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                v[k] = S.cnt2[g * kPer + k];
+                sum += (v[k] & 0xFFFFu) + (v[k] >> 16);
+            }
+            unsigned long long total;
+            uint32_t o = (uint32_t)block_excl64<T>(sum, &total);
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                const uint32_t c = v[k] & 0xFFFFu;
+                S.cnt2[g * kPer + k] = o | ((o + c) << 16);
+                o += c + (v[k] >> 16);
+            }
+            if (g == 0) S.cnt2[kBlockIons / 2] = n;
+        }
+        __syncthreads();
+        for (uint32_t j = g; j < n; j += T) S.arr[cnt[bucket(S.word[j])] + S.pos[j]] = (uint16_t)j;
+        __syncthreads();
+        for (uint32_t j = g; j < n; j += T) {
+            const uint32_t w = S.word[j], k = bucket(w);
+            const uint32_t first = cnt[k], end = cnt[k + 1];
+            uint32_t r = first;
+            for (uint32_t t = first; t < end; ++t) {
+                const uint32_t i = S.arr[t], wi = S.word[i];
+                if (wi < w || (wi == w && i != j && record_id(R, cell_record(b, idx, S.rec[i])) <
+                                                        record_id(R, cell_record(b, idx, S.rec[j]))))
+                    ++r;
+            }
+            ord[done + r] = cell_record(b, idx, S.rec[j]);
+        }
+        done += n;
+        lo += width;
     }
     __syncthreads();
     // the triplet to the last thread, the pairs from the first
     const uint32_t first = (M & 1u) ? 3u : 0u, np = (M - first) / 2u;
-    if (first && g == T - 1u)
-        collide_triplet(R, S.pidx[S.ord[0]], S.pidx[S.ord[1]], S.pidx[S.ord[2]], (float)M);
-    for (uint32_t e = g; e < np; e += T)
-        collide_pair(R, S.pidx[S.ord[first + 2 * e]], S.pidx[S.ord[first + 2 * e + 1]], (float)M);
+    if (first && g == T - 1u) collide_triplet(R, ord[0], ord[1], ord[2], (float)M);
+    for (uint32_t e = g; e < np; e += T) collide_pair(R, ord[first + 2u * e], ord[first + 2u * e + 1u], (float)M);
     __syncthreads();   // the shared memory is used again
 }
 
 // collisions of a cell of m >= 2 ions
 __device__ __forceinline__ uint32_t collisions_of(uint32_t m) { return (m & 1u) ? 3u + (m - 3u) / 2u : m / 2u; }
 
-template <int kT>
-__device__ __forceinline__ void group_sync()
+// A large cell by a warp alone, in global memory, should the block's list of them
+// be full: the rank by counting smaller (word, id)
+__device__ __forceinline__ void collide_warp_large(const RunDev& R, const BigCell& b)
 {
-    if (kT == 32) __syncwarp();
-    else __syncthreads();
-}
-
-// A cell of more than kBlockIons ions, in global memory, by a warp or a block
-// of kT threads of which this is thread g (told: a word they share): its records'
-// indices to cidx, their places to cord, and the rank by counting smaller
-// (word, id)
-template <int kT>
-__device__ __forceinline__ void collide_huge(const RunDev& R, const BigCell b, uint32_t g, uint32_t* told)
-{
-    const uint32_t room = min(b.y, b.z), m = b.z;
-    if (g == 0) *told = atomicAdd(R.cword + kCwHuge, m);
-    group_sync<kT>();
-    const uint32_t off = *told;
-    group_sync<kT>();
+    const uint32_t g = threadIdx.x & 31, m = b.z;
+    uint32_t off = 0u;
+    if (g == 0) off = atomicAdd(R.cword + kCwHuge, m);
+    off = __shfl_sync(0xFFFFFFFFu, off, 0);
     if (off + m > R.cover) return;   // (the scratch holds every participant)
-    uint32_t* idx = R.cidx + off;
-    uint32_t* ord = R.cord + off;
-    for (uint32_t i = g; i < room; i += kT) idx[i] = b.x + i;
+    uint32_t* const idx = R.cidx + off;
+    uint32_t* const ord = R.cord + off;
     if (g == 0) {
         uint32_t at = b.w;
-        for (uint32_t i = room; i < m; ++i) {
+        for (uint32_t i = b.y; i < m; ++i) {
             idx[i] = at ? at - 1u : R.cpool;
             if (at) at = R.cnext[at - 1u - R.cpool];
         }
     }
-    group_sync<kT>();
-    for (uint32_t j = g; j < m; j += kT) {
-        const uint32_t p = idx[j], w = R.crec[2 * (size_t)p + 1].y;
+    __syncwarp();
+    for (uint32_t j = g; j < m; j += 32u) {
+        const uint32_t p = cell_record(b, idx, j), w = R.crec[2 * (size_t)p + 1].y;
         uint32_t r = 0u;
         for (uint32_t i = 0; i < m; ++i) {
-            const uint32_t wo = R.crec[2 * (size_t)idx[i] + 1].y;
-            if (wo < w || (wo == w && i != j && record_id(R, idx[i]) < record_id(R, p))) ++r;
+            const uint32_t pi = cell_record(b, idx, i), wi = R.crec[2 * (size_t)pi + 1].y;
+            if (wi < w || (wi == w && i != j && record_id(R, pi) < record_id(R, p))) ++r;
         }
         ord[r] = p;
     }
-    group_sync<kT>();
+    __syncwarp();
     const uint32_t first = (m & 1u) ? 3u : 0u;
     if (first && g == 0) collide_triplet(R, ord[0], ord[1], ord[2], (float)m);
-    for (uint32_t p = first + 2u * g; p < m; p += 2u * kT) collide_pair(R, ord[p], ord[p + 1], (float)m);
-    group_sync<kT>();
+    for (uint32_t p = first + 2u * g; p < m; p += 64u) collide_pair(R, ord[p], ord[p + 1], (float)m);
+    __syncwarp();
 }
 
 // Shared memory of a warp: up to kWarpIons ions of up to 32 cells
@@ -485,7 +531,7 @@ struct BlockSmem {
     AnySmem a;
     BigCell big[kBigs];
     const RunDev* big_run[kBigs];
-    uint32_t ntrip, nbig, off[kCollideWarps];
+    uint32_t ntrip, nbig, off;
 };
 
 // element exchange of the bitonic network: keep the smaller or the larger
@@ -800,7 +846,7 @@ __device__ __forceinline__ void collide_item(const RunDev& R, WarpSmem& S, Block
                     B.big_run[at] = &R;
                 }
             } else {   // no room for it (more than kBigs such cells in a few items): the warp does it
-                collide_huge<32>(R, big, lane, B.off + threadIdx.x / 32u);
+                collide_warp_large(R, big);
                 ncoll += collisions_of(cm);
             }
             continue;
@@ -831,8 +877,7 @@ __device__ __forceinline__ void collide_item(const RunDev& R, WarpSmem& S, Block
 // a large cell, by the block
 __device__ __forceinline__ void collide_big(const RunDev& R, BlockSmem& B, const BigCell& b)
 {
-    if (b.z <= (uint32_t)kBlockIons) collide_cell(R, B.a.cell, b);
-    else collide_huge<32 * kCollideWarps>(R, b, threadIdx.x, B.off);
+    collide_cell(R, B.a.cell, b, &B.off);
     if (threadIdx.x == 0) atomicAdd(R.tally + kTallyCoulomb, (unsigned long long)collisions_of(b.z));
 }
 

@@ -70,10 +70,10 @@ constexpr double kNanbuSHi = 6.0;
 // entries; then the sets, each the step's unplanned cells and overflow records
 constexpr int kCwPlanned = 0, kCwRanges = 1, kCwSet = 2, kCwHuge = 3, kCwUnplanned = 4, kCwOverflow = 5, kCwWords = 8;
 // Coulomb collisions: room (records) a range of cells spans; ions of several
-// cells that a warp sorts in registers, of one cell that a warp ranks, and of one
-// cell that a block holds in shared memory; warps a block
+// cells that a warp sorts in registers, of one cell that a warp ranks, and that a
+// block ranks at a time; warps a block
 constexpr uint32_t kRange = 128;
-constexpr int kWarpIons = 128, kWarpCell = 512, kBlockIons = 1024, kCollideWarps = 4;
+constexpr int kWarpIons = 128, kWarpCell = 512, kBlockIons = 1792, kCollideWarps = 4;
 
 // Device parameter block of one run: FP32 constants of the kernels (built in
 // FP64 on the host) and the run's device arrays.
