@@ -288,6 +288,10 @@ struct KernelTimer {
 
 }  // namespace
 
+// the counters that a load clears: tallies, first-passage sums, and the words
+// step, nleave[3], ticket, err, bad[2], cword[kCwWords]
+constexpr size_t kZeroBytes = (kTallyWords + kFptdWords) * sizeof(unsigned long long) + (8 + kCwWords) * sizeof(uint32_t);
+
 constexpr uint32_t kSortAfterLoad = 8;   // steps of one ecris_step call that sort a fresh load first
 
 // what a captured step graph bakes in: the parameter block (by value) and
@@ -319,6 +323,11 @@ struct ecris_ctx {
     size_t cap = 0, cap_cells = 0;
     size_t n = 0, n4 = 0;
     uint8_t* d_q8 = nullptr;
+    // arrays that a load clears, in few allocations so that it clears them in
+    // few calls: the counters (d_zero: tallies, first-passage sums, then the
+    // words from d_step on), the time sums per cell (d_dep, d_count, d_charge,
+    // d_mark) and the collisions' counts (d_ccount, d_chead, d_pcount)
+    unsigned long long* d_zero = nullptr;
     unsigned int* d_bad = nullptr;
     uint32_t* d_err = nullptr;
     // Coulomb collisions: see RunDev
@@ -335,7 +344,6 @@ struct ecris_ctx {
     uint32_t* d_cord = nullptr;
     uint32_t* d_cword = nullptr;
     unsigned long long* d_plan = nullptr;   // block sums of the plan
-    bool planned = false;       // the buckets were planned since the load
     int collide_grid = 0;       // most blocks of the collision kernel
     // two sets of particle arrays, each the eight arrays of one allocation
     // (d_set: 8 cap words, so that a set not in use also serves as cap 32-byte
@@ -450,34 +458,24 @@ void free_ions(ecris_ctx* ctx)
     free_async(ctx, ctx->d_hoff);
     free_async(ctx, ctx->d_hblk);
     free_async(ctx, ctx->d_dep);
-    free_async(ctx, ctx->d_count);
-    free_async(ctx, ctx->d_charge);
-    free_async(ctx, ctx->d_mark);
     free_async(ctx, ctx->d_ne64);
-    free_async(ctx, ctx->d_tally);
+    free_async(ctx, ctx->d_zero);
     free_async(ctx, ctx->d_census);
-    free_async(ctx, ctx->d_step);
     free_async(ctx, ctx->d_leave);
     free_async(ctx, ctx->d_birth);
-    free_async(ctx, ctx->d_fptd);
-    free_async(ctx, ctx->d_nleave);
-    free_async(ctx, ctx->d_ticket);
     free_async(ctx, ctx->d_q8);
-    free_async(ctx, ctx->d_bad);
-    free_async(ctx, ctx->d_err);
     free_async(ctx, ctx->d_crec);
     free_async(ctx, ctx->d_cnext);
-    free_async(ctx, ctx->d_chead);
     free_async(ctx, ctx->d_ccount);
     free_async(ctx, ctx->d_cbkt);
     free_async(ctx, ctx->d_pcell);
-    free_async(ctx, ctx->d_pcount);
     free_async(ctx, ctx->d_rstart);
     free_async(ctx, ctx->d_xcell);
     free_async(ctx, ctx->d_cidx);
     free_async(ctx, ctx->d_cord);
-    free_async(ctx, ctx->d_cword);
     free_async(ctx, ctx->d_plan);
+    // (these lie in the allocations above)
+    ctx->d_chead = ctx->d_pcount = ctx->d_cword = nullptr;
     ctx->have_ions = false;
     ctx->loaded = false;
     ctx->cap = ctx->cap_cells = 0;
@@ -932,13 +930,11 @@ ecris_status sort_particles(ecris_ctx* ctx)
     const size_t cap4 = 4 * ctx->n4;
     uint4* aos = ctx->fresh ? reinterpret_cast<uint4*>(dst.x) : nullptr;
     CK(timed(ctx, kKindOther, [&] {
-        return launch_sort(*ctx->h_run, (uint32_t)cap4, dst, ctx->d_hist, ctx->d_hoff, ctx->d_hblk, ctx->d_plan, aos,
-                           ctx->stream);
-    }, (aos ? 7 : 6) + (ctx->d_plan ? 3 : 0)));
+        // (the load planned the collisions' buckets for its own order)
+        return launch_sort(*ctx->h_run, (uint32_t)cap4, dst, ctx->d_hist, ctx->d_hoff, ctx->d_hblk,
+                           aos ? nullptr : ctx->d_plan, aos, ctx->stream);
+    }, aos ? 7 : (ctx->d_plan ? 9 : 6)));
     ctx->since_sort = 0;
-    if (ctx->d_ccount && !ctx->planned)   // the load's counts were for a plan that is not needed now
-        CK(cudaMemsetAsync(ctx->d_ccount, 0, ctx->cap_cells * sizeof(uint32_t), ctx->stream));
-    ctx->planned = true;
     if (ctx->fresh) {
         ctx->fresh = false;
         return ECRIS_OK;
@@ -1237,37 +1233,41 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
                            ctx->stream));
         CK(cudaMemsetAsync(ctx->d_hist, 0, (2 * nc + 1) * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_q8, cap, ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_dep, nc * sizeof(unsigned long long), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_count, nc * sizeof(unsigned long long), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_charge, nc * sizeof(unsigned long long), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_mark, nc * sizeof(unsigned long long), ctx->stream));
+        CK(cudaMallocAsync((void**)&ctx->d_dep, 4 * nc * sizeof(unsigned long long), ctx->stream));
+        ctx->d_count = ctx->d_dep + nc;
+        ctx->d_charge = ctx->d_dep + 2 * nc;
+        ctx->d_mark = ctx->d_dep + 3 * nc;
         CK(cudaMallocAsync((void**)&ctx->d_ne64, nc * sizeof(double), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_tally, kTallyWords * sizeof(unsigned long long), ctx->stream));
+        CK(cudaMallocAsync((void**)&ctx->d_zero, kZeroBytes, ctx->stream));
+        ctx->d_tally = ctx->d_zero;
+        ctx->d_fptd = ctx->d_zero + kTallyWords;
+        {
+            uint32_t* w = reinterpret_cast<uint32_t*>(ctx->d_fptd + kFptdWords);
+            ctx->d_step = w;
+            ctx->d_nleave = w + 1;
+            ctx->d_ticket = w + 4;
+            ctx->d_err = w + 5;
+            ctx->d_bad = w + 6;
+            ctx->d_cword = w + 8;
+        }
         CK(cudaMallocAsync((void**)&ctx->d_census, kQSlots * sizeof(unsigned long long), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_step, sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_leave, cap * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_birth, cap * sizeof(uint32_t), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_fptd, kFptdWords * sizeof(unsigned long long), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_nleave, 3 * sizeof(uint32_t), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_ticket, sizeof(unsigned int), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_bad, 2 * sizeof(unsigned int), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_err, sizeof(uint32_t), ctx->stream));
         if (h.mcc.flags & kFCoulomb) {
             const size_t cells = std::min(nc, cap);   // most cells with ions
             CK(cudaMallocAsync((void**)&ctx->d_crec, 2 * cap * 2 * sizeof(uint4), ctx->stream));
             CK(cudaMallocAsync((void**)&ctx->d_cnext, cap * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_chead, nc * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_ccount, nc * sizeof(uint32_t), ctx->stream));
+            CK(cudaMallocAsync((void**)&ctx->d_ccount, (2 * nc + cells) * sizeof(uint32_t), ctx->stream));
+            ctx->d_chead = ctx->d_ccount + nc;
+            ctx->d_pcount = ctx->d_ccount + 2 * nc;
             CK(cudaMallocAsync((void**)&ctx->d_cbkt, nc * sizeof(uint4), ctx->stream));
             CK(cudaMallocAsync((void**)&ctx->d_pcell, cells * sizeof(uint4), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_pcount, cells * sizeof(uint32_t), ctx->stream));
             // the cells' room is at most 9/8 of the ions and 4 a cell
             CK(cudaMallocAsync((void**)&ctx->d_rstart, ((9 * cap / 8 + 4 * cells) / kRange + 3) * sizeof(uint32_t),
                                ctx->stream));
             CK(cudaMallocAsync((void**)&ctx->d_xcell, cells * sizeof(uint32_t), ctx->stream));
             CK(cudaMallocAsync((void**)&ctx->d_cidx, cap * sizeof(uint32_t), ctx->stream));
             CK(cudaMallocAsync((void**)&ctx->d_cord, cap * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_cword, kCwWords * sizeof(uint32_t), ctx->stream));
             CK(cudaMallocAsync((void**)&ctx->d_plan, plan_blocks((uint32_t)nc) * sizeof(unsigned long long),
                                ctx->stream));
         }
@@ -1283,30 +1283,15 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
             CK(cudaMemcpyAsync(ctx->d_soa[k], xyzv[k], n * sizeof(float), kind, ctx->stream));
         CK(cudaMemcpyAsync(ctx->d_q8, q, n, kind, ctx->stream));
     }
-    if (ctx->d_ccount) {
-        CK(cudaMemsetAsync(ctx->d_ccount, 0, nc * sizeof(uint32_t), ctx->stream));
-        CK(cudaMemsetAsync(ctx->d_chead, 0, nc * sizeof(uint32_t), ctx->stream));
-        CK(cudaMemsetAsync(ctx->d_pcount, 0, std::min(nc, ctx->cap) * sizeof(uint32_t), ctx->stream));
-        CK(cudaMemsetAsync(ctx->d_cword, 0, kCwWords * sizeof(uint32_t), ctx->stream));
-    }
-    ctx->planned = false;
-    CK(cudaMemsetAsync(ctx->d_dep, 0, nc * sizeof(unsigned long long), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_count, 0, nc * sizeof(unsigned long long), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_charge, 0, nc * sizeof(unsigned long long), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_mark, 0, nc * sizeof(unsigned long long), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_tally, 0, kTallyWords * sizeof(unsigned long long), ctx->stream));
+    if (ctx->d_ccount)
+        CK(cudaMemsetAsync(ctx->d_ccount, 0, (2 * nc + std::min(nc, ctx->cap)) * sizeof(uint32_t), ctx->stream));
+    CK(cudaMemsetAsync(ctx->d_dep, 0, 4 * nc * sizeof(unsigned long long), ctx->stream));
+    CK(cudaMemsetAsync(ctx->d_zero, 0, kZeroBytes, ctx->stream));
     CK(cudaMemsetAsync(ctx->d_birth, 0xFF, ctx->cap * sizeof(uint32_t), ctx->stream));   // births unknown
-    CK(cudaMemsetAsync(ctx->d_fptd, 0, kFptdWords * sizeof(unsigned long long), ctx->stream));
     {
         const ecris_status pst = zero_probes(ctx);
         if (pst != ECRIS_OK) return pst;
     }
-    CK(cudaMemsetAsync(ctx->d_step, 0, sizeof(uint32_t), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_nleave, 0, 3 * sizeof(uint32_t), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_ticket, 0, sizeof(unsigned int), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(uint32_t), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_bad, 0, sizeof(unsigned int), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_bad + 1, 0xFF, sizeof(unsigned int), ctx->stream));
     // validate on the device, build the meta words and fill the padding slots
     LoadCheck lc;
     lc.R0sq = (float)(h.geo.R0 * h.geo.R0);
@@ -1337,7 +1322,14 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
         ctx->loaded = false;
         return fail(ctx, ECRIS_EINVAL,
                     "load_ions: %u particle(s) outside the chamber, not finite or with Q > qmax "
-                    "(first index %u)", bad[0], bad[1]);
+                    "(first index %u)", bad[0], ~bad[1]);
+    }
+    if (ctx->d_ccount) {
+        // the collisions' buckets, from the counts taken above: good for the
+        // first steps and for the first sort, which changes no cell
+        RunDev R;
+        fill_rundev(ctx, 1e-9, R);
+        CK(launch_plan(R, ctx->d_ccount, true, ctx->d_plan, ctx->stream));
     }
     ctx->weight = weight;
     ctx->seed = seed;
@@ -1387,11 +1379,6 @@ ecris_status ecris_step(ecris_ctx* ctx, uint32_t nsteps, double dt)
         // a window of steps; timed steps launch the collision kernels of their
         // one step as a graph of their own
         const uint32_t K = window_steps(ctx, nsteps - s, ctx->timer.on);
-        if (coulomb && !ctx->planned && ctx->n4 > 0) {
-            // on the load order: from the load's counts
-            CK(launch_plan(*ctx->h_run, ctx->d_ccount, true, ctx->d_plan, ctx->stream));
-            ctx->planned = true;
-        }
         const RunDev& R = *ctx->h_run;
         CK(timed(ctx, kKindStep, [&] {
             cudaError_t e = launch_quiet(R, K, ctx->sm_count, ctx->stream);

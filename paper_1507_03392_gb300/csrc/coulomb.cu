@@ -5,8 +5,8 @@
 // The ions' pass of a step leaves a 32-byte record of every ion that stayed
 // inside, (v, Q) and (array slot, its three words of the stream-1 Philox
 // block), in its cell's bucket (place_warp in step_kernel.cu):
-//   - buckets are planned at every layout sort (and before the first step on
-//     the load order) from the cells' ion counts at that time: a cell of h ions
+//   - buckets are planned at every load and layout sort from the cells' ion
+//     counts at that time: a cell of h ions
 //     gets room for h + h/8 + 4 (k_plan*), cells without ions none;
 //   - an ion that finds its cell's bucket full, or a cell without one, goes to
 //     the overflow part of the pool and is chained to its cell.

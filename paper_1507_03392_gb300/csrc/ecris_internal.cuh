@@ -432,7 +432,7 @@ struct LoadCheck {
 };
 // check particles [0, n), convert their positions (metres, float) in place to
 // fixed point, build their meta words from q8 and ids, fill pads [n, cap);
-// bad[0] counts invalid particles, bad[1] holds the lowest invalid index
+// bad[0] counts invalid particles, ~bad[1] is the lowest invalid index (bad zeroed before)
 cudaError_t launch_load_init(const LoadCheck& lc, float* const soa[6], const uint8_t* q8, uint32_t* meta,
                              uint32_t* id, uint32_t n, uint32_t cap, unsigned int* bad, cudaStream_t s);
 

@@ -182,17 +182,30 @@ __device__ __forceinline__ bool atom_may_ionize(const RunDev& R, uint32_t w0)
     return w0 < gate || gate == 0xFFFFFFFFu;
 }
 
+// What a particle carries from step to step of a window: its cell's record and
+// what follows from it and the charge state, so that a particle that stays in
+// its cell reads nothing and forms neither again.
+struct Carry {
+    uint32_t cell = kNoCell;   // the cell at X, Y, Z (kNoCell: not known)
+    float4 cr;                 // its record
+    uint32_t qthr = kNoCell;   // charge state that thr holds for (kNoCell: none)
+    uint32_t thr, always;      // the ionisation word fires below thr, or always (~0)
+    uint32_t qD = kNoCell;     // charge state that D holds for
+    float D;                   // the kick's size
+};
+
 // Advance one particle by one step.  pid is its stable id (the Philox counter
 // word).  On return dep_cell is the cell it deposits in and ckey the cell
 // where it takes part in Coulomb collisions (kNoCell if it does not).  A
 // particle that left the chamber keeps its old position and returns true
 // with its pushed velocity: the leaver pass finishes its step.
 // kVar: with the code of the opt-in processes (double ionisation, elastic
-// ion-atom scattering); without it the kernels carry none of their branches
-template <bool kVar>
+// ion-atom scattering); without it the kernels carry none of their branches.
+// kCarry: c holds the particle's cell from its last step
+template <bool kVar, bool kCarry>
 __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uint32_t step, int32_t& X,
                                               int32_t& Y, int32_t& Z, float& vx, float& vy, float& vz,
-                                              uint32_t& meta, uint32_t& ckey, uint32_t& dep_cell)
+                                              uint32_t& meta, uint32_t& ckey, uint32_t& dep_cell, Carry& c)
 {
     ckey = kNoCell;
     dep_cell = kNoCell;
@@ -208,11 +221,11 @@ __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uin
     // an ion's cell record is fetched with its field gather, at the old
     // position; the push moves it far less than a cell, so it is reused
     // unless the particle crossed into another cell
-    uint32_t cell_pre = kNoCell;
-    float4 cr = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (Q > 0) {
-        cell_pre = ngp_cell(R, X, Y, Z);
-        cr = __ldg(R.cell + cell_pre);
+    if (!kCarry) c.cell = kNoCell;
+    if (Q > 0 && c.cell == kNoCell) {
+        c.cell = ngp_cell(R, X, Y, Z);
+        c.cr = __ldg(R.cell + c.cell);
+        if (kCarry) c.qthr = c.qD = kNoCell;
     }
     if ((R.flags & kFPush) && Q > 0) {
         const float x0 = fx_xy(R, X), y0 = fx_xy(R, Y), z0 = fx_z(R, Z);
@@ -247,6 +260,7 @@ __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uin
         Y = Y0;
         Z = Z0;
         meta = status | Q;
+        if (kCarry) c.cell = kNoCell;   // it goes on elsewhere
         return true;
     }
 
@@ -257,18 +271,29 @@ __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uin
     // the densest cell; otherwise no cell can ionise it this step
     const bool ionize = (R.flags & kFIonize) && (int)Q < R.qmax;
     const bool need = Q > 0 || (ionize && atom_may_ionize(R, w.w0));
-    if (need && cell != cell_pre) cr = __ldg(R.cell + cell);   // n_e, zone, delta_x, delta_y
+    if (need && cell != c.cell) {
+        c.cr = __ldg(R.cell + cell);   // n_e, zone, delta_x, delta_y
+        if (kCarry) c.qthr = c.qD = kNoCell;
+    }
+    // (an atom that needed no record has none to carry)
+    if (kCarry) c.cell = need ? cell : kNoCell;
+    const float4 cr = c.cr;
     const int zone = cr.y > 0.5f ? 1 : 0;
     const bool recomb = kVar && (R.flags & kFRecomb) && Q >= 1;
     if ((ionize && need) || recomb) {
-        const float lam = cr.x * __ldg(R.kdt + zone * kQSlots + Q);
-        if constexpr (kVar) {
-            const float p = event_prob(lam);
-            if (fires(w.w0, p)) {
+        if (!kCarry || c.qthr != Q) {
+            const float t = event_prob(cr.x * __ldg(R.kdt + zone * kQSlots + Q)) * 4294967296.0f;
+            c.always = t >= 4294967296.0f ? 0xFFFFFFFFu : 0u;   // (as fires())
+            c.thr = __float2uint_rz(t);
+            if (kCarry) c.qthr = Q;
+        }
+        if (w.w0 < c.thr || c.always) {
+            if constexpr (kVar) {
                 // single, double, triple and recombination share [0, p) in
                 // proportion to their rates: below p k1/k one electron goes,
                 // below p (k1+k2)/k two, below p (k1+k2+k3)/k three, above
                 // that one is captured
+                const float p = event_prob(cr.x * __ldg(R.kdt + zone * kQSlots + Q));
                 int up = 1;
                 if (R.flags & (kFDouble | kFRecomb)) {
                     if (!fires(w.w0, p * __ldg(R.kdt + 2 * kQSlots + zone * kQSlots + Q))) {
@@ -284,11 +309,11 @@ __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uin
                     Q -= 1u;
                     ev |= kEvRecomb;
                 }
+            } else {
+                if (Q == 0) R.birth[pid] = step;   // an ion is born (first-passage clock)
+                Q += 1;
+                ev |= kEvIonize;
             }
-        } else if (fires(w.w0, event_prob(lam))) {
-            if (Q == 0) R.birth[pid] = step;   // an ion is born (first-passage clock)
-            Q += 1;
-            ev |= kEvIonize;
         }
     }
     // collisions with the neutral background: 1 charge exchange, 2 elastic
@@ -335,8 +360,12 @@ __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uin
         }
     }
     if ((R.flags & kFEikick) && Q >= 1) {
-        const float qp = R.ei_pow == 1 ? (float)Q : (float)(Q * Q);
-        const float D = sqrt_approx((zone ? R.ei_coef[1] : R.ei_coef[0]) * cr.x * qp);
+        if (!kCarry || c.qD != Q) {
+            const float qp = R.ei_pow == 1 ? (float)Q : (float)(Q * Q);
+            c.D = sqrt_approx((zone ? R.ei_coef[1] : R.ei_coef[0]) * cr.x * qp);
+            if (kCarry) c.qD = Q;
+        }
+        const float D = c.D;
         const float ct = fmaf(2.0f, unit01(w.w2), -1.0f);
         const float st = sqrt_approx(fmaxf(0.0f, fmaf(-ct, ct, 1.0f)));
         float sp, cp;
@@ -988,10 +1017,11 @@ __device__ __forceinline__ void active_tile(const RunDev& R, uint32_t t, uint32_
     }
     // deposits: summed while the particle stays in a cell
     uint32_t at = kNoCell, n = 0u, q = 0u;
+    Carry carry;
 #pragma unroll 1
     for (uint32_t s = 0; s < K; ++s) {
         uint32_t ck, dc;
-        if (step_particle<kVar>(R, id, step0 + s, x, y, z, vx, vy, vz, meta, ck, dc)) {
+        if (step_particle<kVar, true>(R, id, step0 + s, x, y, z, vx, vy, vz, meta, ck, dc, carry)) {
             const Left l = leave_call(R, id, step0 + s, x, y, z, vx, vy, vz, meta);
             x = l.X; y = l.Y; z = l.Z;
             vx = l.vx; vy = l.vy; vz = l.vz;
@@ -1097,7 +1127,8 @@ __device__ __forceinline__ void ions_tile(const RunDev& R, uint32_t t, uint32_t 
         vx = R.vx[i]; vy = R.vy[i]; vz = R.vz[i];
     }
     uint32_t ck, dc;
-    if (step_particle<kVar>(R, id, step, x, y, z, vx, vy, vz, meta, ck, dc)) {
+    Carry carry;
+    if (step_particle<kVar, false>(R, id, step, x, y, z, vx, vy, vz, meta, ck, dc, carry)) {
         const Left l = leave_call(R, id, step, x, y, z, vx, vy, vz, meta);
         x = l.X; y = l.Y; z = l.Z;
         vx = l.vx; vy = l.vy; vz = l.vz;
@@ -1236,7 +1267,7 @@ __global__ void k_load_init(LoadCheck lc, SoaPtrs soa, const uint8_t* __restrict
                             isfinite(vx) && isfinite(vy) && isfinite(vz) && q <= lc.qmax;
             if (!ok) {
                 atomicAdd(bad, 1u);
-                atomicMin(bad + 1, i);
+                atomicMax(bad + 1, ~i);
             }
             meta[i] = q;
             const int3 p = to_fx(x, y, z, lc);
