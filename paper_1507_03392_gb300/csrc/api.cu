@@ -1610,7 +1610,7 @@ struct ecris_batch {
     int sm_count = 0;
     int blocks_per_sm = 0;          // 0: as many as fit
     int shape = kDefaultShape;      // launch shape of the batch's passes
-    int max_bps[kStepShapes] = {};  // resident blocks per SM of each shape
+    WindowBlocks max_bps[kStepShapes] = {};  // resident blocks per SM of each shape's passes
     uint32_t sort_every = 32;
     size_t budget = 0, used = 0;
     std::string err;
@@ -1774,11 +1774,13 @@ ecris_status batch_items(ecris_batch* b)
     return ECRIS_OK;
 }
 
-// resident blocks per SM of the batch's passes: as many as the tuning asks for
-int batch_bps(const ecris_batch* b)
+// the grid of a pass that has m resident blocks per SM: as many as the tuning
+// asks for.  Each pass has its own number: with one for all of them the pass
+// that could hold more ran too few, or a second wave (2.6e7 atoms and ions:
+// quiet pass 2089 us on the grid of the ions' pass, 1601 on its own).
+int batch_grid(const ecris_batch* b, int m)
 {
-    const int m = b->max_bps[b->shape];
-    return b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, m) : m;
+    return b->sm_count * (b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, m) : m);
 }
 
 cudaError_t batch_side_streams(ecris_batch* b)
@@ -1797,19 +1799,22 @@ cudaError_t batch_side_streams(ecris_batch* b)
 cudaError_t batch_window(ecris_batch* b, uint32_t K)
 {
     const uint32_t nr = (uint32_t)b->runs.size();
-    const int threads = kShapeThreads[b->shape], grid = b->sm_count * batch_bps(b);
+    const int threads = shape_block(b->shape);
+    const WindowBlocks& m = b->max_bps[b->shape];
     if (nr == 0) return cudaSuccess;
-    cudaError_t e = launch_quiet_batch(b->d_runs, nr, b->d_items, b->nitems, shape_tile(b->shape), threads, grid, K,
+    cudaError_t e = launch_quiet_batch(b->d_runs, nr, b->d_items, b->nitems, shape_tile(b->shape), threads,
+                                       batch_grid(b, m.quiet), K,
                                        b->d_pref, b->d_ticket, b->stream);
     if (e == cudaSuccess && b->any_plain)
-        e = launch_active_batch(b->d_runs, nr, threads, grid, b->variants, K, b->d_pref, b->d_ticket, b->stream);
+        e = launch_active_batch(b->d_runs, nr, threads, batch_grid(b, m.active), b->variants, K, b->d_pref, b->d_ticket,
+                                b->stream);
     return e;
 }
 
 cudaError_t batch_ions(ecris_batch* b)
 {
-    return launch_ions_batch(b->d_runs, (uint32_t)b->runs.size(), kShapeThreads[b->shape],
-                             b->sm_count * batch_bps(b), b->variants, b->d_pref, b->stream);
+    return launch_ions_batch(b->d_runs, (uint32_t)b->runs.size(), shape_block(b->shape),
+                             batch_grid(b, b->max_bps[b->shape].ions), b->variants, b->d_pref, b->stream);
 }
 
 // A step of every run with collisions between ions (captured into the batch
@@ -1913,9 +1918,7 @@ ecris_status ecris_batch_create(ecris_batch** out, int device, void* cuda_stream
         return ECRIS_ECUDA;
     }
     b->collide_grid = collide_blocks(b->sm_count);
-    for (int k = 0; k < kStepShapes; ++k) {
-        b->max_bps[k] = window_blocks_per_sm(kShapeThreads[k]);
-    }
+    for (int k = 0; k < kStepShapes; ++k) b->max_bps[k] = window_blocks_per_sm(shape_block(k));
     *out = b;
     return ECRIS_OK;
 }
@@ -2437,7 +2440,8 @@ ecris_status batch_autotune(ecris_batch* b, uint32_t trial_steps, bool cadence, 
     }
     // 2. resident blocks per SM of that shape
     best = 1e30f;
-    for (int bps = 1; bps <= b->max_bps[best_shape] && st == ECRIS_OK; ++bps) {
+    const WindowBlocks& m = b->max_bps[best_shape];
+    for (int bps = 1; bps <= std::max(m.quiet, std::max(m.active, m.ions)) && st == ECRIS_OK; ++bps) {
         apply(best_shape, bps, orig_sort);
         st = time_steps(b, trial_steps, true, &ms);
         if (st == ECRIS_OK && ms < best) {

@@ -403,7 +403,8 @@ cudaError_t launch_active_batch(const RunDev* runs, uint32_t nruns, int threads,
 cudaError_t launch_ions_batch(const RunDev* runs, uint32_t nruns, int threads, int grid, bool variants,
                               const uint32_t* pref, cudaStream_t s);
 // resident blocks per SM of the batch's passes
-int window_blocks_per_sm(int threads);
+struct WindowBlocks { int quiet, active, ions; };
+WindowBlocks window_blocks_per_sm(int threads);
 cudaError_t launch_fold(const RunDev& R, uint32_t ncells, unsigned long long* count,
                         unsigned long long* charge, cudaStream_t s);
 // words of the rate table after its 8 kQSlots rates and shares: the atom gate and the
@@ -470,6 +471,7 @@ constexpr int kDefaultShape = 11;
 constexpr int kShapeThreads[kStepShapes] = {128, 128, 128, 256, 256, 256, 512, 512, 512, 128, 256, 256};
 constexpr int kShapeVec[kStepShapes] = {1, 2, 4, 1, 2, 4, 1, 2, 4, 2, 1, 2};
 constexpr int kShapeStages[kStepShapes] = {2, 2, 2, 2, 2, 2, 2, 2, 2, 3, 3, 3};
+inline int shape_block(int k) { return kShapeThreads[k] < 256 ? kShapeThreads[k] : 256; }   // threads of its blocks
 inline uint32_t shape_tile(int k) { return (uint32_t)(kShapeThreads[k] * kShapeVec[k]); }
 // message returned by ecris_last_error(NULL) on the calling thread
 void ecris_internal_set_thread_error(const char* msg);

@@ -115,10 +115,11 @@ __device__ __forceinline__ int32_t add_wrap(int32_t a, int32_t b, bool& over)
 // sum that leaves the 32-bit range has left the chamber.  On return X, Y, Z
 // hold the new position (clamped into the range for a leaver); true if the
 // particle left.
+template <bool kPush>
 __device__ __forceinline__ bool move(const RunDev& R, int32_t& X, int32_t& Y, int32_t& Z, float vx, float vy,
                                      float vz)
 {
-    const bool push = (R.flags & kFPush) != 0;
+    const bool push = kPush || (R.flags & kFPush) != 0;
     const float dx = push ? vx * R.dt_sxy : 0.0f, dy = push ? vy * R.dt_sxy : 0.0f, dz = push ? vz * R.dt_sz : 0.0f;
     if (fmaxf(fabsf(dx), fmaxf(fabsf(dy), fabsf(dz))) < 1.0e9f) {
         bool ox, oy, oz;
@@ -182,6 +183,15 @@ __device__ __forceinline__ bool atom_may_ionize(const RunDev& R, uint32_t w0)
     return w0 < gate || gate == 0xFFFFFFFFu;
 }
 
+// Is the run one for the step without tests: every process on, neutrals there,
+// no E grid, the kick quadratic in Q?  Testing them for every particle took one
+// instruction in eight.
+__device__ __forceinline__ bool plain_run(const RunDev& R)
+{
+    constexpr uint32_t all = kFPush | kFIonize | kFCx | kFEikick;
+    return (R.flags & (all | kFHasE)) == all && R.n0s1 > 0.0f && R.ei_pow == 2;
+}
+
 // What a particle carries from step to step of a window: its cell's record and
 // what follows from it and the charge state, so that a particle that stays in
 // its cell reads nothing and forms neither again.
@@ -196,13 +206,14 @@ struct Carry {
 
 // Advance one particle by one step.  pid is its stable id (the Philox counter
 // word).  On return dep_cell is the cell it deposits in and ckey the cell
-// where it takes part in Coulomb collisions (kNoCell if it does not).  A
+// where it can take part in Coulomb collisions (kNoCell: no ion, or it left).  A
 // particle that left the chamber keeps its old position and returns true
 // with its pushed velocity: the leaver pass finishes its step.
 // kVar: with the code of the opt-in processes (double ionisation, elastic
 // ion-atom scattering); without it the kernels carry none of their branches.
-// kCarry: c holds the particle's cell from its last step
-template <bool kVar, bool kCarry>
+// kCarry: c holds the particle's cell from its last step.  kPlain: every process
+// is on and there is no E grid (plain_run), so nothing is left to test
+template <bool kVar, bool kCarry, bool kPlain>
 __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uint32_t step, int32_t& X,
                                               int32_t& Y, int32_t& Z, float& vx, float& vy, float& vz,
                                               uint32_t& meta, uint32_t& ckey, uint32_t& dep_cell, Carry& c)
@@ -227,12 +238,12 @@ __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uin
         c.cr = __ldg(R.cell + c.cell);
         if (kCarry) c.qthr = c.qD = kNoCell;
     }
-    if ((R.flags & kFPush) && Q > 0) {
+    if ((kPlain || (R.flags & kFPush)) && Q > 0) {
         const float x0 = fx_xy(R, X), y0 = fx_xy(R, Y), z0 = fx_z(R, Z);
         float Bx, By, Bz, Ex, Ey, Ez;
         if (kVar && R.btab) bfield_table(R, x0, y0, z0, Bx, By, Bz);
         else bfield(R, x0, y0, z0, Bx, By, Bz);
-        if (R.flags & kFHasE) {
+        if (!kPlain && (R.flags & kFHasE)) {
             efield(R, x0, y0, z0, Ex, Ey, Ez);
         } else {
             Ex = 0.0f;   // no E grid: the gather would return zeros
@@ -255,7 +266,7 @@ __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uin
         vz = fmaf(h, Ez, mz);
     }
     const int32_t X0 = X, Y0 = Y, Z0 = Z;
-    if (move(R, X, Y, Z, vx, vy, vz)) {
+    if (move<kPlain>(R, X, Y, Z, vx, vy, vz)) {
         X = X0;   // the leaver pass redoes the move from the old position
         Y = Y0;
         Z = Z0;
@@ -269,7 +280,7 @@ __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uin
     const Words w = rng_words(R, pid, step, 0u);
     // an atom needs its cell only if its ionisation word could fire in
     // the densest cell; otherwise no cell can ionise it this step
-    const bool ionize = (R.flags & kFIonize) && (int)Q < R.qmax;
+    const bool ionize = (kPlain || (R.flags & kFIonize)) && (int)Q < R.qmax;
     const bool need = Q > 0 || (ionize && atom_may_ionize(R, w.w0));
     if (need && cell != c.cell) {
         c.cr = __ldg(R.cell + cell);   // n_e, zone, delta_x, delta_y
@@ -328,7 +339,7 @@ __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uin
             const float pt = event_prob((scx + sel) * vrel * R.dt);
             if (fires(w.w1, pt)) coll = fires(w.w1, pt * (scx / (scx + sel))) ? 1u : 2u;
         }
-    } else if ((R.flags & kFCx) && R.n0s1 > 0.0f && Q >= 1 && Q != 2) {
+    } else if ((kPlain || ((R.flags & kFCx) && R.n0s1 > 0.0f)) && Q >= 1 && Q != 2) {
         const float vrel = sqrt_approx(norm2_plus(vx, vy, vz, R.vth2));
         const float p = event_prob(R.n0s1 * (float)Q * vrel * R.dt);
         if (fires(w.w1, p)) coll = 1u;
@@ -359,9 +370,9 @@ __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uin
             }
         }
     }
-    if ((R.flags & kFEikick) && Q >= 1) {
+    if ((kPlain || (R.flags & kFEikick)) && Q >= 1) {
         if (!kCarry || c.qD != Q) {
-            const float qp = R.ei_pow == 1 ? (float)Q : (float)(Q * Q);
+            const float qp = !kPlain && R.ei_pow == 1 ? (float)Q : (float)(Q * Q);
             c.D = sqrt_approx((zone ? R.ei_coef[1] : R.ei_coef[0]) * cr.x * qp);
             if (kCarry) c.qD = Q;
         }
@@ -379,7 +390,7 @@ __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uin
             vz = fmaf(k, dzv, vz);
         }
     }
-    if (Q >= 1 && (R.flags & kFCoulomb)) ckey = cell;
+    if (Q >= 1) ckey = cell;
     dep_cell = cell;   // NGP deposition at the final position (aggregated over the warp by the caller)
     meta = status | ev | Q;
     return false;
@@ -914,7 +925,7 @@ __device__ __forceinline__ uint32_t list_entries(uint32_t ni, uint32_t na) { ret
 // collisions between ions (k_active_batch), pref[nruns + 1 + r] for those with
 // (k_ions_batch), nruns + 1 entries each
 template <bool kOne>
-__global__ void __launch_bounds__(512, kOne ? 3 : 2) k_quiet_batch(const RunDev* __restrict__ runs,
+__global__ void __launch_bounds__(256, 4) k_quiet_batch(const RunDev* __restrict__ runs,
                                                                    const uint2* __restrict__ items, uint32_t nitems,
                                                                    uint32_t tile, uint32_t K, uint32_t nruns,
                                                                    uint32_t* __restrict__ pref, unsigned int* ticket)
@@ -922,7 +933,7 @@ __global__ void __launch_bounds__(512, kOne ? 3 : 2) k_quiet_batch(const RunDev*
     __shared__ QuietSteps S;
     extern __shared__ QuietWarp warps[];
     __shared__ RunDev rs;
-    __shared__ uint2 s_sum[512];
+    __shared__ uint2 s_sum[256];
     pdl_wait();
     pdl_trigger();
     QuietWarp& W = warps[threadIdx.x >> 5];
@@ -998,7 +1009,7 @@ __device__ __noinline__ Left leave_call(const RunDev& R, uint32_t pid, uint32_t 
 
 // One tile of k_active: entries [t T, (t + 1) T) of the run's list, one a thread
 // of the block of T, K steps each
-template <bool kVar>
+template <bool kVar, bool kPlain>
 __device__ __forceinline__ void active_tile(const RunDev& R, uint32_t t, uint32_t K, uint32_t ni, uint32_t na)
 {
     const uint32_t step0 = *R.step, ni32 = (ni + 31u) & ~31u, nslot = 4u * R.n4;
@@ -1021,7 +1032,7 @@ __device__ __forceinline__ void active_tile(const RunDev& R, uint32_t t, uint32_
 #pragma unroll 1
     for (uint32_t s = 0; s < K; ++s) {
         uint32_t ck, dc;
-        if (step_particle<kVar, true>(R, id, step0 + s, x, y, z, vx, vy, vz, meta, ck, dc, carry)) {
+        if (step_particle<kVar, true, kPlain>(R, id, step0 + s, x, y, z, vx, vy, vz, meta, ck, dc, carry)) {
             const Left l = leave_call(R, id, step0 + s, x, y, z, vx, vy, vz, meta);
             x = l.X; y = l.Y; z = l.Z;
             vx = l.vx; vy = l.vy; vz = l.vz;
@@ -1046,15 +1057,30 @@ __device__ __forceinline__ void active_tile(const RunDev& R, uint32_t t, uint32_
     }
 }
 
+// Resident blocks an SM that the passes over the lists are compiled for.  They
+// wait on gathers and long chains, so more warps hide more, until the spilled
+// registers cost more than that gives.  Times with 3/4/5 blocks of 256 threads
+// (or twice as many of 128), in us: k_ions, 2e6 ions 32.2/30.0/30.9; k_active,
+// 1e4 particles x 32 steps 32.5/34.9/38.1, with variants 1e6 x 32 284/260/273;
+// k_active_batch, 7e6 ions x 32 2711/2744/2864; k_ions_batch, 8e6 ions
+// 167/145/135.
+constexpr int kListBlocks = 8;   // the most, of kActiveTile threads
+constexpr int kActiveBatchBlocks = 3, kIonsBatchBlocks = 5;   // of 256
+
 // the last block clears the lists and advances the step counter
 template <bool kVar>
-__global__ void __launch_bounds__(512, 2) k_active(const __grid_constant__ RunDev R, uint32_t K, unsigned int* ticket)
+__global__ void __launch_bounds__(kActiveTile, kVar ? 8 : 6) k_active(const __grid_constant__ RunDev R, uint32_t K,
+                                                                      unsigned int* ticket)
 {
     pdl_wait();
     pdl_trigger();
     const uint32_t ni = R.nleave[0], na = R.nleave[1];
     const uint32_t nt = (list_entries(ni, na) + blockDim.x - 1u) / blockDim.x;
-    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) active_tile<kVar>(R, t, K, ni, na);
+    const bool plain = !kVar && plain_run(R);
+    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
+        if (!kVar && plain) active_tile<false, true>(R, t, K, ni, na);
+        else active_tile<kVar, false>(R, t, K, ni, na);
+    }
     if (last_block(ticket) && threadIdx.x == 0) {
         R.nleave[0] = 0u;
         R.nleave[1] = 0u;
@@ -1083,7 +1109,7 @@ __device__ __forceinline__ uint32_t batch_tile(const RunDev* __restrict__ runs, 
 }
 
 template <bool kVar>
-__global__ void __launch_bounds__(512, 2) k_active_batch(const RunDev* __restrict__ runs, uint32_t nruns,
+__global__ void __launch_bounds__(256, kActiveBatchBlocks) k_active_batch(const RunDev* __restrict__ runs, uint32_t nruns,
                                                          const uint32_t* __restrict__ pref, uint32_t K,
                                                          unsigned int* ticket)
 {
@@ -1095,7 +1121,8 @@ __global__ void __launch_bounds__(512, 2) k_active_batch(const RunDev* __restric
     uint32_t cur = 0xFFFFFFFFu;
     for (uint32_t v = blockIdx.x; v < nt; v += gridDim.x) {
         const uint32_t t = batch_tile(runs, nruns, pref, v, rs, s_at, cur);
-        active_tile<kVar>(rs, t, K, rs.nleave[0], rs.nleave[1]);
+        if (!kVar && plain_run(rs)) active_tile<false, true>(rs, t, K, rs.nleave[0], rs.nleave[1]);
+        else active_tile<kVar, false>(rs, t, K, rs.nleave[0], rs.nleave[1]);
         __syncthreads();
     }
     if (last_block(ticket))
@@ -1109,7 +1136,7 @@ __global__ void __launch_bounds__(512, 2) k_active_batch(const RunDev* __restric
 
 // One step of a tile of listed particles of a run with collisions between
 // ions; the ions that stay are recorded in their cells' buckets
-template <bool kVar>
+template <bool kVar, bool kPlain>
 __device__ __forceinline__ void ions_tile(const RunDev& R, uint32_t t, uint32_t ni, uint32_t na)
 {
     const uint32_t step = *R.step, ni32 = (ni + 31u) & ~31u, nslot = 4u * R.n4;
@@ -1128,7 +1155,7 @@ __device__ __forceinline__ void ions_tile(const RunDev& R, uint32_t t, uint32_t 
     }
     uint32_t ck, dc;
     Carry carry;
-    if (step_particle<kVar, false>(R, id, step, x, y, z, vx, vy, vz, meta, ck, dc, carry)) {
+    if (step_particle<kVar, false, kPlain>(R, id, step, x, y, z, vx, vy, vz, meta, ck, dc, carry)) {
         const Left l = leave_call(R, id, step, x, y, z, vx, vy, vz, meta);
         x = l.X; y = l.Y; z = l.Z;
         vx = l.vx; vy = l.vy; vz = l.vz;
@@ -1152,18 +1179,22 @@ __device__ __forceinline__ void begin_collisions(const RunDev& R)
 }
 
 template <bool kVar>
-__global__ void __launch_bounds__(512, 2) k_ions(const __grid_constant__ RunDev R)
+__global__ void __launch_bounds__(kActiveTile, 8) k_ions(const __grid_constant__ RunDev R)
 {
     pdl_wait();
     pdl_trigger();
     if (blockIdx.x == 0 && threadIdx.x == 0) begin_collisions(R);
     const uint32_t ni = R.nleave[0], na = R.nleave[1];
     const uint32_t nt = (list_entries(ni, na) + blockDim.x - 1u) / blockDim.x;
-    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) ions_tile<kVar>(R, t, ni, na);
+    const bool plain = !kVar && plain_run(R);
+    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
+        if (!kVar && plain) ions_tile<false, true>(R, t, ni, na);
+        else ions_tile<kVar, false>(R, t, ni, na);
+    }
 }
 
 template <bool kVar>
-__global__ void __launch_bounds__(512, 2) k_ions_batch(const RunDev* __restrict__ runs, uint32_t nruns,
+__global__ void __launch_bounds__(256, kIonsBatchBlocks) k_ions_batch(const RunDev* __restrict__ runs, uint32_t nruns,
                                                        const uint32_t* __restrict__ pref)
 {
     __shared__ RunDev rs;
@@ -1177,7 +1208,8 @@ __global__ void __launch_bounds__(512, 2) k_ions_batch(const RunDev* __restrict_
     uint32_t cur = 0xFFFFFFFFu;
     for (uint32_t v = blockIdx.x; v < nt; v += gridDim.x) {
         const uint32_t t = batch_tile(runs, nruns, pref, v, rs, s_at, cur);
-        ions_tile<kVar>(rs, t, rs.nleave[0], rs.nleave[1]);
+        if (!kVar && plain_run(rs)) ions_tile<false, true>(rs, t, rs.nleave[0], rs.nleave[1]);
+        else ions_tile<kVar, false>(rs, t, rs.nleave[0], rs.nleave[1]);
         __syncthreads();
     }
 }
@@ -1298,19 +1330,21 @@ cudaError_t launch_load_init(const LoadCheck& lc, float* const soa[6], const uin
 }
 
 template <class K>
-static int blocks_per_sm(K kernel, int threads)
+static int blocks_per_sm(K kernel, int threads, int smem)
 {
     int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, 0) != cudaSuccess || b < 1) b = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, smem) != cudaSuccess || b < 1) b = 1;
     return b;
 }
 
-int window_blocks_per_sm(int threads)
+WindowBlocks window_blocks_per_sm(int threads)
 {
-    int b = blocks_per_sm(k_active_batch<false>, threads);
-    b = std::min(b, blocks_per_sm(k_active_batch<true>, threads));
-    b = std::min(b, blocks_per_sm(k_ions_batch<false>, threads));
-    return std::min(b, blocks_per_sm(k_ions_batch<true>, threads));
+    const int smem = (threads / 32) * (int)sizeof(QuietWarp);
+    WindowBlocks b;
+    b.quiet = std::min(blocks_per_sm(k_quiet_batch<false>, threads, smem), blocks_per_sm(k_quiet_batch<true>, threads, smem));
+    b.active = std::min(blocks_per_sm(k_active_batch<false>, threads, 0), blocks_per_sm(k_active_batch<true>, threads, 0));
+    b.ions = std::min(blocks_per_sm(k_ions_batch<false>, threads, 0), blocks_per_sm(k_ions_batch<true>, threads, 0));
+    return b;
 }
 
 cudaError_t launch_quiet(const RunDev& R, uint32_t K, int sm_count, cudaStream_t s)
@@ -1326,7 +1360,7 @@ cudaError_t launch_quiet(const RunDev& R, uint32_t K, int sm_count, cudaStream_t
 // as many blocks as the list could need, at most one wave
 static dim3 list_grid(const RunDev& R, int sm_count)
 {
-    return dim3(std::min(4u * R.n4 / kActiveTile + 2u, 8u * (uint32_t)sm_count));
+    return dim3(std::min(4u * R.n4 / kActiveTile + 2u, (uint32_t)(kListBlocks * sm_count)));
 }
 
 static bool variants(const RunDev& R) { return (R.flags & kFVariants) || R.btab; }
