@@ -201,6 +201,14 @@ __device__ __forceinline__ Words rng_words(const RunDev& R, uint32_t pid, uint32
     return philox(pid, step * 4u + st, R.seed_lo, R.seed_hi);
 }
 
+// the block's copy of a run's parameter block (all threads call it)
+__device__ __forceinline__ void stage_run(RunDev& rs, const RunDev* src)
+{
+    const uint32_t* from = reinterpret_cast<const uint32_t*>(src);
+    uint32_t* to = reinterpret_cast<uint32_t*>(&rs);
+    for (uint32_t k = threadIdx.x; k < sizeof(RunDev) / 4; k += blockDim.x) to[k] = from[k];
+}
+
 // Programmatic dependent launch: a kernel launched with launch_pdl may be
 // scheduled while the kernel before it in the stream finishes (that kernel's
 // blocks signal with pdl_trigger, or by exiting); it calls pdl_wait before it

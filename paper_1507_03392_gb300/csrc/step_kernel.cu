@@ -909,14 +909,6 @@ __global__ void __launch_bounds__(128, kOne ? 8 : kQuietBlocks) k_quiet(const __
     quiet_end(R, S, W, n, K);
 }
 
-// the block's copy of a run's parameter block (all threads call it)
-__device__ __forceinline__ void stage_run(RunDev& rs, const RunDev* src)
-{
-    const uint32_t* from = reinterpret_cast<const uint32_t*>(src);
-    uint32_t* to = reinterpret_cast<uint32_t*>(&rs);
-    for (uint32_t k = threadIdx.x; k < sizeof(RunDev) / 4; k += blockDim.x) to[k] = from[k];
-}
-
 // entries of a run's list: its ions, padded to whole warps, then its atoms
 __device__ __forceinline__ uint32_t list_entries(uint32_t ni, uint32_t na) { return ((ni + 31u) & ~31u) + na; }
 
