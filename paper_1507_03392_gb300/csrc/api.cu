@@ -294,12 +294,6 @@ constexpr size_t kZeroBytes = (kTallyWords + kFptdWords) * sizeof(unsigned long 
 
 constexpr uint32_t kSortAfterLoad = 8;   // steps of one ecris_step call that sort a fresh load first
 
-// what a captured step graph bakes in: the parameter block (by value) and
-// the launch shapes
-struct GraphKey {
-    RunDev R;
-};
-
 struct ecris_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -362,14 +356,6 @@ struct ecris_ctx {
     uint32_t since_sort = 0;
     bool fresh = false;         // loaded, not yet sorted
     uint32_t calls_since_load = 0;
-    int parity = 0;                // which particle set is current (flips at each sort)
-    // captured per-step kernel sequences, by particle set and kind (0: the
-    // whole step, 1: the collision kernels only), each valid for the launch
-    // arguments it was captured with (a reload into the same buffers with
-    // the same step length keeps them, so a load-step-read cycle does not
-    // re-instantiate its graph)
-    cudaGraphExec_t gexec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
-    GraphKey gkey[2][2];
     unsigned long long* d_dep = nullptr;
     unsigned long long* d_count = nullptr;
     unsigned long long* d_charge = nullptr;
@@ -441,18 +427,8 @@ void free_async(ecris_ctx* ctx, T*& p)
     p = nullptr;
 }
 
-void free_graphs(ecris_ctx* ctx)
-{
-    for (auto& row : ctx->gexec)
-        for (auto& x : row) {
-            if (x) cudaGraphExecDestroy(x);
-            x = nullptr;
-        }
-}
-
 void free_ions(ecris_ctx* ctx)
 {
-    free_graphs(ctx);
     for (auto& p : ctx->d_set) free_async(ctx, p);
     free_async(ctx, ctx->d_hist);
     free_async(ctx, ctx->d_hoff);
@@ -862,44 +838,6 @@ ecris_status get_cells(ecris_ctx* ctx, float* ne, float* delta_x, float* delta_y
     return ECRIS_OK;
 }
 
-// the kernel sequence of one step with collisions between ions (after the
-// window's quiet pass), captured once per particle set and parameter block and
-// replayed as a CUDA graph
-ecris_status step_graph(ecris_ctx* ctx, int kind, cudaGraphExec_t* out)
-{
-    const int p = ctx->parity;
-    GraphKey key;
-    std::memset(&key, 0, sizeof key);
-    std::memcpy(&key.R, ctx->h_run, sizeof(RunDev));   // the block was zeroed before it was filled
-    if (ctx->gexec[p][kind] && std::memcmp(&ctx->gkey[p][kind], &key, sizeof key) == 0) {
-        *out = ctx->gexec[p][kind];
-        return ECRIS_OK;
-    }
-    if (ctx->gexec[p][kind]) {
-        cudaGraphExecDestroy(ctx->gexec[p][kind]);
-        ctx->gexec[p][kind] = nullptr;
-    }
-    cudaGraph_t g = nullptr;
-    CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = cudaSuccess;
-    // kind 0, the whole step; kind 1, the collision kernels alone (timed
-    // steps launch the ions' pass on its own before them)
-    if (kind == 0) e = launch_ions(*ctx->h_run, ctx->sm_count, ctx->stream);
-    if (e == cudaSuccess)
-        e = launch_coulomb(*ctx->h_run, (uint32_t)ctx->n, ctx->collide_grid, ctx->stream);
-    const cudaError_t e2 = cudaStreamEndCapture(ctx->stream, &g);
-    CK(e);
-    CK(e2);
-    cudaGraphExec_t x = nullptr;
-    e = cudaGraphInstantiate(&x, g, 0);
-    cudaGraphDestroy(g);
-    CK(e);
-    ctx->gexec[p][kind] = x;
-    ctx->gkey[p][kind] = key;
-    *out = x;
-    return ECRIS_OK;
-}
-
 // Steps of the next window: at most `left`, and no further than the next sort
 // and the next deposit fold.  Timed steps go one by one.
 uint32_t window_steps(const ecris_ctx* ctx, uint32_t left, bool one_by_one)
@@ -951,7 +889,6 @@ ecris_status sort_particles(ecris_ctx* ctx)
     R.vz = ctx->d_soa[5];
     R.meta = ctx->d_meta;
     R.id = ctx->d_id;
-    ctx->parity ^= 1;
     return ECRIS_OK;
 }
 
@@ -1376,21 +1313,22 @@ ecris_status ecris_step(ecris_ctx* ctx, uint32_t nsteps, double dt)
             st = sort_particles(ctx);
             if (st != ECRIS_OK) return st;
         }
-        // a window of steps; timed steps launch the collision kernels of their
-        // one step as a graph of their own
+        // a window of steps (timed steps are windows of one)
         const uint32_t K = window_steps(ctx, nsteps - s, ctx->timer.on);
         const RunDev& R = *ctx->h_run;
         CK(timed(ctx, kKindStep, [&] {
-            cudaError_t e = launch_quiet(R, K, ctx->sm_count, ctx->stream);
-            if (e == cudaSuccess && !coulomb) e = launch_active(R, K, ctx->d_ticket, ctx->sm_count, ctx->stream);
-            if (e == cudaSuccess && coulomb && ctx->timer.on) e = launch_ions(R, ctx->sm_count, ctx->stream);
-            return e;
+            const cudaError_t e = launch_quiet(R, K, ctx->sm_count, ctx->stream);
+            if (e != cudaSuccess) return e;
+            return coulomb ? launch_ions(R, ctx->sm_count, ctx->stream)
+                           : launch_active(R, K, ctx->d_ticket, ctx->sm_count, ctx->stream);
         }));
+        // (each kernel may start while the one before it ends; a graph a step lost
+        // that between steps: 2e4 particles 25.6 us a step, 22.9 without)
         for (uint32_t k = 0; coulomb && k < K; ++k) {
-            cudaGraphExec_t x = nullptr;
-            st = step_graph(ctx, ctx->timer.on ? 1 : 0, &x);
-            if (st != ECRIS_OK) return st;
-            CK(timed(ctx, kKindCoulomb, [&] { return cudaGraphLaunch(x, ctx->stream); }, kCoulombKernels));
+            if (k > 0) CK(launch_ions(R, ctx->sm_count, ctx->stream));
+            CK(timed(ctx, kKindCoulomb, [&] {
+                return launch_coulomb(R, (uint32_t)ctx->n, ctx->collide_grid, ctx->stream);
+            }));
         }
         ctx->since_fold += K;
         if (ctx->since_fold >= ctx->fold_every) {
@@ -1629,8 +1567,6 @@ struct ecris_batch {
     bool variants = false;          // some run has an opt-in process of kFVariants
     bool layout_dirty = true;       // work list must be rebuilt
     bool params_dirty = true;       // parameter blocks must be uploaded
-    cudaGraphExec_t gexec = nullptr;
-    bool graph_dirty = true;
     unsigned int* d_ticket = nullptr;   // last-block ticket of the leaver pass
     KernelTimer timer;              // ecris_batch_set_profiling
     int collide_grid = 0;       // most blocks of the collision kernel
@@ -1646,9 +1582,6 @@ struct ecris_batch {
     uint2* h_items = nullptr;
     size_t h_items_cap = 0;
     cudaEvent_t items_staged = nullptr;
-    // graphs replaced while launches of them may still be queued, each with an
-    // event recorded after its last launch; destroyed once that has passed
-    std::vector<std::pair<cudaEvent_t, cudaGraphExec_t>> old_graphs;
     // pinned host blocks of removed runs (freed with the batch: freeing pinned
     // memory may synchronise the device)
     std::vector<void*> old_host;
@@ -1677,21 +1610,6 @@ bool run_live(const ecris_batch* b, int32_t r)
 
 // upload the parameter blocks of all runs (free slots get a block whose step
 // pointer is NULL, which the kernels skip)
-// destroy the replaced graphs whose last launch has passed
-void batch_reap(ecris_batch* b)
-{
-    size_t k = 0;
-    for (auto& g : b->old_graphs) {
-        if (cudaEventQuery(g.first) == cudaSuccess) {
-            cudaGraphExecDestroy(g.second);
-            cudaEventDestroy(g.first);
-        } else {
-            b->old_graphs[k++] = g;
-        }
-    }
-    b->old_graphs.resize(k);
-}
-
 // Release a removed run without waiting for the batch's queued steps: its
 // device memory is freed in stream order after them (no launch enqueued later
 // reads it), its pinned blocks are kept until the batch goes.
@@ -1719,7 +1637,6 @@ ecris_status batch_upload(ecris_batch* b)
         if (b->d_pref) cudaFreeAsync(b->d_pref, b->stream);
         BCK(cudaMallocAsync((void**)&b->d_pref, 2 * (b->runs_cap + 1) * sizeof(uint32_t), b->stream));
         BCK(cudaMallocHost((void**)&b->h_runs, b->runs_cap * sizeof(RunDev)));
-        b->graph_dirty = true;
     } else {
         BCK(cudaEventSynchronize(b->staged));   // the previous upload has read the staging copy
     }
@@ -1770,7 +1687,6 @@ ecris_status batch_items(ecris_batch* b)
         if (c) ((c->h.mcc.flags & kFCoulomb) ? b->any_coulomb : b->any_plain) = true;
     }
     b->layout_dirty = false;
-    b->graph_dirty = true;
     return ECRIS_OK;
 }
 
@@ -1811,14 +1727,14 @@ cudaError_t batch_window(ecris_batch* b, uint32_t K)
     return e;
 }
 
+// a step of the runs with collisions between ions: the ions' pass of all of
+// them, then their collisions
 cudaError_t batch_ions(ecris_batch* b)
 {
     return launch_ions_batch(b->d_runs, (uint32_t)b->runs.size(), shape_block(b->shape),
                              batch_grid(b, b->max_bps[b->shape].ions), b->variants, b->d_pref, b->stream);
 }
 
-// A step of every run with collisions between ions (captured into the batch
-// graph): the ions' pass of all of them, then their collisions
 cudaError_t batch_coulomb(ecris_batch* b)
 {
     size_t n = 0;
@@ -1826,36 +1742,6 @@ cudaError_t batch_coulomb(ecris_batch* b)
         if (c && (c->h.mcc.flags & kFCoulomb)) n += c->n;
     return launch_coulomb_batch(b->d_runs, (uint32_t)b->runs.size(), (uint32_t)std::min(n, (size_t)0xFFFFFFFFu),
                                 b->collide_grid, b->stream);
-}
-
-cudaError_t batch_launch(ecris_batch* b)
-{
-    const cudaError_t e = batch_ions(b);
-    return e == cudaSuccess ? batch_coulomb(b) : e;
-}
-
-ecris_status batch_graph(ecris_batch* b)
-{
-    if (!b->graph_dirty && b->gexec) return ECRIS_OK;
-    if (b->gexec) {
-        // launches of the old graph may still be queued: destroy it later
-        cudaEvent_t ev = nullptr;
-        BCK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-        BCK(cudaEventRecord(ev, b->stream));
-        b->old_graphs.emplace_back(ev, b->gexec);
-        b->gexec = nullptr;
-    }
-    cudaGraph_t g = nullptr;
-    BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-    const cudaError_t e = batch_launch(b);
-    const cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
-    BCK(e);
-    BCK(e2);
-    const cudaError_t e3 = cudaGraphInstantiate(&b->gexec, g, 0);
-    cudaGraphDestroy(g);
-    BCK(e3);
-    b->graph_dirty = false;
-    return ECRIS_OK;
 }
 
 }  // namespace
@@ -1930,7 +1816,6 @@ void ecris_batch_destroy(ecris_batch* b)
     cudaStreamSynchronize(b->stream);
     for (auto* c : b->runs)
         if (c) ecris_destroy(c);
-    if (b->gexec) cudaGraphExecDestroy(b->gexec);
     if (b->d_runs) cudaFreeAsync(b->d_runs, b->stream);
     if (b->d_pref) cudaFreeAsync(b->d_pref, b->stream);
     if (b->d_items) cudaFreeAsync(b->d_items, b->stream);
@@ -1941,10 +1826,6 @@ void ecris_batch_destroy(ecris_batch* b)
         if (b->sort_join[k]) cudaEventDestroy(b->sort_join[k]);
     }
     if (b->sort_fork) cudaEventDestroy(b->sort_fork);
-    for (auto& g : b->old_graphs) {
-        cudaGraphExecDestroy(g.second);
-        cudaEventDestroy(g.first);
-    }
     for (void* p : b->old_host) cudaFreeHost(p);
     if (b->h_items) cudaFreeHost(b->h_items);
     if (b->items_staged) cudaEventDestroy(b->items_staged);
@@ -1974,7 +1855,6 @@ ecris_status ecris_batch_add_run(ecris_batch* b, const ecris_geometry* geo, cons
         return bfail(b, ECRIS_ENOMEM, "batch_add_run: the run (" + std::to_string(need) + " bytes) would exceed the "
                      "memory budget (" + std::to_string(b->used) + " of " + std::to_string(b->budget) + " used)");
     BCK(cudaSetDevice(b->device));
-    batch_reap(b);
     // set the run up on the setup stream (its waits then cover only its own
     // copies), then hand it to the batch stream
     ecris_ctx* c = nullptr;
@@ -2033,7 +1913,6 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
 {
     if (!b) return ECRIS_EINVAL;
     BCK(cudaSetDevice(b->device));
-    batch_reap(b);
     for (auto* c : b->runs)
         if (c && (c->failed || c->steps_done + nsteps >= kMaxSteps))
             return bfail(b, ECRIS_ESTATE, "batch_step: a run failed earlier or would pass 2^30 steps");
@@ -2083,18 +1962,12 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
             if (c) K = std::min(K, window_steps(c, K, b->timer.on));
         BCK(b->timer.run(kKindStep, b->stream, [&] {
             cudaError_t e = batch_window(b, K);
-            if (e == cudaSuccess && b->timer.on && b->any_coulomb) e = batch_ions(b);
+            if (e == cudaSuccess && b->any_coulomb) e = batch_ions(b);
             return e;
         }));
         for (uint32_t k = 0; b->any_coulomb && k < K; ++k) {
-            if (!b->timer.on) {
-                ecris_status st = batch_graph(b);
-                if (st != ECRIS_OK) return st;
-                BCK(cudaGraphLaunch(b->gexec, b->stream));
-                continue;
-            }
-            // timed: the graph's collision kernels on their own
-            BCK(b->timer.run(kKindCoulomb, b->stream, [&] { return batch_coulomb(b); }, kCoulombKernels));
+            if (k > 0) BCK(batch_ions(b));
+            BCK(b->timer.run(kKindCoulomb, b->stream, [&] { return batch_coulomb(b); }));
         }
         for (size_t r = 0; r < b->runs.size(); ++r) {
             ecris_ctx* c = b->runs[r];
@@ -2270,7 +2143,6 @@ ecris_status ecris_batch_set_tuning(ecris_batch* b, const ecris_tuning* t)
         b->shape = shape;
         b->layout_dirty = true;   // the runs' tiles and the work list change with the tile size
     }
-    b->graph_dirty = true;
     return ECRIS_OK;
 }
 
@@ -2355,7 +2227,7 @@ ecris_status snapshot_restore(ecris_batch* b, ecris_ctx* c, RunSnapshot& sn)
 
 // time per step of `steps` steps of the batch in its current tuning, with
 // no sort among them (hold = true) or in whole sort periods starting with a
-// sort; one untimed step first takes the graph capture out of the timing
+// sort; one untimed step first
 ecris_status time_steps(ecris_batch* b, uint32_t steps, bool hold, float* ms_per_step)
 {
     cudaEvent_t t0 = nullptr, t1 = nullptr;
@@ -2425,7 +2297,6 @@ ecris_status batch_autotune(ecris_batch* b, uint32_t trial_steps, bool cadence, 
         b->shape = shape;
         b->blocks_per_sm = bps;
         b->sort_every = every;
-        b->graph_dirty = true;
     };
     // 1. the launch shape (threads per block x particles per thread: the first
     // nine, the others differ from one of these in name only), as many resident
