@@ -349,7 +349,7 @@ struct ecris_ctx {
     float* d_soa2[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     uint32_t* d_meta2 = nullptr;
     uint32_t* d_id2 = nullptr;
-    uint32_t* d_hist = nullptr;    // sort histogram (2 Nc + 1), kept zero between sorts
+    uint32_t* d_hist = nullptr;    // sort histogram (2 Nc + 1) and ticket, kept zero between sorts
     uint32_t* d_hoff = nullptr;    // its exclusive scan (2 Nc + 2)
     uint32_t* d_hblk = nullptr;    // scan block totals
     uint32_t sort_every = 32;      // steps between sorts
@@ -871,7 +871,7 @@ ecris_status sort_particles(ecris_ctx* ctx)
         // (the load planned the collisions' buckets for its own order)
         return launch_sort(*ctx->h_run, (uint32_t)cap4, dst, ctx->d_hist, ctx->d_hoff, ctx->d_hblk,
                            aos ? nullptr : ctx->d_plan, aos, ctx->stream);
-    }, aos ? 7 : (ctx->d_plan ? 9 : 6)));
+    }, aos ? 4 : (ctx->d_plan ? 5 : 3)));
     ctx->since_sort = 0;
     if (ctx->fresh) {
         ctx->fresh = false;
@@ -1164,11 +1164,11 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
             (set ? ctx->d_meta2 : ctx->d_meta) = ctx->d_set[set] + 6 * cap;
             (set ? ctx->d_id2 : ctx->d_id) = ctx->d_set[set] + 7 * cap;
         }
-        CK(cudaMallocAsync((void**)&ctx->d_hist, (2 * nc + 1) * sizeof(uint32_t), ctx->stream));
+        CK(cudaMallocAsync((void**)&ctx->d_hist, (2 * nc + 2) * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_hoff, (2 * nc + 2) * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_hblk, (size_t)sort_scan_blocks((uint32_t)(2 * nc + 1)) * sizeof(uint32_t),
                            ctx->stream));
-        CK(cudaMemsetAsync(ctx->d_hist, 0, (2 * nc + 1) * sizeof(uint32_t), ctx->stream));
+        CK(cudaMemsetAsync(ctx->d_hist, 0, (2 * nc + 2) * sizeof(uint32_t), ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_q8, cap, ctx->stream));
         CK(cudaMallocAsync((void**)&ctx->d_dep, 4 * nc * sizeof(unsigned long long), ctx->stream));
         ctx->d_count = ctx->d_dep + nc;
@@ -1933,7 +1933,7 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
                 BCK(b->timer.run(kKindOther, b->stream, [&] {
                     st = sort_particles(c);
                     return cudaSuccess;
-                }, 6));
+                }, c->fresh ? 4 : (c->d_plan ? 5 : 3)));
             } else {
                 const int k = nsort % kBatchSideStreams;
                 if (nsort == 0) {

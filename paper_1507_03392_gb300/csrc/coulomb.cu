@@ -86,43 +86,35 @@ __device__ __forceinline__ unsigned long long block_excl64(unsigned long long v,
 }
 
 // (planned cells, room) of the blocks of kPlanBlock cells, packed (<< 32 |);
-// count: ions per cell
-__global__ void __launch_bounds__(kPlanThreads) k_plan_sum(const uint32_t* __restrict__ count, uint32_t ncells,
-                                                           unsigned long long* __restrict__ blk)
+// count: ions per cell.  The last block makes that the exclusive scan, and the
+// plan's words.
+__global__ void __launch_bounds__(kPlanThreads) k_plan_sum(const __grid_constant__ RunDev R,
+                                                           const uint32_t* __restrict__ count, unsigned long long* blk)
 {
     pdl_wait();
     pdl_trigger();
-    const uint32_t base = blockIdx.x * kPlanBlock + threadIdx.x;
+    const uint32_t base = blockIdx.x * kPlanBlock + threadIdx.x, nb = gridDim.x;
     unsigned long long v = 0ull, total;
 #pragma unroll
     for (int j = 0; j < kPlanPer; ++j) {
         const uint32_t c = base + j * kPlanThreads;
-        const uint32_t h = c < ncells ? count[c] : 0u;
+        const uint32_t h = c < R.ncells ? count[c] : 0u;
         v += ((unsigned long long)(h ? 1u : 0u) << 32) + bucket_room(h);
     }
     block_excl64<kPlanThreads>(v, &total);
     if (threadIdx.x == 0) blk[blockIdx.x] = total;
-}
-
-// one block: exclusive scan of the block sums in place, and the plan's words
-__global__ void __launch_bounds__(1024) k_plan_scan(const __grid_constant__ RunDev R, unsigned long long* blk,
-                                                    uint32_t nb)
-{
-    pdl_wait();
-    pdl_trigger();
-    const uint32_t per = (nb + 1023u) / 1024u, base = threadIdx.x * per;
-    unsigned long long sum = 0ull, total;
-    for (uint32_t j = 0; j < per; ++j)
-        if (base + j < nb) sum += blk[base + j];
-    unsigned long long o = block_excl64<1024>(sum, &total);
-    for (uint32_t j = 0; j < per; ++j)
-        if (base + j < nb) {
-            const unsigned long long t = blk[base + j];
-            blk[base + j] = o;
-            o += t;
-        }
+    if (!last_block(R.cword + kCwTicket)) return;
+    unsigned long long carry = 0ull;
+    for (uint32_t b0 = 0; b0 < nb; b0 += kPlanThreads) {
+        const uint32_t b = b0 + threadIdx.x;
+        const unsigned long long t = b < nb ? __ldcg(blk + b) : 0ull;
+        __syncthreads();   // (the scan's shared memory is used again)
+        const unsigned long long o = carry + block_excl64<kPlanThreads>(t, &total);
+        if (b < nb) blk[b] = o;
+        carry += total;
+    }
     if (threadIdx.x == 0) {
-        const uint32_t np = (uint32_t)(total >> 32), room = (uint32_t)total;
+        const uint32_t np = (uint32_t)(carry >> 32), room = (uint32_t)carry;
         R.cword[kCwPlanned] = np;
         R.cword[kCwRanges] = (room + kRange - 1u) / kRange;
         R.rstart[0] = 0u;
@@ -137,6 +129,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_cells(const __grid_consta
                                                              const unsigned long long* __restrict__ blk, int zero)
 {
     pdl_wait();
+    pdl_trigger();
     const uint32_t base = blockIdx.x * kPlanBlock + threadIdx.x * kPlanPer;
     uint32_t h[kPlanPer];
     unsigned long long v = 0ull, total;
@@ -1033,8 +1026,7 @@ uint32_t plan_blocks(uint32_t ncells) { return (ncells + kPlanBlock - 1u) / kPla
 cudaError_t launch_plan(const RunDev& R, uint32_t* count, bool zero, unsigned long long* blk, cudaStream_t s)
 {
     const uint32_t nb = plan_blocks(R.ncells);
-    cudaError_t e = launch_pdl(k_plan_sum, dim3(nb), dim3(kPlanThreads), 0, s, (const uint32_t*)count, R.ncells, blk);
-    if (e == cudaSuccess) e = launch_pdl(k_plan_scan, dim3(1), dim3(1024), 0, s, R, blk, nb);
+    cudaError_t e = launch_pdl(k_plan_sum, dim3(nb), dim3(kPlanThreads), 0, s, R, (const uint32_t*)count, blk);
     if (e == cudaSuccess)
         e = launch_pdl(k_plan_cells, dim3(nb), dim3(kPlanThreads), 0, s, R, count, (const unsigned long long*)blk,
                        zero ? 1 : 0);

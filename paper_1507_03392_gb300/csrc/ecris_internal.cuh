@@ -67,8 +67,10 @@ constexpr double kNanbuSHi = 6.0;
 // words of RunDev::cword: the plan's planned cells and ranges; which of the two
 // sets of a step's counters is in use (the ions' pass of a step sets it, the
 // collision kernel clears the other set for the next step); the scratch
-// entries; then the sets, each the step's unplanned cells and overflow records
-constexpr int kCwPlanned = 0, kCwRanges = 1, kCwSet = 2, kCwHuge = 3, kCwUnplanned = 4, kCwOverflow = 5, kCwWords = 8;
+// entries; then the sets, each the step's unplanned cells and overflow records;
+// the ticket of the plan's kernels
+constexpr int kCwPlanned = 0, kCwRanges = 1, kCwSet = 2, kCwHuge = 3, kCwUnplanned = 4, kCwOverflow = 5, kCwTicket = 8,
+              kCwWords = 10;
 // Coulomb collisions: room (records) a range of cells spans; ions of several
 // cells that a warp sorts in registers, of one cell that a warp ranks, and that a
 // block ranks at a time; warps a block
@@ -241,6 +243,20 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
                               Args&&... args)
 {
     return launch_early(true, kernel, grid, block, smem, s, std::forward<Args>(args)...);
+}
+
+// last block of a grid (after every block's work is visible): ticket reset
+__device__ __forceinline__ bool last_block(unsigned int* ticket)
+{
+    __shared__ int last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1 ? 1 : 0;
+        if (last) *ticket = 0u;
+    }
+    __syncthreads();
+    return last != 0;
 }
 
 // square root through the approximate hardware instruction (relative error
@@ -461,8 +477,8 @@ struct ParticleSet {
 };
 // Counting sort of the run's particles (in R) by (ion/atom, cell) into `dst`:
 // live ions first, then live atoms, each by cell; frozen and padding slots
-// last.  hist (2 Nc + 1 words) must be zero and is left zero; off (2 Nc + 2)
-// and blk (scan block totals) are scratch.  plan (plan_blocks words, or
+// last.  hist (2 Nc + 2 words: the bins and a ticket) must be zero and is left
+// zero; off (2 Nc + 1) and blk (scan block totals) are scratch.  plan (plan_blocks words, or
 // NULL): also plan the collisions' buckets from the counts.  aos (the memory of `dst` as cap
 // 32-byte records, or NULL): for input in arbitrary order (the first sort
 // after a load), move records there and unpack them back into the arrays of

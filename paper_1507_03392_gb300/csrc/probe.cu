@@ -18,6 +18,8 @@ namespace {
 __global__ void __launch_bounds__(256) k_probe(const __grid_constant__ RunDev R, const __grid_constant__ ProbeDev P,
                                                uint32_t n4)
 {
+    pdl_wait();
+    pdl_trigger();
     for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < n4; g += gridDim.x * blockDim.x) {
         const uint4 m4 = reinterpret_cast<const uint4*>(R.meta)[g];
         const uint32_t mm[4] = {m4.x, m4.y, m4.z, m4.w};
@@ -66,8 +68,7 @@ cudaError_t launch_probe(const RunDev& R, const ProbeDev& P, uint32_t n4, int sm
     if (n4 == 0) return cudaSuccess;
     const uint32_t need = (n4 + 255) / 256;
     const uint32_t blocks = need < (uint32_t)(4 * sm_count) ? need : (uint32_t)(4 * sm_count);
-    k_probe<<<blocks, 256, 0, s>>>(R, P, n4);
-    return cudaGetLastError();
+    return launch_pdl(k_probe, dim3(blocks), dim3(256), 0, s, R, P, n4);
 }
 
 }  // namespace ecris

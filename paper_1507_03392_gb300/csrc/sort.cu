@@ -10,9 +10,13 @@
 // for the collision kernels.
 //
 // Passes: count keys into a histogram (2 Nc + 1 bins: ions by cell, atoms by
-// cell, one bin for frozen and padding slots); exclusive scan; move every
-// particle to off[key] + (histogram counted down by one), which leaves the
-// histogram zero for the next sort.  Order inside a bin follows the atomics
+// cell, one bin for frozen and padding slots); exclusive scan of it by blocks,
+// whose totals the last block scans; move every particle to its key's place in
+// the block, the block's offset and (histogram counted down by one), which
+// leaves the histogram zero for the next sort.  A small run's sort is the
+// latency of its launches: three, each free to start while the one before it
+// ends (1000 steps of 1e4 particles with 31 sorts over 65536 cells take 1.63 ms;
+// with the scan in three launches and no overlap 2.10).  Order inside a bin follows the atomics
 // and does not matter.  The move writes the destination arrays directly when
 // the input is mostly in key order already (every sort but the first after a
 // load), since a warp's lanes then land on consecutive places and the eight
@@ -48,6 +52,8 @@ __device__ __forceinline__ uint32_t sort_key(const RunDev& R, uint32_t i)
 // whole warps share a key)
 __global__ void k_sort_count(const __grid_constant__ RunDev R, uint32_t cap, uint32_t* __restrict__ hist)
 {
+    pdl_wait();
+    pdl_trigger();
     const uint32_t stride = gridDim.x * blockDim.x;
     const uint32_t end = (cap + 31u) & ~31u;   // whole warps iterate together
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < end; i += stride) {
@@ -71,19 +77,11 @@ __device__ __forceinline__ uint32_t warp_incl(uint32_t v)
     return v;
 }
 
-// block-local exclusive scan of in[0, n) into out, block totals to blk
-__global__ void __launch_bounds__(kSortThreads) k_scan1(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
-                                                        uint32_t* __restrict__ blk, uint32_t n)
+// exclusive scan over the block's kSortThreads threads; *total: the sum
+__device__ __forceinline__ uint32_t block_excl(uint32_t v, uint32_t* total)
 {
-    __shared__ uint32_t ws[kSortThreads / 32];
-    const uint32_t base = blockIdx.x * kSortScanBlock + threadIdx.x * kSortPerThread;
-    uint32_t v[kSortPerThread], sum = 0;
-#pragma unroll
-    for (int j = 0; j < kSortPerThread; ++j) {
-        v[j] = base + j < n ? in[base + j] : 0u;
-        sum += v[j];
-    }
-    const uint32_t incl = warp_incl(sum);
+    __shared__ uint32_t ws[kSortThreads / 32 + 1];
+    const uint32_t incl = warp_incl(v);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 31) ws[warp] = incl;
     __syncthreads();
@@ -91,61 +89,55 @@ __global__ void __launch_bounds__(kSortThreads) k_scan1(const uint32_t* __restri
         const uint32_t w = lane < kSortThreads / 32 ? ws[lane] : 0u;
         const uint32_t wi = warp_incl(w);
         if (lane < kSortThreads / 32) ws[lane] = wi - w;
-        if (lane == kSortThreads / 32 - 1) blk[blockIdx.x] = wi;
+        if (lane == kSortThreads / 32 - 1) ws[kSortThreads / 32] = wi;
     }
     __syncthreads();
-    uint32_t o = ws[warp] + incl - sum;
+    *total = ws[kSortThreads / 32];
+    return ws[warp] + incl - v;
+}
+
+// exclusive scan of in[0, n) into out within blocks of kSortScanBlock; blk: the
+// blocks' offsets (ticket: a zero word, left zero)
+__global__ void __launch_bounds__(kSortThreads) k_sort_scan(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
+                                                            uint32_t* blk, uint32_t n, uint32_t* ticket)
+{
+    pdl_wait();
+    pdl_trigger();
+    const uint32_t base = blockIdx.x * kSortScanBlock + threadIdx.x * kSortPerThread, nb = gridDim.x;
+    uint32_t v[kSortPerThread], sum = 0, total;
+#pragma unroll
+    for (int j = 0; j < kSortPerThread; ++j) {
+        v[j] = base + j < n ? in[base + j] : 0u;
+        sum += v[j];
+    }
+    uint32_t o = block_excl(sum, &total);
 #pragma unroll
     for (int j = 0; j < kSortPerThread; ++j) {
         if (base + j < n) out[base + j] = o;
         o += v[j];
     }
-}
-
-// one block: exclusive scan of the block totals in place, total to out[n]
-__global__ void __launch_bounds__(1024) k_scan2(uint32_t* __restrict__ blk, uint32_t nb, uint32_t* __restrict__ out,
-                                                uint32_t n)
-{
-    __shared__ uint32_t ws[32];
-    const uint32_t per = (nb + 1023) / 1024, base = threadIdx.x * per;
-    uint32_t sum = 0;
-    for (uint32_t j = 0; j < per; ++j)
-        if (base + j < nb) sum += blk[base + j];
-    const uint32_t incl = warp_incl(sum);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 31) ws[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const uint32_t w = ws[lane];
-        const uint32_t wi = warp_incl(w);
-        ws[lane] = wi - w;
-        if (lane == 31) out[n] = wi;
+    if (threadIdx.x == 0) blk[blockIdx.x] = total;
+    if (!last_block(ticket)) return;
+    uint32_t carry = 0;
+    for (uint32_t b0 = 0; b0 < nb; b0 += kSortThreads) {
+        const uint32_t b = b0 + threadIdx.x;
+        const uint32_t t = b < nb ? __ldcg(blk + b) : 0u;
+        __syncthreads();   // (the scan's shared memory is used again)
+        const uint32_t at = carry + block_excl(t, &total);
+        if (b < nb) blk[b] = at;
+        carry += total;
     }
-    __syncthreads();
-    uint32_t o = ws[warp] + incl - sum;
-    for (uint32_t j = 0; j < per; ++j) {
-        if (base + j < nb) {
-            const uint32_t t = blk[base + j];
-            blk[base + j] = o;
-            o += t;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kSortThreads) k_scan3(uint32_t* __restrict__ out, const uint32_t* __restrict__ blk,
-                                                        uint32_t n)
-{
-    const uint32_t add = blk[blockIdx.x], base = blockIdx.x * kSortScanBlock;
-    for (uint32_t j = threadIdx.x; j < (uint32_t)kSortScanBlock; j += kSortThreads)
-        if (base + j < n) out[base + j] += add;
 }
 
 // kRecords: write 32-byte records to aos (unpacked by k_sort_unpack), else
 // the destination arrays
 template <bool kRecords>
 __global__ void k_sort_move(const __grid_constant__ RunDev R, uint32_t cap, ParticleSet dst, uint4* __restrict__ aos,
-                            uint32_t* __restrict__ hist, const uint32_t* __restrict__ off)
+                            uint32_t* __restrict__ hist, const uint32_t* __restrict__ off,
+                            const uint32_t* __restrict__ blk)
 {
+    pdl_wait();
+    pdl_trigger();
     const uint32_t stride = gridDim.x * blockDim.x;
     const uint32_t end = (cap + 31u) & ~31u;
     const uint32_t lane = threadIdx.x & 31;
@@ -169,7 +161,7 @@ __global__ void k_sort_move(const __grid_constant__ RunDev R, uint32_t cap, Part
         }
         const uint32_t act = __ballot_sync(0xFFFFFFFFu, in);
         if (!in) continue;
-        const uint32_t base = off[key];
+        const uint32_t base = off[key] + blk[key / kSortScanBlock];
         // one atomic per group of lanes with the same key; lanes take
         // consecutive places below the group's previous count
         const uint32_t grp = __match_any_sync(act, key);
@@ -198,6 +190,8 @@ __global__ void k_sort_move(const __grid_constant__ RunDev R, uint32_t cap, Part
 // records in sorted order -> the destination arrays, coalesced both ways
 __global__ void k_sort_unpack(const uint4* __restrict__ aos, uint32_t cap, ParticleSet dst)
 {
+    pdl_wait();
+    pdl_trigger();
     for (uint32_t d = blockIdx.x * blockDim.x + threadIdx.x; d < cap; d += gridDim.x * blockDim.x) {
         const uint4 a = aos[2 * (size_t)d], b = aos[2 * (size_t)d + 1];
         dst.x[d] = (int32_t)a.x;
@@ -221,6 +215,8 @@ struct OutPtrs { float* p[6]; };
 __global__ void k_export_records(const __grid_constant__ RunDev R, uint32_t n, uint32_t cap, uint4* __restrict__ rec,
                                  double sxy, double sz)
 {
+    pdl_wait();
+    pdl_trigger();
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cap; i += gridDim.x * blockDim.x) {
         const uint32_t d = R.id[i];
         if (d >= n) continue;   // padding
@@ -234,6 +230,8 @@ __global__ void k_export_records(const __grid_constant__ RunDev R, uint32_t n, u
 
 __global__ void k_export_unpack(const uint4* __restrict__ rec, uint32_t n, OutPtrs out, uint32_t* __restrict__ meta_out)
 {
+    pdl_wait();
+    pdl_trigger();
     for (uint32_t d = blockIdx.x * blockDim.x + threadIdx.x; d < n; d += gridDim.x * blockDim.x) {
         const uint4 a = rec[2 * (size_t)d], b = rec[2 * (size_t)d + 1];
         if (out.p[0]) out.p[0][d] = __uint_as_float(a.x);
@@ -249,6 +247,8 @@ __global__ void k_export_unpack(const uint4* __restrict__ rec, uint32_t n, OutPt
 __global__ void k_export_ordered(const __grid_constant__ RunDev R, uint32_t n, uint32_t cap, OutPtrs out,
                                  uint32_t* __restrict__ meta_out, double sxy, double sz)
 {
+    pdl_wait();
+    pdl_trigger();
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cap; i += gridDim.x * blockDim.x) {
         const uint32_t d = R.id[i];
         if (d >= n) continue;   // padding
@@ -280,23 +280,18 @@ cudaError_t launch_sort(const RunDev& R, uint32_t cap, const ParticleSet& dst, u
                         uint32_t* blk, unsigned long long* plan, uint4* aos, cudaStream_t s)
 {
     const uint32_t nbins = 2u * R.ncells + 1u;
-    const int nb = sort_scan_blocks(nbins);
-    k_sort_count<<<grid_for(cap, 256, 8192), 256, 0, s>>>(R, cap, hist);
-    k_scan1<<<nb, kSortThreads, 0, s>>>(hist, off, blk, nbins);
-    k_scan2<<<1, 1024, 0, s>>>(blk, (uint32_t)nb, off, nbins);
-    k_scan3<<<nb, kSortThreads, 0, s>>>(off, blk, nbins);
-    if (plan) {
-        const cudaError_t e = launch_plan(R, hist, false, plan, s);
-        if (e != cudaSuccess) return e;
-    }
-    if (aos) {
-        k_sort_move<true><<<grid_for(cap, 256, 8192), 256, 0, s>>>(R, cap, dst, aos, hist, off);
-        const ParticleSet src{R.x, R.y, R.z, R.vx, R.vy, R.vz, R.meta, R.id};
-        k_sort_unpack<<<grid_for(cap, 256, 8192), 256, 0, s>>>(aos, cap, src);
-    } else {
-        k_sort_move<false><<<grid_for(cap, 256, 8192), 256, 0, s>>>(R, cap, dst, nullptr, hist, off);
-    }
-    return cudaGetLastError();
+    const dim3 grid(grid_for(cap, 256, 8192)), block(256);
+    cudaError_t e = launch_pdl(k_sort_count, grid, block, 0, s, R, cap, hist);
+    if (e == cudaSuccess)
+        e = launch_pdl(k_sort_scan, dim3(sort_scan_blocks(nbins)), dim3(kSortThreads), 0, s, (const uint32_t*)hist, off,
+                       blk, nbins, hist + nbins);
+    if (e == cudaSuccess && plan) e = launch_plan(R, hist, false, plan, s);
+    if (e == cudaSuccess)
+        e = launch_pdl(aos ? k_sort_move<true> : k_sort_move<false>, grid, block, 0, s, R, cap, dst, aos, hist,
+                       (const uint32_t*)off, (const uint32_t*)blk);
+    const ParticleSet src{R.x, R.y, R.z, R.vx, R.vy, R.vz, R.meta, R.id};
+    if (e == cudaSuccess && aos) e = launch_pdl(k_sort_unpack, grid, block, 0, s, (const uint4*)aos, cap, src);
+    return e;
 }
 
 cudaError_t launch_export_ordered(const RunDev& R, uint32_t n, uint32_t cap, float* const out[6], uint32_t* meta_out,
@@ -304,13 +299,12 @@ cudaError_t launch_export_ordered(const RunDev& R, uint32_t n, uint32_t cap, flo
 {
     OutPtrs o;
     for (int k = 0; k < 6; ++k) o.p[k] = out ? out[k] : nullptr;
-    if (rec && n >= kExportRecords) {
-        k_export_records<<<grid_for(cap, 256, 8192), 256, 0, s>>>(R, n, cap, rec, sxy, sz);
-        k_export_unpack<<<grid_for(n, 256, 8192), 256, 0, s>>>(rec, n, o, meta_out);
-    } else {
-        k_export_ordered<<<grid_for(cap, 256, 8192), 256, 0, s>>>(R, n, cap, o, meta_out, sxy, sz);
-    }
-    return cudaGetLastError();
+    const dim3 grid(grid_for(cap, 256, 8192)), block(256);
+    if (!rec || n < kExportRecords)
+        return launch_pdl(k_export_ordered, grid, block, 0, s, R, n, cap, o, meta_out, sxy, sz);
+    const cudaError_t e = launch_pdl(k_export_records, grid, block, 0, s, R, n, cap, rec, sxy, sz);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(k_export_unpack, dim3(grid_for(n, 256, 8192)), block, 0, s, (const uint4*)rec, n, o, meta_out);
 }
 
 }  // namespace ecris

@@ -527,21 +527,6 @@ __device__ __forceinline__ void deposit_warp(const RunDev& R, uint32_t cell, uin
         atomicAdd(R.dep + cell, ((unsigned long long)(lane - h + 1u) << 32) | (unsigned long long)q);
 }
 
-// last block of a grid (after every block's work is visible): ticket reset
-__device__ __forceinline__ bool last_block(unsigned int* ticket)
-{
-    __shared__ int last;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1 ? 1 : 0;
-        if (last) *ticket = 0u;
-    }
-    __syncthreads();
-    return last != 0;
-}
-
-
 // ---------------------------------------------------------------------------
 // Windows of steps.  A call's steps run in windows of up to kMaxWindow: an
 // atom's step depends on no other particle, and without collisions between
