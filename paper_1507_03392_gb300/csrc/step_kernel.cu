@@ -897,6 +897,33 @@ __global__ void __launch_bounds__(128, kOne ? 8 : kQuietBlocks) k_quiet(const __
 // entries of a run's list: its ions, padded to whole warps, then its atoms
 __device__ __forceinline__ uint32_t list_entries(uint32_t ni, uint32_t na) { return ((ni + 31u) & ~31u) + na; }
 
+// Entries a warp takes (log2): 32, or fewer if the run's list is so short that
+// the grid has warps to spare.  The lanes of a warp of atoms leave the chamber in
+// different steps, and each one that does takes the whole warp through its FP64
+// geometry (k_active, 1e4 particles x 32 steps: 33 us with 32 a warp, 30 so).
+// Not in k_ions: in one step few do, and more warps add to the deposit and the
+// buckets more often (2e4 and 2e5 particles 2 and 4 % slower).
+__device__ __forceinline__ uint32_t list_lanes(uint32_t entries)
+{
+    uint32_t lw = 5u;
+    while (lw > 0u && (entries >> (lw - 1u)) <= gridDim.x * (blockDim.x >> 5)) --lw;
+    return lw;
+}
+
+// tiles of a run's list
+__device__ __forceinline__ uint32_t list_tiles(uint32_t entries, uint32_t lw)
+{
+    const uint32_t warps = (entries + (1u << lw) - 1u) >> lw, per = blockDim.x >> 5;
+    return (warps + per - 1u) / per;
+}
+
+// this lane's entry of tile t (none: past every list)
+__device__ __forceinline__ uint32_t list_entry(uint32_t t, uint32_t lw)
+{
+    const uint32_t lane = threadIdx.x & 31u, w = t * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    return lane >> lw ? 0xFFFFFFFFu : (w << lw) + lane;
+}
+
 // every run of a batch; the last block works out where each run's tiles of
 // listed particles start in the passes over them: pref[r] for the runs without
 // collisions between ions (k_active_batch), pref[nruns + 1 + r] for those with
@@ -987,10 +1014,11 @@ __device__ __noinline__ Left leave_call(const RunDev& R, uint32_t pid, uint32_t 
 // One tile of k_active: entries [t T, (t + 1) T) of the run's list, one a thread
 // of the block of T, K steps each
 template <bool kVar, bool kPlain>
-__device__ __forceinline__ void active_tile(const RunDev& R, uint32_t t, uint32_t K, uint32_t ni, uint32_t na)
+__device__ __forceinline__ void active_tile(const RunDev& R, uint32_t t, uint32_t K, uint32_t ni, uint32_t na,
+                                            uint32_t lw = 5u)
 {
     const uint32_t step0 = *R.step, ni32 = (ni + 31u) & ~31u, nslot = 4u * R.n4;
-    const uint32_t e = t * blockDim.x + threadIdx.x;
+    const uint32_t e = list_entry(t, lw);
     const bool in = e < ni || (e >= ni32 && e - ni32 < na);
     if (!__any_sync(0xFFFFFFFFu, in)) return;
     uint32_t i = 0u, id = 0u, meta = kStPad;
@@ -1052,11 +1080,11 @@ __global__ void __launch_bounds__(kActiveTile, kVar ? 8 : 6) k_active(const __gr
     pdl_wait();
     pdl_trigger();
     const uint32_t ni = R.nleave[0], na = R.nleave[1];
-    const uint32_t nt = (list_entries(ni, na) + blockDim.x - 1u) / blockDim.x;
+    const uint32_t lw = list_lanes(list_entries(ni, na)), nt = list_tiles(list_entries(ni, na), lw);
     const bool plain = !kVar && plain_run(R);
     for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
-        if (!kVar && plain) active_tile<false, true>(R, t, K, ni, na);
-        else active_tile<kVar, false>(R, t, K, ni, na);
+        if (!kVar && plain) active_tile<false, true>(R, t, K, ni, na, lw);
+        else active_tile<kVar, false>(R, t, K, ni, na, lw);
     }
     if (last_block(ticket) && threadIdx.x == 0) {
         R.nleave[0] = 0u;
