@@ -292,6 +292,7 @@ struct KernelTimer {
 // step, nleave[3], ticket, err, bad[2], cword[kCwWords]
 constexpr size_t kZeroBytes = (kTallyWords + kFptdWords) * sizeof(unsigned long long) + (8 + kCwWords) * sizeof(uint32_t);
 
+constexpr size_t kLoadAside = 1u << 19;   // particles of a load from the host that uses two streams
 constexpr uint32_t kSortAfterLoad = 8;   // steps of one ecris_step call that sort a fresh load first
 
 struct ecris_ctx {
@@ -388,6 +389,9 @@ struct ecris_ctx {
     uint32_t fold_every = 1, since_fold = 0;
 
     KernelTimer timer;          // ecris_set_profiling
+    // large loads from the host (made by the first)
+    cudaStream_t load_stream = nullptr;
+    cudaEvent_t load_event[2] = {nullptr, nullptr};
 };
 
 namespace {
@@ -425,6 +429,17 @@ void free_async(ecris_ctx* ctx, T*& p)
 {
     if (p) cudaFreeAsync(p, ctx->stream);
     p = nullptr;
+}
+
+// the load's stream; its last work was waited for by the context's own stream
+void free_load_stream(ecris_ctx* ctx)
+{
+    for (auto& ev : ctx->load_event) {
+        if (ev) cudaEventDestroy(ev);
+        ev = nullptr;
+    }
+    if (ctx->load_stream) cudaStreamDestroy(ctx->load_stream);
+    ctx->load_stream = nullptr;
 }
 
 void free_ions(ecris_ctx* ctx)
@@ -948,6 +963,7 @@ void ecris_destroy(ecris_ctx* ctx)
     free_fields(ctx);
     cudaStreamSynchronize(ctx->stream);
     ctx->timer.release();
+    free_load_stream(ctx);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     if (ctx->h_run) cudaFreeHost(ctx->h_run);
     if (ctx->h_kdt) cudaFreeHost(ctx->h_kdt);
@@ -1215,16 +1231,30 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
     ctx->n = n;
     ctx->n4 = n4;
     const cudaMemcpyKind kind = src_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    // A large load from the host is bound by the link: while the velocities
+    // cross, the positions are converted and the counters cleared on a stream
+    // of their own (load, one step and read-back of 4e6 particles: 940 us in order, 917 so;
+    // 5.3e5: 281 and 259; 3e5 gain nothing)
+    const bool aside = !src_is_device && n >= kLoadAside;
+    if (aside && !ctx->load_stream) {
+        CK(cudaStreamCreateWithFlags(&ctx->load_stream, cudaStreamNonBlocking));
+        for (auto& ev : ctx->load_event) CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    }
+    cudaStream_t side = aside ? ctx->load_stream : ctx->stream;
     if (n) {
-        for (int k = 0; k < 6; ++k)
+        for (int k = 0; k < (aside ? 3 : 6); ++k)
             CK(cudaMemcpyAsync(ctx->d_soa[k], xyzv[k], n * sizeof(float), kind, ctx->stream));
         CK(cudaMemcpyAsync(ctx->d_q8, q, n, kind, ctx->stream));
     }
+    if (aside) {
+        CK(cudaEventRecord(ctx->load_event[0], ctx->stream));
+        CK(cudaStreamWaitEvent(side, ctx->load_event[0], 0));
+    }
     if (ctx->d_ccount)
-        CK(cudaMemsetAsync(ctx->d_ccount, 0, (2 * nc + std::min(nc, ctx->cap)) * sizeof(uint32_t), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_dep, 0, 4 * nc * sizeof(unsigned long long), ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_zero, 0, kZeroBytes, ctx->stream));
-    CK(cudaMemsetAsync(ctx->d_birth, 0xFF, ctx->cap * sizeof(uint32_t), ctx->stream));   // births unknown
+        CK(cudaMemsetAsync(ctx->d_ccount, 0, (2 * nc + std::min(nc, ctx->cap)) * sizeof(uint32_t), side));
+    CK(cudaMemsetAsync(ctx->d_dep, 0, 4 * nc * sizeof(unsigned long long), side));
+    CK(cudaMemsetAsync(ctx->d_zero, 0, kZeroBytes, side));
+    CK(cudaMemsetAsync(ctx->d_birth, 0xFF, ctx->cap * sizeof(uint32_t), side));   // births unknown
     {
         const ecris_status pst = zero_probes(ctx);
         if (pst != ECRIS_OK) return pst;
@@ -1249,7 +1279,14 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
     lc.nz = h.nz;
     lc.count = ctx->d_ccount;
     CK(launch_load_init(lc, ctx->d_soa, ctx->d_q8, ctx->d_meta, ctx->d_id, (uint32_t)n, (uint32_t)cap, ctx->d_bad,
-                        ctx->stream));
+                        !aside, side));
+    if (aside) {
+        CK(cudaEventRecord(ctx->load_event[1], side));
+        for (int k = 3; k < 6; ++k)
+            CK(cudaMemcpyAsync(ctx->d_soa[k], xyzv[k], n * sizeof(float), kind, ctx->stream));
+        CK(cudaStreamWaitEvent(ctx->stream, ctx->load_event[1], 0));
+        CK(launch_load_check(ctx->d_soa, ctx->d_meta, (uint32_t)n, (uint32_t)cap, ctx->d_bad, ctx->stream));
+    }
     unsigned int bad[2] = {0u, 0u};
     CK(cudaMemcpyAsync(bad, ctx->d_bad, sizeof bad, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
@@ -1487,8 +1524,10 @@ ecris_status ecris_get_state(ecris_ctx* ctx, float* const xyzv[6], uint32_t* met
         // the particles sit in sorted order: scatter them back to load order
         // by their ids (into the caller's device arrays, or via the spare set)
         if (dst_is_device) {
+            // (before the first sort the order is the load's: no scatter, no records;
+            // 4e6 particles 115 us with them, 100 without)
             CK(launch_export_ordered(*ctx->h_run, (uint32_t)n, (uint32_t)(4 * ctx->n4), xyzv, meta, sxy, sz,
-                                     reinterpret_cast<uint4*>(ctx->d_soa2[0]), ctx->stream));
+                                     ctx->fresh ? nullptr : reinterpret_cast<uint4*>(ctx->d_soa2[0]), ctx->stream));
         } else {
             float* spare[6];
             for (int k = 0; k < 6; ++k) spare[k] = (xyzv && xyzv[k]) ? ctx->d_soa2[k] : nullptr;
@@ -1619,6 +1658,7 @@ void batch_release_run(ecris_batch* b, ecris_ctx* c)
     free_ions(c);
     free_fields(c);
     c->timer.release();
+    free_load_stream(c);
     if (c->h_run) b->old_host.push_back(c->h_run);
     if (c->h_kdt) b->old_host.push_back(c->h_kdt);
     delete c;

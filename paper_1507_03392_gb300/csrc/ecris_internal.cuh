@@ -463,11 +463,16 @@ struct LoadCheck {
     int32_t nx, ny, nz;
     uint32_t* count;                // ions per cell, added up for the first plan (nullptr: no collisions)
 };
-// check particles [0, n), convert their positions (metres, float) in place to
-// fixed point, build their meta words from q8 and ids, fill pads [n, cap);
-// bad[0] counts invalid particles, ~bad[1] is the lowest invalid index (bad zeroed before)
+// check the positions and charge states of particles [0, n), convert the
+// positions (metres, float) in place to fixed point, build the meta words from
+// q8 and the ids, fill pads [n, cap); and the velocities, now or in
+// launch_load_check.  bad[0] counts invalid particles, ~bad[1] is the lowest invalid
+// index (bad zeroed before)
 cudaError_t launch_load_init(const LoadCheck& lc, float* const soa[6], const uint8_t* q8, uint32_t* meta,
-                             uint32_t* id, uint32_t n, uint32_t cap, unsigned int* bad, cudaStream_t s);
+                             uint32_t* id, uint32_t n, uint32_t cap, unsigned int* bad, bool velocities,
+                             cudaStream_t s);
+cudaError_t launch_load_check(float* const soa[6], const uint32_t* meta, uint32_t n, uint32_t cap, unsigned int* bad,
+                              cudaStream_t s);
 
 // One set of particle arrays (the sort moves particles between two sets).
 struct ParticleSet {

@@ -1290,32 +1290,56 @@ __device__ __forceinline__ void store_fx(SoaPtrs soa, uint32_t i, const int3& p)
     reinterpret_cast<int32_t*>(soa.p[2])[i] = p.z;
 }
 
+__device__ __forceinline__ bool velocity_ok(const SoaPtrs& soa, uint32_t i)
+{
+    const float vx = soa.p[3][i], vy = soa.p[4][i], vz = soa.p[5][i];
+    return isfinite(vx) & isfinite(vy) & isfinite(vz);   // (three loads at once)
+}
+
+__device__ __forceinline__ void pad_velocity(const SoaPtrs& soa, uint32_t i)
+{
+    soa.p[3][i] = soa.p[4][i] = soa.p[5][i] = 0.0f;
+}
+
 __global__ void k_load_init(LoadCheck lc, SoaPtrs soa, const uint8_t* __restrict__ q8,
                             uint32_t* __restrict__ meta, uint32_t* __restrict__ id, uint32_t n, uint32_t cap,
-                            unsigned int* __restrict__ bad)
+                            unsigned int* __restrict__ bad, int velocities)
 {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cap; i += gridDim.x * blockDim.x) {
         id[i] = i;
         if (i < n) {
             const float x = soa.p[0][i], y = soa.p[1][i], z = soa.p[2][i];
-            const float vx = soa.p[3][i], vy = soa.p[4][i], vz = soa.p[5][i];
             const uint32_t q = q8[i];
-            const bool ok = (x * x + y * y <= lc.R0sq) && (z >= 0.0f) && (z <= lc.L) &&
-                            isfinite(vx) && isfinite(vy) && isfinite(vz) && q <= lc.qmax;
+            bool ok = (x * x + y * y <= lc.R0sq) && (z >= 0.0f) && (z <= lc.L) && q <= lc.qmax;
+            if (velocities) ok = ok && velocity_ok(soa, i);
             if (!ok) {
                 atomicAdd(bad, 1u);
                 atomicMax(bad + 1, ~i);
             }
-            meta[i] = q;
+            meta[i] = ok ? q : kStPad;   // (counted: the velocity check leaves it out)
             const int3 p = to_fx(x, y, z, lc);
             store_fx(soa, i, p);
             if (lc.count && q > 0u) atomicAdd(lc.count + ngp_cell(lc, p.x, p.y, p.z), 1u);
         } else {
             store_fx(soa, i, to_fx(lc.inlet_x, lc.inlet_y, lc.inlet_z, lc));
-            soa.p[3][i] = 0.0f;
-            soa.p[4][i] = 0.0f;
-            soa.p[5][i] = 0.0f;
             meta[i] = kStPad;
+            if (velocities) pad_velocity(soa, i);
+        }
+    }
+}
+
+// the velocities alone
+__global__ void k_load_check(SoaPtrs soa, const uint32_t* __restrict__ meta, uint32_t n, uint32_t cap,
+                             unsigned int* __restrict__ bad)
+{
+    pdl_wait();
+    pdl_trigger();
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cap; i += gridDim.x * blockDim.x) {
+        if (i >= n) {
+            pad_velocity(soa, i);
+        } else if (!velocity_ok(soa, i) && meta[i] != kStPad) {
+            atomicAdd(bad, 1u);
+            atomicMax(bad + 1, ~i);
         }
     }
 }
@@ -1323,15 +1347,24 @@ __global__ void k_load_init(LoadCheck lc, SoaPtrs soa, const uint8_t* __restrict
 }  // namespace
 
 cudaError_t launch_load_init(const LoadCheck& lc, float* const soa[6], const uint8_t* q8, uint32_t* meta,
-                             uint32_t* id, uint32_t n, uint32_t cap, unsigned int* bad, cudaStream_t s)
+                             uint32_t* id, uint32_t n, uint32_t cap, unsigned int* bad, bool velocities,
+                             cudaStream_t s)
 {
     SoaPtrs p;
     for (int k = 0; k < 6; ++k) p.p[k] = soa[k];
     const int threads = 256;
     int blocks = (int)((cap + threads - 1) / threads);
     if (blocks > 8192) blocks = 8192;
-    k_load_init<<<blocks, threads, 0, s>>>(lc, p, q8, meta, id, n, cap, bad);
+    k_load_init<<<blocks, threads, 0, s>>>(lc, p, q8, meta, id, n, cap, bad, velocities ? 1 : 0);
     return cudaGetLastError();
+}
+
+cudaError_t launch_load_check(float* const soa[6], const uint32_t* meta, uint32_t n, uint32_t cap, unsigned int* bad,
+                              cudaStream_t s)
+{
+    SoaPtrs p;
+    for (int k = 0; k < 6; ++k) p.p[k] = soa[k];
+    return launch_pdl(k_load_check, dim3(std::min((cap + 255u) / 256u, 8192u)), dim3(256), 0, s, p, meta, n, cap, bad);
 }
 
 template <class K>
