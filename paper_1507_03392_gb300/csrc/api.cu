@@ -1233,8 +1233,8 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
     const cudaMemcpyKind kind = src_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     // A large load from the host is bound by the link: while the velocities
     // cross, the positions are converted and the counters cleared on a stream
-    // of their own (load, one step and read-back of 4e6 particles: 940 us in order, 917 so;
-    // 5.3e5: 281 and 259; 3e5 gain nothing)
+    // of their own (load, one step and read-back of 4e6 particles: 24 us
+    // less so, of 5.3e5 15 less; 3e5 gain nothing)
     const bool aside = !src_is_device && n >= kLoadAside;
     if (aside && !ctx->load_stream) {
         CK(cudaStreamCreateWithFlags(&ctx->load_stream, cudaStreamNonBlocking));
@@ -1525,7 +1525,7 @@ ecris_status ecris_get_state(ecris_ctx* ctx, float* const xyzv[6], uint32_t* met
         // by their ids (into the caller's device arrays, or via the spare set)
         if (dst_is_device) {
             // (before the first sort the order is the load's: no scatter, no records;
-            // 4e6 particles 115 us with them, 100 without)
+            // 2e6 particles 48 us with them, 22 without)
             CK(launch_export_ordered(*ctx->h_run, (uint32_t)n, (uint32_t)(4 * ctx->n4), xyzv, meta, sxy, sz,
                                      ctx->fresh ? nullptr : reinterpret_cast<uint4*>(ctx->d_soa2[0]), ctx->stream));
         } else {

@@ -205,6 +205,78 @@ __global__ void k_sort_unpack(const uint4* __restrict__ aos, uint32_t cap, Parti
     }
 }
 
+// Fixed point to metres, (float)((double)k s) for the whole number k = hi + lo
+// (both exact in FP32) and s = s_hi + s_lo + what 2^-49 s bounds.  The GPU has
+// few FP64 units, and ten FP64 instructions a particle and loads waiting for
+// stores bound the whole export (4e6 particles in load order 100 us, 40 so).  Here the product is formed as an unevaluated FP32 sum, h = fl(hi s_hi)
+// with its exact error (an FMA) and the cross terms, to 2^-44.8 of its size: terms
+// of 2^-22 and less, rounded twice, and lo s_lo <= 2^-47 left out.  Its rounding to
+// FP32 is that of the FP64 product unless the sum lies within that of the middle
+// between two FP32 numbers (or r is a power of two, below which they lie
+// closer); those few, one in 2^17, take the FP64 product itself.
+struct Scale {
+    double s;
+    float hi, lo;
+};
+
+Scale make_scale(double s) { return Scale{s, (float)s, (float)(s - (double)(float)s)}; }
+
+// (out of line: inlined, its instructions are issued for every particle)
+__device__ __noinline__ float to_metres_fp64(float hi, float lo, double s)
+{
+    return (float)(((double)hi + (double)lo) * s);
+}
+
+__device__ __forceinline__ float to_metres(float hi, float lo, const Scale& c)
+{
+    const float h = __fmul_rn(hi, c.hi);
+    const float t = __fmaf_rn(lo, c.hi, __fmaf_rn(hi, c.lo, __fmaf_rn(hi, c.hi, -h)));
+    const float r = __fadd_rn(h, t);
+    const float d = fabsf(__fsub_rn(t, __fsub_rn(r, h)));   // (exact: |t| < |h|, or both are 0)
+    const uint32_t bits = __float_as_uint(r);
+    const float half = __uint_as_float((bits & 0x7F800000u) - (24u << 23));   // half the spacing above |r|
+    if (fabsf(__fsub_rn(d, half)) <= half * 3.8146973e-6f || !(bits & 0x007FFFFFu))
+        return to_metres_fp64(hi, lo, c.s);
+    return r;
+}
+
+// a signed and an unsigned coordinate (see fx_xy, fx_z), truncated to FP32 and
+// the rest
+__device__ __forceinline__ float metres_xy(int32_t X, const Scale& c)
+{
+    const float hi = __int2float_rz(X);
+    return to_metres(hi, (float)(X - __float2int_rz(hi)), c);
+}
+
+__device__ __forceinline__ float metres_z(int32_t Z, const Scale& c)
+{
+    const uint32_t U = (uint32_t)Z ^ 0x80000000u;
+    const float hi = __uint2float_rz(U);
+    return to_metres(hi, (float)(U - __float2uint_rz(hi)), c);
+}
+
+// a particle's words as the export writes them, all loaded at once (a load
+// behind the store of the word before it waits for each in turn)
+struct Exported {
+    uint32_t d, meta;
+    float v[6];
+};
+
+__device__ __forceinline__ Exported exported(const RunDev& R, uint32_t i, const Scale& sxy, const Scale& sz)
+{
+    Exported e;
+    e.d = R.id[i];
+    const int32_t X = R.x[i], Y = R.y[i], Z = R.z[i];
+    e.v[3] = R.vx[i];
+    e.v[4] = R.vy[i];
+    e.v[5] = R.vz[i];
+    e.meta = R.meta[i];
+    e.v[0] = metres_xy(X, sxy);
+    e.v[1] = metres_xy(Y, sxy);
+    e.v[2] = metres_z(Z, sz);
+    return e;
+}
+
 struct OutPtrs { float* p[6]; };
 
 // Export of a large run, first pass: the particle's 32-byte record to place
@@ -213,18 +285,16 @@ struct OutPtrs { float* p[6]; };
 // fit in L2); the records cost one full sector, and the second pass is
 // coalesced.
 __global__ void k_export_records(const __grid_constant__ RunDev R, uint32_t n, uint32_t cap, uint4* __restrict__ rec,
-                                 double sxy, double sz)
+                                 Scale sxy, Scale sz)
 {
     pdl_wait();
     pdl_trigger();
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cap; i += gridDim.x * blockDim.x) {
-        const uint32_t d = R.id[i];
-        if (d >= n) continue;   // padding
-        const float x = (float)((double)R.x[i] * sxy), y = (float)((double)R.y[i] * sxy);
-        const float z = (float)(((double)R.z[i] + 2147483648.0) * sz);
-        store_record(rec, d, make_uint4(__float_as_uint(x), __float_as_uint(y), __float_as_uint(z),
-                                        __float_as_uint(R.vx[i])),
-                     make_uint4(__float_as_uint(R.vy[i]), __float_as_uint(R.vz[i]), R.meta[i], 0u));
+        const Exported e = exported(R, i, sxy, sz);
+        if (e.d >= n) continue;   // padding
+        store_record(rec, e.d, make_uint4(__float_as_uint(e.v[0]), __float_as_uint(e.v[1]), __float_as_uint(e.v[2]),
+                                          __float_as_uint(e.v[3])),
+                     make_uint4(__float_as_uint(e.v[4]), __float_as_uint(e.v[5]), e.meta, 0u));
     }
 }
 
@@ -245,20 +315,17 @@ __global__ void k_export_unpack(const uint4* __restrict__ rec, uint32_t n, OutPt
 }
 
 __global__ void k_export_ordered(const __grid_constant__ RunDev R, uint32_t n, uint32_t cap, OutPtrs out,
-                                 uint32_t* __restrict__ meta_out, double sxy, double sz)
+                                 uint32_t* __restrict__ meta_out, Scale sxy, Scale sz)
 {
     pdl_wait();
     pdl_trigger();
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cap; i += gridDim.x * blockDim.x) {
-        const uint32_t d = R.id[i];
-        if (d >= n) continue;   // padding
-        if (out.p[0]) out.p[0][d] = (float)((double)R.x[i] * sxy);
-        if (out.p[1]) out.p[1][d] = (float)((double)R.y[i] * sxy);
-        if (out.p[2]) out.p[2][d] = (float)(((double)R.z[i] + 2147483648.0) * sz);
-        if (out.p[3]) out.p[3][d] = R.vx[i];
-        if (out.p[4]) out.p[4][d] = R.vy[i];
-        if (out.p[5]) out.p[5][d] = R.vz[i];
-        if (meta_out) meta_out[d] = R.meta[i];
+        const Exported e = exported(R, i, sxy, sz);
+        if (e.d >= n) continue;   // padding
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            if (out.p[k]) out.p[k][e.d] = e.v[k];
+        if (meta_out) meta_out[e.d] = e.meta;
     }
 }
 
@@ -301,8 +368,8 @@ cudaError_t launch_export_ordered(const RunDev& R, uint32_t n, uint32_t cap, flo
     for (int k = 0; k < 6; ++k) o.p[k] = out ? out[k] : nullptr;
     const dim3 grid(grid_for(cap, 256, 8192)), block(256);
     if (!rec || n < kExportRecords)
-        return launch_pdl(k_export_ordered, grid, block, 0, s, R, n, cap, o, meta_out, sxy, sz);
-    const cudaError_t e = launch_pdl(k_export_records, grid, block, 0, s, R, n, cap, rec, sxy, sz);
+        return launch_pdl(k_export_ordered, grid, block, 0, s, R, n, cap, o, meta_out, make_scale(sxy), make_scale(sz));
+    const cudaError_t e = launch_pdl(k_export_records, grid, block, 0, s, R, n, cap, rec, make_scale(sxy), make_scale(sz));
     if (e != cudaSuccess) return e;
     return launch_pdl(k_export_unpack, dim3(grid_for(n, 256, 8192)), block, 0, s, (const uint4*)rec, n, o, meta_out);
 }
