@@ -2349,15 +2349,21 @@ ecris_status batch_autotune(ecris_batch* b, uint32_t trial_steps, bool cadence, 
             best_shape = k;
         }
     }
-    // 2. resident blocks per SM of that shape
+    // 2. resident blocks per SM of that shape, from as many as fit downwards:
+    // the passes wait on memory, so once fewer are clearly slower the rest are
+    // slower still (a trial of one block an SM alone took as long as eight of
+    // the best: 6 requests of 4.5e6 particles 108 ms with all of them,
+    // 88 so)
     best = 1e30f;
     const WindowBlocks& m = b->max_bps[best_shape];
-    for (int bps = 1; bps <= std::max(m.quiet, std::max(m.active, m.ions)) && st == ECRIS_OK; ++bps) {
+    for (int bps = std::max(m.quiet, std::max(m.active, m.ions)); bps >= 1 && st == ECRIS_OK; --bps) {
         apply(best_shape, bps, orig_sort);
         st = time_steps(b, trial_steps, true, &ms);
         if (st == ECRIS_OK && ms < best) {
             best = ms;
             best_bps = bps;
+        } else if (ms > 1.1f * best) {
+            break;
         }
     }
     // 3. steps between sorts: whole sort periods, each starting with a sort,
