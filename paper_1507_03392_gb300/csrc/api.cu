@@ -1357,6 +1357,7 @@ ecris_status ecris_step(ecris_ctx* ctx, uint32_t nsteps, double dt)
         const uint32_t K = window_steps(ctx, nsteps - s, ctx->timer.on);
         const RunDev& R = *ctx->h_run;
         CK(timed(ctx, kKindStep, [&] {
+            if (K == 1) return launch_one(R, ctx->d_ticket, ctx->sm_count, ctx->stream);
             const cudaError_t e = launch_quiet(R, K, ctx->sm_count, ctx->stream);
             if (e != cudaSuccess) return e;
             return coulomb ? launch_ions(R, ctx->sm_count, ctx->stream)
@@ -1609,7 +1610,7 @@ struct ecris_batch {
     bool variants = false;          // some run has an opt-in process of kFVariants
     bool layout_dirty = true;       // work list must be rebuilt
     bool params_dirty = true;       // parameter blocks must be uploaded
-    unsigned int* d_ticket = nullptr;   // last-block ticket of the leaver pass
+    unsigned int* d_ticket = nullptr;   // ticket of the kernels whose last block ends a pass
     KernelTimer timer;              // ecris_batch_set_profiling
     int collide_grid = 0;       // most blocks of the collision kernel
     // side streams on which the layout sorts of the runs due for one run side
@@ -1753,14 +1754,17 @@ cudaError_t batch_side_streams(ecris_batch* b)
     return e;
 }
 
-// the first launch of a window: the quiet pass of every run, and the whole
-// window of the runs without collisions between ions
+// the first launches of a window: the quiet pass of every run, and the whole
+// window of the runs without collisions between ions; or one step of all runs
 cudaError_t batch_window(ecris_batch* b, uint32_t K)
 {
     const uint32_t nr = (uint32_t)b->runs.size();
     const int threads = shape_block(b->shape);
     const WindowBlocks& m = b->max_bps[b->shape];
     if (nr == 0) return cudaSuccess;
+    if (K == 1)
+        return launch_one_batch(b->d_runs, nr, b->d_items, b->nitems, shape_tile(b->shape), threads,
+                                batch_grid(b, m.one), b->variants, b->d_ticket, b->stream);
     cudaError_t e = launch_quiet_batch(b->d_runs, nr, b->d_items, b->nitems, shape_tile(b->shape), threads,
                                        batch_grid(b, m.quiet), K,
                                        b->d_pref, b->d_ticket, b->stream);
@@ -2005,7 +2009,7 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
             if (c) K = std::min(K, window_steps(c, K, b->timer.on));
         BCK(b->timer.run(kKindStep, b->stream, [&] {
             cudaError_t e = batch_window(b, K);
-            if (e == cudaSuccess && b->any_coulomb) e = batch_ions(b);
+            if (e == cudaSuccess && b->any_coulomb && K > 1) e = batch_ions(b);
             return e;
         }));
         for (uint32_t k = 0; b->any_coulomb && k < K; ++k) {
@@ -2359,7 +2363,7 @@ ecris_status batch_autotune(ecris_batch* b, uint32_t trial_steps, bool cadence, 
     // 88 so)
     best = 1e30f;
     const WindowBlocks& m = b->max_bps[best_shape];
-    for (int bps = std::max(m.quiet, std::max(m.active, m.ions)); bps >= 1 && st == ECRIS_OK; --bps) {
+    for (int bps = std::max(std::max(m.quiet, m.one), std::max(m.active, m.ions)); bps >= 1 && st == ECRIS_OK; --bps) {
         apply(best_shape, bps, orig_sort);
         st = time_steps(b, trial_steps, true, &ms);
         if (st == ECRIS_OK && ms < best) {

@@ -52,7 +52,7 @@ constexpr uint32_t kFDouble = 1u << 7;
 constexpr uint32_t kFElastic = 1u << 8;
 constexpr uint32_t kFRecomb = 1u << 9;
 constexpr uint32_t kFlagMask = 0x3FFu;
-// processes whose code only the variant step kernels carry (with the
+// processes whose code only the variant kernels carry (with the
 // on-axis field table)
 constexpr uint32_t kFVariants = kFDouble | kFElastic | kFRecomb;
 constexpr uint32_t kFHasE = 1u << 16;   // internal: the run has a nonzero E grid (the push gathers it)
@@ -314,7 +314,7 @@ __device__ __forceinline__ void bfield(const RunDev& R, float x, float y, float 
         b1 = R.aRk * s;
         b2 = R.aRk2 * c;
     }
-    // (FMAs written out: the step kernel is compiled without contraction)
+    // (FMAs written out: the kernels that step are compiled without contraction)
     const float hx = -0.5f * b1, hz = -0.25f * b2;
     const float r2 = fmaf(x, x, y * y);
     Bx = fmaf(hx, x, R.hex_c * (2.0f * x * y));
@@ -423,6 +423,9 @@ constexpr uint32_t kActiveTile = 128;   // threads a block of the passes over on
 cudaError_t launch_quiet(const RunDev& R, uint32_t K, int sm_count, cudaStream_t s);
 cudaError_t launch_active(const RunDev& R, uint32_t K, unsigned int* ticket, int sm_count, cudaStream_t s);
 cudaError_t launch_ions(const RunDev& R, int sm_count, cudaStream_t s);
+// instead of launch_quiet and what follows it, a window of one step (with
+// collisions between ions launch_coulomb follows, else the counter is advanced)
+cudaError_t launch_one(const RunDev& R, unsigned int* ticket, int sm_count, cudaStream_t s);
 // the same for every run of a batch: items are the (run, tile) work list of
 // `tile` particles a tile, pref 2 (nruns + 1) words of scratch, grid the
 // blocks; entries of runs with step == NULL are skipped.  variants: some run
@@ -434,8 +437,10 @@ cudaError_t launch_active_batch(const RunDev* runs, uint32_t nruns, int threads,
                                 const uint32_t* pref, unsigned int* ticket, cudaStream_t s);
 cudaError_t launch_ions_batch(const RunDev* runs, uint32_t nruns, int threads, int grid, bool variants,
                               const uint32_t* pref, cudaStream_t s);
+cudaError_t launch_one_batch(const RunDev* runs, uint32_t nruns, const uint2* items, uint32_t nitems, uint32_t tile,
+                             int threads, int grid, bool variants, unsigned int* ticket, cudaStream_t s);
 // resident blocks per SM of the batch's passes
-struct WindowBlocks { int quiet, active, ions; };
+struct WindowBlocks { int quiet, active, ions, one; };
 WindowBlocks window_blocks_per_sm(int threads);
 cudaError_t launch_fold(const RunDev& R, uint32_t ncells, unsigned long long* count,
                         unsigned long long* charge, cudaStream_t s);

@@ -7,7 +7,7 @@
 //      budget and the slot limit allow (a request that does not fit waits, and
 //      the ones behind it wait too, so arrival order is kept); a new run is
 //      set up on its own stream while the batch's queued steps run;
-//   2. enqueue steps_per_tick steps of the batch (one graph replay per step)
+//   2. enqueue steps_per_tick steps of the batch (in windows of up to 32)
 //      and, for every run whose own step count reaches a multiple of its
 //      window, a copy of its tallies into pinned memory (a snapshot);
 //   3. while those steps run, read the snapshots of the previous tick and

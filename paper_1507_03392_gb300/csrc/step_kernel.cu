@@ -61,8 +61,8 @@ __device__ __noinline__ Disp far_displacement(float dx, float dy, float dz)
 }
 
 // Position after the step's straight move with the (already pushed)
-// velocity, in 64-bit fixed point.  The step kernel and the leaver pass both
-// call this, so they get the same integers.  The displacement is rounded to
+// velocity, in 64-bit fixed point, for a particle that left the chamber; move
+// below gets the same integers.  The displacement is rounded to
 // nearest; below 2^30 units a 32-bit conversion gives the same integer,
 // larger (or non-finite) ones take the bounded 64-bit conversion.
 __device__ __forceinline__ void displace(const RunDev& R, int32_t X, int32_t Y, int32_t Z, float vx, float vy,
@@ -208,7 +208,7 @@ struct Carry {
 // word).  On return dep_cell is the cell it deposits in and ckey the cell
 // where it can take part in Coulomb collisions (kNoCell: no ion, or it left).  A
 // particle that left the chamber keeps its old position and returns true
-// with its pushed velocity: the leaver pass finishes its step.
+// with its pushed velocity: leave_particle finishes its step.
 // kVar: with the code of the opt-in processes (double ionisation, elastic
 // ion-atom scattering); without it the kernels carry none of their branches.
 // kCarry: c holds the particle's cell from its last step.  kPlain: every process
@@ -267,7 +267,7 @@ __device__ __forceinline__ bool step_particle(const RunDev& R, uint32_t pid, uin
     }
     const int32_t X0 = X, Y0 = Y, Z0 = Z;
     if (move<kPlain>(R, X, Y, Z, vx, vy, vz)) {
-        X = X0;   // the leaver pass redoes the move from the old position
+        X = X0;   // leave_particle redoes the move from the old position
         Y = Y0;
         Z = Z0;
         meta = status | Q;
@@ -549,14 +549,15 @@ __device__ __forceinline__ void deposit_warp(const RunDev& R, uint32_t cell, uin
 // the front of the list and atoms from its back, so that a warp has one kind.
 //
 // With collisions between ions the listed particles take one step at a time
-// (k_ions), which also records the ions for the collision kernels; the list
-// holds for the window.
+// (k_ions), which also records the ions for the collision kernel; the list
+// holds for the window.  A window of one step takes all particles in place
+// (k_one).
 //
 // Against a step kernel and a leaver pass a step, which read and wrote every
 // particle each time and were bound by instruction issue: 32 steps of the 32
 // oxygen runs of a gas-flow scan (2.6e7 particles, dt 1 ns) took 11.8 ms and
-// take 5.2 (k_quiet 1.7, k_active 3.4); 1000 steps of 1e4 particles, bound by
-// the latency of two launches a step, 9.1 ms and 2.2.
+// take 4.3 (k_quiet 1.6, k_active 2.7); 1000 steps of 1e4 particles, bound by
+// the latency of two launches a step, 9.1 ms and 1.6.
 // ---------------------------------------------------------------------------
 
 // The part of an atom's Philox blocks in a window that does not depend on the
@@ -781,36 +782,29 @@ __device__ __forceinline__ void quiet_details(const RunDev& R, const QuietSteps&
 // looked at one by one are put by and taken 32 at a time: in place they would
 // keep whole warps waiting (at dt 1 ns, 3 % of the atoms were on two thirds of
 // the warps).
-template <bool kOne>
 __device__ __forceinline__ void quiet_group(const RunDev& R, const QuietSteps& S, QuietWarp& W, QuietCount& n,
                                             uint32_t i0, uint32_t K)
 {
-    if (kOne) K = 1u;
     const uint32_t lane = threadIdx.x & 31, i = i0 + lane, nslot = 4u * R.n4;
     const uint32_t meta = i < nslot ? R.meta[i] : kStPad;
-    // the atom's words, in a window of one step before it is known to be one
-    // (such a window waits for memory, not for arithmetic)
     int32_t X = 0, Y = 0, Z = 0;
     uint32_t id = 0u;
     float3 v = make_float3(0.f, 0.f, 0.f);
-    if (kOne && i < nslot) atom_words(R, i, X, Y, Z, id, v);
     const uint32_t status = meta & 0xFFFF0000u, Q = meta & kQMask;
     const bool live = !(status & (kStFrozen | kStPad));
     bool listed = false, detail = false, hit = false;
     uint32_t dep_cell = kNoCell;
     if (live && Q == 0u) {
-        if (!kOne) atom_words(R, i, X, Y, Z, id, v);
+        atom_words(R, i, X, Y, Z, id, v);
         Way w;
         listed = !quiet_way(R, v, X, Y, Z, K, w);
         if (!listed && (R.flags & kFIonize)) {
             const QuietAtom a = quiet_atom(R, id);
             const QuietKeys key = quiet_keys(R);
             uint32_t lo = 0xFFFFFFFFu, s = 0;
-            if (!kOne) {   // four steps' blocks side by side
-                for (; s + 4u <= K; s += 4u)
-                    lo = min(lo, min(min(quiet_word0(key, a, S.rng[s]), quiet_word0(key, a, S.rng[s + 1u])),
-                                     min(quiet_word0(key, a, S.rng[s + 2u]), quiet_word0(key, a, S.rng[s + 3u]))));
-            }
+            for (; s + 4u <= K; s += 4u)   // four steps' blocks side by side
+                lo = min(lo, min(min(quiet_word0(key, a, S.rng[s]), quiet_word0(key, a, S.rng[s + 1u])),
+                                 min(quiet_word0(key, a, S.rng[s + 2u]), quiet_word0(key, a, S.rng[s + 3u]))));
             for (; s < K; ++s) lo = min(lo, quiet_word0(key, a, S.rng[s]));
             hit = atom_may_ionize(R, lo);
         }
@@ -818,7 +812,7 @@ __device__ __forceinline__ void quiet_group(const RunDev& R, const QuietSteps& S
             // the cells it visits: the same one throughout if the first and
             // the last step share it (each coordinate is monotone)
             dep_cell = ngp_cell(R, w.XE, w.YE, w.ZE);
-            detail = hit || (!kOne && ngp_cell(R, X + w.DX, Y + w.DY, Z + w.DZ) != dep_cell);
+            detail = hit || ngp_cell(R, X + w.DX, Y + w.DY, Z + w.DZ) != dep_cell;
             if (detail) {
                 dep_cell = kNoCell;
             } else {
@@ -868,15 +862,12 @@ __device__ __forceinline__ void quiet_start(const RunDev& R, QuietSteps& S, uint
     __syncthreads();
 }
 
-// kOne: a window of one step, which is bound by memory and wants more warps
-// than one whose words fill the multipliers
 // groups: 32-particle groups a warp takes in a row (they stay together in the
 // list).  Fewer resident blocks with four steps' words side by side did better
 // than more with two: 240 us a 32-step window of 3e6 atoms with 6 blocks and
 // four, 257 and 261 with 10 or 8 and two.
 constexpr int kQuietBlocks = 6;
-template <bool kOne>
-__global__ void __launch_bounds__(128, kOne ? 8 : kQuietBlocks) k_quiet(const __grid_constant__ RunDev R, uint32_t K,
+__global__ void __launch_bounds__(128, kQuietBlocks) k_quiet(const __grid_constant__ RunDev R, uint32_t K,
                                                                           uint32_t groups)
 {
     __shared__ QuietSteps S;
@@ -890,7 +881,7 @@ __global__ void __launch_bounds__(128, kOne ? 8 : kQuietBlocks) k_quiet(const __
     const uint32_t nslot = 4u * R.n4, run = 32u * groups, nw = gridDim.x * 4u;
     for (uint32_t g = blockIdx.x * 4u + (threadIdx.x >> 5); g * run < nslot; g += nw)
 #pragma unroll 1
-        for (uint32_t k = 0; k < run; k += 32u) quiet_group<kOne>(R, S, W, n, g * run + k, K);
+        for (uint32_t k = 0; k < run; k += 32u) quiet_group(R, S, W, n, g * run + k, K);
     quiet_end(R, S, W, n, K);
 }
 
@@ -928,7 +919,6 @@ __device__ __forceinline__ uint32_t list_entry(uint32_t t, uint32_t lw)
 // listed particles start in the passes over them: pref[r] for the runs without
 // collisions between ions (k_active_batch), pref[nruns + 1 + r] for those with
 // (k_ions_batch), nruns + 1 entries each
-template <bool kOne>
 __global__ void __launch_bounds__(256, 4) k_quiet_batch(const RunDev* __restrict__ runs,
                                                                    const uint2* __restrict__ items, uint32_t nitems,
                                                                    uint32_t tile, uint32_t K, uint32_t nruns,
@@ -956,7 +946,7 @@ __global__ void __launch_bounds__(256, 4) k_quiet_batch(const RunDev* __restrict
         // the tile's particles, a stretch of them a warp
         const uint32_t per = tile / (blockDim.x >> 5), i0 = it.y * tile + (threadIdx.x >> 5) * per;
 #pragma unroll 1
-        for (uint32_t k = 0; k < per; k += 32u) quiet_group<kOne>(rs, S, W, n, i0 + k, K);
+        for (uint32_t k = 0; k < per; k += 32u) quiet_group(rs, S, W, n, i0 + k, K);
     }
     if (cur != 0xFFFFFFFFu) quiet_end(rs, S, W, n, K);
     if (!last_block(ticket)) return;
@@ -1219,6 +1209,121 @@ __global__ void __launch_bounds__(256, kIonsBatchBlocks) k_ions_batch(const RunD
     }
 }
 
+// A window of one step (a call of one step, a timed one, the step up to a sort):
+// every particle in its place, in one pass over the arrays.  Listing the ions
+// and the atoms with an event to come, and gathering them again, costs more
+// than it saves here (4e6 particles with collisions, cold caches: k_quiet and
+// k_ions 100 us, this 78; 4.8e7 without: k_quiet and k_active 1030 us, this 712,
+// with four blocks of 256 threads an SM instead of five 741).
+template <bool kVar, bool kPlain>
+__device__ __forceinline__ void one_group(const RunDev& R, uint32_t i, uint32_t step)
+{
+    const bool in = i < 4u * R.n4;
+    uint32_t id = 0u, meta = kStPad;
+    int32_t x = 0, y = 0, z = 0;
+    float vx = 0.0f, vy = 0.0f, vz = 0.0f;
+    if (in) {
+        meta = R.meta[i];
+        id = R.id[i];
+        x = R.x[i]; y = R.y[i]; z = R.z[i];
+        vx = R.vx[i]; vy = R.vy[i]; vz = R.vz[i];
+    }
+    const uint32_t was = meta;
+    uint32_t ck = kNoCell, dc = kNoCell;
+    bool left = false;
+    // nearly all atoms: those that neither leave nor can ionise, as in the quiet
+    // pass.  In a mixed warp they would wait for the ions all the same (4e6
+    // particles in load order 2 % slower from 24 atoms a warp on, the same from 29
+    // on; sorted 3 % faster with either).
+    bool quick = false;
+    if (__popc(__ballot_sync(0xFFFFFFFFu, (was & kQMask) == 0u)) >= 29 && !(was & (kStFrozen | kStPad | kQMask))) {
+        Way w;
+        quick = quiet_way(R, make_float3(vx, vy, vz), x, y, z, 1u, w);
+        if (quick && (R.flags & kFIonize))
+            quick = !atom_may_ionize(R, quiet_word0(quiet_keys(R), quiet_atom(R, id), quiet_step(R, step)));
+        if (quick) {
+            x = w.XE; y = w.YE; z = w.ZE;
+            meta = was & 0xFFFF0000u;   // its events are over
+            dc = ngp_cell(R, x, y, z);
+        }
+    }
+    if (!quick) {
+        Carry carry;
+        left = step_particle<kVar, false, kPlain>(R, id, step, x, y, z, vx, vy, vz, meta, ck, dc, carry);
+    }
+    if (left) {
+        const Left l = leave_call(R, id, step, x, y, z, vx, vy, vz, meta);
+        x = l.X; y = l.Y; z = l.Z;
+        vx = l.vx; vy = l.vy; vz = l.vz;
+        meta = l.meta;
+        dc = l.cell;   // (as an atom: no charge)
+    }
+    if (in) {
+        if (!(was & (kStFrozen | kStPad))) {
+            R.x[i] = x; R.y[i] = y; R.z[i] = z;
+            if (((was | meta) & kQMask) || left) {   // (an atom keeps its velocity)
+                R.vx[i] = vx; R.vy[i] = vy; R.vz[i] = vz;
+            }
+        }
+        if (meta != was) R.meta[i] = meta;
+    }
+    deposit_warp(R, dc, meta & kQMask);
+    if (R.flags & kFCoulomb) place_warp(R, i, ck, id, step, vx, vy, vz, meta);
+}
+
+// what the collision kernel of a window of one step finds set (by one thread)
+__device__ __forceinline__ void begin_one(const RunDev& R)
+{
+    begin_collisions(R);
+    R.nleave[2] = 1u;
+}
+
+template <bool kVar>
+__global__ void __launch_bounds__(kActiveTile, 8) k_one(const __grid_constant__ RunDev R, unsigned int* ticket)
+{
+    pdl_wait();
+    pdl_trigger();
+    const bool plain = !kVar && plain_run(R), coulomb = (R.flags & kFCoulomb) != 0;
+    if (coulomb && blockIdx.x == 0 && threadIdx.x == 0) begin_one(R);
+    const uint32_t end = 4u * R.n4, step = *R.step;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; (i & ~31u) < end; i += gridDim.x * blockDim.x) {
+        if (!kVar && plain) one_group<false, true>(R, i, step);
+        else one_group<kVar, false>(R, i, step);
+    }
+    if (!coulomb && last_block(ticket) && threadIdx.x == 0) *R.step += 1u;
+}
+
+template <bool kVar>
+__global__ void __launch_bounds__(256, 5) k_one_batch(const RunDev* __restrict__ runs, uint32_t nruns,
+                                                      const uint2* __restrict__ items, uint32_t nitems, uint32_t tile,
+                                                      unsigned int* ticket)
+{
+    __shared__ RunDev rs;
+    pdl_wait();
+    pdl_trigger();
+    uint32_t cur = 0xFFFFFFFFu;
+    for (uint32_t k = blockIdx.x; k < nitems; k += gridDim.x) {
+        const uint2 it = items[k];
+        if (it.x != cur) {
+            __syncthreads();
+            cur = it.x;
+            stage_run(rs, runs + cur);
+            __syncthreads();
+        }
+        const uint32_t step = *rs.step;
+        for (uint32_t j = threadIdx.x; j < tile; j += blockDim.x) {
+            if (!kVar && plain_run(rs)) one_group<false, true>(rs, it.y * tile + j, step);
+            else one_group<kVar, false>(rs, it.y * tile + j, step);
+        }
+    }
+    if (!last_block(ticket)) return;
+    for (uint32_t r = threadIdx.x; r < nruns; r += blockDim.x) {
+        if (!runs[r].step) continue;
+        if (runs[r].flags & kFCoulomb) begin_one(runs[r]);
+        else *runs[r].step += 1u;
+    }
+}
+
 // Fold the packed per-step deposit into the time-summed count and charge
 // grids and clear it.
 __global__ void k_fold(const __grid_constant__ RunDev R, uint32_t ncells,
@@ -1379,20 +1484,20 @@ WindowBlocks window_blocks_per_sm(int threads)
 {
     const int smem = (threads / 32) * (int)sizeof(QuietWarp);
     WindowBlocks b;
-    b.quiet = std::min(blocks_per_sm(k_quiet_batch<false>, threads, smem), blocks_per_sm(k_quiet_batch<true>, threads, smem));
+    b.quiet = blocks_per_sm(k_quiet_batch, threads, smem);
     b.active = std::min(blocks_per_sm(k_active_batch<false>, threads, 0), blocks_per_sm(k_active_batch<true>, threads, 0));
     b.ions = std::min(blocks_per_sm(k_ions_batch<false>, threads, 0), blocks_per_sm(k_ions_batch<true>, threads, 0));
+    b.one = std::min(blocks_per_sm(k_one_batch<false>, threads, 0), blocks_per_sm(k_one_batch<true>, threads, 0));
     return b;
 }
 
 cudaError_t launch_quiet(const RunDev& R, uint32_t K, int sm_count, cudaStream_t s)
 {
     // at most one wave of blocks; four groups in a row once every warp has some
-    const uint32_t most = (uint32_t)((K == 1u ? 8 : kQuietBlocks) * sm_count), slots = 4u * R.n4;
+    const uint32_t most = (uint32_t)(kQuietBlocks * sm_count), slots = 4u * R.n4;
     const uint32_t groups = slots >= most * 4u * 128u * 2u ? 4u : 1u;
     const uint32_t need = (slots + 128u * groups - 1u) / (128u * groups);
-    return launch_pdl(K == 1u ? k_quiet<true> : k_quiet<false>, dim3(std::max(1u, std::min(need, most))), dim3(128), 0,
-                      s, R, K, groups);
+    return launch_pdl(k_quiet, dim3(std::max(1u, std::min(need, most))), dim3(128), 0, s, R, K, groups);
 }
 
 // as many blocks as the list could need, at most one wave
@@ -1409,17 +1514,36 @@ cudaError_t launch_active(const RunDev& R, uint32_t K, unsigned int* ticket, int
                       R, K, ticket);
 }
 
+// Blocks that start while the collision kernel before them ends get an SM
+// whose memory that kernel has split for its shared memory, with little left
+// for the cache that the gathers live on.  Up to about three blocks' work a
+// resident block the early start gives more than that costs: us a step with
+// and without, 2e5 particles 27.7 and 32.4, 4e5 35.5 and 38.7, 5e5 42.4 and
+// 39.8, 1e6 53.7 and 49.8, 4e6 92.4 and 88.9.
+static bool small_list(const RunDev& R, int sm_count)
+{
+    return 4u * R.n4 <= 3u * kListBlocks * kActiveTile * (uint32_t)sm_count;
+}
+
 cudaError_t launch_ions(const RunDev& R, int sm_count, cudaStream_t s)
 {
-    // Blocks that start while the collision kernel before them ends get an SM
-    // whose memory that kernel has split for its shared memory, with little left
-    // for the cache that the gathers live on.  Up to about three blocks' work a
-    // resident block the early start gives more than that costs: us a step with
-    // and without, 2e5 particles 27.7 and 32.4, 4e5 35.5 and 38.7, 5e5 42.4 and
-    // 39.8, 1e6 53.7 and 49.8, 4e6 92.4 and 88.9.
-    const bool early = 4u * R.n4 <= 3u * kListBlocks * kActiveTile * (uint32_t)sm_count;
-    return launch_early(early, variants(R) ? k_ions<true> : k_ions<false>, list_grid(R, sm_count), dim3(kActiveTile), 0,
+    return launch_early(small_list(R, sm_count), variants(R) ? k_ions<true> : k_ions<false>, list_grid(R, sm_count), dim3(kActiveTile), 0,
                         s, R);
+}
+
+cudaError_t launch_one(const RunDev& R, unsigned int* ticket, int sm_count, cudaStream_t s)
+{
+    const uint32_t need = (4u * R.n4 + kActiveTile - 1u) / kActiveTile, most = (uint32_t)(8 * sm_count);
+    return launch_early(small_list(R, sm_count), variants(R) ? k_one<true> : k_one<false>,
+                        dim3(std::max(1u, std::min(need, most))), dim3(kActiveTile), 0, s, R, ticket);
+}
+
+cudaError_t launch_one_batch(const RunDev* runs, uint32_t nruns, const uint2* items, uint32_t nitems, uint32_t tile,
+                             int threads, int grid, bool variants, unsigned int* ticket, cudaStream_t s)
+{
+    return launch_early(false, variants ? k_one_batch<true> : k_one_batch<false>,
+                        dim3(std::max(1u, std::min(nitems, (uint32_t)grid))), dim3(threads), 0, s, runs, nruns, items,
+                        nitems, tile, ticket);
 }
 
 cudaError_t launch_quiet_batch(const RunDev* runs, uint32_t nruns, const uint2* items, uint32_t nitems, uint32_t tile,
@@ -1427,7 +1551,7 @@ cudaError_t launch_quiet_batch(const RunDev* runs, uint32_t nruns, const uint2* 
                                cudaStream_t s)
 {
     const uint32_t g = std::max(1u, std::min(nitems, (uint32_t)grid));
-    return launch_pdl(K == 1u ? k_quiet_batch<true> : k_quiet_batch<false>, dim3(g), dim3(threads),
+    return launch_pdl(k_quiet_batch, dim3(g), dim3(threads),
                       (threads / 32) * sizeof(QuietWarp), s, runs, items, nitems, tile, K, nruns, pref, ticket);
 }
 
