@@ -7,7 +7,7 @@ density 1e10 cm^-3, every process of the step on.  Inputs are synthetic
 particles.  L2 is flushed (a 512 MB write) between timed steps.
 
 On one GPU the line also carries the batched form (a 64-run oxygen gas-flow
-scan in one persistent kernel and graph, beside the same runs stepped one at a
+scan in one pass over all runs a step, beside the same runs stepped one at a
 time), the served form (a Poisson request stream of O/Ar/Kr runs: scans/s,
 p50/p99 time to converged currents) and a 128-run argon power scan admitted
 under an HBM budget of a third of its total.
@@ -283,8 +283,8 @@ def _percentile(xs, q):
 
 def bench_batched(E, I, args, local, stream, flush, peak, peak_kind):
     """The batched gas-flow scan: oxygen runs (n0 log-spaced 3e9-3e11 cm^-3, N
-    log-uniform 2e5-2e6) advanced together by the persistent batched step
-    kernel, replayed as one CUDA graph per step, launch shape autotuned.
+    log-uniform 2e5-2e6) advanced together a step at a time by the batched
+    passes, launch shape autotuned.
     Reported beside the plain single-run form of the same runs."""
     import torch
     wls = [I.config_oxygen_scan(i) for i in range(args.batch_runs)]
@@ -358,16 +358,16 @@ def bench_batched(E, I, args, local, stream, flush, peak, peak_kind):
         "steps_note": "a whole number of sort periods of the tuned cadence",
         "value": value, "unit": "ion-steps/s", "ms_per_step": ms / nsteps,
         "tuning": tune,
-        "roofline": {"bound": "hbm", "kernel": "k_step_batch", "achieved": achieved, "peak": peak,
+        "roofline": {"bound": "hbm", "kernel": "k_one_batch", "achieved": achieved, "peak": peak,
                      "peak_source": peak_kind, "unit": "GB/s", "frac": achieved / peak,
                      "algorithmic_bytes_per_launch": algo, "kernel_ms": k_ms, "traffic": ktraffic,
-                     "kernel_ms_from": "a profiled pass (the step's kernels launched one by one, after "
-                                       "the timed graph-replayed steps)",
+                     "kernel_ms_from": "a profiled pass (the step's kernels timed one by one, after "
+                                       "the timed steps)",
                      "share_of_step": prof["step_ms"] / max(1e-9, prof["step_ms"] + prof["coulomb_ms"]
                                                             + prof["other_ms"]),
                      "whole_step": {"bytes_per_ion_step": ALGO_BYTES_STEP_KERNEL, "achieved": whole,
                                     "frac": whole / peak,
-                                    "note": "the timed graph-replayed steps' ion-steps/s times 56 B"}},
+                                    "note": "the timed steps' ion-steps/s times 56 B"}},
         "plain_single_run": {"value": plain, "unit": "ion-steps/s",
                              "runs": min(args.plain_runs, len(wls)),
                              "note": "the first runs of the scan stepped one at a time through ecris_step"},
@@ -579,7 +579,7 @@ def main():
         dist.barrier()
     sampler = ClockSampler(local)
     sampler.start()
-    # the timed steps: each one CUDA graph replay, as a user's ecris_step runs
+    # the timed steps: each one call, as a user's ecris_step runs
     starts = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
     ends = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
     torch.cuda.synchronize()
@@ -604,10 +604,8 @@ def main():
     step_ms = [s.elapsed_time(e) for s, e in zip(starts, ends)]
     value, total_s = replica_throughput(n * args.steps, 1e-3 * sum(step_ms), dist, "cuda")
     total_ms = 1e3 * total_s
-    # kernels launched in the timed steps: a graph replay holds the same
-    # kernels the profiled pass launched one by one, step for step (with
-    # collisions the profiled pass, like the graph, runs the leaver pass inside
-    # the scan kernel)
+    # kernels launched in the timed steps: those the profiled pass timed, step
+    # for step
     nprof_steps = min(args.steps, 200)
     launches = int(round((prof["step_launches"] + prof["coulomb_launches"] + prof["other_launches"])
                          * args.steps / nprof_steps))
@@ -619,14 +617,14 @@ def main():
     peak, peak_kind = measured_peaks()
     step_bytes = ALGO_BYTES_STEP_COULOMB if coulomb else ALGO_BYTES_STEP_KERNEL
     whole = value * step_bytes / 1e9
-    roofline = {"bound": "hbm", "kernel": "k_step", "achieved": achieved, "peak": peak,
+    roofline = {"bound": "hbm", "kernel": "k_one", "achieved": achieved, "peak": peak,
                 "peak_source": peak_kind, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": ncu_traffic(n), "algorithmic_bytes_per_launch": algo,
                 "kernel_ms": k_ms,
-                "kernel_ms_from": "a timed pass with per-kernel CUDA events after the graph-replayed steps",
+                "kernel_ms_from": "a timed pass with per-kernel CUDA events after the timed steps",
                 "share_of_step": prof["step_ms"] / max(1e-9, prof["step_ms"] + prof["coulomb_ms"] + prof["other_ms"]),
                 "whole_step": {"bytes_per_ion_step": step_bytes, "achieved": whole, "frac": whole / peak,
-                               "note": "ion-steps/s of the timed (graph-replayed) steps times the algorithmic "
+                               "note": "ion-steps/s of the timed steps times the algorithmic "
                                        "bytes of a whole step"}}
 
     # end to end through the public API with host buffers: H2D of the state,

@@ -355,9 +355,9 @@ ecris_status ecris_set_tuning(ecris_ctx* ctx, const ecris_tuning* t);
 /* ------------------------------------------------------------------------ */
 /* Batched form: many runs advanced together (the paper's parameter scans of */
 /* Sec. III -- gas flow, microwave power via n_e and T_e -- run as one       */
-/* batch).  Each pass of a step is one launch over all active runs, and each   */
-/* step's passes with collisions one CUDA graph.  Each run keeps its particles */
-/* resident on the device and gives exactly the results it gives alone.      */
+/* batch).  Each pass is one launch over all active runs.  Each run keeps    */
+/* its particles resident on the device and gives exactly the results it     */
+/* gives alone.                                                              */
 /* ------------------------------------------------------------------------ */
 typedef struct ecris_batch ecris_batch;
 
@@ -403,7 +403,7 @@ ecris_status ecris_batch_get_cells(ecris_batch* b, int32_t run, float* ne, float
 /* Bytes held by the batch's runs and its budget (0: none). */
 ecris_status ecris_batch_memory(const ecris_batch* b, size_t* used, size_t* budget);
 /* Kernel timing for a batch, as ecris_set_profiling / ecris_get_profile:
- * with profiling on, every step launches its kernels one by one (no graph, no
+ * with profiling on, every step launches its kernels one by one (no
  * windows of several steps) between events; step_* is the step's passes,
  * coulomb_* the collision kernel of all runs, other_* sorts and deposit folds. */
 ecris_status ecris_batch_set_profiling(ecris_batch* b, int enable);
