@@ -89,7 +89,7 @@ __device__ __forceinline__ unsigned long long block_excl64(unsigned long long v,
 // count: ions per cell.  The last block makes that the exclusive scan, and the
 // plan's words.
 __global__ void __launch_bounds__(kPlanThreads) k_plan_sum(const __grid_constant__ RunDev R,
-                                                           const uint32_t* __restrict__ count, unsigned long long* blk)
+                                                           const uint32_t* count, unsigned long long* blk)
 {
     pdl_wait();
     pdl_trigger();
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_sum(const __grid_constant
 // b holds the planned cells whose room starts in [b kRange, (b + 1) kRange)
 __global__ void __launch_bounds__(kPlanThreads) k_plan_cells(const __grid_constant__ RunDev R,
                                                              uint32_t* __restrict__ count,
-                                                             const unsigned long long* __restrict__ blk, int zero)
+                                                             const unsigned long long* blk, int zero)
 {
     pdl_wait();
     pdl_trigger();
@@ -268,7 +268,7 @@ struct Record {
 __device__ __forceinline__ Record load_record(const RunDev& R, uint32_t p)
 {
     uint32_t a[8];
-    asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7])
                  : "l"(R.crec + 2 * (size_t)p));
     return Record{make_float4(__uint_as_float(a[0]), __uint_as_float(a[1]), __uint_as_float(a[2]),

@@ -216,7 +216,10 @@ __device__ __forceinline__ void stage_run(RunDev& rs, const RunDev* src)
 // blocks signal with pdl_trigger, or by exiting); it calls pdl_wait before it
 // touches memory, which waits until the kernel before it has completed and
 // its writes are visible.  This hides the launch latency between the
-// dependent kernels of a step.
+// dependent kernels of a step.  What the kernel before it writes is read through
+// plain pointers: a read-only load (const __restrict__, __ldg) says that the
+// memory does not change while the kernel lives, so the compiler could move it
+// above the wait; a load in inline assembly is volatile, which keeps it below.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -581,7 +584,7 @@ __device__ __forceinline__ void place_warp(const RunDev& R, uint32_t slot, uint3
     const uint32_t tl = after ? (uint32_t)(__ffs(after) - 2) : 31u;  // last lane of this lane's run
     const uint32_t h = 31u - (uint32_t)__clz(heads & upto);           // first lane of this lane's run
     uint4 bk = make_uint4(0u, 0u, 0u, 0u);
-    if (in) bk = R.cbkt ? __ldg(R.cbkt + ck) : make_uint4(ck * R.uroom, R.uroom, ck, 0u);
+    if (in) bk = R.cbkt ? R.cbkt[ck] : make_uint4(ck * R.uroom, R.uroom, ck, 0u);
     uint32_t k = 0u;
     if (in && lane == h) k = atomicAdd(bk.x == kNoCell ? R.ccount + ck : R.pcount + bk.z, tl - h + 1u);
     const Words w = rng_words(R, id, step, 1u);

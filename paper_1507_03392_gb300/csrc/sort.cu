@@ -98,7 +98,7 @@ __device__ __forceinline__ uint32_t block_excl(uint32_t v, uint32_t* total)
 
 // exclusive scan of in[0, n) into out within blocks of kSortScanBlock; blk: the
 // blocks' offsets (ticket: a zero word, left zero)
-__global__ void __launch_bounds__(kSortThreads) k_sort_scan(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
+__global__ void __launch_bounds__(kSortThreads) k_sort_scan(const uint32_t* in, uint32_t* __restrict__ out,
                                                             uint32_t* blk, uint32_t n, uint32_t* ticket)
 {
     pdl_wait();
@@ -133,8 +133,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scan(const uint32_t* __re
 // the destination arrays
 template <bool kRecords>
 __global__ void k_sort_move(const __grid_constant__ RunDev R, uint32_t cap, ParticleSet dst, uint4* __restrict__ aos,
-                            uint32_t* __restrict__ hist, const uint32_t* __restrict__ off,
-                            const uint32_t* __restrict__ blk)
+                            uint32_t* __restrict__ hist, const uint32_t* off, const uint32_t* blk)
 {
     pdl_wait();
     pdl_trigger();
@@ -188,7 +187,7 @@ __global__ void k_sort_move(const __grid_constant__ RunDev R, uint32_t cap, Part
 }
 
 // records in sorted order -> the destination arrays, coalesced both ways
-__global__ void k_sort_unpack(const uint4* __restrict__ aos, uint32_t cap, ParticleSet dst)
+__global__ void k_sort_unpack(const uint4* aos, uint32_t cap, ParticleSet dst)
 {
     pdl_wait();
     pdl_trigger();
@@ -298,7 +297,7 @@ __global__ void k_export_records(const __grid_constant__ RunDev R, uint32_t n, u
     }
 }
 
-__global__ void k_export_unpack(const uint4* __restrict__ rec, uint32_t n, OutPtrs out, uint32_t* __restrict__ meta_out)
+__global__ void k_export_unpack(const uint4* rec, uint32_t n, OutPtrs out, uint32_t* __restrict__ meta_out)
 {
     pdl_wait();
     pdl_trigger();

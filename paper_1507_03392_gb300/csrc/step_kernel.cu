@@ -1086,7 +1086,7 @@ __global__ void __launch_bounds__(kActiveTile, kVar ? 8 : 6) k_active(const __gr
 // the run whose listed tiles hold tile v of a batch pass, and v less the run's
 // first tile: staged in rs, with *s_at = (run, first tile) (all threads call it)
 __device__ __forceinline__ uint32_t batch_tile(const RunDev* __restrict__ runs, uint32_t nruns,
-                                               const uint32_t* __restrict__ pref, uint32_t v, RunDev& rs, uint2& s_at,
+                                               const uint32_t* pref, uint32_t v, RunDev& rs, uint2& s_at,
                                                uint32_t& cur)
 {
     for (uint32_t r = threadIdx.x; r < nruns; r += blockDim.x) {
@@ -1105,7 +1105,7 @@ __device__ __forceinline__ uint32_t batch_tile(const RunDev* __restrict__ runs, 
 
 template <bool kVar>
 __global__ void __launch_bounds__(256, kActiveBatchBlocks) k_active_batch(const RunDev* __restrict__ runs, uint32_t nruns,
-                                                         const uint32_t* __restrict__ pref, uint32_t K,
+                                                         const uint32_t* pref, uint32_t K,
                                                          unsigned int* ticket)
 {
     __shared__ RunDev rs;
@@ -1190,7 +1190,7 @@ __global__ void __launch_bounds__(kActiveTile, 8) k_ions(const __grid_constant__
 
 template <bool kVar>
 __global__ void __launch_bounds__(256, kIonsBatchBlocks) k_ions_batch(const RunDev* __restrict__ runs, uint32_t nruns,
-                                                       const uint32_t* __restrict__ pref)
+                                                       const uint32_t* pref)
 {
     __shared__ RunDev rs;
     __shared__ uint2 s_at;
@@ -1434,7 +1434,7 @@ __global__ void k_load_init(LoadCheck lc, SoaPtrs soa, const uint8_t* __restrict
 }
 
 // the velocities alone
-__global__ void k_load_check(SoaPtrs soa, const uint32_t* __restrict__ meta, uint32_t n, uint32_t cap,
+__global__ void k_load_check(SoaPtrs soa, const uint32_t* meta, uint32_t n, uint32_t cap,
                              unsigned int* __restrict__ bad)
 {
     pdl_wait();
