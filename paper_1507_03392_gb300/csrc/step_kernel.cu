@@ -535,9 +535,10 @@ __device__ __forceinline__ void deposit_warp(const RunDev& R, uint32_t cell, uin
 //
 // k_quiet takes the atoms.  An atom moves on a straight line by the same whole
 // number of grid units every step, so its place after the window is one
-// multiply away; it stays in the chamber throughout if it does at the window's
-// end (the chamber is convex, and the box and r <= R0 tests are exact in the
-// integers).  What is left of its steps is the ionisation word: one Philox
+// multiply away; it stays in the chamber throughout if it is inside at the
+// window's start and end (the chamber is convex, and the box and r <= R0 tests
+// are exact in the integers).  A load tests r <= R0 in FP32 and lets an atom
+// in up to some hundred grid units outside, so the start is tested, too.  What is left of its steps is the ionisation word: one Philox
 // block a step, of which the first two rounds hardly depend on both the
 // particle and the step (see QuietAtom), compared with the atom gate.  An atom
 // that neither leaves nor ionises in the window is done: moved, its deposits
@@ -635,8 +636,8 @@ __device__ __forceinline__ void atom_words(const RunDev& R, uint32_t i, int32_t&
 }
 
 // An atom's straight way through the window: its displacement a step and its
-// end; false if it leaves the chamber within the window (or moves too far in
-// it for 32-bit arithmetic)
+// end; false if it may leave the chamber within the window (it ends outside, or
+// starts outside the cylinder) or moves too far in it for 32-bit arithmetic
 struct Way { int32_t DX, DY, DZ, XE, YE, ZE; };
 
 __device__ __forceinline__ bool quiet_way(const RunDev& R, const float3& v, int32_t X, int32_t Y, int32_t Z,
@@ -645,6 +646,7 @@ __device__ __forceinline__ bool quiet_way(const RunDev& R, const float3& v, int3
     const bool push = (R.flags & kFPush) != 0;
     const float dx = push ? v.x * R.dt_sxy : 0.0f, dy = push ? v.y * R.dt_sxy : 0.0f, dz = push ? v.z * R.dt_sz : 0.0f;
     if (!(fmaxf(fabsf(dx), fmaxf(fabsf(dy), fabsf(dz))) * (float)K < 1.0e9f)) return false;
+    if (K > 1u && (long long)X * X + (long long)Y * Y > (1ll << 62)) return false;
     w.DX = __float2int_rn(dx);
     w.DY = __float2int_rn(dy);
     w.DZ = __float2int_rn(dz);
