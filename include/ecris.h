@@ -560,7 +560,7 @@ ecris_status ecris_server_calib_poll(ecris_server* s, int64_t job, ecris_calib_r
  * the device.  It runs the same Takizawa-Abe pairing and Nanbu scattering as
  * ecris_step (ECRIS_F_COULOMB) on caller-owned device arrays and keeps all its
  * working memory in one fixed-size array that the library holds on every GPU
- * that loads it (about 5 MB, until the process exits); it allocates nothing.
+ * that loads it (about 6 MB, until the process exits); it allocates nothing.
  *
  *   n            particles, at most 65536; arrays are indexed by particle id
  *                (the Philox counter word, as in ecris_step)

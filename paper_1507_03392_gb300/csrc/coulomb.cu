@@ -122,6 +122,14 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_sum(const __grid_constant
     }
 }
 
+// the ranges that start in or just after the room of planned place k
+__device__ __forceinline__ void mark_ranges(const RunDev& R, uint32_t k, uint32_t at, uint32_t room)
+{
+    for (uint32_t b = at / kRange + 1u; b * kRange < at + room; ++b) R.rstart[b] = k + 1u;
+    // a range that starts just where the next cell's room does
+    if ((at + room) % kRange == 0u) R.rstart[(at + room) / kRange] = k + 1u;
+}
+
 // every cell's bucket, the compact list of planned cells, and the ranges: range
 // b holds the planned cells whose room starts in [b kRange, (b + 1) kRange)
 __global__ void __launch_bounds__(kPlanThreads) k_plan_cells(const __grid_constant__ RunDev R,
@@ -150,11 +158,59 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_cells(const __grid_consta
         R.cbkt[c] = room ? make_uint4(at, fits, k, 0u) : make_uint4(kNoCell, 0u, 0u, 0u);
         if (!room) continue;
         R.pcell[k] = make_uint4(at, fits, c, 0u);
-        for (uint32_t b = at / kRange + 1u; b * kRange < at + room; ++b) R.rstart[b] = k + 1u;
-        // a range that starts just where the next cell's room does
-        if ((at + room) % kRange == 0u) R.rstart[(at + room) / kRange] = k + 1u;
+        mark_ranges(R, k, at, room);
         o += (1ull << 32) + room;
     }
+}
+
+// Room of a cell of h ions whose bucket holds them for one step: at least 4, so
+// that a range has at most 32 cells; none where nothing collides.
+__device__ __forceinline__ uint32_t exact_room(uint32_t h) { return h < 2u ? 0u : max(h, 4u); }
+
+// The plan of a call's own counts.  Any order of the cells' buckets will do, so a
+// block takes the places and the records of its cells from one cursor (places << 32
+// | records) instead of a scan over the blocks; the last block sets the plan's words.
+// Two calls that share the working memory and overlap, which they must not, get
+// no bucket past the pool.
+__global__ void __launch_bounds__(kPlanThreads) k_plan_exact(const __grid_constant__ RunDev R, const uint32_t* count,
+                                                             uint32_t* first, unsigned long long* cursor)
+{
+    __shared__ unsigned long long s_start;
+    pdl_wait();
+    pdl_trigger();
+    const uint32_t base = blockIdx.x * kPlanBlock + threadIdx.x * kPlanPer;
+    uint32_t h[kPlanPer];
+    unsigned long long v = 0ull, total;
+#pragma unroll
+    for (int j = 0; j < kPlanPer; ++j) {
+        h[j] = base + j < R.ncells ? count[base + j] : 0u;
+        const uint32_t room = exact_room(h[j]);
+        v += ((unsigned long long)(room ? 1u : 0u) << 32) + room;
+    }
+    unsigned long long o = block_excl64<kPlanThreads>(v, &total);
+    if (threadIdx.x == 0) s_start = atomicAdd(cursor, total);
+    __syncthreads();
+    o += s_start;
+#pragma unroll
+    for (int j = 0; j < kPlanPer; ++j) {
+        const uint32_t c = base + j;
+        if (c >= R.ncells) break;
+        const uint32_t room = exact_room(h[j]), k = (uint32_t)(o >> 32), at = (uint32_t)o;
+        const bool in = room && at < R.cpool && room <= R.cpool - at;
+        first[c] = in ? at : kNoCell;
+        if (!in) continue;
+        R.pcell[k] = make_uint4(at, room, c, h[j]);
+        mark_ranges(R, k, at, room);
+        o += (1ull << 32) + room;
+    }
+    if (!last_block(R.cword + kCwTicket) || threadIdx.x != 0) return;
+    const unsigned long long end = __ldcg(cursor);
+    const uint32_t nr = min(((uint32_t)end + kRange - 1u) / kRange, R.cpool / kRange);
+    const uint32_t np = min((uint32_t)(end >> 32), R.cpool / 4u);
+    R.cword[kCwPlanned] = np;
+    R.cword[kCwRanges] = nr;
+    R.rstart[0] = 0u;
+    R.rstart[nr] = np;
 }
 
 // ---------------------------------------------------------------------------
@@ -241,11 +297,14 @@ __device__ __forceinline__ void collide(const RunDev& R, float4& ra, float4& rb,
 
 __device__ __forceinline__ void write_back(const RunDev& R, uint32_t slot, const float4& r)
 {
+    // (no ids: a caller's arrays, whose event words are not the records' meta
+    // words; a slot past them is another call's that overlaps this one, which
+    // it must not)
+    if (!R.id && slot >= R.n) return;
     R.vx[slot] = r.x;
     R.vy[slot] = r.y;
     R.vz[slot] = r.z;
-    // (a caller's event words are not the records' meta words)
-    if (R.pcell) R.meta[slot] = __float_as_uint(r.w) | kEvCoulomb;
+    if (R.id) R.meta[slot] = __float_as_uint(r.w) | kEvCoulomb;
     else R.meta[slot] |= kEvCoulomb;
 }
 
@@ -678,8 +737,7 @@ __device__ __forceinline__ uint32_t collide_warp(const RunDev& R, PackSmem& S, B
 // ranges and groups of 32 unplanned cells of a run
 __device__ __forceinline__ uint32_t collide_items(const RunDev& R)
 {
-    const uint32_t nr = R.pcell ? R.cword[kCwRanges] : (R.ncells + R.ucells - 1u) / R.ucells;
-    return nr + (R.cword[R.cword[kCwSet] + kCwUnplanned] + 31u) / 32u;
+    return R.cword[kCwRanges] + (R.cword[R.cword[kCwSet] + kCwUnplanned] + 31u) / 32u;
 }
 
 // Order and collide one cell of kWarpIons to kWarpCell ions that all lie in its
@@ -764,25 +822,19 @@ struct ItemCell { uint32_t base, room, m, head; };
 __device__ __forceinline__ ItemCell item_cell(const RunDev& R, uint32_t item)
 {
     const uint32_t lane = threadIdx.x & 31;
-    const uint32_t nr = R.pcell ? R.cword[kCwRanges] : (R.ncells + R.ucells - 1u) / R.ucells;
+    const uint32_t nr = R.cword[kCwRanges];
     uint32_t c = kNoCell;
     uint32_t* count = nullptr;
     ItemCell ic{0u, 0u, 0u, 0u};
     if (item < nr) {
-        if (R.pcell) {
-            const uint32_t k = R.rstart[item] + lane;
-            if (k < R.rstart[item + 1]) {
-                const uint4 p = R.pcell[k];
-                ic.base = p.x;
-                ic.room = p.y;
-                c = p.z;
-                count = R.pcount + k;
-            }
-        } else if (lane < R.ucells && item * R.ucells + lane < R.ncells) {
-            c = item * R.ucells + lane;
-            ic.base = c * R.uroom;
-            ic.room = R.uroom;
-            count = R.pcount + c;
+        const uint32_t k = R.rstart[item] + lane;
+        if (k < R.rstart[item + 1]) {
+            const uint4 p = R.pcell[k];
+            ic.base = p.x;
+            ic.room = p.y;
+            ic.m = p.w;
+            c = p.z;
+            if (R.pcount) count = R.pcount + k;
         }
     } else {
         const uint32_t k = (item - nr) * 32u + lane;
@@ -798,8 +850,8 @@ __device__ __forceinline__ ItemCell item_cell(const RunDev& R, uint32_t item)
             ic.head = R.chead[c];
             R.chead[c] = 0u;
         }
-        if (ic.m < 2u) ic.m = 0u;   // nothing to collide with
     }
+    if (ic.m < 2u) ic.m = 0u;   // nothing to collide with
     return ic;
 }
 
@@ -1031,6 +1083,12 @@ cudaError_t launch_plan(const RunDev& R, uint32_t* count, bool zero, unsigned lo
         e = launch_pdl(k_plan_cells, dim3(nb), dim3(kPlanThreads), 0, s, R, count, (const unsigned long long*)blk,
                        zero ? 1 : 0);
     return e;
+}
+
+cudaError_t launch_plan_exact(const RunDev& R, const uint32_t* count, uint32_t* first, unsigned long long* cursor,
+                              cudaStream_t s)
+{
+    return launch_pdl(k_plan_exact, dim3(plan_blocks(R.ncells)), dim3(kPlanThreads), 0, s, R, count, first, cursor);
 }
 
 int collide_blocks(int sm_count)

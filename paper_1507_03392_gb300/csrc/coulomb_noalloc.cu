@@ -14,7 +14,7 @@
 //
 // Limits: at most kNaMaxIons particles and kNaMaxCells cells per call; larger
 // sizes are rejected with ECRIS_EINVAL.  The array (kNaScratchBytes, about
-// 5 MB) is held by every GPU that loads the library until the process exits.
+// 6 MB) is held by every GPU that loads the library until the process exits.
 // Every call shares it and finds the last call's contents there; what must
 // start at zero is cleared at the start of each call.  Calls whose GPU work
 // overlaps (different streams, or several host threads) race on the array
@@ -23,8 +23,12 @@
 // that first call before any stream capture begins.  That set-up is kept for
 // the life of the process: a device reset (cudaDeviceReset) is not supported,
 // and the entry point must not be called on a device after one.
-// There is no plan of the cells' buckets: the bucket records are shared out
-// evenly among the call's cells, and what does not fit overflows.
+// A call knows its ions only when it is made, so it counts them by cell, plans
+// exact buckets (k_plan_exact) and places the records; nothing overflows, however
+// the ions are spread.  (A pool shared out evenly among the cells needs neither
+// count nor plan, two launches less, but its time hung on the spread: 65521 ions
+// evenly in 65536 cells took 23 us a call and in 4096 cells 37, 60000 ions in 400 of
+// 65536 cells 5559; 30, 36 and 33 so.)
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -40,19 +44,20 @@ namespace {
 
 constexpr uint32_t kNaMaxIons = 65536;
 constexpr uint32_t kNaMaxCells = 65536;
-constexpr uint32_t kNaPool = 49152;    // bucket records, shared out evenly among the call's cells
+constexpr uint32_t kNaPool = 2 * kNaMaxIons;   // bucket records: a cell that collides takes at most 2 an ion
 constexpr size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // byte offsets of the sub-buffers inside the scratch array
 constexpr size_t kOffRec = 0;
-constexpr size_t kOffNext = kOffRec + align256(2 * sizeof(uint4) * (kNaPool + kNaMaxIons));
-constexpr size_t kOffHead = kOffNext + align256(sizeof(uint32_t) * kNaMaxIons);
-constexpr size_t kOffCcount = kOffHead + align256(sizeof(uint32_t) * kNaMaxCells);
-constexpr size_t kOffIdx = kOffCcount + align256(sizeof(uint32_t) * kNaMaxCells);
-constexpr size_t kOffOrd = kOffIdx + align256(sizeof(uint32_t) * kNaMaxIons);
+constexpr size_t kOffCcount = kOffRec + align256(2 * sizeof(uint4) * kNaPool);
+constexpr size_t kOffFirst = kOffCcount + align256(sizeof(uint32_t) * kNaMaxCells);
+constexpr size_t kOffRank = kOffFirst + align256(sizeof(uint32_t) * kNaMaxCells);
+constexpr size_t kOffPcell = kOffRank + align256(sizeof(uint32_t) * kNaMaxIons);
+constexpr size_t kOffRstart = kOffPcell + align256(sizeof(uint4) * (kNaPool / 4));
+constexpr size_t kOffOrd = kOffRstart + align256(sizeof(uint32_t) * (kNaPool / kRange + 1));
 constexpr size_t kOffNanbu = kOffOrd + align256(sizeof(uint32_t) * kNaMaxIons);
 constexpr size_t kOffWords = kOffNanbu + align256(sizeof(float) * kNanbuN);
-// words: step; from word 16 the collisions' counters; then the tally block
+// words: step; from word 16 the collisions' counters; from word 32 the plan's cursor; then the tally block
 constexpr size_t kOffTally = kOffWords + 256;
 constexpr size_t kNaScratchBytes = kOffTally + align256(sizeof(unsigned long long) * kTallyWords);
 
@@ -70,39 +75,60 @@ DeviceSetup g_setup[64];
 // clear the per-call counters and store the step index
 __global__ void k_na_init(unsigned char* base, uint32_t ncells, uint32_t step)
 {
+    pdl_wait();
+    pdl_trigger();
     uint32_t* ccount = reinterpret_cast<uint32_t*>(base + kOffCcount);
-    uint32_t* chead = reinterpret_cast<uint32_t*>(base + kOffHead);
     uint32_t* words = reinterpret_cast<uint32_t*>(base + kOffWords);
     unsigned long long* tally = reinterpret_cast<unsigned long long*>(base + kOffTally);
     const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < ncells; i += stride) ccount[i] = chead[i] = 0u;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < ncells; i += stride) ccount[i] = 0u;
     // (the collisions' counters: the set of this step)
-    if (blockIdx.x == 0 && threadIdx.x < 16 + kCwWords)
+    if (blockIdx.x == 0 && threadIdx.x < 34)
         words[threadIdx.x] = threadIdx.x == 0 ? step : (threadIdx.x == 16 + kCwSet ? 2u * (step & 1u) : 0u);
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < (uint32_t)kTallyWords; i += stride) tally[i] = 0ull;
 }
 
-// record the participants (cell < ncells, Q >= 1) in their cells' buckets, as
-// the ions' pass does for ecris_step (whole warps: n rounded up)
-__global__ void k_na_pack(const __grid_constant__ RunDev R, uint32_t n, const uint32_t* __restrict__ cell,
-                          const uint8_t* __restrict__ q)
+// cell of particle i if it takes part (cell < ncells, 1 <= Q <= 63)
+__device__ __forceinline__ uint32_t na_cell(const RunDev& R, uint32_t i, const uint32_t* cell, const uint8_t* q)
+{
+    const uint32_t c = cell[i], Q = q[i];
+    return c >= R.ncells || Q == 0u || Q > 63u ? kNoCell : c;
+}
+
+// count the participants by cell; rank: each one's arrival in its cell (one atomic per
+// group of lanes in the same cell; whole warps: n rounded up)
+__global__ void k_na_count(const __grid_constant__ RunDev R, const uint32_t* __restrict__ cell,
+                           const uint8_t* __restrict__ q, uint32_t* count, uint32_t* rank)
 {
     pdl_wait();
     pdl_trigger();
-    const uint32_t end = (n + 31u) & ~31u;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < end; i += gridDim.x * blockDim.x) {
-        uint32_t c = kNoCell, Q = 0u;
-        float vx = 0.0f, vy = 0.0f, vz = 0.0f;
-        if (i < n) {
-            c = cell[i];
-            Q = q[i];
-            if (c >= R.ncells || Q == 0u || Q > 63u) c = kNoCell;
-            vx = R.vx[i];
-            vy = R.vy[i];
-            vz = R.vz[i];
-        }
-        place_warp(R, i, c, i, *R.step, vx, vy, vz, Q);   // slot and id are both the array index
-    }
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31u;
+    const uint32_t c = i < R.n ? na_cell(R, i, cell, q) : kNoCell;
+    const uint32_t grp = __match_any_sync(0xFFFFFFFFu, c);
+    const int leader = __ffs(grp) - 1;
+    uint32_t k = 0u;
+    if (c != kNoCell && lane == (uint32_t)leader) k = atomicAdd(count + c, (uint32_t)__popc(grp));
+    k = __shfl_sync(0xFFFFFFFFu, k, leader) + (uint32_t)__popc(grp & ((1u << lane) - 1u));
+    if (i < R.n) rank[i] = k;
+}
+
+// record the participants in their cells' buckets, as the ions' pass does for ecris_step; slot and id are both
+// the array index
+__global__ void k_na_pack(const __grid_constant__ RunDev R, const uint32_t* __restrict__ cell,
+                          const uint8_t* __restrict__ q, const uint32_t* first, const uint32_t* rank)
+{
+    pdl_wait();
+    pdl_trigger();
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= R.n) return;
+    const uint32_t c = na_cell(R, i, cell, q);
+    if (c == kNoCell) return;
+    const uint32_t at = first[c], k = rank[i];
+    if (at == kNoCell || k >= R.cpool - at) return;   // (alone in its cell)
+    const Words w = rng_words(R, i, *R.step, 1u);
+    store_record(R.crec, at + k, make_uint4(__float_as_uint(R.vx[i]), __float_as_uint(R.vy[i]), __float_as_uint(R.vz[i]),
+                                            (uint32_t)q[i]),
+                 make_uint4(i, w.w0, w.w1, w.w2));
 }
 
 ecris_status na_fail(const std::string& msg)
@@ -179,12 +205,12 @@ extern "C" ecris_status ecris_coulomb_collide_noalloc(size_t n, const uint32_t* 
     R.crec = reinterpret_cast<uint4*>(base + kOffRec);
     R.cpool = kNaPool;
     R.cover = kNaMaxIons;
-    R.cnext = reinterpret_cast<uint32_t*>(base + kOffNext);
-    R.chead = reinterpret_cast<uint32_t*>(base + kOffHead);
-    R.pcount = reinterpret_cast<uint32_t*>(base + kOffCcount);
-    R.uroom = kNaPool / ncells;
-    R.ucells = R.uroom > kRange ? 1u : (R.uroom < kRange / 32u ? 32u : kRange / R.uroom);
-    R.cidx = reinterpret_cast<uint32_t*>(base + kOffIdx);
+    R.n = (uint32_t)n;
+    uint32_t* const count = reinterpret_cast<uint32_t*>(base + kOffCcount);
+    uint32_t* const first = reinterpret_cast<uint32_t*>(base + kOffFirst);
+    uint32_t* const rank = reinterpret_cast<uint32_t*>(base + kOffRank);
+    R.pcell = reinterpret_cast<uint4*>(base + kOffPcell);
+    R.rstart = reinterpret_cast<uint32_t*>(base + kOffRstart);
     R.cord = reinterpret_cast<uint32_t*>(base + kOffOrd);
     R.cword = reinterpret_cast<uint32_t*>(base + kOffWords) + 16;
     R.nanbu = reinterpret_cast<const float*>(base + kOffNanbu);
@@ -193,10 +219,15 @@ extern "C" ecris_status ecris_coulomb_collide_noalloc(size_t n, const uint32_t* 
     R.step = reinterpret_cast<uint32_t*>(base + kOffWords);
     R.tally = reinterpret_cast<unsigned long long*>(base + kOffTally);
 
-    k_na_init<<<(ncells + 255) / 256, 256, 0, s>>>(base, ncells, step);
-    e = cudaGetLastError();
-    if (e == cudaSuccess && n > 0)
-        e = launch_pdl(k_na_pack, dim3((uint32_t)((n + 255) / 256)), dim3(256), 0, s, R, (uint32_t)n, cell, q);
+    e = launch_pdl(k_na_init, dim3((ncells + 255) / 256), dim3(256), 0, s, base, ncells, step);
+    if (n > 0) {
+        const dim3 grid((uint32_t)((n + 255) / 256));
+        if (e == cudaSuccess) e = launch_pdl(k_na_count, grid, dim3(256), 0, s, R, cell, q, count, rank);
+        if (e == cudaSuccess)
+            e = launch_plan_exact(R, count, first, reinterpret_cast<unsigned long long*>(R.cword + 16), s);
+        if (e == cudaSuccess)
+            e = launch_pdl(k_na_pack, grid, dim3(256), 0, s, R, cell, q, (const uint32_t*)first, (const uint32_t*)rank);
+    }
     if (e != cudaSuccess) return na_cuda(e, "launch");
     e = launch_coulomb(R, (uint32_t)n, setup.grid, s);
     if (e != cudaSuccess) return na_cuda(e, "launch_coulomb");

@@ -149,11 +149,10 @@ struct alignas(16) RunDev {
     uint32_t *ccount;            // per cell without a plan: its participants (zero between steps)
     uint4 *cbkt;                 // per cell: its bucket (first record, room, planned place, 0); (kNoCell, 0, 0, 0):
                                  // not planned
-    uint4 *pcell;                // planned cells by place: (first record, room, cell, 0) (nullptr: every cell c has
-                                 // place c and uroom records from c uroom)
-    uint32_t *pcount;            // their participants (zero between steps)
+    uint4 *pcell;                // planned cells by place: (first record, room, cell, participants where pcount is
+                                 // nullptr)
+    uint32_t *pcount;            // their participants (zero between steps; nullptr: see pcell)
     uint32_t *rstart;            // first planned place of each range
-    uint32_t ucells, uroom;      // without a plan: cells a range and records a cell
     uint32_t *xcell;             // unplanned cells with participants this step
     uint32_t *cidx, *cord;       // scratch of cells too large for shared memory, one word a participant each
     uint32_t *cword;             // counters (kCw*)
@@ -555,6 +554,11 @@ void batch_snapshot_diag(const ecris_batch* b, int32_t run, const TallySnapshot&
 // batch).
 uint32_t plan_blocks(uint32_t ncells);
 cudaError_t launch_plan(const RunDev& R, uint32_t* count, bool zero, unsigned long long* blk, cudaStream_t s);
+// Exact buckets of the present counts alone, for one step: first[c] is cell c's
+// first record (kNoCell: fewer than two ions, nothing to collide); at most
+// R.cpool = 2 n records for n ions, R.cpool / 4 places; words: a zeroed 64-bit cursor
+cudaError_t launch_plan_exact(const RunDev& R, const uint32_t* count, uint32_t* first, unsigned long long* cursor,
+                              cudaStream_t s);
 int collide_blocks(int sm_count);    // most blocks of the collision kernel
 cudaError_t launch_coulomb(const RunDev& R, uint32_t n, int most, cudaStream_t s);
 cudaError_t launch_coulomb_batch(const RunDev* runs, uint32_t nruns, uint32_t n, int most, cudaStream_t s);
@@ -584,7 +588,7 @@ __device__ __forceinline__ void place_warp(const RunDev& R, uint32_t slot, uint3
     const uint32_t tl = after ? (uint32_t)(__ffs(after) - 2) : 31u;  // last lane of this lane's run
     const uint32_t h = 31u - (uint32_t)__clz(heads & upto);           // first lane of this lane's run
     uint4 bk = make_uint4(0u, 0u, 0u, 0u);
-    if (in) bk = R.cbkt ? R.cbkt[ck] : make_uint4(ck * R.uroom, R.uroom, ck, 0u);
+    if (in) bk = R.cbkt[ck];
     uint32_t k = 0u;
     if (in && lane == h) k = atomicAdd(bk.x == kNoCell ? R.ccount + ck : R.pcount + bk.z, tl - h + 1u);
     const Words w = rng_words(R, id, step, 1u);
