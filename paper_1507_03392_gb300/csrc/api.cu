@@ -292,6 +292,8 @@ struct KernelTimer {
 constexpr size_t kZeroBytes = (kTallyWords + kFptdWords) * sizeof(unsigned long long) + (8 + kCwWords) * sizeof(uint32_t);
 
 constexpr size_t kLoadAside = 1u << 19;   // particles of a load from the host that uses two streams
+// steps that a plan of the collisions' buckets is used for, where no sort makes a new one
+constexpr uint32_t kPlanEvery = 32;
 constexpr uint32_t kSortAfterLoad = 8;   // steps of one ecris_step call that sort a fresh load first
 
 struct ecris_ctx {
@@ -326,7 +328,8 @@ struct ecris_ctx {
     uint32_t* d_err = nullptr;
     // Coulomb collisions: see RunDev
     uint4* d_crec = nullptr;
-    uint32_t* d_cnext = nullptr;
+    uint2* d_cnext = nullptr;
+    uint4* d_cbig = nullptr;
     uint32_t* d_chead = nullptr;
     uint32_t* d_ccount = nullptr;
     uint4* d_cbkt = nullptr;
@@ -354,6 +357,7 @@ struct ecris_ctx {
     uint32_t* d_hblk = nullptr;    // scan block totals
     uint32_t sort_every = 32;      // steps between sorts
     uint32_t since_sort = 0;
+    uint32_t plan_steps = 0, last_plan = 0;   // steps since the load, and at the last plan of the collisions' buckets
     bool fresh = false;         // loaded, not yet sorted
     uint32_t calls_since_load = 0;
     unsigned long long* d_dep = nullptr;
@@ -456,6 +460,7 @@ void free_ions(ecris_ctx* ctx)
     free_async(ctx, ctx->d_q8);
     free_async(ctx, ctx->d_crec);
     free_async(ctx, ctx->d_cnext);
+    free_async(ctx, ctx->d_cbig);
     free_async(ctx, ctx->d_ccount);
     free_async(ctx, ctx->d_cbkt);
     free_async(ctx, ctx->d_pcell);
@@ -586,8 +591,10 @@ void fill_rundev(ecris_ctx* ctx, double dt, RunDev& R)
     R.dep = ctx->d_dep;
     R.tally = ctx->d_tally;
     R.crec = ctx->d_crec;
-    R.cpool = R.cover = (uint32_t)ctx->cap;
+    R.cpool = (uint32_t)ctx->cap;
+    R.cover = (uint32_t)ctx->cap + 32u;
     R.cnext = ctx->d_cnext;
+    R.cbig = ctx->d_cbig;
     R.chead = ctx->d_chead;
     R.ccount = ctx->d_ccount;
     R.cbkt = ctx->d_cbkt;
@@ -891,6 +898,7 @@ ecris_status sort_particles(ecris_ctx* ctx)
         ctx->fresh = false;
         return ECRIS_OK;
     }
+    ctx->last_plan = ctx->plan_steps;
     for (int k = 0; k < 6; ++k) std::swap(ctx->d_soa[k], ctx->d_soa2[k]);
     std::swap(ctx->d_meta, ctx->d_meta2);
     std::swap(ctx->d_id, ctx->d_id2);
@@ -903,6 +911,30 @@ ecris_status sort_particles(ecris_ctx* ctx)
     R.vz = ctx->d_soa[5];
     R.meta = ctx->d_meta;
     R.id = ctx->d_id;
+    return ECRIS_OK;
+}
+
+// Is a plan of the collisions' buckets due that no sort makes?  Ions without room in a
+// bucket collide all the same, but are found through their cells' chains; so a plan
+// is made anew every kPlanEvery steps (4e6 particles from atoms, dt 1e-7 s, a sort
+// every 512 steps: 1566 us a step with plans at sorts alone and a chain link an ion,
+// 222 so) and, where an
+// eighth of the atoms or more may ionise in that time, whenever the steps since the
+// load have grown by half (1e6 atoms on 16x16x32 cells, 1 % of them ionising a step:
+// 32 steps 4.0 ms without these, 2.9 at every doubling, 2.5 so).
+bool plan_due(const ecris_ctx* ctx)
+{
+    if (!(ctx->h.mcc.flags & kFCoulomb) || ctx->n4 == 0) return false;
+    const bool fast = ctx->h_run->atom_gate >= (1u << 24);   // (0: the device knows the gate)
+    return ctx->plan_steps - ctx->last_plan >= (fast ? std::min(std::max(ctx->last_plan / 2u, 2u), kPlanEvery) : kPlanEvery);
+}
+
+ecris_status plan_collisions(ecris_ctx* ctx)
+{
+    CK(timed(ctx, kKindOther, [&] {
+        return launch_replan(*ctx->h_run, (uint32_t)(4 * ctx->n4), ctx->d_hist, ctx->d_plan, ctx->stream);
+    }, 3));
+    ctx->last_plan = ctx->plan_steps;
     return ECRIS_OK;
 }
 
@@ -1211,8 +1243,10 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
         CK(cudaMallocAsync((void**)&ctx->d_birth, cap * sizeof(uint32_t), ctx->stream));
         if (h.mcc.flags & kFCoulomb) {
             const size_t cells = std::min(nc, cap);   // most cells with ions
-            CK(cudaMallocAsync((void**)&ctx->d_crec, 2 * cap * 2 * sizeof(uint4), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_cnext, cap * sizeof(uint32_t), ctx->stream));
+            // (list entries: the ions are padded to whole warps)
+            CK(cudaMallocAsync((void**)&ctx->d_crec, (2 * cap + 32) * 2 * sizeof(uint4), ctx->stream));
+            CK(cudaMallocAsync((void**)&ctx->d_cnext, (cap + 32) * sizeof(uint2), ctx->stream));
+            CK(cudaMallocAsync((void**)&ctx->d_cbig, (cap / kWarpIons + 1) * 2 * sizeof(uint4), ctx->stream));
             CK(cudaMallocAsync((void**)&ctx->d_ccount, (2 * nc + cells) * sizeof(uint32_t), ctx->stream));
             ctx->d_chead = ctx->d_ccount + nc;
             ctx->d_pcount = ctx->d_ccount + 2 * nc;
@@ -1315,6 +1349,7 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
     ctx->time_s = 0.0;
     ctx->dt_loaded = -1.0;
     ctx->since_fold = 0;
+    ctx->plan_steps = ctx->last_plan = 0;
     // a load leaves the particles in load order.  The first ecris_step call
     // after it groups them first only if it runs kSortAfterLoad or more
     // steps; a shorter first call (a load, a step and a read-back, say) steps
@@ -1353,6 +1388,10 @@ ecris_status ecris_step(ecris_ctx* ctx, uint32_t nsteps, double dt)
             st = sort_particles(ctx);
             if (st != ECRIS_OK) return st;
         }
+        if (plan_due(ctx)) {
+            st = plan_collisions(ctx);
+            if (st != ECRIS_OK) return st;
+        }
         // a window of steps (timed steps are windows of one)
         const uint32_t K = window_steps(ctx, nsteps - s, ctx->timer.on);
         const RunDev& R = *ctx->h_run;
@@ -1366,7 +1405,14 @@ ecris_status ecris_step(ecris_ctx* ctx, uint32_t nsteps, double dt)
         // (each kernel may start while the one before it ends; a graph a step lost
         // that between steps: 2e4 particles 25.6 us a step, 22.9 without)
         for (uint32_t k = 0; coulomb && k < K; ++k) {
-            if (k > 0) CK(launch_ions(R, ctx->sm_count, ctx->stream));
+            if (k > 0) {
+                if (plan_due(ctx)) {
+                    st = plan_collisions(ctx);
+                    if (st != ECRIS_OK) return st;
+                }
+                CK(launch_ions(R, ctx->sm_count, ctx->stream));
+            }
+            ++ctx->plan_steps;
             CK(timed(ctx, kKindCoulomb, [&] {
                 return launch_coulomb(R, (uint32_t)ctx->n, ctx->collide_grid, ctx->stream);
             }));
@@ -1974,13 +2020,15 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
         // work the batch stream then waits for; timed steps sort one by one)
         int nsort = 0;
         for (auto* c : b->runs) {
-            if (!c || c->n4 == 0 || c->since_sort < c->sort_every) continue;
+            if (!c || c->n4 == 0) continue;
+            const bool sort = c->since_sort >= c->sort_every;
+            if (!sort && !plan_due(c)) continue;
             ecris_status st = ECRIS_OK;
             if (b->timer.on) {
                 BCK(b->timer.run(kKindOther, b->stream, [&] {
-                    st = sort_particles(c);
+                    st = sort ? sort_particles(c) : plan_collisions(c);
                     return cudaSuccess;
-                }, c->fresh ? 4 : (c->d_plan ? 5 : 3)));
+                }, !sort ? 3 : c->fresh ? 4 : (c->d_plan ? 5 : 3)));
             } else {
                 const int k = nsort % kBatchSideStreams;
                 if (nsort == 0) {
@@ -1989,12 +2037,12 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
                 }
                 if (nsort < kBatchSideStreams) BCK(cudaStreamWaitEvent(b->side[k], b->sort_fork, 0));
                 c->stream = b->side[k];
-                st = sort_particles(c);
+                st = sort ? sort_particles(c) : plan_collisions(c);
                 c->stream = b->stream;
                 ++nsort;
             }
             if (st != ECRIS_OK) return bfail(b, st, "batch_step: " + c->err);
-            b->params_dirty = true;
+            if (sort) b->params_dirty = true;
         }
         for (int k = 0; k < nsort && k < kBatchSideStreams; ++k) {
             BCK(cudaEventRecord(b->sort_join[k], b->side[k]));
@@ -2013,6 +2061,14 @@ ecris_status ecris_batch_step(ecris_batch* b, uint32_t nsteps)
             return e;
         }));
         for (uint32_t k = 0; b->any_coulomb && k < K; ++k) {
+            for (auto* c : b->runs) {
+                if (!c) continue;
+                if (k > 0 && plan_due(c)) {
+                    const ecris_status st = plan_collisions(c);
+                    if (st != ECRIS_OK) return bfail(b, st, "batch_step: " + c->err);
+                }
+                ++c->plan_steps;
+            }
             if (k > 0) BCK(batch_ions(b));
             BCK(b->timer.run(kKindCoulomb, b->stream, [&] { return batch_coulomb(b); }));
         }

@@ -5,17 +5,18 @@
 // The ions' pass of a step leaves a 32-byte record of every ion that stayed
 // inside, (v, Q) and (array slot, its three words of the stream-1 Philox
 // block), in its cell's bucket (place_warp in step_kernel.cu):
-//   - buckets are planned at every load and layout sort from the cells' ion
-//     counts at that time: a cell of h ions
-//     gets room for h + h/8 + 4 (k_plan*), cells without ions none;
+//   - buckets are planned from the cells' ion counts at every load and layout
+//     sort, and in between where plan_due in api.cu says so: a cell of h ions gets
+//     room for h + h/8 + 4 (k_plan*), cells without ions none;
 //   - an ion that finds its cell's bucket full, or a cell without one, goes to
-//     the overflow part of the pool and is chained to its cell.
+//     the overflow part of the pool, where a warp's run of ions of one cell is
+//     chained to the cell as one link.
 // So a cell's records lie together without a count, a scan and a scatter in
 // every step.  Then k_collide orders each cell's ions by (first word, particle
 // id), which is independent of the order of arrival, pairs consecutive ones and
 // collides them; a cell with an odd count puts ranks 0, 1, 2 in a triplet that
 // collides (0,1), (1,2), (2,0) over dt/2 each:
-//   - a warp takes a range of planned cells (kRange records' room) or 32
+//   - a warp takes a range of planned cells (kRange records' room) or up to 32
 //     unplanned ones.  It sorts up to kWarpIons ions of several cells at once in
 //     registers, by cell, the first word's high 20 bits and the ion's place (a
 //     bitonic network over 32 lanes x 4); words that tie in those bits are put in
@@ -383,13 +384,14 @@ __device__ __forceinline__ uint32_t record_id(const RunDev& R, uint32_t p)
     return slot_id(R, R.crec[2 * (size_t)p + 1].x);
 }
 
-// a cell that takes a block: (first record, room, ions, chain)
+// a cell that takes a block: (first record, room, ions, where in cidx the records
+// past its bucket are, less the room)
 using BigCell = uint4;
 
-// the record of ion j of a cell (idx: those past its bucket)
-__device__ __forceinline__ uint32_t cell_record(const BigCell& b, const uint32_t* idx, uint32_t j)
+// the record of ion j of a cell
+__device__ __forceinline__ uint32_t cell_record(const RunDev& R, const BigCell& b, uint32_t j)
 {
-    return j < b.y ? b.x + j : idx[j];
+    return j < b.y ? b.x + j : R.cidx[b.w + j];
 }
 
 // Order and collide the ions of one cell by the block.  The words are uniform,
@@ -404,15 +406,7 @@ __device__ __forceinline__ void collide_cell(const RunDev& R, CellSmem& S, const
     __syncthreads();
     const uint32_t off = *s_off;
     if (off + M > R.cover) return;   // (the scratch holds every participant)
-    uint32_t* const idx = R.cidx + off;
     uint32_t* const ord = R.cord + off;
-    if (g == 0) {
-        uint32_t at = b.w;
-        for (uint32_t i = b.y; i < M; ++i) {
-            idx[i] = at ? at - 1u : R.cpool;   // (a chain holds as many as the count says)
-            if (at) at = R.cnext[at - 1u - R.cpool];
-        }
-    }
     unsigned long long width = (1ull << 32) / ((M + kBlockIons * 7u / 8u - 1u) / (kBlockIons * 7u / 8u)) + 1ull;
     if (M <= (uint32_t)kBlockIons) width = 1ull << 32;
     uint32_t done = 0u;
@@ -423,7 +417,7 @@ __device__ __forceinline__ void collide_cell(const RunDev& R, CellSmem& S, const
         for (uint32_t k = g; k < (uint32_t)kBlockIons / 2u + 1u; k += T) S.cnt2[k] = 0u;
         __syncthreads();
         for (uint32_t j = g; j < M; j += T) {
-            const uint32_t w = R.crec[2 * (size_t)cell_record(b, idx, j) + 1].y;
+            const uint32_t w = R.crec[2 * (size_t)cell_record(R, b, j) + 1].y;
             if (w < lo || w - lo >= width) continue;
             const uint32_t at = atomicAdd(&S.n, 1u);
             if (at < (uint32_t)kBlockIons) {
@@ -439,11 +433,11 @@ __device__ __forceinline__ void collide_cell(const RunDev& R, CellSmem& S, const
         }
         if (n > (uint32_t)kBlockIons) {   // one word for so many ions: in the order of their ids
             for (uint32_t j = g; j < M; j += T) {
-                const uint32_t p = cell_record(b, idx, j), id = record_id(R, p);
+                const uint32_t p = cell_record(R, b, j), id = record_id(R, p);
                 if (R.crec[2 * (size_t)p + 1].y != (uint32_t)lo) continue;
                 uint32_t r = 0u;
                 for (uint32_t i = 0; i < M; ++i) {
-                    const uint32_t pi = cell_record(b, idx, i);
+                    const uint32_t pi = cell_record(R, b, i);
                     if (R.crec[2 * (size_t)pi + 1].y == (uint32_t)lo && record_id(R, pi) < id) ++r;
                 }
                 ord[done + r] = p;
@@ -488,11 +482,11 @@ __device__ __forceinline__ void collide_cell(const RunDev& R, CellSmem& S, const
             uint32_t r = first;
             for (uint32_t t = first; t < end; ++t) {
                 const uint32_t i = S.arr[t], wi = S.word[i];
-                if (wi < w || (wi == w && i != j && record_id(R, cell_record(b, idx, S.rec[i])) <
-                                                        record_id(R, cell_record(b, idx, S.rec[j]))))
+                if (wi < w || (wi == w && i != j && record_id(R, cell_record(R, b, S.rec[i])) <
+                                                        record_id(R, cell_record(R, b, S.rec[j]))))
                     ++r;
             }
-            ord[done + r] = cell_record(b, idx, S.rec[j]);
+            ord[done + r] = cell_record(R, b, S.rec[j]);
         }
         done += n;
         lo += width;
@@ -508,48 +502,14 @@ __device__ __forceinline__ void collide_cell(const RunDev& R, CellSmem& S, const
 // collisions of a cell of m >= 2 ions
 __device__ __forceinline__ uint32_t collisions_of(uint32_t m) { return (m & 1u) ? 3u + (m - 3u) / 2u : m / 2u; }
 
-// A large cell by a warp alone, in global memory, should the block's list of them
-// be full: the rank by counting smaller (word, id)
-__device__ __forceinline__ void collide_warp_large(const RunDev& R, const BigCell& b)
-{
-    const uint32_t g = threadIdx.x & 31, m = b.z;
-    uint32_t off = 0u;
-    if (g == 0) off = atomicAdd(R.cword + kCwHuge, m);
-    off = __shfl_sync(0xFFFFFFFFu, off, 0);
-    if (off + m > R.cover) return;   // (the scratch holds every participant)
-    uint32_t* const idx = R.cidx + off;
-    uint32_t* const ord = R.cord + off;
-    if (g == 0) {
-        uint32_t at = b.w;
-        for (uint32_t i = b.y; i < m; ++i) {
-            idx[i] = at ? at - 1u : R.cpool;
-            if (at) at = R.cnext[at - 1u - R.cpool];
-        }
-    }
-    __syncwarp();
-    for (uint32_t j = g; j < m; j += 32u) {
-        const uint32_t p = cell_record(b, idx, j), w = R.crec[2 * (size_t)p + 1].y;
-        uint32_t r = 0u;
-        for (uint32_t i = 0; i < m; ++i) {
-            const uint32_t pi = cell_record(b, idx, i), wi = R.crec[2 * (size_t)pi + 1].y;
-            if (wi < w || (wi == w && i != j && record_id(R, pi) < record_id(R, p))) ++r;
-        }
-        ord[r] = p;
-    }
-    __syncwarp();
-    const uint32_t first = (m & 1u) ? 3u : 0u;
-    if (first && g == 0) collide_triplet(R, ord[0], ord[1], ord[2], (float)m);
-    for (uint32_t p = first + 2u * g; p < m; p += 64u) collide_pair(R, ord[p], ord[p + 1], (float)m);
-    __syncwarp();
-}
-
 // Shared memory of a warp: up to kWarpIons ions of up to 32 cells
 struct PackSmem {
     float4 v[kWarpIons];             // the ions' records, cell after cell
     uint4 w[kWarpIons];
     uint4 cell[32];                  // (first record - first place, places in the bucket end, first place, ions)
     uint32_t pidx[kWarpIons];        // where the records are in the pool
-    uint32_t list[kWarpIons];        // pairs; or the keys while ties are put in order
+    uint32_t list[kWarpIons];        // the cells' places in cidx (see BigCell), less the first place; then the
+                                     // keys while ties are put in order; then pairs
 };
 
 // or one cell of up to kWarpCell
@@ -565,15 +525,13 @@ union WarpSmem {
     RankSmem rank;
 };
 
-// what a block's warps put by for the block
-constexpr uint32_t kTrips = 128, kBigs = 32;
-struct Trip {
-    uint32_t a, b, c, m;
-    const RunDev* run;
-};
+// what a block's warps put by for the block: triplets (three records, the cell's
+// ions) and, in a list in R.cbig, large cells (big: the first + 1, 0: none)
+constexpr uint32_t kTrips = 128;
 struct WarpsSmem {
     WarpSmem warp[kCollideWarps];
-    Trip trip[kTrips];
+    uint32_t past[kCollideWarps][32];   // of a warp's item: see item_overflow
+    uint4 trip[kTrips];
 };
 union AnySmem {
     WarpsSmem w;
@@ -581,9 +539,7 @@ union AnySmem {
 };
 struct BlockSmem {
     AnySmem a;
-    BigCell big[kBigs];
-    const RunDev* big_run[kBigs];
-    uint32_t ntrip, nbig, off;
+    uint32_t ntrip, big, off;
 };
 
 // element exchange of the bitonic network: keep the smaller or the larger
@@ -645,7 +601,7 @@ __device__ __forceinline__ uint32_t collide_warp(const RunDev& R, PackSmem& S, B
             const uint32_t bf = word == 0u ? before[0] : word == 1u ? before[1] : word == 2u ? before[2] : before[3];
             q[k] = bf + (uint32_t)__popc(st & (0xFFFFFFFFu >> (31u - (j & 31u)))) - 1u;
             const uint4 c = S.cell[q[k]];
-            p[k] = j < c.y ? c.x + j : S.pidx[j];
+            p[k] = j < c.y ? c.x + j : R.cidx[S.list[q[k]] + j];
         }
 #pragma unroll
         for (int k = 0; k < 2; ++k) rec[k] = load_record(R, p[k]);
@@ -705,7 +661,7 @@ __device__ __forceinline__ uint32_t collide_warp(const RunDev& R, PackSmem& S, B
         if (kind == 2u) {
             const uint32_t ia = S.pidx[key[r] & 127u], ib = S.pidx[kb & 127u], ic = S.pidx[kc & 127u];
             const uint32_t at = atomicAdd(&B.ntrip, 1u);
-            if (at < kTrips) B.a.w.trip[at] = Trip{ia, ib, ic, m, &R};
+            if (at < kTrips) B.a.w.trip[at] = make_uint4(ia, ib, ic, m);
             else collide_triplet(R, ia, ib, ic, (float)m);
             S.w[key[r] & 127u].x = S.w[kb & 127u].x = S.w[kc & 127u].x = kNoCell;   // written back there
         }
@@ -734,10 +690,20 @@ __device__ __forceinline__ uint32_t collide_warp(const RunDev& R, PackSmem& S, B
     return np + 3u * nt;
 }
 
-// ranges and groups of 32 unplanned cells of a run
+// Unplanned cells an item (log2), of n of them: 32, or fewer while the grid has
+// warps to spare
+__device__ __forceinline__ uint32_t unplanned_lanes(uint32_t n)
+{
+    uint32_t lw = 0u;
+    while (lw < 5u && (n >> (lw + 1u)) >= gridDim.x * (uint32_t)kCollideWarps) ++lw;
+    return lw;
+}
+
+// ranges and groups of unplanned cells of a run
 __device__ __forceinline__ uint32_t collide_items(const RunDev& R)
 {
-    return R.cword[kCwRanges] + (R.cword[R.cword[kCwSet] + kCwUnplanned] + 31u) / 32u;
+    const uint32_t n = R.cword[kCwUnplanned + R.cword[kCwSet]], lw = unplanned_lanes(n);
+    return R.cword[kCwRanges] + ((n + (1u << lw) - 1u) >> lw);
 }
 
 // Order and collide one cell of kWarpIons to kWarpCell ions that all lie in its
@@ -805,7 +771,7 @@ __device__ __forceinline__ uint32_t collide_warp_cell(const RunDev& R, RankSmem&
     if (first && lane == 0) {
         const uint32_t ia = base + S.pos[0], ib = base + S.pos[1], ic = base + S.pos[2];
         const uint32_t at = atomicAdd(&B.ntrip, 1u);
-        if (at < kTrips) B.a.w.trip[at] = Trip{ia, ib, ic, M, &R};
+        if (at < kTrips) B.a.w.trip[at] = make_uint4(ia, ib, ic, M);
         else collide_triplet(R, ia, ib, ic, (float)M);
     }
     for (uint32_t e = lane; e < np; e += 32u)
@@ -837,8 +803,9 @@ __device__ __forceinline__ ItemCell item_cell(const RunDev& R, uint32_t item)
             if (R.pcount) count = R.pcount + k;
         }
     } else {
-        const uint32_t k = (item - nr) * 32u + lane;
-        if (k < R.cword[R.cword[kCwSet] + kCwUnplanned]) {
+        const uint32_t n = R.cword[kCwUnplanned + R.cword[kCwSet]], lw = unplanned_lanes(n);
+        const uint32_t k = ((item - nr) << lw) + lane;
+        if (!(lane >> lw) && k < n) {
             c = R.xcell[k];
             count = R.ccount + c;
         }
@@ -855,12 +822,40 @@ __device__ __forceinline__ ItemCell item_cell(const RunDev& R, uint32_t item)
     return ic;
 }
 
+// The records past the buckets of an item's cells, written to cidx: each lane walks
+// its cell's chain, all of them at once.  past: the lanes' places there less their
+// rooms.
+__device__ __forceinline__ void item_overflow(const RunDev& R, const ItemCell ic, uint32_t* past)
+{
+    const uint32_t lane = threadIdx.x & 31, n = ic.m > ic.room ? ic.m - ic.room : 0u;
+    uint32_t incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= (uint32_t)o) incl += t;
+    }
+    uint32_t first = 0u;
+    if (lane == 31u) first = atomicAdd(R.cword + kCwOverflow, incl);   // (all of a step's are at most cover)
+    first = __shfl_sync(0xFFFFFFFFu, first, 31) + incl - n;
+    uint32_t at = ic.head;
+    for (uint32_t i = 0; i < n && at;) {   // (a chain holds as many as the count says)
+        const uint32_t p = R.cpool + at - 1u;
+        const uint2 run = R.cnext[at - 1u];
+        for (uint32_t k = 0; k < run.y && i < n; ++k, ++i) R.cidx[first + i] = p + k;
+        at = run.x;
+    }
+    past[lane] = first - ic.room;
+    __syncwarp();
+}
+
 // One item of a run by a warp.  Returns the collisions.
 __device__ __forceinline__ uint32_t collide_item(const RunDev& R, WarpSmem& S, BlockSmem& B, const ItemCell& ic)
 {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t m = ic.m;
     uint32_t ncoll = 0u;
+    const uint32_t* const past = B.a.w.past[threadIdx.x >> 5];
+    if (__any_sync(0xFFFFFFFFu, m > ic.room)) item_overflow(R, ic, B.a.w.past[threadIdx.x >> 5]);
     uint32_t left = __ballot_sync(0xFFFFFFFFu, m > 0u);
     while (left) {
         // the next cells that fit together
@@ -881,38 +876,27 @@ __device__ __forceinline__ uint32_t collide_item(const RunDev& R, WarpSmem& S, B
                 ncoll += collide_warp_cell(R, S.rank, B, base, cm);
                 continue;
             }
-            const BigCell big = make_uint4(base, room, cm, __shfl_sync(0xFFFFFFFFu, ic.head, src));
-            uint32_t at = 0u;
-            if (lane == 0) at = atomicAdd(&B.nbig, 1u);
-            at = __shfl_sync(0xFFFFFFFFu, at, 0);
-            if (at < kBigs) {
-                if (lane == 0) {
-                    B.big[at] = big;
-                    B.big_run[at] = &R;
-                }
-            } else {   // no room for it (more than kBigs such cells in a few items): the warp does it
-                collide_warp_large(R, big);
-                ncoll += collisions_of(cm);
+            const BigCell big = make_uint4(base, room, cm, past[src]);
+            if (lane == 0) {
+                const uint32_t at = atomicAdd(R.cword + kCwBig, 1u);
+                R.cbig[2 * at] = big;
+                R.cbig[2 * at + 1].x = atomicExch(&B.big, at + 1u);
             }
             continue;
         }
         left &= ~take;
         const bool taken = (take >> lane) & 1u;
         const uint32_t seg = incl - m;
-        if (taken)
-            S.pack.cell[__popc(take & ((1u << lane) - 1u))] = make_uint4(ic.base - seg, seg + min(ic.room, m), seg, m);
+        if (taken) {
+            const uint32_t at = (uint32_t)__popc(take & ((1u << lane) - 1u));
+            S.pack.cell[at] = make_uint4(ic.base - seg, seg + min(ic.room, m), seg, m);
+            if (m > ic.room) S.pack.list[at] = past[lane] - seg;
+        }
         const uint32_t M = __shfl_sync(0xFFFFFFFFu, incl, 31 - __clz((int)take));
         uint32_t starts[4];
 #pragma unroll
         for (uint32_t r = 0; r < 4u; ++r)
             starts[r] = __reduce_or_sync(0xFFFFFFFFu, taken && (seg >> 5) == r ? 1u << (seg & 31u) : 0u);
-        if (taken && m > ic.room) {   // ions past the bucket: walk the chain
-            uint32_t at = ic.head;
-            for (uint32_t i = ic.room; i < m; ++i) {
-                S.pack.pidx[seg + i] = at ? at - 1u : R.cpool;   // (a chain holds as many as the count says)
-                if (at) at = R.cnext[at - 1u - R.cpool];
-            }
-        }
         __syncwarp();
         ncoll += collide_warp(R, S.pack, B, M, starts);
     }
@@ -927,19 +911,23 @@ __device__ __forceinline__ void collide_big(const RunDev& R, BlockSmem& B, const
 }
 
 // what the block's warps have put by (all threads call it, at the same point)
-__device__ __forceinline__ void collide_rest(BlockSmem& B)
+__device__ __forceinline__ void collide_rest(const RunDev& R, BlockSmem& B)
 {
     __syncthreads();
-    const uint32_t nt = min(B.ntrip, kTrips), nb = min(B.nbig, kBigs);
+    const uint32_t nt = min(B.ntrip, kTrips);
     static_assert(kTrips == 32 * kCollideWarps, "a triplet a thread");
     if (threadIdx.x < nt) {
-        const Trip t = B.a.w.trip[threadIdx.x];
-        collide_triplet(*t.run, t.a, t.b, t.c, (float)t.m);
+        const uint4 t = B.a.w.trip[threadIdx.x];
+        collide_triplet(R, t.x, t.y, t.z, (float)t.w);
     }
     __syncthreads();   // the list's memory is the large cells' too
-    for (uint32_t e = 0; e < nb; ++e) collide_big(*B.big_run[e], B, B.big[e]);
+    for (uint32_t e = B.big; e;) {
+        const BigCell b = R.cbig[2 * (e - 1u)];
+        e = R.cbig[2 * (e - 1u) + 1].x;
+        collide_big(R, B, b);
+    }
     __syncthreads();
-    if (threadIdx.x == 0) B.ntrip = B.nbig = 0u;
+    if (threadIdx.x == 0) B.ntrip = B.big = 0u;
     __syncthreads();
 }
 
@@ -949,9 +937,7 @@ __device__ __forceinline__ void collide_rest(BlockSmem& B)
 __device__ __forceinline__ void step_done(const RunDev& R)
 {
     *R.step += 1u;
-    uint32_t* const other = R.cword + (2u - R.cword[kCwSet]);
-    other[kCwUnplanned] = 0u;
-    other[kCwOverflow] = 0u;
+    R.cword[kCwUnplanned + (1u - R.cword[kCwSet])] = 0u;
     if (R.nleave && --R.nleave[2] == 0u) R.nleave[0] = R.nleave[1] = 0u;   // the window's list is done with
 }
 
@@ -1012,10 +998,10 @@ __device__ __forceinline__ void collide_share(const RunDev& R, BlockSmem& B, uin
         next = ItemCell{0u, 0u, 0u, 0u};
         if (v0 + stride + warp < end) next = item_cell(R, v0 + stride + warp);
         ncoll += collide_item(R, B.a.w.warp[warp], B, ic);
-        if (++n % kVisit == 0u) collide_rest(B);
+        if (++n % kVisit == 0u) collide_rest(R, B);
     }
     if ((threadIdx.x & 31u) == 0u && ncoll) atomicAdd(R.tally + kTallyCoulomb, (unsigned long long)ncoll);
-    collide_rest(B);
+    collide_rest(R, B);
 }
 
 __global__ void __launch_bounds__(32 * kCollideWarps, 8) k_collide(const __grid_constant__ RunDev R)
@@ -1023,7 +1009,7 @@ __global__ void __launch_bounds__(32 * kCollideWarps, 8) k_collide(const __grid_
     __shared__ BlockSmem B;
     pdl_wait();
     pdl_trigger();
-    if (threadIdx.x == 0) B.ntrip = B.nbig = 0u;
+    if (threadIdx.x == 0) B.ntrip = B.big = 0u;
     if (blockIdx.x == 0 && threadIdx.x == 32) step_done(R);
     __syncthreads();
     collide_share(R, B, blockIdx.x * kCollideWarps, collide_items(R), gridDim.x * kCollideWarps);
@@ -1041,7 +1027,7 @@ __global__ void __launch_bounds__(32 * kCollideWarps, 8) k_collide_batch(const R
     __shared__ uint32_t s_pref[kRunChunk + 1];
     pdl_wait();
     pdl_trigger();
-    if (threadIdx.x == 0) B.ntrip = B.nbig = 0u;
+    if (threadIdx.x == 0) B.ntrip = B.big = 0u;
     if (blockIdx.x == 0)
         for (uint32_t r = threadIdx.x; r < nruns; r += blockDim.x)
             if (runs[r].step && (runs[r].flags & kFCoulomb)) step_done(runs[r]);

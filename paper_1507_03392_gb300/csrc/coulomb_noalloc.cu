@@ -55,7 +55,8 @@ constexpr size_t kOffRank = kOffFirst + align256(sizeof(uint32_t) * kNaMaxCells)
 constexpr size_t kOffPcell = kOffRank + align256(sizeof(uint32_t) * kNaMaxIons);
 constexpr size_t kOffRstart = kOffPcell + align256(sizeof(uint4) * (kNaPool / 4));
 constexpr size_t kOffOrd = kOffRstart + align256(sizeof(uint32_t) * (kNaPool / kRange + 1));
-constexpr size_t kOffNanbu = kOffOrd + align256(sizeof(uint32_t) * kNaMaxIons);
+constexpr size_t kOffBig = kOffOrd + align256(sizeof(uint32_t) * kNaMaxIons);
+constexpr size_t kOffNanbu = kOffBig + align256(2 * sizeof(uint4) * (kNaMaxIons / kWarpIons + 1));
 constexpr size_t kOffWords = kOffNanbu + align256(sizeof(float) * kNanbuN);
 // words: step; from word 16 the collisions' counters; from word 32 the plan's cursor; then the tally block
 constexpr size_t kOffTally = kOffWords + 256;
@@ -82,9 +83,9 @@ __global__ void k_na_init(unsigned char* base, uint32_t ncells, uint32_t step)
     unsigned long long* tally = reinterpret_cast<unsigned long long*>(base + kOffTally);
     const uint32_t stride = gridDim.x * blockDim.x;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < ncells; i += stride) ccount[i] = 0u;
-    // (the collisions' counters: the set of this step)
+    // (the collisions' counters: this step's)
     if (blockIdx.x == 0 && threadIdx.x < 34)
-        words[threadIdx.x] = threadIdx.x == 0 ? step : (threadIdx.x == 16 + kCwSet ? 2u * (step & 1u) : 0u);
+        words[threadIdx.x] = threadIdx.x == 0 ? step : (threadIdx.x == 16 + kCwSet ? step & 1u : 0u);
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < (uint32_t)kTallyWords; i += stride) tally[i] = 0ull;
 }
 
@@ -212,6 +213,7 @@ extern "C" ecris_status ecris_coulomb_collide_noalloc(size_t n, const uint32_t* 
     R.pcell = reinterpret_cast<uint4*>(base + kOffPcell);
     R.rstart = reinterpret_cast<uint32_t*>(base + kOffRstart);
     R.cord = reinterpret_cast<uint32_t*>(base + kOffOrd);
+    R.cbig = reinterpret_cast<uint4*>(base + kOffBig);
     R.cword = reinterpret_cast<uint32_t*>(base + kOffWords) + 16;
     R.nanbu = reinterpret_cast<const float*>(base + kOffNanbu);
     R.nanbu_lnlo = (float)std::log(kNanbuSLo);

@@ -65,12 +65,12 @@ constexpr double kNanbuSLo = 1e-3;
 constexpr double kNanbuSHi = 6.0;
 
 // words of RunDev::cword: the plan's planned cells and ranges; which of the two
-// sets of a step's counters is in use (the ions' pass of a step sets it, the
-// collision kernel clears the other set for the next step); the scratch
-// entries; then the sets, each the step's unplanned cells and overflow records;
-// the ticket of the plan's kernels
-constexpr int kCwPlanned = 0, kCwRanges = 1, kCwSet = 2, kCwHuge = 3, kCwUnplanned = 4, kCwOverflow = 5, kCwTicket = 8,
-              kCwWords = 10;
+// counts of a step's unplanned cells is in use (the ions' pass of a step sets it,
+// the collision kernel clears the other one for the next step); the entries taken
+// of the scratch of large cells, of their list and of overflow records; then those
+// two counts; the ticket of the plan's kernels
+constexpr int kCwPlanned = 0, kCwRanges = 1, kCwSet = 2, kCwHuge = 3, kCwBig = 4, kCwOverflow = 5, kCwUnplanned = 6,
+              kCwTicket = 8, kCwWords = 10;
 // Coulomb collisions: room (records) a range of cells spans; ions of several
 // cells that a warp sorts in registers, of one cell that a warp ranks, and that a
 // block ranks at a time; warps a block
@@ -142,10 +142,11 @@ struct alignas(16) RunDev {
     unsigned long long *tally;   // kTallyWords
     uint4 *crec;                 // pool of 32-byte records of the step's Coulomb participants: (vx, vy, vz,
                                  // meta word as bits), (array slot, words 0, 1, 2 of the stream-1 Philox block); the
-                                 // first cpool are the cells' buckets, the next cover the overflow
+                                 // first cpool are the cells' buckets, the next cover the overflow, by list entry
     uint32_t cpool, cover;
-    uint32_t *cnext;             // per overflow record: the next of its cell's chain (record + 1, 0: none)
-    uint32_t *chead;             // per cell: its chain of overflow records (zero between steps)
+    uint2 *cnext;                // per run of overflow records of a cell, at its first: (next run of the cell's chain
+                                 // + 1, 0: none; records)
+    uint32_t *chead;             // per cell: its chain (zero between steps)
     uint32_t *ccount;            // per cell without a plan: its participants (zero between steps)
     uint4 *cbkt;                 // per cell: its bucket (first record, room, planned place, 0); (kNoCell, 0, 0, 0):
                                  // not planned
@@ -154,7 +155,9 @@ struct alignas(16) RunDev {
     uint32_t *pcount;            // their participants (zero between steps; nullptr: see pcell)
     uint32_t *rstart;            // first planned place of each range
     uint32_t *xcell;             // unplanned cells with participants this step
-    uint32_t *cidx, *cord;       // scratch of cells too large for shared memory, one word a participant each
+    uint32_t *cidx, *cord;       // scratch, one word a participant each: the overflow records of each cell, the ions
+                                 // in order of cells too large for shared memory
+    uint4 *cbig;                 // cells that take a block: (first record, room, ions, see BigCell), (next + 1, 0, 0, 0)
     uint32_t *cword;             // counters (kCw*)
     const float *nanbu;          // ln A at ln s = nanbu_lnlo + i / nanbu_inv_dln, i < kNanbuN
     float nanbu_lnlo, nanbu_inv_dln;
@@ -497,6 +500,8 @@ struct ParticleSet {
 // R, which then hold the sorted particles; NULL writes `dst` directly.
 cudaError_t launch_sort(const RunDev& R, uint32_t cap, const ParticleSet& dst, uint32_t* hist, uint32_t* off,
                         uint32_t* blk, unsigned long long* plan, uint4* aos, cudaStream_t s);
+// the collisions' buckets planned anew without a sort (hist as above)
+cudaError_t launch_replan(const RunDev& R, uint32_t cap, uint32_t* hist, unsigned long long* plan, cudaStream_t s);
 int sort_scan_blocks(uint32_t nbins);
 // state in load order: out[id[slot]] = state[slot] for id < n (positions to
 // metres), into device arrays; rec: scratch of n 32-byte records (not `out`),
@@ -571,11 +576,12 @@ __device__ __forceinline__ void store_record(uint4* rec, size_t d, const uint4& 
                  : "memory");
 }
 
-// Record this lane's Coulomb participant (ck != kNoCell) in its cell's bucket,
-// or in the overflow chained to the cell when the bucket is full; the whole warp
+// Record this lane's Coulomb participant (ck != kNoCell) in its cell's bucket or,
+// when that is full, at place e of the overflow (e: the warp's first plus the lane),
+// where the lanes of a cell are chained to it together; the whole warp
 // calls this.  One returning atomic per run of neighbouring lanes in the same
 // cell.
-__device__ __forceinline__ void place_warp(const RunDev& R, uint32_t slot, uint32_t ck, uint32_t id, uint32_t step,
+__device__ __forceinline__ void place_warp(const RunDev& R, uint32_t e, uint32_t slot, uint32_t ck, uint32_t id, uint32_t step,
                                            float vx, float vy, float vz, uint32_t meta)
 {
     const uint32_t lane = threadIdx.x & 31;
@@ -593,22 +599,22 @@ __device__ __forceinline__ void place_warp(const RunDev& R, uint32_t slot, uint3
     if (in && lane == h) k = atomicAdd(bk.x == kNoCell ? R.ccount + ck : R.pcount + bk.z, tl - h + 1u);
     const Words w = rng_words(R, id, step, 1u);
     k = __shfl_sync(0xFFFFFFFFu, k, h) + (lane - h);
-    uint32_t p = k < bk.y ? bk.x + k : kNoCell;
-    const uint32_t over = __ballot_sync(0xFFFFFFFFu, in && k >= bk.y);
-    if (over) {
+    const bool over = in && k >= bk.y;
+    const uint32_t om = __ballot_sync(0xFFFFFFFFu, over);
+    if (over && (lane == h || !((om >> (lane - 1u)) & 1u)))
+        R.cnext[e] = make_uint2(atomicExch(R.chead + ck, e + 1u), tl - lane + 1u);
+    // the first ion of a cell without a bucket lists it
+    const bool lists = over && bk.x == kNoCell && k == 0u;
+    const uint32_t lm = __ballot_sync(0xFFFFFFFFu, lists);
+    if (lm) {
         uint32_t o = 0u;
-        const uint32_t first = (uint32_t)(__ffs(over) - 1);
-        uint32_t* const words = R.cword + 2u * (step & 1u);   // the step's set of counters
-        if (lane == first) o = atomicAdd(words + kCwOverflow, (uint32_t)__popc(over));
-        o = __shfl_sync(0xFFFFFFFFu, o, first) + (uint32_t)__popc(over & (upto >> 1));
-        if (in && k >= bk.y && o < R.cover) {
-            p = R.cpool + o;
-            R.cnext[o] = atomicExch(R.chead + ck, p + 1u);
-            if (bk.x == kNoCell && k == 0u) R.xcell[atomicAdd(words + kCwUnplanned, 1u)] = ck;
-        }
+        const uint32_t first = (uint32_t)(__ffs(lm) - 1);
+        if (lane == first) o = atomicAdd(R.cword + kCwUnplanned + (step & 1u), (uint32_t)__popc(lm));
+        o = __shfl_sync(0xFFFFFFFFu, o, first) + (uint32_t)__popc(lm & (upto >> 1));
+        if (lists) R.xcell[o] = ck;
     }
-    if (in && p != kNoCell)
-        store_record(R.crec, p, make_uint4(__float_as_uint(vx), __float_as_uint(vy), __float_as_uint(vz), meta),
+    if (in)
+        store_record(R.crec, over ? R.cpool + e : bk.x + k, make_uint4(__float_as_uint(vx), __float_as_uint(vy), __float_as_uint(vz), meta),
                      make_uint4(slot, w.w0, w.w1, w.w2));
 }
 

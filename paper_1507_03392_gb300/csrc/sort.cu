@@ -49,7 +49,8 @@ __device__ __forceinline__ uint32_t sort_key(const RunDev& R, uint32_t i)
 }
 
 // lanes with equal keys add once per group (input already in order makes
-// whole warps share a key)
+// whole warps share a key); kIons: the ions alone
+template <bool kIons>
 __global__ void k_sort_count(const __grid_constant__ RunDev R, uint32_t cap, uint32_t* __restrict__ hist)
 {
     pdl_wait();
@@ -57,8 +58,9 @@ __global__ void k_sort_count(const __grid_constant__ RunDev R, uint32_t cap, uin
     const uint32_t stride = gridDim.x * blockDim.x;
     const uint32_t end = (cap + 31u) & ~31u;   // whole warps iterate together
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < end; i += stride) {
-        const bool in = i < cap;
-        const uint32_t key = in ? sort_key(R, i) : 0xFFFFFFFFu;
+        uint32_t key = i < cap ? sort_key(R, i) : 0xFFFFFFFFu;
+        if (kIons && key >= R.ncells) key = 0xFFFFFFFFu;
+        const bool in = key != 0xFFFFFFFFu;
         const uint32_t act = __ballot_sync(0xFFFFFFFFu, in);
         if (!in) continue;
         const uint32_t grp = __match_any_sync(act, key);
@@ -347,7 +349,7 @@ cudaError_t launch_sort(const RunDev& R, uint32_t cap, const ParticleSet& dst, u
 {
     const uint32_t nbins = 2u * R.ncells + 1u;
     const dim3 grid(grid_for(cap, 256, 8192)), block(256);
-    cudaError_t e = launch_pdl(k_sort_count, grid, block, 0, s, R, cap, hist);
+    cudaError_t e = launch_pdl(k_sort_count<false>, grid, block, 0, s, R, cap, hist);
     if (e == cudaSuccess)
         e = launch_pdl(k_sort_scan, dim3(sort_scan_blocks(nbins)), dim3(kSortThreads), 0, s, (const uint32_t*)hist, off,
                        blk, nbins, hist + nbins);
@@ -358,6 +360,12 @@ cudaError_t launch_sort(const RunDev& R, uint32_t cap, const ParticleSet& dst, u
     const ParticleSet src{R.x, R.y, R.z, R.vx, R.vy, R.vz, R.meta, R.id};
     if (e == cudaSuccess && aos) e = launch_pdl(k_sort_unpack, grid, block, 0, s, (const uint4*)aos, cap, src);
     return e;
+}
+
+cudaError_t launch_replan(const RunDev& R, uint32_t cap, uint32_t* hist, unsigned long long* plan, cudaStream_t s)
+{
+    const cudaError_t e = launch_pdl(k_sort_count<true>, dim3(grid_for(cap, 256, 8192)), dim3(256), 0, s, R, cap, hist);
+    return e == cudaSuccess ? launch_plan(R, hist, true, plan, s) : e;
 }
 
 cudaError_t launch_export_ordered(const RunDev& R, uint32_t n, uint32_t cap, float* const out[6], uint32_t* meta_out,
