@@ -592,7 +592,7 @@ void fill_rundev(ecris_ctx* ctx, double dt, RunDev& R)
     R.tally = ctx->d_tally;
     R.crec = ctx->d_crec;
     R.cpool = (uint32_t)ctx->cap;
-    R.cover = (uint32_t)ctx->cap + 32u;
+    R.cover = (uint32_t)ctx->cap + 32u;   // (list entries: the ions are padded to whole warps)
     R.cnext = ctx->d_cnext;
     R.cbig = ctx->d_cbig;
     R.chead = ctx->d_chead;
@@ -1243,7 +1243,6 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
         CK(cudaMallocAsync((void**)&ctx->d_birth, cap * sizeof(uint32_t), ctx->stream));
         if (h.mcc.flags & kFCoulomb) {
             const size_t cells = std::min(nc, cap);   // most cells with ions
-            // (list entries: the ions are padded to whole warps)
             CK(cudaMallocAsync((void**)&ctx->d_crec, (2 * cap + 32) * 2 * sizeof(uint4), ctx->stream));
             CK(cudaMallocAsync((void**)&ctx->d_cnext, (cap + 32) * sizeof(uint2), ctx->stream));
             CK(cudaMallocAsync((void**)&ctx->d_cbig, (cap / kWarpIons + 1) * 2 * sizeof(uint4), ctx->stream));

@@ -508,8 +508,7 @@ struct PackSmem {
     uint4 w[kWarpIons];
     uint4 cell[32];                  // (first record - first place, places in the bucket end, first place, ions)
     uint32_t pidx[kWarpIons];        // where the records are in the pool
-    uint32_t list[kWarpIons];        // the cells' places in cidx (see BigCell), less the first place; then the
-                                     // keys while ties are put in order; then pairs
+    uint32_t list[kWarpIons];        // pairs; or the keys while ties are put in order
 };
 
 // or one cell of up to kWarpCell
@@ -601,7 +600,7 @@ __device__ __forceinline__ uint32_t collide_warp(const RunDev& R, PackSmem& S, B
             const uint32_t bf = word == 0u ? before[0] : word == 1u ? before[1] : word == 2u ? before[2] : before[3];
             q[k] = bf + (uint32_t)__popc(st & (0xFFFFFFFFu >> (31u - (j & 31u)))) - 1u;
             const uint4 c = S.cell[q[k]];
-            p[k] = j < c.y ? c.x + j : R.cidx[S.list[q[k]] + j];
+            p[k] = j < c.y ? c.x + j : S.pidx[j];
         }
 #pragma unroll
         for (int k = 0; k < 2; ++k) rec[k] = load_record(R, p[k]);
@@ -690,19 +689,22 @@ __device__ __forceinline__ uint32_t collide_warp(const RunDev& R, PackSmem& S, B
     return np + 3u * nt;
 }
 
-// Unplanned cells an item (log2), of n of them: 32, or fewer while the grid has
-// warps to spare
-__device__ __forceinline__ uint32_t unplanned_lanes(uint32_t n)
+// Unplanned cells an item (log2), of n of them: 32, or fewer if they have so many
+// ions that a warp would take these in several turns.  (One a warp, as long as the
+// grid had warps, cost 6 runs at dt 1e-7 s 45.3 ms a 256 steps, and 41.2 so; 32
+// always, a run with 156 ions in each of its cells a multiple.)
+__device__ __forceinline__ uint32_t unplanned_lanes(const RunDev& R, uint32_t n)
 {
+    const unsigned long long ions = (unsigned long long)R.cword[kCwLoose + R.cword[kCwSet]] * kLooseEvery;
     uint32_t lw = 0u;
-    while (lw < 5u && (n >> (lw + 1u)) >= gridDim.x * (uint32_t)kCollideWarps) ++lw;
+    while (lw < 5u && (ions << (lw + 1u)) <= (unsigned long long)n * kWarpIons) ++lw;
     return lw;
 }
 
 // ranges and groups of unplanned cells of a run
 __device__ __forceinline__ uint32_t collide_items(const RunDev& R)
 {
-    const uint32_t n = R.cword[kCwUnplanned + R.cword[kCwSet]], lw = unplanned_lanes(n);
+    const uint32_t n = R.cword[kCwUnplanned + R.cword[kCwSet]], lw = unplanned_lanes(R, n);
     return R.cword[kCwRanges] + ((n + (1u << lw) - 1u) >> lw);
 }
 
@@ -803,7 +805,7 @@ __device__ __forceinline__ ItemCell item_cell(const RunDev& R, uint32_t item)
             if (R.pcount) count = R.pcount + k;
         }
     } else {
-        const uint32_t n = R.cword[kCwUnplanned + R.cword[kCwSet]], lw = unplanned_lanes(n);
+        const uint32_t n = R.cword[kCwUnplanned + R.cword[kCwSet]], lw = unplanned_lanes(R, n);
         const uint32_t k = ((item - nr) << lw) + lane;
         if (!(lane >> lw) && k < n) {
             c = R.xcell[k];
@@ -822,10 +824,13 @@ __device__ __forceinline__ ItemCell item_cell(const RunDev& R, uint32_t item)
     return ic;
 }
 
+// Records past a bucket from which an item's go through cidx
+constexpr uint32_t kFewPast = 16;
+
 // The records past the buckets of an item's cells, written to cidx: each lane walks
 // its cell's chain, all of them at once.  past: the lanes' places there less their
-// rooms.
-__device__ __forceinline__ void item_overflow(const RunDev& R, const ItemCell ic, uint32_t* past)
+// rooms.  (Out of line: its registers are not the others'.)
+__device__ __noinline__ void item_overflow(const RunDev& R, const ItemCell ic, uint32_t* past)
 {
     const uint32_t lane = threadIdx.x & 31, n = ic.m > ic.room ? ic.m - ic.room : 0u;
     uint32_t incl = n;
@@ -854,8 +859,11 @@ __device__ __forceinline__ uint32_t collide_item(const RunDev& R, WarpSmem& S, B
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t m = ic.m;
     uint32_t ncoll = 0u;
-    const uint32_t* const past = B.a.w.past[threadIdx.x >> 5];
-    if (__any_sync(0xFFFFFFFFu, m > ic.room)) item_overflow(R, ic, B.a.w.past[threadIdx.x >> 5]);
+    // (the few records past a bucket of a small cell are found as it is taken: 1.7e7
+    // particles in 12 runs, 32 steps, 12.7 ms with all of them through cidx, 12.3 so)
+    uint32_t* const past = B.a.w.past[threadIdx.x >> 5];
+    const bool many = __any_sync(0xFFFFFFFFu, m > ic.room && (m - ic.room > kFewPast || m > (uint32_t)kWarpIons));
+    if (many) item_overflow(R, ic, past);
     uint32_t left = __ballot_sync(0xFFFFFFFFu, m > 0u);
     while (left) {
         // the next cells that fit together
@@ -887,16 +895,23 @@ __device__ __forceinline__ uint32_t collide_item(const RunDev& R, WarpSmem& S, B
         left &= ~take;
         const bool taken = (take >> lane) & 1u;
         const uint32_t seg = incl - m;
-        if (taken) {
-            const uint32_t at = (uint32_t)__popc(take & ((1u << lane) - 1u));
-            S.pack.cell[at] = make_uint4(ic.base - seg, seg + min(ic.room, m), seg, m);
-            if (m > ic.room) S.pack.list[at] = past[lane] - seg;
-        }
+        if (taken)
+            S.pack.cell[__popc(take & ((1u << lane) - 1u))] = make_uint4(ic.base - seg, seg + min(ic.room, m), seg, m);
         const uint32_t M = __shfl_sync(0xFFFFFFFFu, incl, 31 - __clz((int)take));
         uint32_t starts[4];
 #pragma unroll
         for (uint32_t r = 0; r < 4u; ++r)
             starts[r] = __reduce_or_sync(0xFFFFFFFFu, taken && (seg >> 5) == r ? 1u << (seg & 31u) : 0u);
+        if (taken && m > ic.room) {   // the ions past the bucket
+            uint32_t at = ic.head, i = ic.room;
+            if (many)
+                for (; i < m; ++i) S.pack.pidx[seg + i] = R.cidx[past[lane] + i];
+            while (i < m && at) {   // (a chain holds as many as the count says)
+                const uint2 link = R.cnext[at - 1u];
+                for (uint32_t k = 0; k < link.y && i < m; ++k, ++i) S.pack.pidx[seg + i] = R.cpool + at - 1u + k;
+                at = link.x;
+            }
+        }
         __syncwarp();
         ncoll += collide_warp(R, S.pack, B, M, starts);
     }
@@ -937,7 +952,9 @@ __device__ __forceinline__ void collide_rest(const RunDev& R, BlockSmem& B)
 __device__ __forceinline__ void step_done(const RunDev& R)
 {
     *R.step += 1u;
-    R.cword[kCwUnplanned + (1u - R.cword[kCwSet])] = 0u;
+    const uint32_t other = 1u - R.cword[kCwSet];
+    R.cword[kCwUnplanned + other] = 0u;
+    R.cword[kCwLoose + other] = 0u;
     if (R.nleave && --R.nleave[2] == 0u) R.nleave[0] = R.nleave[1] = 0u;   // the window's list is done with
 }
 

@@ -65,12 +65,14 @@ constexpr double kNanbuSLo = 1e-3;
 constexpr double kNanbuSHi = 6.0;
 
 // words of RunDev::cword: the plan's planned cells and ranges; which of the two
-// counts of a step's unplanned cells is in use (the ions' pass of a step sets it,
-// the collision kernel clears the other one for the next step); the entries taken
-// of the scratch of large cells, of their list and of overflow records; then those
-// two counts; the ticket of the plan's kernels
+// sets of a step's counts is in use (the ions' pass of a step sets it, the
+// collision kernel clears the other set for the next step); the entries taken of
+// the scratch of large cells, of their list and of overflow records; then the
+// counts, two words each: the step's unplanned cells, and their ions in one warp of
+// kLooseEvery; the ticket of the plan's kernels
 constexpr int kCwPlanned = 0, kCwRanges = 1, kCwSet = 2, kCwHuge = 3, kCwBig = 4, kCwOverflow = 5, kCwUnplanned = 6,
-              kCwTicket = 8, kCwWords = 10;
+              kCwLoose = 8, kCwTicket = 10, kCwWords = 12;
+constexpr uint32_t kLooseEvery = 8;
 // Coulomb collisions: room (records) a range of cells spans; ions of several
 // cells that a warp sorts in registers, of one cell that a warp ranks, and that a
 // block ranks at a time; warps a block
@@ -144,8 +146,8 @@ struct alignas(16) RunDev {
                                  // meta word as bits), (array slot, words 0, 1, 2 of the stream-1 Philox block); the
                                  // first cpool are the cells' buckets, the next cover the overflow, by list entry
     uint32_t cpool, cover;
-    uint2 *cnext;                // per run of overflow records of a cell, at its first: (next run of the cell's chain
-                                 // + 1, 0: none; records)
+    uint2 *cnext;                // per link of overflow records in a row of one cell, at the first one's place: (place
+                                 // of the next link of the cell's chain + 1, 0: none; records)
     uint32_t *chead;             // per cell: its chain (zero between steps)
     uint32_t *ccount;            // per cell without a plan: its participants (zero between steps)
     uint4 *cbkt;                 // per cell: its bucket (first record, room, planned place, 0); (kNoCell, 0, 0, 0):
@@ -578,11 +580,11 @@ __device__ __forceinline__ void store_record(uint4* rec, size_t d, const uint4& 
 
 // Record this lane's Coulomb participant (ck != kNoCell) in its cell's bucket or,
 // when that is full, at place e of the overflow (e: the warp's first plus the lane),
-// where the lanes of a cell are chained to it together; the whole warp
+// chained to the cell; the whole warp
 // calls this.  One returning atomic per run of neighbouring lanes in the same
 // cell.
-__device__ __forceinline__ void place_warp(const RunDev& R, uint32_t e, uint32_t slot, uint32_t ck, uint32_t id, uint32_t step,
-                                           float vx, float vy, float vz, uint32_t meta)
+__device__ __forceinline__ void place_warp(const RunDev& R, uint32_t e, uint32_t slot, uint32_t ck, uint32_t id,
+                                           uint32_t step, float vx, float vy, float vz, uint32_t meta)
 {
     const uint32_t lane = threadIdx.x & 31;
     const bool in = ck != kNoCell;
@@ -600,21 +602,30 @@ __device__ __forceinline__ void place_warp(const RunDev& R, uint32_t e, uint32_t
     const Words w = rng_words(R, id, step, 1u);
     k = __shfl_sync(0xFFFFFFFFu, k, h) + (lane - h);
     const bool over = in && k >= bk.y;
+    uint32_t p = bk.x + k;
     const uint32_t om = __ballot_sync(0xFFFFFFFFu, over);
-    if (over && (lane == h || !((om >> (lane - 1u)) & 1u)))
-        R.cnext[e] = make_uint2(atomicExch(R.chead + ck, e + 1u), tl - lane + 1u);
-    // the first ion of a cell without a bucket lists it
-    const bool lists = over && bk.x == kNoCell && k == 0u;
-    const uint32_t lm = __ballot_sync(0xFFFFFFFFu, lists);
-    if (lm) {
-        uint32_t o = 0u;
-        const uint32_t first = (uint32_t)(__ffs(lm) - 1);
-        if (lane == first) o = atomicAdd(R.cword + kCwUnplanned + (step & 1u), (uint32_t)__popc(lm));
-        o = __shfl_sync(0xFFFFFFFFu, o, first) + (uint32_t)__popc(lm & (upto >> 1));
-        if (lists) R.xcell[o] = ck;
+    if (om) {
+        if (over) {   // the lanes of a cell are one link
+            p = R.cpool + e;
+            if (lane == h || !((om >> (lane - 1u)) & 1u))
+                R.cnext[e] = make_uint2(atomicExch(R.chead + ck, e + 1u), tl - lane + 1u);
+        }
+        const uint32_t loose = __ballot_sync(0xFFFFFFFFu, over && bk.x == kNoCell);
+        if (loose && lane == 0 && (e >> 5) % kLooseEvery == 0u)
+            atomicAdd(R.cword + kCwLoose + (step & 1u), (uint32_t)__popc(loose));
+        // the first ion of a cell without a bucket lists it
+        const bool lists = over && bk.x == kNoCell && k == 0u;
+        const uint32_t lm = __ballot_sync(0xFFFFFFFFu, lists);
+        if (lm) {
+            uint32_t o = 0u;
+            const uint32_t first = (uint32_t)(__ffs(lm) - 1);
+            if (lane == first) o = atomicAdd(R.cword + kCwUnplanned + (step & 1u), (uint32_t)__popc(lm));
+            o = __shfl_sync(0xFFFFFFFFu, o, first) + (uint32_t)__popc(lm & (upto >> 1));
+            if (lists) R.xcell[o] = ck;
+        }
     }
     if (in)
-        store_record(R.crec, over ? R.cpool + e : bk.x + k, make_uint4(__float_as_uint(vx), __float_as_uint(vy), __float_as_uint(vz), meta),
+        store_record(R.crec, p, make_uint4(__float_as_uint(vx), __float_as_uint(vy), __float_as_uint(vz), meta),
                      make_uint4(slot, w.w0, w.w1, w.w2));
 }
 
