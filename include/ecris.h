@@ -369,8 +369,10 @@ void ecris_batch_destroy(ecris_batch* b);
 /* message for the last failure on the batch (empty if none) */
 const char* ecris_batch_last_error(const ecris_batch* b);
 
-/* Device bytes a run of n particles on an nx x ny x nz mesh holds in a batch
- * (an upper estimate used for admission). */
+/* Device bytes a run of n particles on an nx x ny x nz mesh holds in a batch,
+ * used for admission: the sum of its arrays, an E grid and the longest on-axis
+ * table among them whether it has them or not (at most 16 bytes a cell and 1 MB
+ * more than it holds).  Probes are not counted. */
 size_t ecris_run_bytes(size_t n, int32_t nx, int32_t ny, int32_t nz, int coulomb);
 
 /* Add a run: the arguments of ecris_init_fields and ecris_load_ions plus its

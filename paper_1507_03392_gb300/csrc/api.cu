@@ -434,6 +434,56 @@ void free_async(ecris_ctx* ctx, T*& p)
     p = nullptr;
 }
 
+constexpr size_t kMaxAxial = 65537;   // samples of an on-axis table
+
+// slots of the arrays of n particles: arrays of a set start at 128-byte boundaries
+size_t capacity(size_t n) { return n > 0 ? (n + 31) / 32 * 32 : 32; }
+
+// The device arrays of a run, f(array, bytes) for each: those of its fields (E: an E
+// grid that is not all zero, nseg: the segments of its on-axis table) and those of its
+// particles.  What is allocated and what ecris_run_bytes charges.
+template <class F>
+void field_arrays(ecris_ctx* c, size_t nc, bool E, size_t nseg, F f)
+{
+    f((void**)&c->d_cell, nc * sizeof(float4));
+    if (E) f((void**)&c->d_E, nc * sizeof(float4));
+    f((void**)&c->d_kdt, kKdtWords * sizeof(float));
+    f((void**)&c->d_rlc, nc * sizeof(double));
+    if (nseg) f((void**)&c->d_btab, nseg * sizeof(float4));
+    f((void**)&c->d_nanbu, kNanbuN * sizeof(float));
+}
+
+template <class F>
+void ion_arrays(ecris_ctx* c, size_t cap, size_t nc, bool coulomb, F f)
+{
+    for (auto& set : c->d_set) f((void**)&set, 8 * cap * sizeof(uint32_t));
+    f((void**)&c->d_hist, (2 * nc + 2) * sizeof(uint32_t));
+    f((void**)&c->d_hoff, (2 * nc + 2) * sizeof(uint32_t));
+    f((void**)&c->d_hblk, (size_t)sort_scan_blocks((uint32_t)(2 * nc + 1)) * sizeof(uint32_t));
+    f((void**)&c->d_q8, cap);
+    f((void**)&c->d_dep, 4 * nc * sizeof(unsigned long long));   // deposit, count, charge, mark
+    f((void**)&c->d_ne64, nc * sizeof(double));
+    f((void**)&c->d_zero, kZeroBytes);
+    f((void**)&c->d_census, kQSlots * sizeof(unsigned long long));
+    f((void**)&c->d_leave, cap * sizeof(uint32_t));
+    f((void**)&c->d_birth, cap * sizeof(uint32_t));
+    if (!coulomb) return;
+    const size_t cells = std::min(nc, cap);   // most cells with ions
+    // (list entries of overflow records: the ions are padded to whole warps)
+    f((void**)&c->d_crec, (2 * cap + 32) * 2 * sizeof(uint4));
+    f((void**)&c->d_cnext, (cap + 32) * sizeof(uint2));
+    f((void**)&c->d_cbig, (cap / kWarpIons + 1) * 2 * sizeof(uint4));
+    f((void**)&c->d_ccount, (2 * nc + cells) * sizeof(uint32_t));   // with chead, pcount
+    f((void**)&c->d_cbkt, nc * sizeof(uint4));
+    f((void**)&c->d_pcell, cells * sizeof(uint4));
+    // the cells' room is at most 9/8 of the ions and 4 a cell
+    f((void**)&c->d_rstart, ((9 * cap / 8 + 4 * cells) / kRange + 3) * sizeof(uint32_t));
+    f((void**)&c->d_xcell, cells * sizeof(uint32_t));
+    f((void**)&c->d_cidx, cap * sizeof(uint32_t));
+    f((void**)&c->d_cord, cap * sizeof(uint32_t));
+    f((void**)&c->d_plan, plan_blocks((uint32_t)nc) * sizeof(unsigned long long));
+}
+
 // the load's stream; its last work was waited for by the context's own stream
 void free_load_stream(ecris_ctx* ctx)
 {
@@ -1024,7 +1074,7 @@ ecris_status ecris_init_fields(ecris_ctx* ctx, const ecris_geometry* geo, const 
             return fail(ctx, ECRIS_EINVAL, "init_fields: gas inlet must lie inside the chamber");
     }
     if (bf->n_axial != 0) {
-        if (bf->n_axial < 4 || bf->n_axial > 65537 || !bf->B_axial)
+        if (bf->n_axial < 4 || bf->n_axial > (int32_t)kMaxAxial || !bf->B_axial)
             return fail(ctx, ECRIS_EINVAL, "init_fields: the axial table needs 4 <= n_axial <= 65537 samples");
         for (int32_t k = 0; k < bf->n_axial; ++k)
             if (!(std::isfinite(bf->B_axial[k]) && bf->B_axial[k] >= 0.0))
@@ -1149,10 +1199,11 @@ ecris_status ecris_init_fields(ecris_ctx* ctx, const ecris_geometry* geo, const 
             if (ex != 0.0f || ey != 0.0f || ez != 0.0f) h.has_e = true;
         }
     }
-    CK(cudaMallocAsync((void**)&ctx->d_cell, nc * sizeof(float4), ctx->stream));
-    if (h.has_e) CK(cudaMallocAsync((void**)&ctx->d_E, nc * sizeof(float4), ctx->stream));
-    CK(cudaMallocAsync((void**)&ctx->d_kdt, kKdtWords * sizeof(float), ctx->stream));
-    CK(cudaMallocAsync((void**)&ctx->d_rlc, nc * sizeof(double), ctx->stream));
+    cudaError_t alloc = cudaSuccess;
+    field_arrays(ctx, nc, h.has_e, h.ax_y.empty() ? 0 : h.ax_y.size() - 1, [&](void** p, size_t bytes) {
+        if (alloc == cudaSuccess) alloc = cudaMallocAsync(p, bytes, ctx->stream);
+    });
+    CK(alloc);
     // R_L n_e per cell for the device's rebuild of delta, in the order the
     // host's records take it: 2.38e-6 sqrt(T_e) / (B dX)
     std::vector<double> rlc(nc);
@@ -1173,10 +1224,8 @@ ecris_status ecris_init_fields(ecris_ctx* ctx, const ecris_geometry* geo, const 
             btab[k] = make_float4((float)y0, (float)(y1 - y0 - hz * hz * (2.0 * m0 + m1) / 6.0),
                                   (float)(hz * hz * m0 / 2.0), (float)(hz * hz * (m1 - m0) / 6.0));
         }
-        CK(cudaMallocAsync((void**)&ctx->d_btab, nseg * sizeof(float4), ctx->stream));
         CK(cudaMemcpyAsync(ctx->d_btab, btab.data(), nseg * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream));
     }
-    CK(cudaMallocAsync((void**)&ctx->d_nanbu, kNanbuN * sizeof(float), ctx->stream));
     CK(cudaMemcpyAsync(ctx->d_nanbu, nanbu_table(), kNanbuN * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(ctx->d_cell, cell.data(), nc * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(ctx->d_rlc, rlc.data(), nc * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
@@ -1207,62 +1256,38 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
     }
     CK(cudaSetDevice(ctx->device));
     const size_t n4 = (n + 3) / 4;
-    const size_t cap = n4 > 0 ? (4 * n4 + 31) / 32 * 32 : 32;   // arrays of a set start at 128-byte boundaries
+    const size_t cap = capacity(n);
     const size_t nc = (size_t)h.nx * h.ny * h.nz;
     // device buffers are kept across loads while they are large enough
     if (!ctx->have_ions || cap > ctx->cap || nc != ctx->cap_cells) {
         free_ions(ctx);
+        cudaError_t alloc = cudaSuccess;
+        ion_arrays(ctx, cap, nc, (h.mcc.flags & kFCoulomb) != 0, [&](void** p, size_t bytes) {
+            if (alloc == cudaSuccess) alloc = cudaMallocAsync(p, bytes, ctx->stream);
+        });
+        CK(alloc);
         for (int set = 0; set < 2; ++set) {
-            CK(cudaMallocAsync((void**)&ctx->d_set[set], 8 * cap * sizeof(uint32_t), ctx->stream));
             for (int k = 0; k < 6; ++k)
                 (set ? ctx->d_soa2 : ctx->d_soa)[k] = reinterpret_cast<float*>(ctx->d_set[set] + k * cap);
             (set ? ctx->d_meta2 : ctx->d_meta) = ctx->d_set[set] + 6 * cap;
             (set ? ctx->d_id2 : ctx->d_id) = ctx->d_set[set] + 7 * cap;
         }
-        CK(cudaMallocAsync((void**)&ctx->d_hist, (2 * nc + 2) * sizeof(uint32_t), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_hoff, (2 * nc + 2) * sizeof(uint32_t), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_hblk, (size_t)sort_scan_blocks((uint32_t)(2 * nc + 1)) * sizeof(uint32_t),
-                           ctx->stream));
         CK(cudaMemsetAsync(ctx->d_hist, 0, (2 * nc + 2) * sizeof(uint32_t), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_q8, cap, ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_dep, 4 * nc * sizeof(unsigned long long), ctx->stream));
         ctx->d_count = ctx->d_dep + nc;
         ctx->d_charge = ctx->d_dep + 2 * nc;
         ctx->d_mark = ctx->d_dep + 3 * nc;
-        CK(cudaMallocAsync((void**)&ctx->d_ne64, nc * sizeof(double), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_zero, kZeroBytes, ctx->stream));
         ctx->d_tally = ctx->d_zero;
         ctx->d_fptd = ctx->d_zero + kTallyWords;
-        {
-            uint32_t* w = reinterpret_cast<uint32_t*>(ctx->d_fptd + kFptdWords);
-            ctx->d_step = w;
-            ctx->d_nleave = w + 1;
-            ctx->d_ticket = w + 4;
-            ctx->d_err = w + 5;
-            ctx->d_bad = w + 6;
-            ctx->d_cword = w + 8;
-        }
-        CK(cudaMallocAsync((void**)&ctx->d_census, kQSlots * sizeof(unsigned long long), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_leave, cap * sizeof(uint32_t), ctx->stream));
-        CK(cudaMallocAsync((void**)&ctx->d_birth, cap * sizeof(uint32_t), ctx->stream));
+        uint32_t* const words = reinterpret_cast<uint32_t*>(ctx->d_fptd + kFptdWords);
+        ctx->d_step = words;
+        ctx->d_nleave = words + 1;
+        ctx->d_ticket = words + 4;
+        ctx->d_err = words + 5;
+        ctx->d_bad = words + 6;
+        ctx->d_cword = words + 8;
         if (h.mcc.flags & kFCoulomb) {
-            const size_t cells = std::min(nc, cap);   // most cells with ions
-            CK(cudaMallocAsync((void**)&ctx->d_crec, (2 * cap + 32) * 2 * sizeof(uint4), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_cnext, (cap + 32) * sizeof(uint2), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_cbig, (cap / kWarpIons + 1) * 2 * sizeof(uint4), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_ccount, (2 * nc + cells) * sizeof(uint32_t), ctx->stream));
             ctx->d_chead = ctx->d_ccount + nc;
             ctx->d_pcount = ctx->d_ccount + 2 * nc;
-            CK(cudaMallocAsync((void**)&ctx->d_cbkt, nc * sizeof(uint4), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_pcell, cells * sizeof(uint4), ctx->stream));
-            // the cells' room is at most 9/8 of the ions and 4 a cell
-            CK(cudaMallocAsync((void**)&ctx->d_rstart, ((9 * cap / 8 + 4 * cells) / kRange + 3) * sizeof(uint32_t),
-                               ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_xcell, cells * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_cidx, cap * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_cord, cap * sizeof(uint32_t), ctx->stream));
-            CK(cudaMallocAsync((void**)&ctx->d_plan, plan_blocks((uint32_t)nc) * sizeof(unsigned long long),
-                               ctx->stream));
         }
         ctx->cap = cap;
         ctx->cap_cells = nc;
@@ -1846,16 +1871,13 @@ extern "C" {
 
 size_t ecris_run_bytes(size_t n, int32_t nx, int32_t ny, int32_t nz, int coulomb)
 {
-    const size_t cap = 4 * ((n + 3) / 4) + 4;
     const size_t nc = (size_t)(nx > 0 ? nx : 0) * (ny > 0 ? ny : 0) * (nz > 0 ? nz : 0);
-    // two particle sets with ids, the first sort's records (held while it
-    // runs), leaver list, births, load bytes, Coulomb lists
-    size_t per_p = 2 * 32 + 32 + 4 + 4 + 4 + 1;
-    if (coulomb) per_p += 16 + 16 + 8 + 16 + 4 + 4 + 1;
-    // cell records, E, deposit, time sums, sort histogram and scan, the n_e
-    // update's mark, scratch and R_L coefficients, Coulomb counts
-    size_t per_c = 16 + 16 + 8 + 8 + 8 + 4 + 4 + 8 + 8 + 8 + (coulomb ? 12 : 0);
-    return cap * per_p + nc * per_c + (1u << 20);
+    size_t bytes = 0;
+    const auto add = [&](void**, size_t b) { bytes += (b + 511) / 512 * 512; };   // (the allocator's granularity)
+    ecris_ctx c;
+    field_arrays(&c, nc, true, kMaxAxial - 1, add);
+    ion_arrays(&c, capacity(n), nc, coulomb != 0, add);
+    return bytes;
 }
 
 ecris_status ecris_batch_create(ecris_batch** out, int device, void* cuda_stream, size_t hbm_budget_bytes)
