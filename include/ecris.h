@@ -343,8 +343,9 @@ ecris_status ecris_get_profile(ecris_ctx* ctx, ecris_profile* out);
 typedef struct {
     int32_t sort_every;
     int32_t blocks_per_sm;  /* batches: resident blocks per SM of the step's passes (0: as many as fit) */
-    int32_t threads;        /* batches: their threads per block, 128, 256 or 512 (0: 256) */
-    int32_t particles_per_thread;   /* batches: particles per thread and tile of the atoms' pass, 1, 2 or 4
+    int32_t threads;        /* batches: with particles_per_thread the tile of the passes, 128, 256 or 512
+                               (0: 256); their blocks have at most 256 threads */
+    int32_t particles_per_thread;   /* batches: threads x this is the tile of the atoms' pass, 1, 2 or 4
                                (0: 2) */
     int32_t stages;         /* batches: 2, or 3 for 128 x 2, 256 x 1 and 256 x 2 (0: 3 for these, else 2);
                                no pass has stages, so 2 and 3 are the same */
@@ -411,11 +412,12 @@ ecris_status ecris_batch_memory(const ecris_batch* b, size_t* used, size_t* budg
 ecris_status ecris_batch_set_profiling(ecris_batch* b, int enable);
 ecris_status ecris_batch_get_profile(ecris_batch* b, ecris_profile* out);
 /* Launch-shape autotuner.  Times `trial_steps` steps of the batch (no sort
- * among them) in each launch shape of its passes -- threads per block 128, 256
- * or 512 times particles per thread 1, 2 or 4 -- with as many resident blocks as
- * fit; then, in the fastest shape, each count of resident
- * blocks per SM; then each sort cadence (8, 32, 128, 256, 512 steps), in whole sort
- * periods that each start with a sort.  Keeps the fastest of each and returns
+ * among them) in each launch shape of its passes -- 128 x 1, 2 or 4, 256 x 1, 2
+ * or 4 and 512 x 4 (512 x 1 and 512 x 2 launch what 256 x 2 and 256 x 4 do) --
+ * with as many resident blocks as fit; then, in the fastest shape, fewer resident
+ * blocks per SM, one at a time until they are a tenth slower; then each sort
+ * cadence (8, 32, 128, 256, 512 steps), in whole sort periods that each start
+ * with a sort.  Keeps the fastest of each and returns
  * the choice in *chosen (may be NULL).  Before the trials every run's state
  * (particles, tallies, deposit and time sums, first-passage records, step
  * counter) is copied aside in device memory, and it is restored afterwards:

@@ -2426,10 +2426,11 @@ ecris_status batch_autotune(ecris_batch* b, uint32_t trial_steps, bool cadence, 
         b->blocks_per_sm = bps;
         b->sort_every = every;
     };
-    // 1. the launch shape (threads per block x particles per thread: the first
-    // nine, the others differ from one of these in name only), as many resident
-    // blocks as fit, no sorts among the timed steps
-    for (int k = 0; k < 9 && st == ECRIS_OK; ++k) {
+    // 1. the launch shape (threads per block x particles per thread: seven of the
+    // twelve, the others launch the same blocks over the same tiles as one of these),
+    // as many resident blocks as fit, no sorts among the timed steps
+    for (int k = 0; k < kStepShapes && st == ECRIS_OK; ++k) {
+        if (shape_repeats(k)) continue;
         apply(k, 0, orig_sort);
         st = time_steps(b, trial_steps, true, &ms);
         if (st == ECRIS_OK && ms < best) {

@@ -514,9 +514,9 @@ cudaError_t launch_census(const RunDev& R, uint32_t n4, unsigned long long* cens
 // add the current particles to the probes' sums (probe.cu)
 cudaError_t launch_probe(const RunDev& R, const ProbeDev& P, uint32_t n4, int sm_count, cudaStream_t s);
 
-// Launch shapes of a batch's passes: threads per block x particles per thread
-// and tile of the atoms' pass.  (The stages of a shape belong to its name in
-// ecris_tuning; no kernel has stages.)
+// Launch shapes of a batch's passes by their names in ecris_tuning, threads per
+// block x particles per thread x stages: tiles of threads x particles of the atoms'
+// pass and of single steps, blocks of at most 256 threads; no kernel has stages.
 constexpr int kStepShapes = 12;
 constexpr int kDefaultShape = 11;
 constexpr int kShapeThreads[kStepShapes] = {128, 128, 128, 256, 256, 256, 512, 512, 512, 128, 256, 256};
@@ -524,6 +524,13 @@ constexpr int kShapeVec[kStepShapes] = {1, 2, 4, 1, 2, 4, 1, 2, 4, 2, 1, 2};
 constexpr int kShapeStages[kStepShapes] = {2, 2, 2, 2, 2, 2, 2, 2, 2, 3, 3, 3};
 inline int shape_block(int k) { return kShapeThreads[k] < 256 ? kShapeThreads[k] : 256; }   // threads of its blocks
 inline uint32_t shape_tile(int k) { return (uint32_t)(kShapeThreads[k] * kShapeVec[k]); }
+// does a shape before it launch the same?
+inline bool shape_repeats(int k)
+{
+    for (int j = 0; j < k; ++j)
+        if (shape_block(j) == shape_block(k) && shape_tile(j) == shape_tile(k)) return true;
+    return false;
+}
 // message returned by ecris_last_error(NULL) on the calling thread
 void ecris_internal_set_thread_error(const char* msg);
 // host: ln A(s) of Nanbu's scattering law on kNanbuN points uniform in ln s
