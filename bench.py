@@ -22,7 +22,6 @@ FP64 CPU oracle on the host cores instead (rank 0 only).
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import math
 import os
@@ -60,29 +59,6 @@ def measured_peaks():
         return float(d["hbm_gbs"]), "measured"
     except Exception:
         return 6800.0, "fallback"
-
-
-def kernel_source_hash():
-    h = hashlib.sha256()
-    for f in ("step_kernel.cu", "ecris_internal.cuh"):
-        with open(os.path.join(ROOT, "paper_1507_03392_gb300", "csrc", f), "rb") as fh:
-            h.update(fh.read())
-    return h.hexdigest()[:16]
-
-
-def ncu_traffic(n_particles, name="k_step_traffic.json"):
-    """DRAM bytes per launch of a step kernel from the committed ncu summary
-    (a capture on a smaller case, scaled by the particle count); None if the
-    kernel's sources changed since it was measured."""
-    path = os.path.join(ROOT, "profiles", name)
-    try:
-        with open(path) as f:
-            d = json.load(f)
-    except Exception:
-        return None
-    if d.get("source_sha") != kernel_source_hash():
-        return None
-    return d["dram_bytes_per_particle"] * n_particles
 
 
 class ClockSampler:
@@ -328,7 +304,6 @@ def bench_batched(E, I, args, local, stream, flush, peak, peak_kind):
     algo = total * ALGO_BYTES_STEP_KERNEL
     achieved = algo / (k_ms * 1e-3) / 1e9
     whole = value * ALGO_BYTES_STEP_KERNEL / 1e9
-    ktraffic = ncu_traffic(total, "k_step_batch_traffic.json")
     # the plain single-run form: the first runs of the scan, one at a time
     plain_ion_steps, plain_ms = 0, 0.0
     for wl, st in list(zip(wls, states))[: args.plain_runs]:
@@ -360,7 +335,7 @@ def bench_batched(E, I, args, local, stream, flush, peak, peak_kind):
         "tuning": tune,
         "roofline": {"bound": "hbm", "kernel": "k_one_batch", "achieved": achieved, "peak": peak,
                      "peak_source": peak_kind, "unit": "GB/s", "frac": achieved / peak,
-                     "algorithmic_bytes_per_launch": algo, "kernel_ms": k_ms, "traffic": ktraffic,
+                     "algorithmic_bytes_per_launch": algo, "kernel_ms": k_ms,
                      "kernel_ms_from": "a profiled pass (the step's kernels timed one by one, after "
                                        "the timed steps)",
                      "share_of_step": prof["step_ms"] / max(1e-9, prof["step_ms"] + prof["coulomb_ms"]
@@ -619,7 +594,7 @@ def main():
     whole = value * step_bytes / 1e9
     roofline = {"bound": "hbm", "kernel": "k_one", "achieved": achieved, "peak": peak,
                 "peak_source": peak_kind, "unit": "GB/s", "frac": achieved / peak,
-                "traffic": ncu_traffic(n), "algorithmic_bytes_per_launch": algo,
+                "algorithmic_bytes_per_launch": algo,
                 "kernel_ms": k_ms,
                 "kernel_ms_from": "a timed pass with per-kernel CUDA events after the timed steps",
                 "share_of_step": prof["step_ms"] / max(1e-9, prof["step_ms"] + prof["coulomb_ms"] + prof["other_ms"]),

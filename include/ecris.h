@@ -54,7 +54,7 @@ typedef enum {
     ECRIS_EINVAL = 1,   /* invalid argument; nothing was changed */
     ECRIS_ENOMEM = 2,   /* device or host allocation failed */
     ECRIS_ECUDA = 3,    /* a CUDA call failed; the message names it */
-    ECRIS_ETIMEOUT = 4, /* a bounded device wait ran out (no kernel waits at present) */
+    ECRIS_ETIMEOUT = 4, /* a bounded device wait ran out (no kernel waits: not returned at present) */
     ECRIS_ESTATE = 5    /* call out of order (e.g. step before load), or the
                            context is unusable after an earlier device error */
 } ecris_status;
@@ -323,12 +323,12 @@ ecris_status ecris_get_state(ecris_ctx* ctx, float* const xyzv[6], uint32_t* met
  * CUDA events; ecris_get_profile synchronises and reports, per kernel kind,
  * the number of launches and their summed device time since the last reset. */
 typedef struct {
-    int64_t step_launches;     /* push/MCC/boundary/deposit passes, counted once a step (the atoms' pass
-                                  and the pass over all other particles; timed steps are windows of one) */
+    int64_t step_launches;     /* push/MCC/boundary/deposit passes, one a step (timed steps are windows of
+                                  one, whose pass takes all particles in place) */
     double step_ms;
     int64_t coulomb_launches;  /* ion-ion collision kernels */
     double coulomb_ms;
-    int64_t other_launches;    /* sorts, deposit fold and bookkeeping kernels */
+    int64_t other_launches;    /* sorts, plans of the collisions' buckets, deposit folds */
     double other_ms;
 } ecris_profile;
 

@@ -288,8 +288,8 @@ struct KernelTimer {
 }  // namespace
 
 // the counters that a load clears: tallies, first-passage sums, and the words
-// step, nleave[3], ticket, err, bad[2], cword[kCwWords]
-constexpr size_t kZeroBytes = (kTallyWords + kFptdWords) * sizeof(unsigned long long) + (8 + kCwWords) * sizeof(uint32_t);
+// step, nleave[3], ticket, bad[2], cword[kCwWords]
+constexpr size_t kZeroBytes = (kTallyWords + kFptdWords) * sizeof(unsigned long long) + (7 + kCwWords) * sizeof(uint32_t);
 
 constexpr size_t kLoadAside = 1u << 19;   // particles of a load from the host that uses two streams
 // steps that a plan of the collisions' buckets is used for, where no sort makes a new one
@@ -325,7 +325,6 @@ struct ecris_ctx {
     // d_mark) and the collisions' counts (d_ccount, d_chead, d_pcount)
     unsigned long long* d_zero = nullptr;
     unsigned int* d_bad = nullptr;
-    uint32_t* d_err = nullptr;
     // Coulomb collisions: see RunDev
     uint4* d_crec = nullptr;
     uint2* d_cnext = nullptr;
@@ -659,7 +658,6 @@ void fill_rundev(ecris_ctx* ctx, double dt, RunDev& R)
     R.nanbu_lnlo = (float)std::log(kNanbuSLo);
     R.nanbu_inv_dln = (float)((kNanbuN - 1) / std::log(kNanbuSHi / kNanbuSLo));
     R.step = ctx->d_step;
-    R.err = ctx->d_err;
     R.leave = ctx->d_leave;
     R.birth = ctx->d_birth;
     R.fptd = ctx->d_fptd;
@@ -1282,9 +1280,8 @@ ecris_status ecris_load_ions(ecris_ctx* ctx, size_t n, const float* const xyzv[6
         ctx->d_step = words;
         ctx->d_nleave = words + 1;
         ctx->d_ticket = words + 4;
-        ctx->d_err = words + 5;
-        ctx->d_bad = words + 6;
-        ctx->d_cword = words + 8;
+        ctx->d_bad = words + 5;
+        ctx->d_cword = words + 7;
         if (h.mcc.flags & kFCoulomb) {
             ctx->d_chead = ctx->d_ccount + nc;
             ctx->d_pcount = ctx->d_ccount + 2 * nc;
@@ -1512,8 +1509,6 @@ ecris_status ecris_diag(ecris_ctx* ctx, ecris_diag_out* out)
     CK(cudaMemsetAsync(ctx->d_census, 0, kQSlots * sizeof(unsigned long long), ctx->stream));
     CK(launch_census(*ctx->h_run, (uint32_t)ctx->n4, ctx->d_census, ctx->stream));
     unsigned long long tally[kTallyWords], census[kQSlots];
-    uint32_t err = 0;
-    CK(cudaMemcpyAsync(&err, ctx->d_err, sizeof err, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaMemcpyAsync(tally, ctx->d_tally, sizeof tally, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaMemcpyAsync(census, ctx->d_census, sizeof census, cudaMemcpyDeviceToHost, ctx->stream));
     if (out->cell_count)
@@ -1521,10 +1516,6 @@ ecris_status ecris_diag(ecris_ctx* ctx, ecris_diag_out* out)
     if (out->cell_charge)
         CK(cudaMemcpyAsync(out->cell_charge, ctx->d_charge, nc * 8, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    if (err) {
-        ctx->failed = true;
-        return fail(ctx, ECRIS_ETIMEOUT, "diag: a kernel's bounded wait ran out; reload");
-    }
     fill_diag(h, ctx->weight, tally, census, ctx->steps_done, ctx->time_s, out);
     return ECRIS_OK;
 }
@@ -2280,8 +2271,8 @@ namespace {
 
 // Everything a step of a batch run changes, copied aside so that the
 // autotuner's trial steps can be undone: the current particle set, the
-// tallies, deposit and time sums, first-passage records, step counter and
-// error word on the device, and the host's step bookkeeping.
+// tallies, deposit and time sums, first-passage records and step counter on
+// the device, and the host's step bookkeeping.
 struct RunSnapshot {
     unsigned char* buf = nullptr;
     size_t bytes = 0;
@@ -2304,7 +2295,6 @@ void snapshot_parts(ecris_ctx* c, F f)
     f((void*)c->d_birth, cap * 4);
     f((void*)c->d_fptd, kFptdWords * sizeof(unsigned long long));
     f((void*)c->d_step, sizeof(uint32_t));
-    f((void*)c->d_err, sizeof(uint32_t));
 }
 
 ecris_status snapshot_take(ecris_batch* b, ecris_ctx* c, RunSnapshot& sn)
@@ -2537,7 +2527,6 @@ ecris_status batch_snapshot(ecris_batch* b, int32_t run, TallySnapshot* dst)
     if (!run_live(b, run)) return bfail(b, ECRIS_EINVAL, "batch_snapshot: no such run");
     const ecris_ctx* c = b->runs[run];
     BCK(cudaMemcpyAsync(dst->tally, c->d_tally, sizeof dst->tally, cudaMemcpyDeviceToHost, b->stream));
-    BCK(cudaMemcpyAsync(&dst->err, c->d_err, sizeof dst->err, cudaMemcpyDeviceToHost, b->stream));
     return ECRIS_OK;
 }
 

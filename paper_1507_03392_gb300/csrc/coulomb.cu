@@ -1034,7 +1034,7 @@ __global__ void __launch_bounds__(32 * kCollideWarps, 8) k_collide(const __grid_
 
 // Every run of a batch.  A block takes one stretch of the runs' items, so that
 // it has a run's parameter block in shared memory for many items, and reads
-// ahead as above (8e6 ions in 12 runs: 205 us with the items dealt out in turn
+// ahead as above (4.2e6 ions in 12 runs: 205 us with the items dealt out in turn
 // and the parameters read from global memory, 180 so).
 __global__ void __launch_bounds__(32 * kCollideWarps, 8) k_collide_batch(const RunDev* __restrict__ runs,
                                                                         uint32_t nruns)

@@ -168,7 +168,6 @@ struct alignas(16) RunDev {
                                  // back (of 4 n4 entries)
     uint32_t *nleave;            // [0], [1] their numbers (zero between windows), [2] with collisions between
                                  // ions, the steps left in the window
-    uint32_t *err;               // device error word (0; a kernel that gave up would leave its status)
     uint32_t *birth;             // by particle id: step of the last ionisation from Q = 0 (~0: unknown)
     unsigned long long *fptd;    // [Q][kFptdBins] extraction counts by age bin, [Q] summed ages (steps),
                                  // [Q] summed extraction radii (nm)
@@ -541,12 +540,11 @@ const float* nanbu_table();
 float coulomb_s_coef(double lnL_ii, double mass_amu, double weight, double cell_volume_m3);
 
 // Hooks of the served form (defined in api.cu, used by server.cu).  A tally
-// snapshot is a run's tally words and device error word, copied in stream
-// order into pinned host memory at a step boundary; the served loop reads it
-// a tick later, while the batch keeps stepping.
+// snapshot is a run's tally words, copied in stream order into pinned host
+// memory at a step boundary; the served loop reads it a tick later, while the
+// batch keeps stepping.
 struct TallySnapshot {
     unsigned long long tally[kTallyWords];
-    uint32_t err, pad;
 };
 // enqueue the copies of run `run`'s tallies into *dst (pinned) on the batch stream
 ecris_status batch_snapshot(ecris_batch* b, int32_t run, TallySnapshot* dst);

@@ -155,14 +155,12 @@ void give_slot(ecris_server* s, Served* v)
     v->ev = nullptr;
 }
 
-// the run's result at its latest snapshot (landed) into res; false on a
-// device error
-bool read_snapshot(ecris_server* s, Served* v, std::vector<int64_t>& ext, ecris_result& res)
+// the run's result at its latest snapshot (landed) into res
+void read_snapshot(ecris_server* s, Served* v, std::vector<int64_t>& ext, ecris_result& res)
 {
     const int q1 = v->req->r.sp.qmax + 1;
     ext.assign(q1, 0);
     std::vector<int64_t> lost(q1, 0);
-    if (v->snap->err) return false;
     ecris_diag_out d;
     std::memset(&d, 0, sizeof d);
     d.extracted = ext.data();
@@ -176,7 +174,6 @@ bool read_snapshot(ecris_server* s, Served* v, std::vector<int64_t>& ext, ecris_
         res.extracted[q] = ext[q];
         res.lost[q] = lost[q];
     }
-    return true;
 }
 
 // the convergence rule at a window boundary (currents into res)
@@ -399,7 +396,8 @@ void serve_loop(ecris_server* s)
                 std::lock_guard<std::mutex> lock(s->mu);
                 res = v->res;
             }
-            const bool ok_diag = landed && !v->ne_failed && read_snapshot(s, v, ext, res);
+            const bool ok_diag = landed && !v->ne_failed;
+            if (ok_diag) read_snapshot(s, v, ext, res);
             const bool conv = ok_diag && converged(v, ext, res);
             const bool cap = v->snap_steps >= r.max_steps;
             res.converged = conv ? 1 : 0;
@@ -425,7 +423,7 @@ void serve_loop(ecris_server* s)
             finish(s, v, rv.second,
                    rv.second == ECRIS_REQ_DONE ? nullptr
                    : v->ne_failed              ? "self-consistent n_e update failed"
-                                               : "device error word set (bounded wait ran out)");
+                                               : "the copy of its tallies failed");
             if (v->job) calib_advance(s, v, rv.second == ECRIS_REQ_DONE);
             v->req.reset();   // the host copy of the inputs is no longer needed
             s->active.erase(std::find(s->active.begin(), s->active.end(), v));

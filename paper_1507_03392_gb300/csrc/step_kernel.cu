@@ -1061,9 +1061,9 @@ __device__ __forceinline__ void active_tile(const RunDev& R, uint32_t t, uint32_
 // Resident blocks an SM that the passes over the lists are compiled for.  They
 // wait on gathers and long chains, so more warps hide more, until the spilled
 // registers cost more than that gives.  Times with 3/4/5 blocks of 256 threads
-// (or twice as many of 128), in us: k_ions, 2e6 ions 32.2/30.0/30.9; k_active,
+// (or twice as many of 128), in us: k_ions, 1.0e6 ions 32.2/30.0/30.9; k_active,
 // 1e4 particles x 32 steps 32.5/34.9/38.1, with variants 1e6 x 32 284/260/273;
-// k_active_batch, 7e6 ions x 32 2711/2744/2864; k_ions_batch, 8e6 ions
+// k_active_batch, 7e6 ions x 32 2711/2744/2864; k_ions_batch, 4.2e6 ions
 // 167/145/135.
 constexpr int kListBlocks = 8;   // the most, of kActiveTile threads
 constexpr int kActiveBatchBlocks = 3, kIonsBatchBlocks = 5;   // of 256
@@ -1516,7 +1516,8 @@ cudaError_t launch_quiet(const RunDev& R, uint32_t K, int sm_count, cudaStream_t
     return launch_pdl(k_quiet, dim3(std::max(1u, std::min(need, most))), dim3(128), 0, s, R, K, groups);
 }
 
-// as many blocks as the list could need, at most one wave
+// as many blocks as the list could need, at most kListBlocks an SM: one wave, but of
+// k_active<false> a third more than the six it holds at a time
 static dim3 list_grid(const RunDev& R, int sm_count)
 {
     return dim3(std::min(4u * R.n4 / kActiveTile + 2u, (uint32_t)(kListBlocks * sm_count)));
