@@ -468,9 +468,8 @@ void ion_arrays(ecris_ctx* c, size_t cap, size_t nc, bool coulomb, F f)
     f((void**)&c->d_birth, cap * sizeof(uint32_t));
     if (!coulomb) return;
     const size_t cells = std::min(nc, cap);   // most cells with ions
-    // (list entries of overflow records: the ions are padded to whole warps)
-    f((void**)&c->d_crec, (2 * cap + 32) * 2 * sizeof(uint4));
-    f((void**)&c->d_cnext, (cap + 32) * sizeof(uint2));
+    f((void**)&c->d_crec, 2 * cap * 2 * sizeof(uint4));
+    f((void**)&c->d_cnext, cap * sizeof(uint2));
     f((void**)&c->d_cbig, (cap / kWarpIons + 1) * 2 * sizeof(uint4));
     f((void**)&c->d_ccount, (2 * nc + cells) * sizeof(uint32_t));   // with chead, pcount
     f((void**)&c->d_cbkt, nc * sizeof(uint4));
@@ -640,8 +639,7 @@ void fill_rundev(ecris_ctx* ctx, double dt, RunDev& R)
     R.dep = ctx->d_dep;
     R.tally = ctx->d_tally;
     R.crec = ctx->d_crec;
-    R.cpool = (uint32_t)ctx->cap;
-    R.cover = (uint32_t)ctx->cap + 32u;   // (list entries: the ions are padded to whole warps)
+    R.cpool = R.cover = (uint32_t)ctx->cap;
     R.cnext = ctx->d_cnext;
     R.cbig = ctx->d_cbig;
     R.chead = ctx->d_chead;

@@ -824,12 +824,12 @@ __device__ __forceinline__ ItemCell item_cell(const RunDev& R, uint32_t item)
     return ic;
 }
 
-// Records past a bucket from which an item's go through cidx
-constexpr uint32_t kFewPast = 16;
+// does a cell that takes a block have records past its bucket?
+__device__ __forceinline__ bool past_large(const ItemCell& ic) { return ic.m > ic.room && ic.m > (uint32_t)kWarpIons; }
 
-// The records past the buckets of an item's cells, written to cidx: each lane walks
-// its cell's chain, all of them at once.  past: the lanes' places there less their
-// rooms.  (Out of line: its registers are not the others'.)
+// The records past the buckets of an item with such a cell, written to cidx: each
+// lane walks its cell's chain, all of them at once.  past: the lanes' places there
+// less their rooms.  (Out of line: its registers are not the others'.)
 __device__ __noinline__ void item_overflow(const RunDev& R, const ItemCell ic, uint32_t* past)
 {
     const uint32_t lane = threadIdx.x & 31, n = ic.m > ic.room ? ic.m - ic.room : 0u;
@@ -840,7 +840,7 @@ __device__ __noinline__ void item_overflow(const RunDev& R, const ItemCell ic, u
         if (lane >= (uint32_t)o) incl += t;
     }
     uint32_t first = 0u;
-    if (lane == 31u) first = atomicAdd(R.cword + kCwOverflow, incl);   // (all of a step's are at most cover)
+    if (lane == 31u) first = atomicAdd(R.cword + kCwPast, incl);   // (all of a step's are at most cover)
     first = __shfl_sync(0xFFFFFFFFu, first, 31) + incl - n;
     uint32_t at = ic.head;
     for (uint32_t i = 0; i < n && at;) {   // (a chain holds as many as the count says)
@@ -859,10 +859,10 @@ __device__ __forceinline__ uint32_t collide_item(const RunDev& R, WarpSmem& S, B
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t m = ic.m;
     uint32_t ncoll = 0u;
-    // (the few records past a bucket of a small cell are found as it is taken: 1.7e7
-    // particles in 12 runs, 32 steps, 12.7 ms with all of them through cidx, 12.3 so)
+    // (else the records past a cell's bucket are found as it is taken: 1.7e7 particles in
+    // 12 runs, 32 steps, 12.7 ms with all of them through cidx, 12.2 so)
     uint32_t* const past = B.a.w.past[threadIdx.x >> 5];
-    const bool many = __any_sync(0xFFFFFFFFu, m > ic.room && (m - ic.room > kFewPast || m > (uint32_t)kWarpIons));
+    const bool many = __any_sync(0xFFFFFFFFu, past_large(ic));
     if (many) item_overflow(R, ic, past);
     uint32_t left = __ballot_sync(0xFFFFFFFFu, m > 0u);
     while (left) {
@@ -955,6 +955,7 @@ __device__ __forceinline__ void step_done(const RunDev& R)
     const uint32_t other = 1u - R.cword[kCwSet];
     R.cword[kCwUnplanned + other] = 0u;
     R.cword[kCwLoose + other] = 0u;
+    R.cword[kCwOverflow + other] = 0u;
     if (R.nleave && --R.nleave[2] == 0u) R.nleave[0] = R.nleave[1] = 0u;   // the window's list is done with
 }
 

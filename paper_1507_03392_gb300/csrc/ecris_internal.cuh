@@ -68,10 +68,10 @@ constexpr double kNanbuSHi = 6.0;
 // sets of a step's counts is in use (the ions' pass of a step sets it, the
 // collision kernel clears the other set for the next step); the entries taken of
 // the scratch of large cells, of their list and of overflow records; then the
-// counts, two words each: the step's unplanned cells, and their ions in one warp of
-// kLooseEvery; the ticket of the plan's kernels
-constexpr int kCwPlanned = 0, kCwRanges = 1, kCwSet = 2, kCwHuge = 3, kCwBig = 4, kCwOverflow = 5, kCwUnplanned = 6,
-              kCwLoose = 8, kCwTicket = 10, kCwWords = 12;
+// counts, two words each: the step's unplanned cells, their ions in one warp of
+// kLooseEvery, and the overflow records; the ticket of the plan's kernels
+constexpr int kCwPlanned = 0, kCwRanges = 1, kCwSet = 2, kCwHuge = 3, kCwBig = 4, kCwPast = 5, kCwUnplanned = 6,
+              kCwLoose = 8, kCwOverflow = 10, kCwTicket = 12, kCwWords = 14;
 constexpr uint32_t kLooseEvery = 8;
 // Coulomb collisions: room (records) a range of cells spans; ions of several
 // cells that a warp sorts in registers, of one cell that a warp ranks, and that a
@@ -144,7 +144,7 @@ struct alignas(16) RunDev {
     unsigned long long *tally;   // kTallyWords
     uint4 *crec;                 // pool of 32-byte records of the step's Coulomb participants: (vx, vy, vz,
                                  // meta word as bits), (array slot, words 0, 1, 2 of the stream-1 Philox block); the
-                                 // first cpool are the cells' buckets, the next cover the overflow, by list entry
+                                 // first cpool are the cells' buckets, the next cover the overflow
     uint32_t cpool, cover;
     uint2 *cnext;                // per link of overflow records in a row of one cell, at the first one's place: (place
                                  // of the next link of the cell's chain + 1, 0: none; records)
@@ -584,12 +584,13 @@ __device__ __forceinline__ void store_record(uint4* rec, size_t d, const uint4& 
 }
 
 // Record this lane's Coulomb participant (ck != kNoCell) in its cell's bucket or,
-// when that is full, at place e of the overflow (e: the warp's first plus the lane),
-// chained to the cell; the whole warp
+// when that is full, in the overflow, chained to the cell (one record after the other:
+// at their slots' places each took a line of the cache to itself, and 6 served requests
+// 78 ms, 70 so); the whole warp
 // calls this.  One returning atomic per run of neighbouring lanes in the same
 // cell.
-__device__ __forceinline__ void place_warp(const RunDev& R, uint32_t e, uint32_t slot, uint32_t ck, uint32_t id,
-                                           uint32_t step, float vx, float vy, float vz, uint32_t meta)
+__device__ __forceinline__ void place_warp(const RunDev& R, uint32_t slot, uint32_t ck, uint32_t id, uint32_t step,
+                                           float vx, float vy, float vz, uint32_t meta)
 {
     const uint32_t lane = threadIdx.x & 31;
     const bool in = ck != kNoCell;
@@ -610,13 +611,16 @@ __device__ __forceinline__ void place_warp(const RunDev& R, uint32_t e, uint32_t
     uint32_t p = bk.x + k;
     const uint32_t om = __ballot_sync(0xFFFFFFFFu, over);
     if (om) {
+        uint32_t o = 0u;
+        if (lane == 0) o = atomicAdd(R.cword + kCwOverflow + (step & 1u), (uint32_t)__popc(om));
+        o = __shfl_sync(0xFFFFFFFFu, o, 0) + (uint32_t)__popc(om & (upto >> 1));
         if (over) {   // the lanes of a cell are one link
-            p = R.cpool + e;
+            p = R.cpool + o;
             if (lane == h || !((om >> (lane - 1u)) & 1u))
-                R.cnext[e] = make_uint2(atomicExch(R.chead + ck, e + 1u), tl - lane + 1u);
+                R.cnext[o] = make_uint2(atomicExch(R.chead + ck, o + 1u), tl - lane + 1u);
         }
         const uint32_t loose = __ballot_sync(0xFFFFFFFFu, over && bk.x == kNoCell);
-        if (loose && lane == 0 && (e >> 5) % kLooseEvery == 0u)
+        if (loose && lane == 0 && (slot >> 5) % kLooseEvery == 0u)
             atomicAdd(R.cword + kCwLoose + (step & 1u), (uint32_t)__popc(loose));
         // the first ion of a cell without a bucket lists it
         const bool lists = over && bk.x == kNoCell && k == 0u;

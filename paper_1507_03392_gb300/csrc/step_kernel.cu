@@ -1169,7 +1169,7 @@ __device__ __forceinline__ void ions_tile(const RunDev& R, uint32_t t, uint32_t 
         R.meta[i] = meta;
     }
     deposit_warp(R, dc, meta & kQMask);
-    place_warp(R, e, i, ck, id, step, vx, vy, vz, meta);
+    place_warp(R, i, ck, id, step, vx, vy, vz, meta);
 }
 
 // what the collision kernel of the step finds set (by one thread)
@@ -1178,7 +1178,7 @@ __device__ __forceinline__ void begin_collisions(const RunDev& R)
     R.cword[kCwSet] = *R.step & 1u;
     R.cword[kCwHuge] = 0u;
     R.cword[kCwBig] = 0u;
-    R.cword[kCwOverflow] = 0u;
+    R.cword[kCwPast] = 0u;
 }
 
 template <bool kVar>
@@ -1284,7 +1284,7 @@ __device__ __forceinline__ void one_group(const RunDev& R, uint32_t i, uint32_t 
         if (meta != was) R.meta[i] = meta;
     }
     deposit_warp(R, dc, meta & kQMask);
-    if (R.flags & kFCoulomb) place_warp(R, i, i, ck, id, step, vx, vy, vz, meta);
+    if (R.flags & kFCoulomb) place_warp(R, i, ck, id, step, vx, vy, vz, meta);
 }
 
 // what the collision kernel of a window of one step finds set (by one thread)
