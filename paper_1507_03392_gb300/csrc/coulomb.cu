@@ -56,36 +56,6 @@ constexpr uint32_t kPlanBlock = kPlanThreads * kPlanPer;
 // room of a cell of h ions
 __device__ __forceinline__ uint32_t bucket_room(uint32_t h) { return h ? h + (h >> 3) + 4u : 0u; }
 
-__device__ __forceinline__ unsigned long long warp_incl64(unsigned long long v)
-{
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long t = __shfl_up_sync(0xFFFFFFFFu, v, o);
-        if ((int)(threadIdx.x & 31) >= o) v += t;
-    }
-    return v;
-}
-
-// exclusive scan over the block of v; *total: the block's sum (kT threads)
-template <int kT>
-__device__ __forceinline__ unsigned long long block_excl64(unsigned long long v, unsigned long long* total)
-{
-    __shared__ unsigned long long ws[kT / 32 + 1];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned long long incl = warp_incl64(v);
-    if (lane == 31) ws[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const unsigned long long w = lane < kT / 32 ? ws[lane] : 0ull;
-        const unsigned long long wi = warp_incl64(w);
-        if (lane < kT / 32) ws[lane] = wi - w;
-        if (lane == kT / 32 - 1) ws[kT / 32] = wi;
-    }
-    __syncthreads();
-    *total = ws[kT / 32];
-    return ws[warp] + incl - v;
-}
-
 // (planned cells, room) of the blocks of kPlanBlock cells, packed (<< 32 |);
 // count: ions per cell.  The last block makes that the exclusive scan, and the
 // plan's words.
@@ -123,14 +93,6 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_sum(const __grid_constant
     }
 }
 
-// the ranges that start in or just after the room of planned place k
-__device__ __forceinline__ void mark_ranges(const RunDev& R, uint32_t k, uint32_t at, uint32_t room)
-{
-    for (uint32_t b = at / kRange + 1u; b * kRange < at + room; ++b) R.rstart[b] = k + 1u;
-    // a range that starts just where the next cell's room does
-    if ((at + room) % kRange == 0u) R.rstart[(at + room) / kRange] = k + 1u;
-}
-
 // every cell's bucket, the compact list of planned cells, and the ranges: range
 // b holds the planned cells whose room starts in [b kRange, (b + 1) kRange)
 __global__ void __launch_bounds__(kPlanThreads) k_plan_cells(const __grid_constant__ RunDev R,
@@ -162,56 +124,6 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_cells(const __grid_consta
         mark_ranges(R, k, at, room);
         o += (1ull << 32) + room;
     }
-}
-
-// Room of a cell of h ions whose bucket holds them for one step: at least 4, so
-// that a range has at most 32 cells; none where nothing collides.
-__device__ __forceinline__ uint32_t exact_room(uint32_t h) { return h < 2u ? 0u : max(h, 4u); }
-
-// The plan of a call's own counts.  Any order of the cells' buckets will do, so a
-// block takes the places and the records of its cells from one cursor (places << 32
-// | records) instead of a scan over the blocks; the last block sets the plan's words.
-// Two calls that share the working memory and overlap, which they must not, get
-// no bucket past the pool.
-__global__ void __launch_bounds__(kPlanThreads) k_plan_exact(const __grid_constant__ RunDev R, const uint32_t* count,
-                                                             uint32_t* first, unsigned long long* cursor)
-{
-    __shared__ unsigned long long s_start;
-    pdl_wait();
-    pdl_trigger();
-    const uint32_t base = blockIdx.x * kPlanBlock + threadIdx.x * kPlanPer;
-    uint32_t h[kPlanPer];
-    unsigned long long v = 0ull, total;
-#pragma unroll
-    for (int j = 0; j < kPlanPer; ++j) {
-        h[j] = base + j < R.ncells ? count[base + j] : 0u;
-        const uint32_t room = exact_room(h[j]);
-        v += ((unsigned long long)(room ? 1u : 0u) << 32) + room;
-    }
-    unsigned long long o = block_excl64<kPlanThreads>(v, &total);
-    if (threadIdx.x == 0) s_start = atomicAdd(cursor, total);
-    __syncthreads();
-    o += s_start;
-#pragma unroll
-    for (int j = 0; j < kPlanPer; ++j) {
-        const uint32_t c = base + j;
-        if (c >= R.ncells) break;
-        const uint32_t room = exact_room(h[j]), k = (uint32_t)(o >> 32), at = (uint32_t)o;
-        const bool in = room && at < R.cpool && room <= R.cpool - at;
-        first[c] = in ? at : kNoCell;
-        if (!in) continue;
-        R.pcell[k] = make_uint4(at, room, c, h[j]);
-        mark_ranges(R, k, at, room);
-        o += (1ull << 32) + room;
-    }
-    if (!last_block(R.cword + kCwTicket) || threadIdx.x != 0) return;
-    const unsigned long long end = __ldcg(cursor);
-    const uint32_t nr = min(((uint32_t)end + kRange - 1u) / kRange, R.cpool / kRange);
-    const uint32_t np = min((uint32_t)(end >> 32), R.cpool / 4u);
-    R.cword[kCwPlanned] = np;
-    R.cword[kCwRanges] = nr;
-    R.rstart[0] = 0u;
-    R.rstart[nr] = np;
 }
 
 // ---------------------------------------------------------------------------
@@ -1087,12 +999,6 @@ cudaError_t launch_plan(const RunDev& R, uint32_t* count, bool zero, unsigned lo
         e = launch_pdl(k_plan_cells, dim3(nb), dim3(kPlanThreads), 0, s, R, count, (const unsigned long long*)blk,
                        zero ? 1 : 0);
     return e;
-}
-
-cudaError_t launch_plan_exact(const RunDev& R, const uint32_t* count, uint32_t* first, unsigned long long* cursor,
-                              cudaStream_t s)
-{
-    return launch_pdl(k_plan_exact, dim3(plan_blocks(R.ncells)), dim3(kPlanThreads), 0, s, R, count, first, cursor);
 }
 
 int collide_blocks(int sm_count)

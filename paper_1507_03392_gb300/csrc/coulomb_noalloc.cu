@@ -24,7 +24,7 @@
 // the life of the process: a device reset (cudaDeviceReset) is not supported,
 // and the entry point must not be called on a device after one.
 // A call knows its ions only when it is made, so it counts them by cell, plans
-// exact buckets (k_plan_exact) and places the records; nothing overflows, however
+// exact buckets (k_na_plan) and places the records; nothing overflows, however
 // the ions are spread.  (A pool shared out evenly among the cells needs neither
 // count nor plan, two launches less, but its time hung on the spread: 65521 ions
 // evenly in 65536 cells took 23 us a call and in 4096 cells 37, 60000 ions in 400 of
@@ -73,11 +73,13 @@ struct DeviceSetup {
 std::mutex g_setup_mutex;
 DeviceSetup g_setup[64];
 
+constexpr int kNaThreads = 256;
+constexpr int kNaSmallThreads = 1024;
+constexpr int kNaPer = 8;               // cells a thread of the plan
+
 // clear the per-call counters and store the step index
-__global__ void k_na_init(unsigned char* base, uint32_t ncells, uint32_t step)
+__device__ __forceinline__ void na_clear(unsigned char* base, uint32_t ncells, uint32_t step)
 {
-    pdl_wait();
-    pdl_trigger();
     uint32_t* ccount = reinterpret_cast<uint32_t*>(base + kOffCcount);
     uint32_t* words = reinterpret_cast<uint32_t*>(base + kOffWords);
     unsigned long long* tally = reinterpret_cast<unsigned long long*>(base + kOffTally);
@@ -92,19 +94,17 @@ __global__ void k_na_init(unsigned char* base, uint32_t ncells, uint32_t step)
 // cell of particle i if it takes part (cell < ncells, 1 <= Q <= 63)
 __device__ __forceinline__ uint32_t na_cell(const RunDev& R, uint32_t i, const uint32_t* cell, const uint8_t* q)
 {
+    if (i >= R.n) return kNoCell;
     const uint32_t c = cell[i], Q = q[i];
     return c >= R.ncells || Q == 0u || Q > 63u ? kNoCell : c;
 }
 
 // count the participants by cell; rank: each one's arrival in its cell (one atomic per
-// group of lanes in the same cell; whole warps: n rounded up)
-__global__ void k_na_count(const __grid_constant__ RunDev R, const uint32_t* __restrict__ cell,
-                           const uint8_t* __restrict__ q, uint32_t* count, uint32_t* rank)
+// group of lanes in the same cell; the whole warp calls it)
+__device__ __forceinline__ void na_count(const RunDev& R, uint32_t i, const uint32_t* cell, const uint8_t* q,
+                                         uint32_t* count, uint32_t* rank)
 {
-    pdl_wait();
-    pdl_trigger();
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31u;
-    const uint32_t c = i < R.n ? na_cell(R, i, cell, q) : kNoCell;
+    const uint32_t lane = threadIdx.x & 31u, c = na_cell(R, i, cell, q);
     const uint32_t grp = __match_any_sync(0xFFFFFFFFu, c);
     const int leader = __ffs(grp) - 1;
     uint32_t k = 0u;
@@ -113,23 +113,133 @@ __global__ void k_na_count(const __grid_constant__ RunDev R, const uint32_t* __r
     if (i < R.n) rank[i] = k;
 }
 
-// record the participants in their cells' buckets, as the ions' pass does for ecris_step; slot and id are both
-// the array index
-__global__ void k_na_pack(const __grid_constant__ RunDev R, const uint32_t* __restrict__ cell,
-                          const uint8_t* __restrict__ q, const uint32_t* first, const uint32_t* rank)
+// Room of a cell of h ions whose bucket holds them for this step: at least 4, so
+// that a range has at most 32 cells; none where nothing collides.  So n ions take at most
+// 2 n records and n / 2 places.
+__device__ __forceinline__ uint32_t na_room(uint32_t h) { return h < 2u ? 0u : max(h, 4u); }
+
+// The plan: first[c] is cell c's first record (kNoCell: nothing to collide).  Any order
+// of the cells' buckets will do, so a block takes the places and the records of kT kNaPer
+// cells from one cursor (places << 32 | records) instead of a scan over the
+// blocks.  (Two calls that share the working memory and overlap, which they must not, get
+// no bucket past the pool.)
+template <int kT>
+__device__ __forceinline__ void na_plan(const RunDev& R, const uint32_t* count, uint32_t* first,
+                                        unsigned long long* cursor)
 {
-    pdl_wait();
-    pdl_trigger();
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= R.n) return;
+    __shared__ unsigned long long s_start;
+    const uint32_t base = (blockIdx.x * kT + threadIdx.x) * kNaPer;
+    uint32_t h[kNaPer];
+    unsigned long long v = 0ull, total;
+#pragma unroll
+    for (int j = 0; j < kNaPer; ++j) {
+        h[j] = base + j < R.ncells ? __ldcg(count + base + j) : 0u;
+        const uint32_t room = na_room(h[j]);
+        v += ((unsigned long long)(room ? 1u : 0u) << 32) + room;
+    }
+    unsigned long long o = block_excl64<kT>(v, &total);
+    if (threadIdx.x == 0) s_start = atomicAdd(cursor, total);
+    __syncthreads();
+    o += s_start;
+#pragma unroll
+    for (int j = 0; j < kNaPer; ++j) {
+        const uint32_t c = base + j;
+        if (c >= R.ncells) break;
+        const uint32_t room = na_room(h[j]), k = (uint32_t)(o >> 32), at = (uint32_t)o;
+        const bool in = room && at < R.cpool && room <= R.cpool - at;
+        first[c] = in ? at : kNoCell;
+        if (!in) continue;
+        R.pcell[k] = make_uint4(at, room, c, h[j]);
+        mark_ranges(R, k, at, room);
+        o += (1ull << 32) + room;
+    }
+}
+
+// its words, by one thread after all blocks
+__device__ __forceinline__ void na_plan_end(const RunDev& R, const unsigned long long* cursor)
+{
+    const unsigned long long end = __ldcg(cursor);
+    const uint32_t nr = min(((uint32_t)end + kRange - 1u) / kRange, R.cpool / kRange);
+    const uint32_t np = min((uint32_t)(end >> 32), R.cpool / 4u);
+    R.cword[kCwPlanned] = np;
+    R.cword[kCwRanges] = nr;
+    R.rstart[0] = 0u;
+    R.rstart[nr] = np;
+}
+
+// record a participant in its cell's bucket, as the ions' pass does for ecris_step; slot
+// and id are both the array index
+__device__ __forceinline__ void na_pack(const RunDev& R, uint32_t i, const uint32_t* cell, const uint8_t* q,
+                                        const uint32_t* first, const uint32_t* rank, uint32_t step)
+{
     const uint32_t c = na_cell(R, i, cell, q);
     if (c == kNoCell) return;
     const uint32_t at = first[c], k = rank[i];
     if (at == kNoCell || k >= R.cpool - at) return;   // (alone in its cell)
-    const Words w = rng_words(R, i, *R.step, 1u);
+    const Words w = rng_words(R, i, step, 1u);
     store_record(R.crec, at + k, make_uint4(__float_as_uint(R.vx[i]), __float_as_uint(R.vy[i]), __float_as_uint(R.vz[i]),
                                             (uint32_t)q[i]),
                  make_uint4(i, w.w0, w.w1, w.w2));
+}
+
+// what the passes before the collision kernel share
+struct Front {
+    unsigned char* base;
+    const uint32_t* cell;
+    const uint8_t* q;
+    uint32_t *count, *first, *rank;
+    unsigned long long* cursor;
+    uint32_t step;
+};
+
+__global__ void k_na_init(Front f, uint32_t ncells)
+{
+    pdl_wait();
+    pdl_trigger();
+    na_clear(f.base, ncells, f.step);
+}
+
+__global__ void k_na_count(const __grid_constant__ RunDev R, Front f)
+{
+    pdl_wait();
+    pdl_trigger();
+    na_count(R, blockIdx.x * blockDim.x + threadIdx.x, f.cell, f.q, f.count, f.rank);
+}
+
+__global__ void __launch_bounds__(kNaThreads) k_na_plan(const __grid_constant__ RunDev R, Front f)
+{
+    pdl_wait();
+    pdl_trigger();
+    na_plan<kNaThreads>(R, f.count, f.first, f.cursor);
+    if (last_block(R.cword + kCwTicket) && threadIdx.x == 0) na_plan_end(R, f.cursor);
+}
+
+__global__ void k_na_pack(const __grid_constant__ RunDev R, Front f)
+{
+    pdl_wait();
+    pdl_trigger();
+    na_pack(R, blockIdx.x * blockDim.x + threadIdx.x, f.cell, f.q, f.first, f.rank, f.step);
+}
+
+// All of it by one block, up to kNaSmallIons particles and as many cells as it plans in one
+// round: the four launches cost more there than their work.  us a call alone, with them and
+// so: 1001 particles in 4096 cells 67 and 63; 8001 70 and 74; 1001 in 32768 cells, four
+// rounds of the plan, 61 and 80.
+constexpr uint32_t kNaSmallIons = 4096, kNaSmallCells = kNaSmallThreads * kNaPer;
+__global__ void __launch_bounds__(kNaSmallThreads) k_na_small(const __grid_constant__ RunDev R, Front f)
+{
+    pdl_wait();
+    pdl_trigger();
+    const uint32_t end = (R.n + 31u) & ~31u;
+    na_clear(f.base, R.ncells, f.step);
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < end; i += kNaSmallThreads) na_count(R, i, f.cell, f.q, f.count, f.rank);
+    __syncthreads();
+    na_plan<kNaSmallThreads>(R, f.count, f.first, f.cursor);
+    __syncthreads();
+    if (threadIdx.x == 0) na_plan_end(R, f.cursor);
+    for (uint32_t i = threadIdx.x; i < end; i += kNaSmallThreads)
+        na_pack(R, i, f.cell, f.q, f.first, f.rank, f.step);
 }
 
 ecris_status na_fail(const std::string& msg)
@@ -207,9 +317,14 @@ extern "C" ecris_status ecris_coulomb_collide_noalloc(size_t n, const uint32_t* 
     R.cpool = kNaPool;
     R.cover = kNaMaxIons;
     R.n = (uint32_t)n;
-    uint32_t* const count = reinterpret_cast<uint32_t*>(base + kOffCcount);
-    uint32_t* const first = reinterpret_cast<uint32_t*>(base + kOffFirst);
-    uint32_t* const rank = reinterpret_cast<uint32_t*>(base + kOffRank);
+    Front f{};
+    f.base = base;
+    f.cell = cell;
+    f.q = q;
+    f.count = reinterpret_cast<uint32_t*>(base + kOffCcount);
+    f.first = reinterpret_cast<uint32_t*>(base + kOffFirst);
+    f.rank = reinterpret_cast<uint32_t*>(base + kOffRank);
+    f.step = step;
     R.pcell = reinterpret_cast<uint4*>(base + kOffPcell);
     R.rstart = reinterpret_cast<uint32_t*>(base + kOffRstart);
     R.cord = reinterpret_cast<uint32_t*>(base + kOffOrd);
@@ -221,14 +336,18 @@ extern "C" ecris_status ecris_coulomb_collide_noalloc(size_t n, const uint32_t* 
     R.step = reinterpret_cast<uint32_t*>(base + kOffWords);
     R.tally = reinterpret_cast<unsigned long long*>(base + kOffTally);
 
-    e = launch_pdl(k_na_init, dim3((ncells + 255) / 256), dim3(256), 0, s, base, ncells, step);
-    if (n > 0) {
-        const dim3 grid((uint32_t)((n + 255) / 256));
-        if (e == cudaSuccess) e = launch_pdl(k_na_count, grid, dim3(256), 0, s, R, cell, q, count, rank);
-        if (e == cudaSuccess)
-            e = launch_plan_exact(R, count, first, reinterpret_cast<unsigned long long*>(R.cword + 16), s);
-        if (e == cudaSuccess)
-            e = launch_pdl(k_na_pack, grid, dim3(256), 0, s, R, cell, q, (const uint32_t*)first, (const uint32_t*)rank);
+    f.cursor = reinterpret_cast<unsigned long long*>(R.cword + 16);
+    if (n <= kNaSmallIons && ncells <= kNaSmallCells) {
+        e = launch_pdl(k_na_small, dim3(1), dim3(kNaSmallThreads), 0, s, R, f);
+    } else {
+        const dim3 block(kNaThreads), grid((uint32_t)((n + kNaThreads - 1) / kNaThreads));
+        e = launch_pdl(k_na_init, dim3((ncells + kNaThreads - 1) / kNaThreads), block, 0, s, f, ncells);
+        if (n > 0) {
+            if (e == cudaSuccess) e = launch_pdl(k_na_count, grid, block, 0, s, R, f);
+            if (e == cudaSuccess)
+                e = launch_pdl(k_na_plan, dim3((ncells + kNaThreads * kNaPer - 1) / (kNaThreads * kNaPer)), block, 0, s, R, f);
+            if (e == cudaSuccess) e = launch_pdl(k_na_pack, grid, block, 0, s, R, f);
+        }
     }
     if (e != cudaSuccess) return na_cuda(e, "launch");
     e = launch_coulomb(R, (uint32_t)n, setup.grid, s);

@@ -566,14 +566,47 @@ void batch_snapshot_diag(const ecris_batch* b, int32_t run, const TallySnapshot&
 // batch).
 uint32_t plan_blocks(uint32_t ncells);
 cudaError_t launch_plan(const RunDev& R, uint32_t* count, bool zero, unsigned long long* blk, cudaStream_t s);
-// Exact buckets of the present counts alone, for one step: first[c] is cell c's
-// first record (kNoCell: fewer than two ions, nothing to collide); at most
-// R.cpool = 2 n records for n ions, R.cpool / 4 places; words: a zeroed 64-bit cursor
-cudaError_t launch_plan_exact(const RunDev& R, const uint32_t* count, uint32_t* first, unsigned long long* cursor,
-                              cudaStream_t s);
 int collide_blocks(int sm_count);    // most blocks of the collision kernel
 cudaError_t launch_coulomb(const RunDev& R, uint32_t n, int most, cudaStream_t s);
 cudaError_t launch_coulomb_batch(const RunDev* runs, uint32_t nruns, uint32_t n, int most, cudaStream_t s);
+
+__device__ __forceinline__ unsigned long long warp_incl64(unsigned long long v)
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(0xFFFFFFFFu, v, o);
+        if ((int)(threadIdx.x & 31) >= o) v += t;
+    }
+    return v;
+}
+
+// exclusive scan over the block of v; *total: the block's sum (kT threads)
+template <int kT>
+__device__ __forceinline__ unsigned long long block_excl64(unsigned long long v, unsigned long long* total)
+{
+    __shared__ unsigned long long ws[kT / 32 + 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned long long incl = warp_incl64(v);
+    if (lane == 31) ws[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned long long w = lane < kT / 32 ? ws[lane] : 0ull;
+        const unsigned long long wi = warp_incl64(w);
+        if (lane < kT / 32) ws[lane] = wi - w;
+        if (lane == kT / 32 - 1) ws[kT / 32] = wi;
+    }
+    __syncthreads();
+    *total = ws[kT / 32];
+    return ws[warp] + incl - v;
+}
+
+// the ranges that start in or just after the room of planned place k
+__device__ __forceinline__ void mark_ranges(const RunDev& R, uint32_t k, uint32_t at, uint32_t room)
+{
+    for (uint32_t b = at / kRange + 1u; b * kRange < at + room; ++b) R.rstart[b] = k + 1u;
+    // a range that starts just where the next cell's room does
+    if ((at + room) % kRange == 0u) R.rstart[(at + room) / kRange] = k + 1u;
+}
 
 // a 32-byte record in one store: one full sector, one request to L2
 __device__ __forceinline__ void store_record(uint4* rec, size_t d, const uint4& a, const uint4& b)

@@ -18,6 +18,10 @@ pytestmark = pytest.mark.gpu
     ((16, 16, 32), [2] * 900 + [1] * 900 + [3, 4, 5, 126, 127, 128, 129, 130, 255, 257, 511, 512, 513, 514]),
     ((16, 16, 32), [1791, 1792, 1793, 1990, 1991, 1992, 3600, 9001]),   # (a tenth of them atoms)
     ((16, 16, 32), [65_536]),
+    ((16, 16, 32), [64] * 64),                               # the most particles and cells that one block prepares
+    ((16, 16, 32), [64] * 64 + [1]),
+    ((16, 19, 27), [64] * 40 + [3] * 7),                     # more cells than that
+    ((4, 4, 4), [5]),
 ])
 def test_equal_to_ecris_step(mesh, sizes):
     from paper_1507_03392_gb300 import inputs as I
