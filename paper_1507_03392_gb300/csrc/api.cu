@@ -916,7 +916,7 @@ uint32_t window_steps(const ecris_ctx* ctx, uint32_t left, bool one_by_one)
     // (two steps are two windows of one: listing the particles that need their
     // steps one by one pays from three on; 4e6 particles 69.1 us a step in windows of
     // one, 77.9 of two, 60.8 of three, with collisions 118.3, 127.6 and 115.1; 32 runs of
-    // 2.6e7 in a batch 399, 418 and 338)
+    // 2.5e7 in a batch 399, 418 and 338)
     return K == 2 ? 1 : K;
 }
 

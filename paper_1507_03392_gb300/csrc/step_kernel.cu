@@ -1255,7 +1255,7 @@ __device__ __forceinline__ void one_group(const RunDev& R, uint32_t i, uint32_t 
             dc = ngp_cell(R, x, y, z);
         }
     }
-    // a warp of such atoms is done here, past no test of the others (32 runs of 2.6e7
+    // a warp of such atoms is done here, past no test of the others (32 runs of 2.5e7
     // particles in a batch 402 us a step, 385 so)
     if (__all_sync(0xFFFFFFFFu, quick)) {
         R.x[i] = x; R.y[i] = y; R.z[i] = z;
