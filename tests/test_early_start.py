@@ -11,8 +11,8 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1507_03392_gb300", "csrc")
 SOURCES = sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh")))
 # what no kernel writes (copies in stream order, which start after and end before every kernel): parameter blocks
-# and work list of a batch; the caller's arrays of the allocation-free step, which first launch waits for
-CONSTANT_PARAMETERS = {"runs", "items", "cell", "q"}
+# and work list of a batch
+CONSTANT_PARAMETERS = {"runs", "items"}
 # tables uploaded or rebuilt by copies and by kernels that let nothing start early
 CONSTANT_TABLES = ("R.cell", "R.kdt", "R.nanbu", "R.btab", "reinterpret_cast<const uint32_t*>(R.kdt)", "e")
 
